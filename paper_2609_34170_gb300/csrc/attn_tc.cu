@@ -78,17 +78,6 @@ struct AtMaps {
   CUtensorMap q, k, v, pk0, pk1, pv0, pv1;
 };
 
-// The idx-th chunk this CTA processes (prefix chunks past the valid prefix
-// length are skipped), or -1.
-__device__ __forceinline__ int chunk_at(const AtParams& p, int P, int c0, int c1, int idx) {
-  const int pre_end = min(min(c1, p.n_pre), (P + AT_BKV - 1) / AT_BKV);
-  const int npre = max(0, pre_end - c0);
-  if (idx < npre) return c0 + idx;
-  const int c = max(c0, p.n_pre) + (idx - npre);
-  return c < c1 ? c : -1;
-}
-
-
 __device__ __forceinline__ int chunk_count(const AtParams& p, int P, int c0, int c1) {
   int n = 0;
   for (int c = c0; c < c1; ++c)
@@ -213,7 +202,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   uint32_t* tmem_slot = (uint32_t*)(sdone + 1);
   int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] K issued, [2] K consumed, [3] V issued, [4] V consumed
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (through a shuffle, so that the compiler knows it is uniform in the warp)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int qt = blockIdx.x, bg = blockIdx.y, split = blockIdx.z;
   const int b = bg / p.Hkv, g = bg % p.Hkv;
   const int rows_per_robot = p.H + p.F;
@@ -238,7 +228,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   // the active context (slot, length and its prefix K/V) is fixed for the
   // whole step, so the first prefix chunks are fetched before the wait on the
   // previous kernel (the QKV projection)
-  int npre = 0, c_next = c0;
+  int npre = 0;
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -267,42 +257,59 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   if (p.xch == 2) cluster_sync();
   const CUtensorMap* pk = slot ? &maps.pk1 : &maps.pk0;
   const CUtensorMap* pv = slot ? &maps.pv1 : &maps.pv0;
-  // K and V of chunk c into stage s, each CTA loading its own copy (query
+  uint32_t el = 0;   // the issuing lane of warps 0 (TMA) and 1 (MMA)
+  const uint32_t q0 = smem_u32(q_s), k0 = smem_u32(kv_s), v0 = smem_u32(v_ring);
+  // K and V of chunk c into stage s (warp 0), each CTA loading its own copy (query
   // tiles of one (b, g) pair read the same chunk, which L2 serves to all)
   auto load_k = [&](int c, int s, uint64_t pol) {
-    uint8_t* ks = kv_s + (size_t)s * k_bytes;
-    mbar_expect_tx(&k_full[s], k_bytes);
+    const uint32_t ks = k0 + (uint32_t)s * k_bytes, bar = smem_u32(&k_full[s]);
+    mbar_expect_tx_el(&k_full[s], k_bytes, el);
     const bool pre = c < p.n_pre;
     const int cc = c - p.n_pre;
     const CUtensorMap* km = pre ? pk : &maps.k;
     const int ky = pre ? c * AT_BKV : g, kz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
-    for (int blk = 0; blk < p.nblk; ++blk) tma_load_3d(km, &k_full[s], ks + (size_t)blk * AT_KBLK, blk * 64, ky, kz, pol);
+    #pragma unroll 1
+    for (int blk = 0; blk < p.nblk; ++blk)
+      tma_load_3d_el(km, bar, ks + (uint32_t)blk * AT_KBLK, blk * 64, ky, kz, pol, el);
   };
   auto load_v = [&](int c, int s, uint64_t pol) {
-    uint8_t* vs = v_ring + (size_t)s * k_bytes;
-    mbar_expect_tx(&v_full[s], k_bytes);
+    const uint32_t vs = v0 + (uint32_t)s * k_bytes, bar = smem_u32(&v_full[s]);
+    mbar_expect_tx_el(&v_full[s], k_bytes, el);
     const bool pre = c < p.n_pre;
     const int cc = c - p.n_pre;
     const CUtensorMap* vm = pre ? pv : &maps.v;
     const int vy = pre ? c * AT_BKV : g, vz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
-    for (int blk = 0; blk < p.nblk; ++blk) tma_load_3d(vm, &v_full[s], vs + (size_t)blk * AT_KBLK, blk * 64, vy, vz, pol);
+    #pragma unroll 1
+    for (int blk = 0; blk < p.nblk; ++blk)
+      tma_load_3d_el(vm, bar, vs + (uint32_t)blk * AT_KBLK, blk * 64, vy, vz, pol, el);
   };
-  if (threadIdx.x == 0) {
-    uint64_t pol_kv;
+  // prefix chunk c into L2
+  auto warm = [&](int c) {
+    #pragma unroll 1
+    for (int blk = 0; blk < p.nblk; ++blk) {
+      prefetch_l2_3d_el(pk, blk * 64, c * AT_BKV, ctx_z, el);
+      prefetch_l2_3d_el(pv, blk * 64, c * AT_BKV, ctx_z, el);
+    }
+  };
+  // this CTA's chunks: prefix chunks c0 .. c0 + n_pre_here - 1 that hold keys, then
+  // the step's own chunks from c_own on
+  const int n_pre_here = max(0, min(min(c1, p.n_pre), (P + AT_BKV - 1) / AT_BKV) - c0);
+  const int c_own = max(c0, p.n_pre) - n_pre_here;
+  uint64_t pol_q = 0, pol_kv = 0;
+  if (warp == 0) {
+    __syncwarp();   // the barriers initialised above
+    el = elect_one();
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_q));
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_kv));
-    for (; c_next < c1 && c_next < p.n_pre && npre < min(SK, SV); ++c_next) {
-      if (c_next * AT_BKV >= P) continue;
-      load_k(c_next, npre, pol_kv);
-      load_v(c_next, npre, pol_kv);
-      ++npre;
+    npre = min(n_pre_here, min(SK, SV));
+    #pragma unroll 1
+    for (int i = 0; i < npre; ++i) {
+      load_k(c0 + i, i, pol_kv);
+      load_v(c0 + i, i, pol_kv);
     }
     // and warm L2 with the prefix chunks that will refill those stages
-    for (int k = 0; k < SK; ++k) {
-      const int c = chunk_at(p, P, c0, c1, npre + k);
-      if (c < 0 || c >= p.n_pre) break;
-      for (int blk = 0; blk < p.nblk; ++blk) prefetch_l2_3d(pk, blk * 64, c * AT_BKV, ctx_z);
-      prefetch_l2_3d(pv, c * AT_BKV, 0, ctx_z);
-    }
+    #pragma unroll 1
+    for (int i = npre; i < min(npre + SK, n_pre_here); ++i) warm(c0 + i);
   }
   // rows of the Q tile that no query fills are zeroed (their scores are unused)
   const int q_rows = p.TQ * p.G;
@@ -314,6 +321,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   pdl_wait();
+  if (warp == 0) {   // Q, before the TMEM set-up, which it does not need
+    mbar_expect_tx_el(q_full, (uint32_t)p.nblk * 128u * (uint32_t)q_rows, el);
+    #pragma unroll 1
+    for (int blk = 0; blk < p.nblk; ++blk)
+      tma_load_3d_el(&maps.q, smem_u32(q_full), q0 + (uint32_t)blk * AT_QBLK, blk * 64, g * p.G,
+                     b * rows_per_robot + qt * p.TQ, pol_q, el);
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(ncols)
@@ -327,43 +341,42 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   const uint32_t o_col = 128;
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint64_t pol_q, pol_kv;
-      asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_q));
-      asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_kv));
-      mbar_expect_tx(q_full, (uint32_t)p.nblk * 128u * (uint32_t)q_rows);
-      for (int blk = 0; blk < p.nblk; ++blk)
-        tma_load_3d(&maps.q, q_full, q_s + (size_t)blk * AT_QBLK, blk * 64, g * p.G, b * rows_per_robot + qt * p.TQ,
-                    pol_q);
-      // K of chunk nk and V of chunk nv (nv <= nk), each as soon as its slot
-      // is free; K may run ahead of V
-      int nk = npre, nv = npre;
-      unsigned long long t_last = globaltimer();
-      bool ok = true;
-      while (ok && (nk < n || nv < n)) {
-        bool progress = false;
-        if (nk < n && mbar_test_wait(&k_empty[nk % SK], ((uint32_t)(nk / SK) & 1u) ^ 1u)) {
-          const int c = chunk_at(p, P, c0, c1, nk);
-          load_k(c, nk % SK, c < p.n_pre ? pol_kv : pol_q);
-          {   // keep the L2 warm 2 SK chunks ahead of the loads (prefix chunks only)
-            const int cf = chunk_at(p, P, c0, c1, nk + 2 * SK);
-            if (cf >= 0 && cf < p.n_pre) {
-              for (int blk = 0; blk < p.nblk; ++blk) prefetch_l2_3d(pk, blk * 64, cf * AT_BKV, ctx_z);
-              prefetch_l2_3d(pv, cf * AT_BKV, 0, ctx_z);
-            }
-          }
-          ++nk;
-          progress = true;
+    // K of chunk nk and V of chunk nv (nv <= nk), each as soon as its slot
+    // is free; K may run ahead of V.  Ring positions: slot and the parity its
+    // `empty` wait takes (npre <= SK <= SV).
+    int nk = npre, nv = npre;
+    int sk = npre == SK ? 0 : npre, sv = npre == SV ? 0 : npre;
+    uint32_t phk = npre == SK ? 0u : 1u, phv = npre == SV ? 0u : 1u;
+    unsigned long long t_last = globaltimer();
+    bool ok = true;
+    while (ok && (nk < n || nv < n)) {
+      bool progress = false;
+      if (nk < n && mbar_test_warp(&k_empty[sk], phk)) {
+        const bool pre = nk < n_pre_here;
+        load_k(pre ? c0 + nk : c_own + nk, sk, pre ? pol_kv : pol_q);
+        // keep the L2 warm 2 SK chunks ahead of the loads (prefix chunks only)
+        if (nk + 2 * SK < n_pre_here) warm(c0 + nk + 2 * SK);
+        ++nk;
+        if (++sk == SK) {
+          sk = 0;
+          phk ^= 1u;
         }
-        if (nv < nk && mbar_test_wait(&v_empty[nv % SV], ((uint32_t)(nv / SV) & 1u) ^ 1u)) {
-          const int c = chunk_at(p, P, c0, c1, nv);
-          load_v(c, nv % SV, c < p.n_pre ? pol_kv : pol_q);
-          ++nv;
-          progress = true;
-        }
-        if (progress) t_last = globaltimer();
-        else if (globaltimer() - t_last > kTcTimeoutNs) ok = false;
+        progress = true;
       }
+      if (nv < nk && mbar_test_warp(&v_empty[sv], phv)) {
+        const bool pre = nv < n_pre_here;
+        load_v(pre ? c0 + nv : c_own + nv, sv, pre ? pol_kv : pol_q);
+        ++nv;
+        if (++sv == SV) {
+          sv = 0;
+          phv ^= 1u;
+        }
+        progress = true;
+      }
+      if (progress) t_last = globaltimer();
+      else ok = __all_sync(0xffffffffu, globaltimer() - t_last <= kTcTimeoutNs);
+    }
+    if (lane == 0) {
       if (!ok) flags[0] = 1;
       flags[1] = nk;
       flags[3] = nv;
@@ -373,70 +386,73 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     // exchange (the softmax warps arrive once their last PV is complete)
     if (p.xch == 1) cluster_arrive_release();
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc_s = idesc_bf16(AT_BM, AT_BKV);
-      const uint32_t idesc_o = idesc_bf16_bmn(AT_BM, p.hdp);
-      bool ok = mbar_wait(q_full, 0);
-      // Issue S of the next chunk and PV of the oldest chunk whose P is ready,
-      // whichever can go: PV(i) never waits for chunk i+1's K/V (that would
-      // chain every chunk's load behind the previous PV).  S runs at most one
-      // chunk ahead of PV (two S buffers in TMEM).
-      int ns = 0, i = 0;   // next S, next PV
-      bool sdone_sent = false;
-      // xch 2: every split learns when this split's last S has completed
-      // (its Q and K ring may then receive the partials of the merge)
-      const uint16_t smask = (uint16_t)((1u << p.splits) - 1u);
-      unsigned long long t_last = globaltimer();
-      while (ok && i < n) {
-        bool progress = false;
-        if (ns < n && ns <= i + 1) {
-          const int s = ns % SK;
-          if (mbar_test_wait(&k_full[s], (uint32_t)(ns / SK) & 1u) &&
-              (ns < 2 || mbar_test_wait(&s_free[ns & 1], (uint32_t)((ns >> 1) - 1) & 1u))) {
-            tc_fence_after();
-            const uint8_t* ks = kv_s + (size_t)s * k_bytes;
-            for (int blk = 0; blk < p.nblk; ++blk) {
-              const uint64_t ad = sw128_desc(smem_u32(q_s + (size_t)blk * AT_QBLK));
-              const uint64_t bd = sw128_desc(smem_u32(ks + (size_t)blk * AT_KBLK));
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                umma_bf16(tmem + (uint32_t)(ns & 1) * AT_BKV, ad + 2 * k, bd + 2 * k, idesc_s,
-                          (blk > 0 || k > 0) ? 1u : 0u);
-            }
-            umma_commit(&s_full[ns & 1]);
-            umma_commit(&k_empty[s]);   // K of this stage is free once S is done
-            ++ns;
-            if (p.xch == 2 && ns == n) {
-              umma_commit_mc(sdone, smask);
-              sdone_sent = true;
-            }
-            progress = true;
-          }
-        }
-        if (i < ns && mbar_test_wait(&p_full[i & 1], (uint32_t)(i >> 1) & 1u) &&
-            mbar_test_wait(&v_full[i % SV], (uint32_t)(i / SV) & 1u)) {
-          tc_fence_after();
-          const int s = i % SV;
-          // A = P from TMEM (the S tile's first 32 columns, two bf16 per column)
-          const uint32_t pa = tmem + (uint32_t)(i & 1) * AT_BKV;
-          // B = V [64 keys][hd], MN-major: 16 keys (two 8-row groups) per K step
-          const uint64_t bd = sw128_mn_desc(smem_u32(v_ring + (size_t)s * k_bytes), AT_KBLK);
+    el = elect_one();
+    const uint32_t idesc_s = idesc_bf16(AT_BM, AT_BKV);
+    const uint32_t idesc_o = idesc_bf16_bmn(AT_BM, p.hdp);
+    const uint64_t qd0 = sw128_desc(q0), kd0 = sw128_desc(k0), vd0 = sw128_mn_desc(v0, AT_KBLK);
+    bool ok = mbar_wait_warp(q_full, 0);
+    // Issue S of the next chunk and PV of the oldest chunk whose P is ready,
+    // whichever can go: PV(i) never waits for chunk i+1's K/V (that would
+    // chain every chunk's load behind the previous PV).  S runs at most one
+    // chunk ahead of PV (two S buffers in TMEM).
+    int ns = 0, i = 0;   // next S, next PV
+    int sk = 0, sv = 0;  // their ring slots, and the parities of their waits
+    uint32_t phk = 0, phv = 0;
+    bool sdone_sent = false;
+    // xch 2: every split learns when this split's last S has completed
+    // (its Q and K ring may then receive the partials of the merge)
+    const uint16_t smask = (uint16_t)((1u << p.splits) - 1u);
+    unsigned long long t_last = globaltimer();
+    while (ok && i < n) {
+      bool progress = false;
+      if (ns < n && ns <= i + 1 && mbar_test_warp(&k_full[sk], phk) &&
+          (ns < 2 || mbar_test_warp(&s_free[ns & 1], (uint32_t)((ns >> 1) - 1) & 1u))) {
+        tc_fence_after();
+        uint64_t ad = qd0, bd = kd0 + (uint32_t)sk * (k_bytes >> 4);
+        const uint32_t sd = tmem + (uint32_t)(ns & 1) * AT_BKV;
+        #pragma unroll 1
+        for (int blk = 0; blk < p.nblk; ++blk, ad += AT_QBLK >> 4, bd += AT_KBLK >> 4) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            umma_bf16_ts(tmem + o_col, pa + 8 * k, bd + 128 * k, idesc_o, (i > 0 || k > 0) ? 1u : 0u);
-          umma_commit(&v_empty[s]);
-          umma_commit(&pv_done[i & 1]);
-          ++i;
-          progress = true;
+            umma_bf16(sd, ad + 2 * k, bd + 2 * k, idesc_s, (blk > 0 || k > 0) ? 1u : 0u, el);
         }
-        if (progress) {
-          t_last = globaltimer();
-        } else if (globaltimer() - t_last > kTcTimeoutNs) {
-          ok = false;
+        umma_commit(&s_full[ns & 1], el);
+        umma_commit(&k_empty[sk], el);   // K of this stage is free once S is done
+        ++ns;
+        if (++sk == SK) {
+          sk = 0;
+          phk ^= 1u;
         }
+        if (p.xch == 2 && ns == n) {
+          umma_commit_mc(sdone, smask, el);
+          sdone_sent = true;
+        }
+        progress = true;
       }
-      // (no chunk, or an abort: arrive all the same, once earlier MMAs are done)
-      if (p.xch == 2 && !sdone_sent) umma_commit_mc(sdone, smask);
+      if (i < ns && mbar_test_warp(&p_full[i & 1], (uint32_t)(i >> 1) & 1u) && mbar_test_warp(&v_full[sv], phv)) {
+        tc_fence_after();
+        // A = P from TMEM (the S tile's first 32 columns, two bf16 per column)
+        const uint32_t pa = tmem + (uint32_t)(i & 1) * AT_BKV;
+        // B = V [64 keys][hd], MN-major: 16 keys (two 8-row groups) per K step
+        const uint64_t bd = vd0 + (uint32_t)sv * (k_bytes >> 4);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          umma_bf16_ts(tmem + o_col, pa + 8 * k, bd + 128 * k, idesc_o, (i > 0 || k > 0) ? 1u : 0u, el);
+        umma_commit(&v_empty[sv], el);
+        umma_commit(&pv_done[i & 1], el);
+        ++i;
+        if (++sv == SV) {
+          sv = 0;
+          phv ^= 1u;
+        }
+        progress = true;
+      }
+      if (progress) t_last = globaltimer();
+      else ok = __all_sync(0xffffffffu, globaltimer() - t_last <= kTcTimeoutNs);
+    }
+    // (no chunk, or an abort: arrive all the same, once earlier MMAs are done)
+    if (p.xch == 2 && !sdone_sent) umma_commit_mc(sdone, smask, el);
+    if (lane == 0) {
       if (!ok) flags[0] = 1;
       flags[2] = ns;   // chunks whose K arrival was consumed
       flags[4] = i;    // chunks whose V arrival was consumed

@@ -424,7 +424,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   uint32_t* tmem_slot = (uint32_t*)(rcv_bar + 1);
   int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] last split, [2] issued, [3] consumed
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (through a shuffle, so that the compiler knows it is uniform in the warp)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t ncols = (p.splits > 1) ? p.acc_cols : 2 * p.acc_cols;
   int tn0 = 0, tm0 = 0, sp0 = 0;
   const bool has_work = work_item(p, 0, tn0, tm0, sp0);
@@ -439,59 +440,81 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 
   pdl_trigger();
   uint64_t pol_w = 0, pol_x = 0;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+  uint32_t el = 0;   // the issuing lane of warps 0 (TMA) and 1 (MMA)
+  const uint32_t full0 = smem_u32(full), a0 = smem_u32(a_s), b0 = smem_u32(b_s);
+  if (warp == 0) {
+    el = elect_one();
+    if (el) {
+      for (int s = 0; s < S; ++s) {
+        mbar_init(&full[s], 1);
+        mbar_init(&empty[s], 1);
+      }
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&acc_full[b], 1);
+        mbar_init(&acc_empty[b], 128);
+      }
+      mbar_init(rcv_bar, 1);   // RED_DSMEM*: the partials' arrival; otherwise armed by nobody
+      flags[0] = flags[1] = flags[2] = flags[3] = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      // the slices of all splits (this one's included): 128 rows x cpr tokens each
+      if constexpr (DSM) mbar_expect_tx(rcv_bar, (uint32_t)(BN * TC_BM * (RED == RED_DSMEM ? 2 : 4)));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      // Weights never depend on earlier kernels: stream the first stages' weight
+      // tiles while the previous kernel is still finishing.
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
+      if (TMA_OUT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 128);
-    }
-    mbar_init(rcv_bar, 1);   // RED_DSMEM*: the partials' arrival; otherwise armed by nobody
-    flags[0] = flags[1] = flags[2] = flags[3] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // the slices of all splits (this one's included): 128 rows x cpr tokens each
-    if constexpr (DSM) mbar_expect_tx(rcv_bar, (uint32_t)(BN * TC_BM * (RED == RED_DSMEM ? 2 : 4)));
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // Weights never depend on earlier kernels: stream the first stages' weight
-    // tiles while the previous kernel is still finishing.
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
-    if (TMA_OUT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_w));
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_x));
+    __syncwarp();
   }
   // A launch that may be skipped at run time (p.skip) issues nothing before
   // it has read its flag after the wait; every other launch streams its first
   // weight tiles now, while the previous kernel is still finishing.
-  auto issue_weight_prologue = [&]() {
+  auto issue_weight_prologue = [&]() {   // warp 0
     if (p.oneshot) {
       // every weight k-tile of this CTA in one box; the token k-tiles follow
       // after the wait into the same barrier
       // (the boxes are S = the largest split's k-tile count deep; a shorter
       // split ignores the extra tile)
-      mbar_expect_tx(&full[0], (uint32_t)S * (TC_A_BYTES + b_bytes));
-      tma_load_3d(&tmW, &full[0], a_s, 0, tn0 * TC_BM, kb0_first, pol_w);
+      mbar_expect_tx_el(&full[0], (uint32_t)S * (TC_A_BYTES + b_bytes), el);
+      tma_load_3d_el(&tmW, full0, a0, 0, tn0 * TC_BM, kb0_first, pol_w, el);
     } else {
+      #pragma unroll 1
       for (int i = 0; i < npre; ++i) {
-        mbar_expect_tx(&full[i], TC_A_BYTES + b_bytes);
-        tma_load_2d(&tmW, &full[i], a_s + (size_t)i * TC_A_BYTES, (kb0_first + i) * TC_BK, tn0 * TC_BM, pol_w);
+        mbar_expect_tx_el(&full[i], TC_A_BYTES + b_bytes, el);
+        tma_load_2d_el(&tmW, full0 + 8u * (uint32_t)i, a0 + (uint32_t)i * TC_A_BYTES, (kb0_first + i) * TC_BK,
+                       tn0 * TC_BM, pol_w, el);
       }
       // a split CTA has one short K range: the rest of its weight slice goes
       // to L2 now, so that after the wait every operand load is an L2 hit
-      if (p.splits > 1)
-        for (int kb = kb0_first + npre; kb < kb1_first; ++kb) prefetch_l2_2d(&tmW, kb * TC_BK, tn0 * TC_BM);
+      if (p.splits > 1) {
+        #pragma unroll 1
+        for (int kb = kb0_first + npre; kb < kb1_first; ++kb) prefetch_l2_2d_el(&tmW, kb * TC_BK, tn0 * TC_BM, el);
+      }
     }
   };
-  if (threadIdx.x == 0 && !p.skip) issue_weight_prologue();
+  if (warp == 0 && !p.skip) issue_weight_prologue();
   // everything below may read what earlier kernels wrote; TMEM is taken only
   // now, so a CTA waiting here never holds columns its predecessor needs
   pdl_wait();
   if (p.skip) {
     // nothing is in flight yet; the flag is the same for every CTA
     if (*p.skip) return;
-    if (threadIdx.x == 0) issue_weight_prologue();
+    if (warp == 0) issue_weight_prologue();
+  }
+  if (warp == 0) {
+    // the tokens of the stages whose weights are on their way: before the
+    // TMEM set-up, which they do not need
+    if (p.oneshot) {
+      tma_load_3d_el(&tmX, full0, b0, 0, tm0 * BN, kb0_first, pol_x, el);
+    } else {
+      #pragma unroll 1
+      for (int i = 0; i < npre; ++i)
+        tma_load_2d_el(&tmX, full0 + 8u * (uint32_t)i, b0 + (uint32_t)i * b_bytes, (kb0_first + i) * TC_BK, tm0 * BN,
+                       pol_x, el);
+    }
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -505,96 +528,95 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0 && p.oneshot) {
-      tma_load_3d(&tmX, &full[0], b_s, 0, tm0 * BN, kb0_first, pol_x);
-      flags[2] = 1;
-    } else if (lane == 0) {
-      int it = 0;   // ring position across all work items
+    int it = p.oneshot ? 1 : npre;   // stages issued, across all work items
+    if (!p.oneshot && has_work) {
+      int s = npre == S ? 0 : npre;          // ring position and the parity its `empty` wait takes
+      uint32_t ph = npre == S ? 0u : 1u;
       bool ok = true;
-      int tn, tm, sp;
-      for (int i = 0; ok && work_item(p, i, tn, tm, sp); ++i) {
-        const int kb0 = (int)((long)sp * p.num_kb / p.splits), kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
+      int tn = tn0, tm = tm0, sp = sp0, i = 0;
+      int kb = kb0_first + npre, kb1 = kb1_first;
+      while (true) {
         #pragma unroll 1
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          if (it < npre) {   // weight tile already in flight
-            tma_load_2d(&tmX, &full[s], b_s + (size_t)s * b_bytes, kb * TC_BK, tm * BN, pol_x);
-            continue;
+        for (; kb < kb1; ++kb, ++it) {
+          ok = mbar_wait_warp(&empty[s], ph, p.wait_ns);
+          if (!ok) break;
+          mbar_expect_tx_el(&full[s], TC_A_BYTES + b_bytes, el);
+          tma_load_2d_el(&tmW, full0 + 8u * (uint32_t)s, a0 + (uint32_t)s * TC_A_BYTES, kb * TC_BK, tn * TC_BM, pol_w,
+                         el);
+          tma_load_2d_el(&tmX, full0 + 8u * (uint32_t)s, b0 + (uint32_t)s * b_bytes, kb * TC_BK, tm * BN, pol_x, el);
+          if (++s == S) {
+            s = 0;
+            ph ^= 1u;
           }
-          if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u, p.wait_ns)) {
-            flags[0] = 1;
-            ok = false;
-            break;
-          }
-          mbar_expect_tx(&full[s], TC_A_BYTES + b_bytes);
-          tma_load_2d(&tmW, &full[s], a_s + (size_t)s * TC_A_BYTES, kb * TC_BK, tn * TC_BM, pol_w);
-          tma_load_2d(&tmX, &full[s], b_s + (size_t)s * b_bytes, kb * TC_BK, tm * BN, pol_x);
         }
+        if (!ok || !work_item(p, ++i, tn, tm, sp)) break;
+        kb = (int)((long)sp * p.num_kb / p.splits);
+        kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
       }
-      flags[2] = it;
+      if (!ok && lane == 0) flags[0] = 1;
     }
+    if (lane == 0) flags[2] = it;
     __syncwarp();
     // RED_DSMEM*: one arrival per thread on the cluster barrier that opens the
     // exchange (the epilogue warps arrive once their MMAs are complete)
     if constexpr (DSM) cluster_arrive_release();
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(TC_BM, BN);
-      int it = 0;
-      bool ok = true;
-      int tn, tm, sp;
-      // fault injection: an arrival that never comes (rcv_bar is armed by
-      // nobody outside the RED_DSMEM modes, which the host never combines with this)
-      if (p.withhold && !mbar_wait(rcv_bar, 0, p.wait_ns)) {
-        flags[0] = 1;
-        ok = false;
-      }
-      if (ok && p.oneshot) {   // one item, every k-tile behind one barrier
-        ok = mbar_wait(&full[0], 0, p.wait_ns);
-        if (ok) {
-          tc_fence_after();
-          #pragma unroll 1
-          for (int kb = 0; kb < kb1_first - kb0_first; ++kb) {
-            const uint64_t ad = sw128_desc(smem_u32(a_s + (size_t)kb * TC_A_BYTES));
-            const uint64_t bd = sw128_desc(smem_u32(b_s + (size_t)kb * b_bytes));
-#pragma unroll
-            for (int k = 0; k < TC_BK / 16; ++k)
-              umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          }
-          umma_commit(&acc_full[0]);
-          it = 1;
-        } else {
-          flags[0] = 1;
-        }
-      }
-      for (int i = 0; !p.oneshot && ok && work_item(p, i, tn, tm, sp); ++i) {
-        const int b = i & 1;
-        // the accumulator of item i - 2 must have been drained by the epilogue
-        if (i >= 2 && !mbar_wait(&acc_empty[b], (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns)) {
-          flags[0] = 1;
-          break;
-        }
+    el = elect_one();
+    const uint32_t idesc = idesc_bf16(TC_BM, BN);
+    const uint64_t ad0 = sw128_desc(a0), bd0 = sw128_desc(b0);
+    int it = 0;
+    bool ok = true;
+    // fault injection: an arrival that never comes (rcv_bar is armed by
+    // nobody outside the RED_DSMEM modes, which the host never combines with this)
+    if (p.withhold) ok = mbar_wait_warp(rcv_bar, 0, p.wait_ns);
+    if (ok && p.oneshot) {   // one item, every k-tile behind one barrier
+      ok = mbar_wait_warp(&full[0], 0, p.wait_ns);
+      if (ok) {
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)b * p.acc_cols;
-        const int kb0 = (int)((long)sp * p.num_kb / p.splits), kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
+        uint64_t ad = ad0, bd = bd0;
         #pragma unroll 1
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u, p.wait_ns)) {
-            flags[0] = 1;
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint64_t ad = sw128_desc(smem_u32(a_s + (size_t)s * TC_A_BYTES));
-          const uint64_t bd = sw128_desc(smem_u32(b_s + (size_t)s * b_bytes));
+        for (int kb = 0; kb < kb1_first - kb0_first; ++kb, ad += TC_A_BYTES >> 4, bd += b_bytes >> 4) {
 #pragma unroll
           for (int k = 0; k < TC_BK / 16; ++k)
-            umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-          umma_commit(&empty[s]);
+            umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u, el);
         }
-        umma_commit(&acc_full[b]);   // arrives once every MMA issued above has completed
+        umma_commit(&acc_full[0], el);
+        it = 1;
       }
+    }
+    int tn, tm, sp, s = 0;
+    uint32_t ph = 0, aoff = 0, boff = 0;   // ring position: parity and descriptor offsets of stage s
+    for (int i = 0; !p.oneshot && ok && work_item(p, i, tn, tm, sp); ++i) {
+      const int b = i & 1;
+      // the accumulator of item i - 2 must have been drained by the epilogue
+      if (i >= 2) ok = mbar_wait_warp(&acc_empty[b], (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)b * p.acc_cols;
+      const int kb0 = (int)((long)sp * p.num_kb / p.splits), kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
+      #pragma unroll 1
+      for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        ok = mbar_wait_warp(&full[s], ph, p.wait_ns);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t ad = ad0 + aoff, bd = bd0 + boff;
+#pragma unroll
+        for (int k = 0; k < TC_BK / 16; ++k)
+          umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u, el);
+        umma_commit(&empty[s], el);
+        aoff += TC_A_BYTES >> 4;
+        boff += b_bytes >> 4;
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+          aoff = boff = 0;
+        }
+      }
+      if (!ok) break;
+      umma_commit(&acc_full[b], el);   // arrives once every MMA issued above has completed
+    }
+    if (lane == 0) {
+      if (!ok) flags[0] = 1;
       flags[3] = it;
     }
     __syncwarp();
@@ -938,7 +960,7 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
   int* flags = (int*)(tmem_slot + 1);  // [0] abort, [2] stages issued, [3] stages consumed
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
@@ -975,29 +997,43 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   const uint32_t full0 = mapa_shared(smem_u32(full), 0);          // the even CTA's full[0]
   const uint32_t acc_empty0 = mapa_shared(smem_u32(acc_empty), 0);
   uint64_t pol_w = 0, pol_x = 0;
-  if (threadIdx.x == 0) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
+  uint32_t el = 0;   // the issuing lane of warps 0 (TMA) and 1 (MMA)
+  const uint32_t a0 = smem_u32(a_s), b0 = smem_u32(b_s);
+  if (warp == 0) {
+    el = elect_one();
+    if (el) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmO) : "memory");
+    }
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_w));
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_x));
+    __syncwarp();
   }
+  const uint32_t el_lead = leader ? el : 0u;   // the even CTA's issuing lane
   // the first stages' weight halves, before the wait on the previous kernel
   // (after it, for a launch that may be skipped at run time)
-  auto issue_weight_prologue = [&]() {
+  auto issue_weight_prologue = [&]() {   // warp 0
+    #pragma unroll 1
     for (int i = 0; i < npre; ++i) {
-      if (leader) mbar_expect_tx(&full[i], stage_tx);
-      tma_load_2d_pair(&tmW, full0 + 8u * (uint32_t)i, a_s + (size_t)i * TC_A_BYTES, i * TC_BK,
-                       (2 * tn0 + (int)rank) * TC_BM, pol_w);
+      mbar_expect_tx_el(&full[i], stage_tx, el_lead);
+      tma_load_2d_pair_el(&tmW, full0 + 8u * (uint32_t)i, a0 + (uint32_t)i * TC_A_BYTES, i * TC_BK,
+                          (2 * tn0 + (int)rank) * TC_BM, pol_w, el);
     }
   };
-  if (threadIdx.x == 0 && !p.skip) issue_weight_prologue();
+  if (warp == 0 && !p.skip) issue_weight_prologue();
   pdl_wait();
   if (p.skip) {
     // nothing has been issued yet and the flag is the same for both CTAs of
     // the pair: they leave together, with no copy or arrival in flight
     if (*p.skip) return;
-    if (threadIdx.x == 0) issue_weight_prologue();
+    if (warp == 0) issue_weight_prologue();
+  }
+  if (warp == 0) {   // their token halves, before the TMEM set-up
+    #pragma unroll 1
+    for (int i = 0; i < npre; ++i)
+      tma_load_2d_pair_el(&tmX, full0 + 8u * (uint32_t)i, b0 + (uint32_t)i * bh_bytes, i * TC_BK,
+                          tm0 * BN + (int)rank * BNh, pol_x, el);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -1010,64 +1046,75 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {   // producer (both CTAs): this CTA's A rows and B half of each stage
-      int it = 0;
+  if (warp == 0) {   // producer (both CTAs): this CTA's A rows and B half of each stage
+    int it = npre;
+    if (has_work) {
+      int s = npre == S ? 0 : npre;   // ring position and the parity its `empty` wait takes
+      uint32_t ph = npre == S ? 0u : 1u;
       bool ok = true;
-      int tn2, tm;
-      for (int i = 0; ok && item(i, tn2, tm); ++i) {
-        for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
-          const int s = it % S;
+      int tn2 = tn0, tm = tm0, i = 0, kb = npre;
+      while (true) {
+        #pragma unroll 1
+        for (; kb < p.num_kb; ++kb, ++it) {
+          ok = mbar_wait_warp(&empty[s], ph);
+          if (!ok) break;
           const uint32_t fb = full0 + 8u * (uint32_t)s;
-          if (it < npre) {   // weight half already in flight
-            tma_load_2d_pair(&tmX, fb, b_s + (size_t)s * bh_bytes, kb * TC_BK, tm * BN + (int)rank * BNh, pol_x);
-            continue;
+          mbar_expect_tx_el(&full[s], stage_tx, el_lead);
+          tma_load_2d_pair_el(&tmW, fb, a0 + (uint32_t)s * TC_A_BYTES, kb * TC_BK, (2 * tn2 + (int)rank) * TC_BM,
+                              pol_w, el);
+          tma_load_2d_pair_el(&tmX, fb, b0 + (uint32_t)s * bh_bytes, kb * TC_BK, tm * BN + (int)rank * BNh, pol_x, el);
+          if (++s == S) {
+            s = 0;
+            ph ^= 1u;
           }
-          if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u)) {
-            flags[0] = 1;
-            ok = false;
-            break;
-          }
-          if (leader) mbar_expect_tx(&full[s], stage_tx);
-          tma_load_2d_pair(&tmW, fb, a_s + (size_t)s * TC_A_BYTES, kb * TC_BK, (2 * tn2 + (int)rank) * TC_BM, pol_w);
-          tma_load_2d_pair(&tmX, fb, b_s + (size_t)s * bh_bytes, kb * TC_BK, tm * BN + (int)rank * BNh, pol_x);
         }
+        if (!ok || !item(++i, tn2, tm)) break;
+        kb = 0;
       }
-      flags[2] = it;
+      if (!ok && lane == 0) flags[0] = 1;
     }
+    if (lane == 0) flags[2] = it;
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && leader) {   // MMA issuer: the even CTA only
+    if (leader) {   // MMA issuer: the even CTA only
+      el = elect_one();
       const uint32_t idesc = idesc_bf16(2 * TC_BM, BN);
-      int it = 0;
+      const uint64_t ad0 = sw128_desc(a0), bd0 = sw128_desc(b0);
+      int it = 0, s = 0;
+      uint32_t ph = 0, aoff = 0, boff = 0;   // ring position: parity and descriptor offsets of stage s
       bool ok = true;
       int tn2, tm;
       for (int i = 0; ok && item(i, tn2, tm); ++i) {
         const int b = i & 1;
         // both CTAs' epilogues must have drained the accumulator of item i - 2
-        if (i >= 2 && !mbar_wait(&acc_empty[b], (uint32_t)((i >> 1) - 1) & 1u)) {
-          flags[0] = 1;
-          break;
-        }
+        if (i >= 2) ok = mbar_wait_warp(&acc_empty[b], (uint32_t)((i >> 1) - 1) & 1u);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)b * p.acc_cols;
+        #pragma unroll 1
         for (int kb = 0; kb < p.num_kb; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u)) {
-            flags[0] = 1;
-            ok = false;
-            break;
-          }
+          ok = mbar_wait_warp(&full[s], ph);
+          if (!ok) break;
           tc_fence_after();
-          const uint64_t ad = sw128_desc(smem_u32(a_s + (size_t)s * TC_A_BYTES));
-          const uint64_t bd = sw128_desc(smem_u32(b_s + (size_t)s * bh_bytes));
+          const uint64_t ad = ad0 + aoff, bd = bd0 + boff;
 #pragma unroll
-          for (int k = 0; k < TC_BK / 16; ++k) umma_bf16_pair(d, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit_pair_mc(&empty[s], 3);   // both CTAs' halves of the stage are free
+          for (int k = 0; k < TC_BK / 16; ++k)
+            umma_bf16_pair(d, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u, el);
+          umma_commit_pair_mc(&empty[s], 3, el);   // both CTAs' halves of the stage are free
+          aoff += TC_A_BYTES >> 4;
+          boff += bh_bytes >> 4;
+          if (++s == S) {
+            s = 0;
+            ph ^= 1u;
+            aoff = boff = 0;
+          }
         }
-        if (ok) umma_commit_pair_mc(&acc_full[b], 3);
+        if (ok) umma_commit_pair_mc(&acc_full[b], 3, el);
       }
-      flags[3] = it;
+      if (lane == 0) {
+        if (!ok) flags[0] = 1;
+        flags[3] = it;
+      }
     }
     __syncwarp();
   } else {
