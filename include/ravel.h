@@ -292,16 +292,14 @@ ravel_status ravel_gemm(ravel_t* r, const void* X, int M, int K, int lda, const 
  * (X and W bf16, 16-byte aligned, K, lda, ldw multiples of 8), on the
  * current CUDA device.  It calls no cudaMalloc / cudaFree: its split-K
  * scratch is one fixed device array inside the library (8 MiB of partial
- * sums plus tile counters), held by every GPU that loads the library until
- * the process exits.  The split plan is chosen to fit that array.  M, N, K
+ * sums), held by every GPU that loads the library until the process exits.  The split plan is chosen to fit that array.  M, N, K
  * above RAVEL_NOALLOC_MAX_M / _N / _K return RAVEL_ESHAPE; bad pointers or
  * modes RAVEL_EINVAL.  The first call on a device resolves the array's device
  * address (and the kernel set-up) for that device; make that first call
  * before any stream capture (a first call on a capturing stream returns
- * RAVEL_EINVAL and does nothing).  Each call clears the scratch's tile
- * counters on `stream` before the GEMM; every call shares the array, so calls
- * that overlap on the GPU race and must be serialised by the caller.  The
- * array also holds a device error word that calls never clear: a bounded wait
+ * RAVEL_EINVAL and does nothing).  Every call shares the array, so calls
+ * that overlap on the GPU race and must be serialised by the caller.  It
+ * also holds a device error word that calls never clear: a bounded wait
  * that runs out inside the GEMM (its output is then not valid) stays recorded
  * until ravel_gemm_noalloc_status reads it. */
 #define RAVEL_NOALLOC_MAX_M 32768

@@ -26,14 +26,12 @@
 //    in order (deterministic) and applies the epilogue.  The partials travel
 //    by st.async straight into rank q's shared memory, completing on an
 //    mbarrier there (slices of up to 32 tokens), else through L2 and the
-//    cluster barrier;
-//  * workspace mode (no cluster, for callers that bring their own scratch):
-//    the last split to arrive (per-tile counter) sums all partials.
+//    cluster barrier.
 // Epilogue: a chunk of tokens is written into a shared-memory box in the
 // output layout and leaves through one TMA store (or a TMA reduce-add for the
 // residual-stream epilogue), double-buffered so that the epilogue threads
-// never wait on global memory; the workspace mode (and unaligned outputs)
-// store from the threads instead.
+// never wait on global memory; unaligned outputs are stored by the threads
+// instead.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -62,15 +60,14 @@ constexpr int STG_LD = 132;                  // SIMT staging pitch (floats): 16 
 constexpr uint32_t STG_BYTES = 16 * STG_LD * 4;
 constexpr uint32_t XCH_BYTES = 32 * STG_LD * 4;  // GeGLU transpose tile (TMA epilogue): <= 32 tokens x 128 rows
 
-enum { RED_NONE = 0, RED_L2_CLUSTER = 1, RED_WORKSPACE = 2, RED_DSMEM = 3, RED_DSMEM32 = 4 };
+enum { RED_NONE = 0, RED_L2_CLUSTER = 1, RED_DSMEM = 2, RED_DSMEM32 = 3 };
 // Epilogue kind of an instantiation: outputs through TMA boxes as fp32, bf16,
 // a reduce-add into the fp32 residual stream or the GeGLU pair -- fixed, so
 // that a long persistent launch carries only the code of its own epilogue --
 // or any of these chosen at run time (EK_TMA_ANY: the
 // short split-K launches of one step then all run one binary, whose code the
 // previous launch has left in the SM's instruction cache), or stored by the
-// threads (EK_GENERIC: any epilogue; unaligned outputs and the workspace
-// reduction).
+// threads (EK_GENERIC: any epilogue; unaligned outputs).
 enum { EK_F32 = 0, EK_BF16 = 1, EK_ADD = 2, EK_GEGLU = 3, EK_GENERIC = 4, EK_TMA_ANY = 5 };
 
 
@@ -80,6 +77,7 @@ struct TcParams {
   int reduce;           // how the splits of a tile are combined (splits > 1)
   uint32_t ring_bytes;  // operand ring bytes (1024-aligned)
   uint32_t acc_cols;    // TMEM columns of one accumulator
+  int lacc;             // log2 of the accumulators an item's K range is cut into (short_sums)
   int tiles_n, tiles_m, num_tiles;
   int epi;              // Epi
   int out_bf16;
@@ -87,7 +85,6 @@ struct TcParams {
   int ldo;
   const float* bias;
   float* ws;
-  int* counters;
   int* err;
   int tma_out;          // outputs leave through TMA boxes
   int oneshot;          // split launch whose whole K range fits the ring: tmW / tmX are 3-D maps
@@ -230,6 +227,27 @@ __device__ __forceinline__ void reduce_slice_smem(const float4* b0, int S, float
       v[4 * g + 1] += x[g].y;
       v[4 * g + 2] += x[g].z;
       v[4 * g + 3] += x[g].w;
+    }
+  }
+}
+
+// v[k] += the item's other accumulators (in K order) at this thread's row,
+// columns taddr + k of the first one.
+__device__ __forceinline__ void add_accumulators(uint32_t taddr, uint32_t acc_cols, int lacc, uint32_t v[16]) {
+  #pragma unroll 1
+  for (int j = 1; j < (1 << lacc); j += 3) {   // up to three loads in flight
+    const int n = (1 << lacc) - j;
+    uint32_t x[3][16];
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (u < n) tmem_ld16_async(taddr + (uint32_t)(j + u) * acc_cols, x[u]);
+    tmem_wait_ld();
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      tmem_reg_fence16(x[u]);
+      if (u >= n) break;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(x[u][k]));
     }
   }
 }
@@ -422,11 +440,15 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   uint64_t* acc_empty = acc_full + 2;  // [2]
   uint64_t* rcv_bar = acc_empty + 2;    // RED_DSMEM*: every split's slice of this rank has arrived
   uint32_t* tmem_slot = (uint32_t*)(rcv_bar + 1);
-  int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] last split, [2] issued, [3] consumed
+  int* flags = (int*)(tmem_slot + 1);   // [0] abort, [2] issued, [3] consumed
 
   // (through a shuffle, so that the compiler knows it is uniform in the warp)
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const uint32_t ncols = (p.splits > 1) ? p.acc_cols : 2 * p.acc_cols;
+  // the K range of an item in 1 << lacc accumulators, summed in the epilogue
+  constexpr bool MULTI = RED != RED_DSMEM;
+  const int lacc = MULTI ? p.lacc : 0;
+  const uint32_t item_cols = p.acc_cols << lacc;
+  const uint32_t ncols = (p.splits > 1) ? item_cols : 2 * item_cols;
   int tn0 = 0, tm0 = 0, sp0 = 0;
   const bool has_work = work_item(p, 0, tn0, tm0, sp0);
   const int kb0_first = (int)((long)sp0 * p.num_kb / p.splits);
@@ -454,7 +476,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         mbar_init(&acc_empty[b], 128);
       }
       mbar_init(rcv_bar, 1);   // RED_DSMEM*: the partials' arrival; otherwise armed by nobody
-      flags[0] = flags[1] = flags[2] = flags[3] = 0;
+      flags[0] = flags[2] = flags[3] = 0;
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       // the slices of all splits (this one's included): 128 rows x cpr tokens each
       if constexpr (DSM) mbar_expect_tx(rcv_bar, (uint32_t)(BN * TC_BM * (RED == RED_DSMEM ? 2 : 4)));
@@ -574,11 +596,19 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       if (ok) {
         tc_fence_after();
         uint64_t ad = ad0, bd = bd0;
+        const int cnt = kb1_first - kb0_first;
+        int j = 0, first = 0, next = cnt >> lacc;   // accumulator j takes k-tiles [first, next)
+        uint32_t d = tmem;
         #pragma unroll 1
-        for (int kb = 0; kb < kb1_first - kb0_first; ++kb, ad += TC_A_BYTES >> 4, bd += b_bytes >> 4) {
+        for (int kb = 0; kb < cnt; ++kb, ad += TC_A_BYTES >> 4, bd += b_bytes >> 4) {
+          if (MULTI && kb == next) {
+            first = kb;
+            next = (cnt * (++j + 1)) >> lacc;
+            d += p.acc_cols;
+          }
 #pragma unroll
           for (int k = 0; k < TC_BK / 16; ++k)
-            umma_bf16(tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u, el);
+            umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb > first || k > 0) ? 1u : 0u, el);
         }
         umma_commit(&acc_full[0], el);
         it = 1;
@@ -592,17 +622,23 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       if (i >= 2) ok = mbar_wait_warp(&acc_empty[b], (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t d = tmem + (uint32_t)b * p.acc_cols;
+      uint32_t d = tmem + (uint32_t)b * item_cols;
       const int kb0 = (int)((long)sp * p.num_kb / p.splits), kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
+      int j = 0, first = kb0, next = kb0 + ((kb1 - kb0) >> lacc);   // accumulator j takes k-tiles [first, next)
       #pragma unroll 1
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        if (MULTI && kb == next) {
+          first = kb;
+          next = kb0 + (((kb1 - kb0) * (++j + 1)) >> lacc);
+          d += p.acc_cols;
+        }
         ok = mbar_wait_warp(&full[s], ph, p.wait_ns);
         if (!ok) break;
         tc_fence_after();
         const uint64_t ad = ad0 + aoff, bd = bd0 + boff;
 #pragma unroll
         for (int k = 0; k < TC_BK / 16; ++k)
-          umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u, el);
+          umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb > first || k > 0) ? 1u : 0u, el);
         umma_commit(&empty[s], el);
         aoff += TC_A_BYTES >> 4;
         boff += b_bytes >> 4;
@@ -642,7 +678,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         break;
       }
       tc_fence_after();
-      const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * p.acc_cols;
+      const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * item_cols;
       const int m_base = tm * BN;
       const int n = tn * TC_BM + r;
       const float brow = (p.bias && n < p.N) ? p.bias[n] : 0.f;
@@ -656,6 +692,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 16) {
           float v[16];
+          add_accumulators(trow + c0, p.acc_cols, lacc, nxt);
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(nxt[k]);
           const bool more = c0 + 16 < BN;
@@ -732,6 +769,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
           tmem_wait_ld();
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq) tmem_reg_fence16(raw + 16 * qq);
+#pragma unroll
+          for (int qq = 0; qq < 4; ++qq)
+            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, lacc, raw + 16 * qq);
           for_upto<16>(4 * nq, [&](int qq) {
             st_async_f4(mapa_shared(rcv0 + (uint32_t)gl * (TC_BM * 16), (uint32_t)dst),
                         make_float4(__uint_as_float(raw[4 * qq]), __uint_as_float(raw[4 * qq + 1]),
@@ -742,7 +782,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             dst += wrap ? 1 : 0;
           });
         }
-      } else if constexpr (RED == RED_L2_CLUSTER) {
+      } else {   // RED_L2_CLUSTER
         // this split's fp32 partial to the workspace as [col/4][row][4]: each
         // thread stores float4 of 4 consecutive columns, a warp one 512-byte run
         const size_t cl = (size_t)tm * gridDim.x + tn;
@@ -758,6 +798,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq) tmem_reg_fence16(raw + 16 * qq);
 #pragma unroll
+          for (int qq = 0; qq < 4; ++qq)
+            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, lacc, raw + 16 * qq);
+#pragma unroll
           for (int qq = 0; qq < 16; ++qq)
             if (qq < 4 * nq)
               __stcg((float4*)(w + (size_t)(c0 / 4 + qq) * (TC_BM * 4)),
@@ -765,44 +808,6 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
                                  __uint_as_float(raw[4 * qq + 2]), __uint_as_float(raw[4 * qq + 3])));
         }
         __threadfence();
-      } else {
-        // workspace mode: [split][tile][col][row] partials, last arrival reduces
-        const int tiles = gridDim.x * gridDim.y;
-        const int tile_id = tm * gridDim.x + tn;
-        #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-          float v[16];
-          tmem_ld16(trow + c0, v);
-          float* w = p.ws + ((size_t)(sp * tiles + tile_id) * BN + c0) * TC_BM + r;
-#pragma unroll
-          for (int k = 0; k < 16; ++k) __stcg(w + (size_t)k * TC_BM, v[k]);
-        }
-        __threadfence();
-        epi_bar();
-        if (threadIdx.x == 64) {
-          const int prev = atomicAdd(&p.counters[tile_id], 1);
-          flags[1] = (prev == p.splits - 1);
-        }
-        epi_bar();
-        if (flags[1]) {
-          __threadfence();
-          #pragma unroll 1
-          for (int c0 = 0; c0 < BN; c0 += 16) {
-            float v[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) v[k] = 0.f;
-            for (int s = 0; s < p.splits; ++s) {
-              const float* w = p.ws + ((size_t)(s * tiles + tile_id) * BN + c0) * TC_BM + r;
-              float x[16];
-#pragma unroll
-              for (int k = 0; k < 16; ++k) x[k] = __ldcg(w + (size_t)k * TC_BM);
-#pragma unroll
-              for (int k = 0; k < 16; ++k) v[k] += x[k];
-            }
-            epilogue_chunk(p, tn, m_base + c0, 16, r, v, stage);
-          }
-          if (threadIdx.x == 64) p.counters[tile_id] = 0;
-        }
       }
     }
     // every TMA output box has been read out of shared memory (the grid's
@@ -989,7 +994,7 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], 512);
     }
-    flags[0] = flags[1] = flags[2] = flags[3] = 0;
+    flags[0] = flags[2] = flags[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // both CTAs' barriers exist before either signals the other's
@@ -1203,8 +1208,7 @@ TcKernel tc_pair_kernel(int ek) {
 }
 
 // The instantiation for a reduction mode and epilogue kind (nullptr where the
-// pair cannot occur: the workspace mode stores from the threads, the
-// shared-memory exchange needs TMA outputs).
+// two cannot occur together: the shared-memory exchange needs TMA outputs).
 TcKernel tc_kernel(int red, int ek) {
 #define RAVEL_TC_K(R, E) \
   if (red == R && ek == E) return tc_gemm_kernel<R, E>;
@@ -1212,7 +1216,6 @@ TcKernel tc_kernel(int red, int ek) {
   RAVEL_TC_K(RED_NONE, EK_GEGLU) RAVEL_TC_K(RED_NONE, EK_GENERIC)
   RAVEL_TC_K(RED_L2_CLUSTER, EK_TMA_ANY) RAVEL_TC_K(RED_L2_CLUSTER, EK_GENERIC)
   RAVEL_TC_K(RED_DSMEM, EK_TMA_ANY) RAVEL_TC_K(RED_DSMEM32, EK_TMA_ANY)
-  RAVEL_TC_K(RED_WORKSPACE, EK_GENERIC)
 #undef RAVEL_TC_K
   return nullptr;
 }
@@ -1316,6 +1319,15 @@ int pick_bn_pair(int M, int tiles_n2, int slots) {
   return bn;
 }
 
+// The tensor cores truncate each fp32 accumulation, so a sum's error grows
+// with its length: about 1e-9 of the result per K element (N(0, 1) x N(0,
+// 0.02) operands: 2.7e-7 at K = 256, 1.7e-6 at 2048).  Where the result is
+// stored in fp32 and the splits' shares are exchanged in fp32 too, an item's
+// K range therefore goes through accumulators of at most 192 elements each
+// (as far as TMEM holds them), added in the epilogue; bf16 results round at
+// 2e-3.
+bool short_sums(const GemmArgs& g) { return !g.xbf16 && (g.epi == EPI_ADD_F32 || (g.epi != EPI_GEGLU && g.out_dt == DT_F32)); }
+
 cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st, int ek,
                              bool out_bf, int es) {
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
@@ -1351,8 +1363,8 @@ cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_s
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, stages, 1, num_kb, RED_NONE, (uint32_t)ring, acc_cols, tiles_n, tiles_m, num_tiles,
-             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.counters, ws.err,
+  TcParams p{g.M, g.N, g.K, bn, stages, 1, num_kb, RED_NONE, (uint32_t)ring, acc_cols, 0, tiles_n, tiles_m, num_tiles,
+             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
              1, 0, box_m, box_bytes, stg_off, xch_off, 0, bar_off, kTcTimeoutNs, 0, g.skip};
   p.set_bytes = (uint32_t)set_bytes;
   const int npairs = std::min(num_tiles, slots);
@@ -1368,7 +1380,7 @@ cudaError_t init_tc_gemm() {
   cudaError_t e = get_encoder();
   if (e != cudaSuccess) return e;
   std::vector<const void*> kernels;
-  for (int red = 0; red < 5; ++red)
+  for (int red = 0; red <= RED_DSMEM32; ++red)
     for (int ek = 0; ek <= EK_TMA_ANY; ++ek)
       if (TcKernel k = tc_kernel(red, ek)) kernels.push_back((const void*)k);
   for (int ek = 0; ek < EK_GENERIC; ++ek) kernels.push_back((const void*)tc_pair_kernel(ek));
@@ -1407,7 +1419,7 @@ bool tc_gemm_supported(const GemmArgs& g) {
   return g.M > 0 && g.N > 0 && g.K > 0;
 }
 
-cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st, bool cluster) {
+cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st) {
   if (!g_encode) return cudaErrorInitializationError;
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
   const int bn = pick_bn(g.M, tiles_n, num_sms);
@@ -1417,19 +1429,15 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   int splits = 1;
   if (tiles < num_sms) splits = std::min(num_kb, std::max(1, num_sms / tiles));
   if (g.max_splits > 0) splits = std::min(splits, g.max_splits);
-  if (cluster) {
-    // the splits of a tile form one cluster: a power of two, at most the cluster
-    // limit, whose partials fit the workspace and whose column slices are
-    // multiples of 4
-    int c = 1;
-    while (c * 2 <= std::min(splits, g_max_cluster) && (bn / (c * 2)) % 4 == 0 &&
-           (size_t)(c * 2) * tiles * bn * TC_BM * 4 <= ws.ws_bytes)
-      c *= 2;
-    splits = c;
-  } else {
-    while (splits > 1 && ((size_t)splits * tiles * bn * TC_BM * 4 > ws.ws_bytes || tiles > ws.n_counters)) --splits;
-  }
-  int reduce = splits == 1 ? RED_NONE : (cluster ? RED_L2_CLUSTER : RED_WORKSPACE);
+  // the splits of a tile form one cluster: a power of two, at most the cluster
+  // limit, whose partials fit the workspace and whose column slices are
+  // multiples of 4
+  int c = 1;
+  while (c * 2 <= std::min(splits, g_max_cluster) && (bn / (c * 2)) % 4 == 0 &&
+         (size_t)(c * 2) * tiles * bn * TC_BM * 4 <= ws.ws_bytes)
+    c *= 2;
+  splits = c;
+  int reduce = splits == 1 ? RED_NONE : RED_L2_CLUSTER;
   {
     // two-SM tiles for a persistent launch whose pair tiles fill at least
     // three quarters of the pairs of SMs
@@ -1439,7 +1447,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
     const int tn2 = (g.N + 2 * TC_BM - 1) / (2 * TC_BM), slots = num_sms / 2;
     const int pbn = pick_bn_pair(g.M, tn2, slots);
     const long pair_tiles = (long)tn2 * ((g.M + pbn - 1) / pbn);
-    if (cluster && g_pair_gemm && splits == 1 && aligned && 4 * pair_tiles >= 3 * slots) {
+    if (g_pair_gemm && splits == 1 && aligned && 4 * pair_tiles >= 3 * slots) {
       const int ek = g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : obf ? EK_BF16 : EK_F32;
       return launch_gemm_pair(g, ws, num_sms, st, ek, obf, oes);
     }
@@ -1449,6 +1457,10 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   while ((int)acc_cols < bn) acc_cols <<= 1;
   const int stage_bytes = TC_A_BYTES + bn * TC_BK * 2;
   const int kb_per_item = (num_kb + splits - 1) / splits;
+  // (more than one k-tile per accumulator, so every one is written)
+  int lacc = 0;
+  if (short_sums(g))
+    while (kb_per_item > (3 << lacc) && (acc_cols << (lacc + (splits > 1 ? 1 : 2))) <= 512u) ++lacc;
   const int grid_ctas = splits > 1 ? tiles * splits : std::min(tiles, num_sms);
   const int items = splits > 1 ? 1 : (tiles + grid_ctas - 1) / grid_ctas;
   int stages = std::min(8, TC_SMEM_BUDGET / stage_bytes);
@@ -1458,14 +1470,14 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   stages = std::max(2, std::min(stages, std::max(2, kb_per_item * items)));
   // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
   // takes its weight and token k-tiles in one box each (K a multiple of 64)
-  const bool oneshot = splits > 1 && cluster && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
+  const bool oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
                        (size_t)kb_per_item * stage_bytes <= (size_t)TC_SMEM_BUDGET;
   if (oneshot) stages = kb_per_item;   // the ring is exactly one box deep
   const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
   // outputs through TMA boxes when the output rows are 16-byte aligned
   const bool out_bf = g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16);
   const int es = out_bf ? 2 : 4;
-  const bool tma_out = reduce != RED_WORKSPACE && ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * es) % 16 == 0;
+  const bool tma_out = ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * es) % 16 == 0;
   int box_m = 0;
   // partials exchanged in bf16 where the caller allows it, else in fp32
   const bool xbf = g.xbf16 != 0;
@@ -1506,13 +1518,13 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, stages, splits, num_kb, reduce, (uint32_t)ring, acc_cols, tiles_n, tiles_m, tiles,
-             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.counters, ws.err,
+  TcParams p{g.M, g.N, g.K, bn, stages, splits, num_kb, reduce, (uint32_t)ring, acc_cols, lacc, tiles_n, tiles_m, tiles,
+             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
              tma_out ? 1 : 0, oneshot ? 1 : 0, box_m, box_bytes, stg_off, xch_off, rcv_off, bar_off, kTcTimeoutNs, 0,
              g.skip};
   // fault injection (tests): a launch without a cluster may be told to wait
   // for an arrival that never comes, with a short limit
-  if ((reduce == RED_NONE || reduce == RED_WORKSPACE) && g_withhold.load() > 0 && g_withhold.fetch_sub(1) > 0) {
+  if (reduce == RED_NONE && g_withhold.load() > 0 && g_withhold.fetch_sub(1) > 0) {
     p.withhold = 1;
     p.wait_ns = kWithholdWaitNs;
   }
@@ -1525,8 +1537,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
                  : g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32;
   const TcKernel k = tc_kernel(reduce, ek);
   if (!k) return cudaErrorInvalidConfiguration;
-  const bool clustered = reduce == RED_L2_CLUSTER || reduce == RED_DSMEM || reduce == RED_DSMEM32;
-  return launch_kernel(k, grid, block, smem, st, clustered ? (unsigned)splits : 1u, mw, mx, mo, p);
+  return launch_kernel(k, grid, block, smem, st, (unsigned)splits, mw, mx, mo, p);
 }
 
 }  // namespace ravel

@@ -96,17 +96,12 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, Dtype dt, cudaStream_t st);
 // 128-row blocks of 64 gate rows then the 64 matching up rows; out is bf16
 // [M][N/2] with out[m][f] = gelu_tanh(gate_f) * up_f.
 struct TcWorkspace {
-  float* ws; size_t ws_bytes;   // split-K partial tiles
-  int* counters; int n_counters;   // per-tile arrival counters, zero between launches
+  float* ws; size_t ws_bytes;   // split-K partial tiles (outputs that TMA cannot store)
   int* err;                     // device error word
 };
 cudaError_t init_tc_gemm();
 bool tc_gemm_supported(const GemmArgs& g);
-// cluster = true: split-K partials are reduced through distributed shared
-// memory inside a thread-block cluster (no workspace); false: through the
-// workspace `ws` with a last-arriving-CTA fix-up.
-cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st,
-                           bool cluster = true);
+cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st);
 // Fault injection for tests: the next `launches` tensor-core GEMM launches
 // that run without a thread-block cluster make their MMA thread wait for an
 // mbarrier arrival that nobody makes, with a 2 ms limit; each gives up,

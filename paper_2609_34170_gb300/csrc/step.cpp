@@ -147,9 +147,7 @@ ravel_status plan_create(StepPlan* p, const ravel_config& c, const ravel_weights
   p->attn_ws_bytes = (size_t)32 << 20;
   AL(p->attn_ws, p->attn_ws_bytes);
   p->tcws.ws_bytes = (size_t)24 << 20;
-  p->tcws.n_counters = 4096;
   AL(p->tcws.ws, p->tcws.ws_bytes);
-  AL(p->tcws.counters, p->tcws.n_counters * sizeof(int));
   AL(p->dn_times, rows_t * sizeof(float));
   AL(p->rel_mask, (size_t)A * sizeof(float));
   p->n_adapters = c.fop_adapter_every > 0 ? L / c.fop_adapter_every : 0;
