@@ -165,32 +165,6 @@ __device__ __forceinline__ void reduce_splits_l2(const float* b0, int S, size_t 
   }
 }
 
-// v[4g + e] (g < NG <= 8: up to 32 tokens) = sum over splits s = 0..S-1 (in
-// order) of this thread's row at column group g; as reduce_splits_l2, with up
-// to 24 float4 loads in flight per batch (one batch for every launch here).
-template <int NG>
-__device__ __forceinline__ void reduce_slice_l2(const float* b0, int S, size_t sstride, float v[32]) {
-  constexpr int GB = (24 / NG) > 0 ? 24 / NG : 1;
-  for (int s0 = 0; s0 < S; s0 += GB) {
-    float4 x[GB][NG];
-#pragma unroll
-    for (int u = 0; u < GB; ++u)
-#pragma unroll
-      for (int g = 0; g < NG; ++g)
-        x[u][g] = (s0 + u < S) ? __ldcg((const float4*)(b0 + (size_t)(s0 + u) * sstride + (size_t)g * 512))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < GB; ++u)
-#pragma unroll
-      for (int g = 0; g < NG; ++g) {
-        v[4 * g] += x[u][g].x;
-        v[4 * g + 1] += x[u][g].y;
-        v[4 * g + 2] += x[u][g].z;
-        v[4 * g + 3] += x[u][g].w;
-      }
-  }
-}
-
 // v[4g + e] (g < NG <= 8) = sum over splits s = 0..S-1 (in order) of the
 // received bf16 partials: b0 points at this thread's four tokens of split 0,
 // group 0 (half of a two-row message); group g of split s is (s * NG + g) *
@@ -885,30 +859,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       const size_t cl = (size_t)tm0 * gridDim.x + tn0;
       const float* base = p.ws + (cl * Sp * (size_t)(BN / 4) + rank * cpr / 4) * (TC_BM * 4) + (size_t)r * 4;
       const size_t sstride = (size_t)(BN / 4) * (TC_BM * 4);
-      const int n = tn0 * TC_BM + r;
-      const float brow = (p.bias && n < p.N) ? p.bias[n] : 0.f;
-      int ebuf = 0;
-      // a slice that would take three or more 4- or 8-token chunks goes out
-      // whole: one L2 round trip, one output box
-      const bool whole = TMA_OUT && cpr <= 32 && cpr > 8 && cpr % 16 != 0;
-      if (whole) {
-        float v[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = 0.f;
-        switch (cpr / 4) {
-          case 1: reduce_slice_l2<1>(base, Sp, sstride, v); break;
-          case 2: reduce_slice_l2<2>(base, Sp, sstride, v); break;
-          case 3: reduce_slice_l2<3>(base, Sp, sstride, v); break;
-          case 4: reduce_slice_l2<4>(base, Sp, sstride, v); break;
-          case 5: reduce_slice_l2<5>(base, Sp, sstride, v); break;
-          case 6: reduce_slice_l2<6>(base, Sp, sstride, v); break;
-          case 7: reduce_slice_l2<7>(base, Sp, sstride, v); break;
-          default: reduce_slice_l2<8>(base, Sp, sstride, v); break;
-        }
-        if constexpr (TMA_OUT) epilogue_tma<EK, 32>(p, &tmO, tn0, tm0 * BN + rank * cpr, r, v, brow, stg_raw, xch, ebuf);
-      }
       #pragma unroll 1
-      for (int cc = 0; !whole && cc < cpr; cc += p.box_m) {
+      for (int cc = 0; cc < cpr; cc += p.box_m) {
         const int nc = p.box_m;
         float v[16];
 #pragma unroll
@@ -917,11 +869,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         if (nc == 16) reduce_splits_l2<4>(b0, Sp, sstride, v);
         else if (nc == 8) reduce_splits_l2<2>(b0, Sp, sstride, v);
         else reduce_splits_l2<1>(b0, Sp, sstride, v);
-        const int m0 = tm0 * BN + rank * cpr + cc;
-        if constexpr (TMA_OUT) epilogue_tma<EK>(p, &tmO, tn0, m0, r, v, brow, stg_raw, xch, ebuf);
-        else epilogue_chunk(p, tn0, m0, nc, r, v, stage);
+        epilogue_chunk(p, tn0, tm0 * BN + rank * cpr + cc, nc, r, v, stage);
       }
-      if (TMA_OUT && threadIdx.x == 64) bulk_wait_read<0>();
     }
   }
   if (warp == 1) {
@@ -1214,7 +1163,7 @@ TcKernel tc_kernel(int red, int ek) {
   if (red == R && ek == E) return tc_gemm_kernel<R, E>;
   RAVEL_TC_K(RED_NONE, EK_F32) RAVEL_TC_K(RED_NONE, EK_BF16) RAVEL_TC_K(RED_NONE, EK_ADD)
   RAVEL_TC_K(RED_NONE, EK_GEGLU) RAVEL_TC_K(RED_NONE, EK_GENERIC)
-  RAVEL_TC_K(RED_L2_CLUSTER, EK_TMA_ANY) RAVEL_TC_K(RED_L2_CLUSTER, EK_GENERIC)
+  RAVEL_TC_K(RED_L2_CLUSTER, EK_GENERIC)
   RAVEL_TC_K(RED_DSMEM, EK_TMA_ANY) RAVEL_TC_K(RED_DSMEM32, EK_TMA_ANY)
 #undef RAVEL_TC_K
   return nullptr;
@@ -1274,49 +1223,74 @@ cudaError_t encode_out(CUtensorMap* m, void* base, int rows, int cols, int ld, b
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Token-tile width: up to 128 tokens, the smallest of 32, 48, .., 128 (the
-// MMA's N steps by 16) that holds M; beyond 128 tokens, the multiple of 16 in
-// [128, 256] whose tile count fills whole waves of the SMs best (per-CTA work
-// ~ waves x BN), larger BN on ties.
-int pick_bn(int M, int tiles_n, int num_sms) {
-  if (M <= 128) return std::max(32, (M + 15) / 16 * 16);
-  int best = 256;
-  long best_cost = -1;
-  for (int bn = 256; bn >= 128; bn -= 16) {
-    const long tiles = (long)tiles_n * ((M + bn - 1) / bn);
-    const long waves = (tiles + num_sms - 1) / num_sms;
-    const long cost = waves * bn;
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = bn;
-    }
-  }
-  return best;
-}
-
-int g_max_cluster = 8;   // largest power-of-two cluster the split-K reduction may use
 std::atomic<int> g_withhold{0};   // launches left to run with a withheld arrival (fault injection)
 constexpr unsigned long long kWithholdWaitNs = 2000000ull;   // their wait limit: 2 ms
-bool g_pair_gemm = true;  // persistent launches of many tiles on SM pairs
-int g_pair_bn_max = 256;  // widest token tile of a pair launch
 
-// Two-SM launch of a persistent GEMM (see tc_gemm_pair_kernel): token-tile
-// width BN (a multiple of 32 in [128, 256]) minimising waves x (BN + 64) --
-// the work of a pair's tiles plus a fixed cost per tile of about 64 token
-// columns (accumulator hand-off and epilogue pipeline, ~1 us) -- larger BN on
-// ties; then the usual TMA epilogue layout.
-int pick_bn_pair(int M, int tiles_n2, int slots) {
-  int bn = 256;
-  long best = -1;
-  for (int c = g_pair_bn_max; c >= 128; c -= 32) {
-    const long tiles = (long)tiles_n2 * ((M + c - 1) / c);
-    const long cost = (tiles + slots - 1) / slots * (c + 64);
-    if (best < 0 || cost < best) {
-      best = cost;
-      bn = c;
+// Resident clusters of 2, 4, 8, 16 split CTAs (one CTA per SM; 0: that
+// cluster size is not to be had).  The split-K kernels take a whole SM each,
+// and clusters stay inside a GPC: 76, 36, 15 and 7 on this part.
+int g_max_clusters[4] = {0, 0, 0, 0};
+
+// How a GEMM is cut: token-tile width, K splits (a cluster), or SM pairs.
+struct TcPlan {
+  bool pair = false;
+  int bn = 0, splits = 1;
+};
+
+// The plan of least estimated time.  The estimate, in microseconds, was fitted
+// to 3,900 measured launches (a chain of dependent launches with weights from
+// HBM; N x K of 2560 x 1024, 1024 x 2048, 8192 x 1024, 1024 x 4096, 1536 x
+// 1024, 1024 x 1024, 2048 x 1024 and 75776 x 1024, 8 to 4224 tokens, all
+// widths and splits): a launch costs a fixed 2.6 (SM pairs: 3.4), its
+// epilogue grows with the tile width (GeGLU's more), a k-tile takes as long as
+// its operands need to arrive (168 GB/s per SM, 142 in pairs, whose MMA then
+// needs 0.295 at 256 tokens), splits add their exchange, and clusters that do
+// not fit at once add a wave.  Over the measured shapes the plan chosen is
+// 0.7 % slower than the best measured one; the widest-tile-and-most-splits
+// rule before it was 19 % slower (M 50 x N 1024 x K 2048: 16 splits, 5.9 us;
+// now 4 splits, 3.8 us; M 240 x 1024 x 4096: 12.4, now 7.3 us).
+TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t ws_bytes, bool pairs, int num_sms) {
+  const int tiles_n = (N + TC_BM - 1) / TC_BM, num_kb = (K + TC_BK - 1) / TC_BK;
+  TcPlan best;
+  float cost = 3.4e38f;
+  auto consider = [&](bool pair, int bn, int splits, float t) {
+    if (t < cost) {
+      cost = t;
+      best.pair = pair;
+      best.bn = bn;
+      best.splits = splits;
+    }
+  };
+  // (tiles wider than the tokens, rounded up to the MMA's step, only pad)
+  const int bn_max = std::min(256, std::max(32, (M + 15) / 16 * 16));
+  for (int bn = 32; bn <= bn_max; bn += 16) {
+    const int tiles = tiles_n * ((M + bn - 1) / bn);
+    const float step = (float)((128 + bn) * 128) / 168e3f, epi = 0.0135f * (float)bn * (geglu ? 2.18f : 1.f);
+    const int waves = (tiles + num_sms - 1) / num_sms;
+    consider(false, bn, 1,
+             2.6f + epi + (float)waves * (float)num_kb * step + (float)(waves - 1) * 0.0067f * (float)bn);
+    for (int i = 0; i < 4; ++i) {
+      // the splits of a tile form one cluster; each sums a slice of whole
+      // 4-token groups, of at most 32 tokens through shared memory, and
+      // through L2 the partials have to fit the workspace
+      const int sp = 2 << i;
+      if (sp > num_kb || bn % (4 * sp) || !g_max_clusters[i] || (long)tiles * sp > 2L * num_sms) break;
+      if (dsmem ? bn / sp > 32 : (size_t)sp * tiles * bn * TC_BM * 4 > ws_bytes) continue;
+      const int w = (tiles + g_max_clusters[i] - 1) / g_max_clusters[i];
+      consider(false, bn, sp,
+               2.6f + epi / (float)sp + (float)w * (float)((num_kb + sp - 1) / sp) * step +
+                   1.07f * (float)(bn * (xbf16 ? 1 : 2)) / 64.f + (float)(w - 1) * 2.5f);
     }
   }
-  return bn;
+  const int tiles_n2 = (N + 2 * TC_BM - 1) / (2 * TC_BM), slots = num_sms / 2;
+  for (int bn = 64; pairs && bn <= std::max(64, std::min(256, (M + 31) / 32 * 32)); bn += 32) {
+    const int waves = (tiles_n2 * ((M + bn - 1) / bn) + slots - 1) / slots;
+    const float step = std::max((float)((128 + bn / 2) * 128) / 142e3f, 0.295f * (float)bn / 256.f);
+    consider(true, bn, 1,
+             3.4f + 0.0119f * (float)bn * (geglu ? 1.35f : 1.f) + (float)waves * (float)num_kb * step +
+                 (float)(waves - 1) * 1.1f);
+  }
+  return best;
 }
 
 // The tensor cores truncate each fp32 accumulation, so a sum's error grows
@@ -1328,12 +1302,14 @@ int pick_bn_pair(int M, int tiles_n2, int slots) {
 // 2e-3.
 bool short_sums(const GemmArgs& g) { return !g.xbf16 && (g.epi == EPI_ADD_F32 || (g.epi != EPI_GEGLU && g.out_dt == DT_F32)); }
 
+// Two-SM launch of a persistent GEMM (see tc_gemm_pair_kernel) with token
+// tiles of bn (a multiple of 32 in [64, 256]) and the usual TMA epilogue
+// layout.
 cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st, int ek,
-                             bool out_bf, int es) {
+                             bool out_bf, int es, int bn) {
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
   const int tiles_n2 = (g.N + 2 * TC_BM - 1) / (2 * TC_BM);
   const int slots = num_sms / 2;
-  const int bn = pick_bn_pair(g.M, tiles_n2, slots);
   const int tiles_m = (g.M + bn - 1) / bn;
   const int num_tiles = tiles_n2 * tiles_m;
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
@@ -1391,21 +1367,21 @@ cudaError_t init_tc_gemm() {
   // clusters of 16 are beyond the portable limit: use them only if allowed
   bool big = true;
   for (const void* k : kernels) big = big && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-  if (big) {
+  for (int i = 0; i < (big ? 4 : 3); ++i) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 1;
     attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 16;
-    cfg.gridDim = dim3(1, 1, 16);
+    attr.val.clusterDim.z = 2u << i;
+    cfg.gridDim = dim3(1, 1, 2u << i);
     cfg.blockDim = dim3(TC_THREADS);
     cfg.dynamicSmemBytes = TC_SMEM_MAX;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_kernel(RED_L2_CLUSTER, EK_GENERIC), &cfg) == cudaSuccess && n > 0)
-      g_max_cluster = 16;
+    g_max_clusters[i] =
+        cudaOccupancyMaxActiveClusters(&n, tc_kernel(RED_DSMEM, EK_TMA_ANY), &cfg) == cudaSuccess && n > 0 ? n : 0;
   }
   cudaGetLastError();
   return cudaSuccess;
@@ -1421,37 +1397,20 @@ bool tc_gemm_supported(const GemmArgs& g) {
 
 cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st) {
   if (!g_encode) return cudaErrorInitializationError;
+  // outputs through TMA boxes when the output rows are 16-byte aligned
+  const bool out_bf = g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16);
+  const int es = out_bf ? 2 : 4;
+  const bool tma_out = ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * es) % 16 == 0;
+  const TcPlan plan = plan_gemm(g.M, g.N, g.K, g.epi == EPI_GEGLU, g.xbf16 != 0, tma_out, ws.ws_bytes, tma_out, num_sms);
+  if (plan.pair)
+    return launch_gemm_pair(g, ws, num_sms, st,
+                            g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32,
+                            out_bf, es, plan.bn);
+  const int bn = plan.bn, splits = plan.splits;
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
-  const int bn = pick_bn(g.M, tiles_n, num_sms);
   const int tiles_m = (g.M + bn - 1) / bn;
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
   const int tiles = tiles_n * tiles_m;
-  int splits = 1;
-  if (tiles < num_sms) splits = std::min(num_kb, std::max(1, num_sms / tiles));
-  if (g.max_splits > 0) splits = std::min(splits, g.max_splits);
-  // the splits of a tile form one cluster: a power of two, at most the cluster
-  // limit, whose partials fit the workspace and whose column slices are
-  // multiples of 4
-  int c = 1;
-  while (c * 2 <= std::min(splits, g_max_cluster) && (bn / (c * 2)) % 4 == 0 &&
-         (size_t)(c * 2) * tiles * bn * TC_BM * 4 <= ws.ws_bytes)
-    c *= 2;
-  splits = c;
-  int reduce = splits == 1 ? RED_NONE : RED_L2_CLUSTER;
-  {
-    // two-SM tiles for a persistent launch whose pair tiles fill at least
-    // three quarters of the pairs of SMs
-    const bool obf = g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16);
-    const int oes = obf ? 2 : 4;
-    const bool aligned = ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * oes) % 16 == 0;
-    const int tn2 = (g.N + 2 * TC_BM - 1) / (2 * TC_BM), slots = num_sms / 2;
-    const int pbn = pick_bn_pair(g.M, tn2, slots);
-    const long pair_tiles = (long)tn2 * ((g.M + pbn - 1) / pbn);
-    if (g_pair_gemm && splits == 1 && aligned && 4 * pair_tiles >= 3 * slots) {
-      const int ek = g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : obf ? EK_BF16 : EK_F32;
-      return launch_gemm_pair(g, ws, num_sms, st, ek, obf, oes);
-    }
-  }
   const int cpr = bn / splits;   // a multiple of 4 whenever the splits form a cluster
   uint32_t acc_cols = 32;
   while ((int)acc_cols < bn) acc_cols <<= 1;
@@ -1474,40 +1433,25 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
                        (size_t)kb_per_item * stage_bytes <= (size_t)TC_SMEM_BUDGET;
   if (oneshot) stages = kb_per_item;   // the ring is exactly one box deep
   const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
-  // outputs through TMA boxes when the output rows are 16-byte aligned
-  const bool out_bf = g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16);
-  const int es = out_bf ? 2 : 4;
-  const bool tma_out = ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * es) % 16 == 0;
-  int box_m = 0;
   // partials exchanged in bf16 where the caller allows it, else in fp32
   const bool xbf = g.xbf16 != 0;
-  uint32_t box_bytes = 0, stg_off = (uint32_t)ring, xch_off = 0, rcv_off = 0, bar_off = 0;
-  size_t smem = 0;
-  auto layout = [&](bool dsmem) {
-    box_m = splits == 1 ? 16
-            : (tma_out && cpr <= 32 && (dsmem || (cpr > 8 && cpr % 16 != 0))) ? cpr   // the whole slice in one box
-            : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
-    box_bytes = (uint32_t)(((size_t)box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
-    const size_t stg_bytes = tma_out ? 2 * (size_t)box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
-    const size_t xch_bytes = (tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
-    // received partials (all splits' slices of this rank) overlay the operand
-    // ring, else the boxes + exchange
-    const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
-    const bool in_ring = rcv_bytes <= ring;
-    xch_off = stg_off + (uint32_t)stg_bytes;
-    rcv_off = in_ring ? 0u : stg_off;
-    bar_off = stg_off + (uint32_t)std::max(stg_bytes + xch_bytes, in_ring ? (size_t)0 : rcv_bytes);
-    smem = 1024 + bar_off + (size_t)(2 * stages + 5) * 8 + 4 + 16 + 64;
-  };
-  // partials by st.async into the owning rank's shared memory when the token
-  // slice fits one output box (<= 32 tokens) and the receive area fits
-  bool dsmem = reduce == RED_L2_CLUSTER && tma_out && cpr <= 32;
-  layout(dsmem);
-  if (dsmem && smem > (size_t)TC_SMEM_MAX) {
-    dsmem = false;
-    layout(false);
-  }
-  if (dsmem) reduce = xbf ? RED_DSMEM : RED_DSMEM32;
+  const bool dsmem = splits > 1 && tma_out;
+  const int reduce = splits == 1 ? RED_NONE : !dsmem ? RED_L2_CLUSTER : xbf ? RED_DSMEM : RED_DSMEM32;
+  // tokens per output box: a split's whole slice through shared memory
+  const int box_m = splits == 1 ? 16 : dsmem ? cpr : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
+  const uint32_t box_bytes =
+      (uint32_t)(((size_t)box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
+  const size_t stg_bytes = tma_out ? 2 * (size_t)box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
+  const size_t xch_bytes = (tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
+  // received partials (all splits' slices of this rank) overlay the operand
+  // ring, else the boxes + exchange
+  const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
+  const bool in_ring = rcv_bytes <= ring;
+  const uint32_t stg_off = (uint32_t)ring, xch_off = stg_off + (uint32_t)stg_bytes;
+  const uint32_t rcv_off = in_ring ? 0u : stg_off;
+  const uint32_t bar_off = stg_off + (uint32_t)std::max(stg_bytes + xch_bytes, in_ring ? (size_t)0 : rcv_bytes);
+  const size_t smem = 1024 + bar_off + (size_t)(2 * stages + 5) * 8 + 4 + 16 + 64;
+  if (smem > (size_t)TC_SMEM_MAX) return cudaErrorInvalidConfiguration;
   CUtensorMap mw, mx, mo;
   memset(&mo, 0, sizeof(mo));
   cudaError_t e = oneshot ? encode_kt(&mw, g.W, g.N, g.K, g.ldw, TC_BM, kb_per_item)

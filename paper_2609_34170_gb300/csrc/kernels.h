@@ -83,7 +83,6 @@ struct GemmArgs {
   void* out; int ldo;           // EPI_STORE*: dtype `out_dt`; EPI_ADD_F32: float, += result
   Dtype out_dt;
   const float* bias;            // [N] or null
-  int max_splits = 0;           // tcgen05 path: cap on the split-K factor (0: chosen from the shape)
   const int* skip = nullptr;    // optional device flag: nonzero at run time -> the launch computes nothing
   // tcgen05 split-K inside a cluster: the splits' partials may travel between
   // the SMs in bf16 (half the bytes of fp32; the sum itself stays fp32), which

@@ -308,9 +308,8 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     }                                   \
   } while (0)
   auto gemm = [&](const void* Aop, int lda, const void* W, int M, int N, int K, Epi epi, void* out, int ldo,
-                  Dtype out_dt, const float* bias, int split_cap = 0, const int* skip = nullptr, int xbf16 = 0) {
+                  Dtype out_dt, const float* bias, const int* skip = nullptr, int xbf16 = 0) {
     GemmArgs g{Aop, lda, W, K, M, N, K, epi, out, ldo, out_dt, bias};
-    g.max_splits = split_cap;
     g.skip = skip;
     g.xbf16 = xbf16;
     return run_gemm(p, g, st);
@@ -335,13 +334,13 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
   RUN(KK_COND_CACHE, launch_cond_check(ca, st));
   pdl_enabled() = p.use_pdl && !trace;
   RUN(KK_EMBED, launch_embed(io.slot_times, Ht, io.delta, B, D, p.omega, p.E, dt, st, skip));
-  RUN(KK_GEMM_COND, gemm(p.E, D, p.t_w1, Ht, D, D, EPI_STORE_SILU, p.H1, D, dt, p.t_b1, 0, skip));
+  RUN(KK_GEMM_COND, gemm(p.E, D, p.t_w1, Ht, D, D, EPI_STORE_SILU, p.H1, D, dt, p.t_b1, skip));
   RUN(KK_GEMM_COND, gemm(rowp(p.E, Ht, D), D, p.d_w1, B, D, D, EPI_STORE_SILU, (void*)rowp(p.H1, Ht, D), D, dt, p.d_b1,
-                         0, skip));
-  RUN(KK_GEMM_COND, gemm(p.H1, D, p.t_w2, Ht, D, D, EPI_STORE, p.HC, D, dt, p.t_b2, 0, skip));
-  RUN(KK_GEMM_COND, gemm(rowp(p.H1, Ht, D), D, p.d_w2, B, D, D, EPI_STORE, (void*)rowp(p.HC, Ht, D), D, dt, p.d_b2, 0,
                          skip));
-  RUN(KK_GEMM_MOD, gemm(p.HC, D, p.mod_w, Ht + B, p.mod_dim, D, EPI_STORE, p.modv, p.mod_dim, DT_F32, nullptr, 0,
+  RUN(KK_GEMM_COND, gemm(p.H1, D, p.t_w2, Ht, D, D, EPI_STORE, p.HC, D, dt, p.t_b2, skip));
+  RUN(KK_GEMM_COND, gemm(rowp(p.H1, Ht, D), D, p.d_w2, B, D, D, EPI_STORE, (void*)rowp(p.HC, Ht, D), D, dt, p.d_b2,
+                         skip));
+  RUN(KK_GEMM_MOD, gemm(p.HC, D, p.mod_w, Ht + B, p.mod_dim, D, EPI_STORE, p.modv, p.mod_dim, DT_F32, nullptr,
                         skip));
   RUN(KK_COND_CACHE, launch_cond_commit(ca, st));
   // residual stream
@@ -371,7 +370,6 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     if (p.use_tc_attn) {
       // the tensor-core attention reads K and V straight from the QKV rows
       GemmArgs gq{p.Y, D, wqkv, D, BY, p.nqkv, D, EPI_STORE, p.QKV, p.nqkv, dt, nullptr};
-      gq.max_splits = p.split_cap[0];
       gq.xbf16 = 1;
       RUN(KK_GEMM_QKV, run_gemm(p, gq, st));
       AttnTcArgs at{p.QKV, p.nqkv, {p.ctx_k[0], p.ctx_k[1]}, {p.ctx_v[0], p.ctx_v[1]}, L, l,
@@ -388,7 +386,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
       RUN(KK_ATTENTION, launch_attention_simt(at, dt, st));
     }
     RUN(KK_GEMM_O, gemm(p.O, p.qdim, (const char*)p.w_o + (size_t)l * D * p.qdim * es, BH, D, p.qdim, EPI_ADD_F32, p.x,
-                        D, DT_F32, nullptr, p.split_cap[1], nullptr, 1));
+                        D, DT_F32, nullptr, nullptr, 1));
     if (adapters && (l + 1) % c.fop_adapter_every == 0) {
       // gated cross-attention adapter: the action rows attend to the FOP tokens
       const int ai = (l + 1) / c.fop_adapter_every - 1, nkv = 2 * c.n_kv_heads * c.head_dim;
@@ -411,7 +409,6 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     RUN(KK_NORM, launch_ada_norm(n2, dt, st));
     const void* wgu = (const char*)p.w_gu + (size_t)l * 2 * Fm * D * es;
     GemmArgs gu{p.Y, D, wgu, D, BH, 2 * Fm, D, EPI_GEGLU, p.Hm, Fm, dt, nullptr};
-    gu.max_splits = p.split_cap[2];
     gu.xbf16 = 1;
     if (p.use_tc && tc_gemm_supported(gu)) {
       RUN(KK_GEMM_GATE_UP, launch_gemm_tc(gu, p.tcws, p.num_sms, st));   // GeGLU fused in the epilogue
@@ -420,7 +417,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
       RUN(KK_GEGLU, launch_geglu(p.GU, BH, Fm, p.Hm, dt, st));
     }
     RUN(KK_GEMM_DOWN, gemm(p.Hm, Fm, (const char*)p.w_down + (size_t)l * D * Fm * es, BH, D, Fm, EPI_ADD_F32, p.x, D,
-                           DT_F32, nullptr, p.split_cap[3], nullptr, 1));
+                           DT_F32, nullptr, nullptr, 1));
   }
   if (!dn && dt == DT_BF16 && A <= 32 && D % 4 == 0) {
     // final norm, velocity head and tail in one launch, about eight CTAs per SM

@@ -59,6 +59,28 @@ def test_gemm_bf16(handles, M, N, K, epi):
     np.testing.assert_allclose(got, ref, rtol=1e-4, atol=1e-4 * scale)
 
 
+# Token counts between one robot's and many robots': every kind of plan (token
+# tiles of 32 to 256, 1 to 8 splits with slices of 8 to 32 tokens, SM pairs with
+# narrow tiles, several TMEM accumulators per item) with a ragged last tile.
+# Tolerance: fp32 sums of K products of N(0, 1) and N(0, 0.05^2), as above.
+@pytest.mark.parametrize("M", [33, 100, 137, 240, 431, 601, 1300, 1999])
+@pytest.mark.parametrize("N,K", [(1024, 2048), (1024, 4096), (1536, 1024), (2500, 1032)])
+def test_gemm_bf16_plans(handles, M, N, K):
+    from paper_2609_34170_gb300 import ravel_gemm
+    g = torch.Generator("cuda").manual_seed(M * N + K)
+    X = torch.randn((M, K), generator=g, device="cuda").bfloat16()
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.05).bfloat16()
+    out = torch.randn((M, N), generator=g, device="cuda")
+    ref = (X.double() @ W.double().T + out.double()).cpu().numpy()
+    ravel_gemm(handles["bf16"], X, W, 2, out)
+    scale = np.sqrt(K) * 0.05 + 1
+    np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-4, atol=1e-4 * scale)
+    half = torch.empty((M, N), device="cuda", dtype=torch.bfloat16)
+    ravel_gemm(handles["bf16"], X, W, 0, half)
+    np.testing.assert_allclose(half.float().cpu().numpy(), (X.double() @ W.double().T).cpu().numpy(), rtol=1e-2,
+                               atol=1e-2 * scale)
+
+
 @pytest.mark.parametrize("M,N,K", [(50, 256, 1024), (50, 8192, 1024), (66, 4096, 1024), (66, 8192, 1024),
                                    (300, 1024, 256), (3200, 2048, 1024), (3200, 8192, 1024)])
 @pytest.mark.parametrize("with_bias", [False, True])
