@@ -1248,7 +1248,14 @@ struct TcPlan {
 // not fit at once add a wave.  Over the measured shapes the plan chosen is
 // 0.7 % slower than the best measured one; the widest-tile-and-most-splits
 // rule before it was 19 % slower (M 50 x N 1024 x K 2048: 16 splits, 5.9 us;
-// now 4 splits, 3.8 us; M 240 x 1024 x 4096: 12.4, now 7.3 us).
+// now 4.1 us; M 240 x 1024 x 4096: 12.4, now 7.3 us).  Inside a step (xbf16)
+// the neighbours of a launch are other kernels: there the exchange of bf16
+// shares weighs less, an unsplit launch 0.3 more (its code is another
+// binary's than the split launches'), and split CTAs past half the SMs, which
+// the next kernel could have started on, up to 0.7 more.  Whole steps at 1 to
+// 64 robots, each projection's width and splits varied in turn: the rule is
+// 0 to 3.5 % of the step away from the best combination (batch 1 at it: 652
+// us, 685 with the chain's terms alone).
 TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t ws_bytes, bool pairs, int num_sms) {
   const int tiles_n = (N + TC_BM - 1) / TC_BM, num_kb = (K + TC_BK - 1) / TC_BK;
   TcPlan best;
@@ -1268,7 +1275,7 @@ TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t
     const float step = (float)((128 + bn) * 128) / 168e3f, epi = 0.0135f * (float)bn * (geglu ? 2.18f : 1.f);
     const int waves = (tiles + num_sms - 1) / num_sms;
     consider(false, bn, 1,
-             2.6f + epi + (float)waves * (float)num_kb * step + (float)(waves - 1) * 0.0067f * (float)bn);
+             (xbf16 ? 2.9f : 2.6f) + epi + (float)waves * (float)num_kb * step + (float)(waves - 1) * 0.0067f * (float)bn);
     for (int i = 0; i < 4; ++i) {
       // the splits of a tile form one cluster; each sums a slice of whole
       // 4-token groups, of at most 32 tokens through shared memory, and
@@ -1279,7 +1286,8 @@ TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t
       const int w = (tiles + g_max_clusters[i] - 1) / g_max_clusters[i];
       consider(false, bn, sp,
                2.6f + epi / (float)sp + (float)w * (float)((num_kb + sp - 1) / sp) * step +
-                   1.07f * (float)(bn * (xbf16 ? 1 : 2)) / 64.f + (float)(w - 1) * 2.5f);
+                   (xbf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * 2.5f +
+                   (xbf16 ? 0.7f * (float)std::max(0, tiles * sp - num_sms / 2) / (float)(num_sms / 2) : 0.f));
     }
   }
   const int tiles_n2 = (N + 2 * TC_BM - 1) / (2 * TC_BM), slots = num_sms / 2;
