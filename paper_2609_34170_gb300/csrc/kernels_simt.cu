@@ -195,6 +195,14 @@ cudaError_t launch_cond_commit(const CondArgs& a, cudaStream_t st) {
   return launch_kernel(cond_commit_kernel, dim3(64), dim3(256), 0, st, 1, a);
 }
 
+// four consecutive values as fp32 (16- / 8-byte aligned)
+__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+  const uint2 u = *(const uint2*)p;
+  const __nv_bfloat162 lo = *(const __nv_bfloat162*)&u.x, hi = *(const __nv_bfloat162*)&u.y;
+  return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
+}
+
 // ============================================================================ GEMM (SIMT)
 
 // 64x64 output tile, K step 32, 256 threads, 4x4 outputs per thread spread
@@ -253,6 +261,85 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
   }
 }
 
+// Few rows (the fp32 mode's small experts): a warp owns 8 rows x 2 columns, its
+// lanes split K in float4 steps, so W streams once per 8 rows in 512-byte
+// requests and the rows come from L1 (the 8 warps of a block read the same
+// ones); the 16 sums then halve across the lanes.  Bound by load latency and
+// the L1: at M 10, K 1024 the tile kernel above, whose only CTAs walk K in
+// serial 32-wide steps with two barriers each, takes 75 us, this one 4.
+constexpr int RG_M = 8, RG_N = 2, RG_WARPS = 8;
+
+template <int EPI, typename TO>
+__global__ void __launch_bounds__(RG_WARPS * 32) gemm_rows_kernel(const float* __restrict__ A, int lda,
+                                                                  const float* __restrict__ W, int ldw, int M, int N,
+                                                                  int K, TO* __restrict__ out, int ldo,
+                                                                  const float* __restrict__ bias,
+                                                                  const int* __restrict__ skip) {
+  pdl_trigger();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.y * RG_M, n0 = (blockIdx.x * RG_WARPS + warp) * RG_N;
+  const int mr = min(RG_M, M - m0);
+  const float* w0 = W + (size_t)min(n0, N - 1) * ldw;
+  const float* w1 = W + (size_t)min(n0 + 1, N - 1) * ldw;
+  pdl_wait();
+  if (skip && *skip) return;
+  float acc[RG_M][RG_N] = {};
+  for (int k = 4 * lane; k < K; k += 128) {
+    const float4 wa = ld4(w0 + k), wb = ld4(w1 + k);
+#pragma unroll
+    for (int r = 0; r < RG_M; ++r) {
+      if (r >= mr) break;
+      const float4 x = ld4(A + (size_t)(m0 + r) * lda + k);
+      acc[r][0] = fmaf(x.x, wa.x, fmaf(x.y, wa.y, fmaf(x.z, wa.z, fmaf(x.w, wa.w, acc[r][0]))));
+      acc[r][1] = fmaf(x.x, wb.x, fmaf(x.y, wb.y, fmaf(x.z, wb.z, fmaf(x.w, wb.w, acc[r][1]))));
+    }
+  }
+  // lanes 2i and 2i + 1 end with the warp's sum i (row i / 2, column i % 2):
+  // each step keeps half of the sums and adds the partner's half
+  float v[RG_M * RG_N];
+#pragma unroll
+  for (int i = 0; i < RG_M * RG_N; ++i) v[i] = acc[i / RG_N][i % RG_N];
+#pragma unroll
+  for (int off = 16; off >= 2; off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < off / 2; ++i) {
+      const float send = up ? v[i] : v[i + off / 2];
+      const float keep = up ? v[i + off / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  float t = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+  const int m = m0 + (lane >> 2), n = n0 + ((lane >> 1) & 1);
+  if ((lane & 1) || (lane >> 2) >= mr || n >= N) return;
+  t += bias ? bias[n] : 0.f;
+  if (EPI == EPI_STORE_SILU) t = silu_f(t);
+  TO* o = out + (size_t)m * ldo + n;
+  if (EPI == EPI_ADD_F32) *(float*)o += t;
+  else *o = from_f32<TO>(t);
+}
+
+// The row kernel re-reads W for every 8 rows (from L2): up to 256 rows, where
+// the tile kernel would leave SMs idle.
+static bool rows_gemm_supported(const GemmArgs& g) {
+  return g.M <= 256 && g.K % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
+         (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
+}
+
+template <int EPI, typename TO>
+static cudaError_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st) {
+  const dim3 grid((g.N + RG_WARPS * RG_N - 1) / (RG_WARPS * RG_N), (g.M + RG_M - 1) / RG_M);
+  return launch_kernel(gemm_rows_kernel<EPI, TO>, grid, dim3(RG_WARPS * 32), 0, st, 1, (const float*)g.A, g.lda,
+                       (const float*)g.W, g.ldw, g.M, g.N, g.K, (TO*)g.out, g.ldo, g.bias, g.skip);
+}
+
+static cudaError_t gemm_rows_dispatch(const GemmArgs& g, cudaStream_t st) {
+  if (g.epi == EPI_ADD_F32) return launch_gemm_rows<EPI_ADD_F32, float>(g, st);
+  if (g.out_dt == DT_BF16)
+    return g.epi == EPI_STORE_SILU ? launch_gemm_rows<EPI_STORE_SILU, bf16>(g, st) : launch_gemm_rows<EPI_STORE, bf16>(g, st);
+  return g.epi == EPI_STORE_SILU ? launch_gemm_rows<EPI_STORE_SILU, float>(g, st) : launch_gemm_rows<EPI_STORE, float>(g, st);
+}
+
 template <typename T>
 static cudaError_t gemm_simt_dispatch(const GemmArgs& g, cudaStream_t st) {
   dim3 grid((g.N + 63) / 64, (g.M + 63) / 64);
@@ -281,12 +368,12 @@ static cudaError_t gemm_simt_dispatch(const GemmArgs& g, cudaStream_t st) {
 
 cudaError_t launch_gemm_simt(const GemmArgs& g, Dtype dt, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  if (dt == DT_F32 && rows_gemm_supported(g)) return gemm_rows_dispatch(g, st);
   return dt == DT_BF16 ? gemm_simt_dispatch<bf16>(g, st) : gemm_simt_dispatch<float>(g, st);
 }
 
 // ============================================================================ adaRMSNorm
 
-__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
 __device__ __forceinline__ float4 add3(float4 a, float4 b, float4 c) {
   return make_float4(a.x + b.x + c.x, a.y + b.y + c.y, a.z + b.z + c.z, a.w + b.w + c.w);
 }
@@ -301,11 +388,6 @@ __device__ __forceinline__ void st4(bf16* p, float4 v) {
 
 __device__ __forceinline__ float4 add2(float4 a, float4 b) {
   return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
-__device__ __forceinline__ float4 ld4(const bf16* p) {
-  const uint2 u = *(const uint2*)p;
-  const __nv_bfloat162 lo = *(const __nv_bfloat162*)&u.x, hi = *(const __nv_bfloat162*)&u.y;
-  return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
 }
 
 // adaRMSNorm over a block of rows of one robot (Sec. 3.1, Eq. 2):
@@ -622,7 +704,12 @@ cudaError_t launch_geglu(const float* GU, int M, int Fm, void* Hm, Dtype dt, cud
 // One CTA per (robot b, KV head g, tile of QT query rows).  Query row r of a
 // (b, g) pair is slot j = r / G of query head g*G + r % G.  Keys are visited
 // in chunks of KT: [0, P) the active context's prefix, [P, P+F) the FOP
-// tokens, [P+F, P+F+H) the action slots; online softmax in fp32.
+// tokens, [P+F, P+F+H) the action slots; online softmax in fp32.  Eight
+// threads copy a key's K and V row in float4 steps; rows of Q and K are padded
+// by four floats, so that the 16-byte reads of a score (8 keys per phase) fall
+// into distinct banks.  (Unpadded rows put the 16 keys of a request into one
+// bank, and an integer division found every element's row: 40 us at 40 query
+// rows, 78 keys and head dim 64, against 8 now.)
 constexpr int ATT_QT = 16, ATT_KT = 32, ATT_THREADS = 256;
 
 template <typename T>
@@ -630,10 +717,10 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
   pdl_trigger();
   pdl_wait();
   extern __shared__ float sm[];
-  const int hd = a.hd;
-  float* Qs = sm;                      // [QT][hd]
-  float* Ks = Qs + ATT_QT * hd;        // [KT][hd]
-  float* Vs = Ks + ATT_KT * hd;        // [KT][hd]
+  const int hd = a.hd, ld = hd + 4;
+  float* Qs = sm;                      // [QT][hd + 4]
+  float* Ks = Qs + ATT_QT * ld;        // [KT][hd + 4]
+  float* Vs = Ks + ATT_KT * ld;        // [KT][hd]
   float* Ss = Vs + ATT_KT * hd;        // [QT][KT]
   const int bg = blockIdx.x;
   const int b = bg / a.Hkv, g = bg % a.Hkv;
@@ -654,57 +741,59 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
   const int nk = P + a.F + a.H;
   const int rpr = a.H + a.F;   // QKV rows per robot: H action slots, then F FOP tokens
   const float scale = rsqrtf((float)hd);
-
-  for (int i = threadIdx.x; i < ATT_QT * hd; i += ATT_THREADS) {
-    const int rr = i / hd, c = i % hd, r = r0 + rr;
-    float v = 0.f;
-    if (r < nrows) {
-      const int j = r / G, h = g * G + r % G;
-      v = to_f32(qkv[(size_t)(b * rpr + j) * a.ld_qkv + h * hd + c]);
-    }
-    Qs[i] = v * scale;
+  // 16 threads per query row: its Q, its scores (keys qlane, qlane + 16), its
+  // softmax and its output columns qlane + 16 i
+  const int qrow = threadIdx.x >> 4, qlane = threadIdx.x & 15;
+  const int r = r0 + qrow, j = r < nrows ? r / G : -1, h = g * G + r % G;
+  for (int c = 4 * qlane; c < hd; c += 64) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < nrows) v = ld4(qkv + (size_t)(b * rpr + j) * a.ld_qkv + h * hd + c);
+    st4(Qs + qrow * ld + c, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
   }
-  // thread layout for scores / softmax: 16 threads per query row
-  const int srow = threadIdx.x >> 4, slane = threadIdx.x & 15;
   float m_run = -INFINITY, l_run = 0.f;
-  // output accumulators: row orow, columns ocol + 16*i
-  const int orow = threadIdx.x >> 4, ocol = threadIdx.x & 15;
   float acc[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-  const int qrow_slot = (r0 + srow < nrows) ? (r0 + srow) / G : -1;
 
   for (int k0 = 0; k0 < nk; k0 += ATT_KT) {
     __syncthreads();
-    for (int i = threadIdx.x; i < ATT_KT * hd; i += ATT_THREADS) {
-      const int kk = i / hd, c = i % hd, key = k0 + kk;
-      float kv = 0.f, vv = 0.f;
+    {
+      const int kk = threadIdx.x >> 3, key = k0 + kk;
+      const T *kr = nullptr, *vr = nullptr;
       if (key < P) {
-        kv = to_f32(pk[(size_t)key * hd + c]);
-        vv = to_f32(pv[(size_t)key * hd + c]);
-      } else if (key < P + a.F) {
-        const size_t row = (size_t)(b * rpr + a.H + (key - P)) * a.ld_qkv;
-        kv = to_f32(qkv[row + kofs + c]);
-        vv = to_f32(qkv[row + vofs + c]);
-      } else if (key < nk) {
-        const size_t row = (size_t)(b * rpr + (key - P - a.F)) * a.ld_qkv;
-        kv = to_f32(qkv[row + kofs + c]);
-        vv = to_f32(qkv[row + vofs + c]);
+        kr = pk + (size_t)key * hd;
+        vr = pv + (size_t)key * hd;
+      } else if (key < nk) {   // the step's own rows: FOP tokens, then slots
+        const int row = key < P + a.F ? a.H + (key - P) : key - P - a.F;
+        kr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + kofs;
+        vr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + vofs;
       }
-      Ks[i] = kv;
-      Vs[i] = vv;
+      for (int c = 4 * (threadIdx.x & 7); c < hd; c += 32) {
+        float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
+        if (kr) {
+          kv = ld4(kr + c);
+          vv = ld4(vr + c);
+        }
+        st4(Ks + kk * ld + c, kv);
+        st4(Vs + kk * hd + c, vv);
+      }
     }
     __syncthreads();
-    // scores: row srow, keys slane and slane + 16
     float s[2];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-      const int kk = slane + 16 * t, key = k0 + kk;
-      float d = 0.f;
-      for (int c = 0; c < hd; ++c) d = fmaf(Qs[srow * hd + c], Ks[kk * hd + c], d);
+      const int kk = qlane + 16 * t, key = k0 + kk;
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int c = 0; c < hd; c += 4) {
+        const float4 q = ld4(Qs + qrow * ld + c), k = ld4(Ks + kk * ld + c);
+        d.x = fmaf(q.x, k.x, d.x);
+        d.y = fmaf(q.y, k.y, d.y);
+        d.z = fmaf(q.z, k.z, d.z);
+        d.w = fmaf(q.w, k.w, d.w);
+      }
       bool vis = key < nk;
-      if (a.mask_mode == 1 && key >= P + a.F && key < nk) vis = vis && (key - P - a.F == qrow_slot);
-      s[t] = vis ? d : -INFINITY;
+      if (a.mask_mode == 1 && key >= P + a.F && key < nk) vis = vis && (key - P - a.F == j);
+      s[t] = vis ? (d.x + d.y) + (d.z + d.w) : -INFINITY;
     }
     float cmax = fmaxf(s[0], s[1]);
 #pragma unroll
@@ -715,46 +804,50 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       const float p = (s[t] == -INFINITY) ? 0.f : __expf(s[t] - m_new);
-      Ss[srow * ATT_KT + slane + 16 * t] = p;
+      Ss[qrow * ATT_KT + qlane + 16 * t] = p;
       psum += p;
     }
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
     l_run = l_run * corr + psum;
     m_run = m_new;
-    __syncthreads();
-    // P V: orow == srow, so corr is this thread's own row correction
+    __syncwarp();   // a row's 16 threads are half a warp
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const int c = ocol + 16 * i;
+      const int c = qlane + 16 * i;
       if (c < hd) {
-        float v = acc[i] * corr;
-        for (int kk = 0; kk < ATT_KT; ++kk) v = fmaf(Ss[orow * ATT_KT + kk], Vs[kk * hd + c], v);
-        acc[i] = v;
+        float v0 = acc[i] * corr, v1 = 0.f;
+#pragma unroll 8
+        for (int kk = 0; kk < ATT_KT; kk += 2) {
+          v0 = fmaf(Ss[qrow * ATT_KT + kk], Vs[kk * hd + c], v0);
+          v1 = fmaf(Ss[qrow * ATT_KT + kk + 1], Vs[(kk + 1) * hd + c], v1);
+        }
+        acc[i] = v0 + v1;
       }
     }
   }
-  const int r = r0 + orow;
   if (r < nrows) {
-    const int j = r / G, h = g * G + r % G;
     T* o = (T*)a.out + (size_t)(b * a.H + j) * a.ld_out + h * hd;
     const float inv = 1.f / l_run;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const int c = ocol + 16 * i;
+      const int c = qlane + 16 * i;
       if (c < hd) o[c] = from_f32<T>(acc[i] * inv);
     }
   }
+}
+
+static size_t att_smem(int hd) {
+  return (size_t)((ATT_QT + ATT_KT) * (hd + 4) + ATT_KT * hd + ATT_QT * ATT_KT) * sizeof(float);
 }
 
 cudaError_t launch_attention_simt(const AttnArgs& a, Dtype dt, cudaStream_t st) {
   if (a.hd > 256 || a.hd % 8) return cudaErrorInvalidValue;
   const int G = a.Hq / a.Hkv;
   dim3 grid(a.B * a.Hkv, (a.H * G + ATT_QT - 1) / ATT_QT);
-  const size_t smem = (size_t)(ATT_QT * a.hd + 2 * ATT_KT * a.hd + ATT_QT * ATT_KT) * sizeof(float);
-  if (dt == DT_BF16) return launch_kernel(attention_simt_kernel<bf16>, grid, dim3(ATT_THREADS), smem, st, 1, a);
-  return launch_kernel(attention_simt_kernel<float>, grid, dim3(ATT_THREADS), smem, st, 1, a);
-  return cudaGetLastError();
+  if (dt == DT_BF16)
+    return launch_kernel(attention_simt_kernel<bf16>, grid, dim3(ATT_THREADS), att_smem(a.hd), st, 1, a);
+  return launch_kernel(attention_simt_kernel<float>, grid, dim3(ATT_THREADS), att_smem(a.hd), st, 1, a);
 }
 
 // ============================================================================ FOP adapter cross-attention
@@ -1046,7 +1139,7 @@ cudaError_t launch_chunk_noise(float* buffer, const uint64_t* seeds, uint64_t* c
 }
 
 cudaError_t init_simt_kernels() {
-  const int att = (ATT_QT * 256 + 2 * ATT_KT * 256 + ATT_QT * ATT_KT) * (int)sizeof(float);
+  const int att = (int)att_smem(256);
   cudaError_t e = cudaFuncSetAttribute(attention_simt_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attention_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);

@@ -131,6 +131,23 @@ def test_gemm_two_sm_is_deterministic(handles):
     np.testing.assert_allclose(outs[0].cpu().numpy(), ref, rtol=1e-4, atol=1e-4 * (np.sqrt(K) * 0.05 + 1))
 
 
+# the row kernel: one ragged 8-row chunk, exact chunks, its last M and the
+# first of the tile kernel; odd N, K that ends inside a lane's stride, and a K
+# that is not whole float4s (the tile kernel)
+@pytest.mark.parametrize("M,N,K", [(1, 1, 4), (8, 16, 128), (10, 1027, 1024), (256, 33, 516), (257, 33, 516), (7, 40, 250)])
+@pytest.mark.parametrize("epi", [0, 1, 2])
+def test_gemm_fp32_rows(handles, M, N, K, epi):
+    from paper_2609_34170_gb300 import ravel_gemm
+    g = torch.Generator("cuda").manual_seed(M + N + K)
+    X, W = (torch.randn(s, generator=g, device="cuda") for s in ((M, K), (N, K)))
+    bias, out = torch.randn(N, generator=g, device="cuda"), torch.randn((M, N), generator=g, device="cuda")
+    ref = X.double() @ W.double().T + bias.double()
+    ref = torch.nn.functional.silu(ref) if epi == 1 else ref + out.double() if epi == 2 else ref
+    ravel_gemm(handles["fp32"], X, W, epi, out, bias)
+    # K products of N(0, 1) values: |sum| errors below K 2^-24 sqrt(K)
+    np.testing.assert_allclose(out.cpu().numpy(), ref.cpu().numpy(), rtol=1e-5, atol=max(1e-6, K ** 1.5 * 6e-8))
+
+
 @pytest.mark.parametrize("M,N,K", [(10, 100, 256), (66, 300, 200)])
 def test_gemm_fp32_simt(handles, M, N, K):
     from paper_2609_34170_gb300 import ravel_gemm
