@@ -57,7 +57,7 @@ constexpr uint32_t AT_KBLK = AT_BKV * 128;    // bytes of one 64-wide head-dim b
 struct AtParams {
   int B, H, F, Hq, Hkv, G, hd, hdp;   // hdp: head dim rounded up to 16 (MMA N of P V)
   int TQ, q_tiles;
-  int Pmax, n_pre, n_kv, splits;
+  int Pmax, n_kv, splits;
   int layer, Bmax, mask_mode;
   int nblk, k_slots, v_slots;         // head-dim blocks of 64; K and V ring depths
   int xch;                            // splits > 1: partials through L2 (0) or shared memory, sent once every
@@ -77,13 +77,6 @@ struct AtParams {
 struct AtMaps {
   CUtensorMap q, k, v, pk0, pk1, pv0, pv1;
 };
-
-__device__ __forceinline__ int chunk_count(const AtParams& p, int P, int c0, int c1) {
-  int n = 0;
-  for (int c = c0; c < c1; ++c)
-    if (!(c < p.n_pre && c * AT_BKV >= P)) ++n;
-  return n;
-}
 
 // Rows of the split-KV combine: out = sum_s wgt[s] * O_s * inv over float4
 // columns [c4b, c4e) of this thread's row, the SP partials of a column batch
@@ -209,8 +202,12 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   const int rows_per_robot = p.H + p.F;
   const int slot = p.ctx_state[2 * b];       // this robot's active context
   const int P = p.ctx_state[2 * b + 1];
-  const int C = p.n_pre + p.n_kv;
-  const int c0 = (int)((long)split * C / p.splits), c1 = (int)((long)(split + 1) * C / p.splits);
+  // this robot's chunks: npv of its prefix, then n_kv of the step's own keys; this
+  // split's are c0 .. c1 - 1 (an even share of the keys that exist, whatever the
+  // context's capacity)
+  const int npv = (P + AT_BKV - 1) / AT_BKV;
+  const int C = npv + p.n_kv;
+  const int c0 = split * C / p.splits, c1 = (split + 1) * C / p.splits;
   const uint32_t ncols = (128 + p.hdp <= 256) ? 256u : 512u;
   const int ctx_z = (p.layer * p.Bmax + b) * p.Hkv + g;
   // query rows of this tile that hold a slot (rows 0 .. vrows-1)
@@ -224,7 +221,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     if (threadIdx.x == 0) raise_error(p.err, ERR_PREFIX_LEN);
     return;
   }
-  const int n = chunk_count(p, P, c0, c1);
+  const int n = c1 - c0;
   // the active context (slot, length and its prefix K/V) is fixed for the
   // whole step, so the first prefix chunks are fetched before the wait on the
   // previous kernel (the QKV projection)
@@ -264,8 +261,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   auto load_k = [&](int c, int s, uint64_t pol) {
     const uint32_t ks = k0 + (uint32_t)s * k_bytes, bar = smem_u32(&k_full[s]);
     mbar_expect_tx_el(&k_full[s], k_bytes, el);
-    const bool pre = c < p.n_pre;
-    const int cc = c - p.n_pre;
+    const bool pre = c < npv;
+    const int cc = c - npv;
     const CUtensorMap* km = pre ? pk : &maps.k;
     const int ky = pre ? c * AT_BKV : g, kz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
     #pragma unroll 1
@@ -275,8 +272,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   auto load_v = [&](int c, int s, uint64_t pol) {
     const uint32_t vs = v0 + (uint32_t)s * k_bytes, bar = smem_u32(&v_full[s]);
     mbar_expect_tx_el(&v_full[s], k_bytes, el);
-    const bool pre = c < p.n_pre;
-    const int cc = c - p.n_pre;
+    const bool pre = c < npv;
+    const int cc = c - npv;
     const CUtensorMap* vm = pre ? pv : &maps.v;
     const int vy = pre ? c * AT_BKV : g, vz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
     #pragma unroll 1
@@ -291,10 +288,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       prefetch_l2_3d_el(pv, blk * 64, c * AT_BKV, ctx_z, el);
     }
   };
-  // this CTA's chunks: prefix chunks c0 .. c0 + n_pre_here - 1 that hold keys, then
-  // the step's own chunks from c_own on
-  const int n_pre_here = max(0, min(min(c1, p.n_pre), (P + AT_BKV - 1) / AT_BKV) - c0);
-  const int c_own = max(c0, p.n_pre) - n_pre_here;
+  const int n_pre_here = max(0, min(c1, npv) - c0);   // prefix chunks of this split (its first ones)
   uint64_t pol_q = 0, pol_kv = 0;
   if (warp == 0) {
     __syncwarp();   // the barriers initialised above
@@ -353,7 +347,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       bool progress = false;
       if (nk < n && mbar_test_warp(&k_empty[sk], phk)) {
         const bool pre = nk < n_pre_here;
-        load_k(pre ? c0 + nk : c_own + nk, sk, pre ? pol_kv : pol_q);
+        load_k(c0 + nk, sk, pre ? pol_kv : pol_q);
         // keep the L2 warm 2 SK chunks ahead of the loads (prefix chunks only)
         if (nk + 2 * SK < n_pre_here) warm(c0 + nk + 2 * SK);
         ++nk;
@@ -365,7 +359,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       }
       if (nv < nk && mbar_test_warp(&v_empty[sv], phv)) {
         const bool pre = nv < n_pre_here;
-        load_v(pre ? c0 + nv : c_own + nv, sv, pre ? pol_kv : pol_q);
+        load_v(c0 + nv, sv, pre ? pol_kv : pol_q);
         ++nv;
         if (++sv == SV) {
           sv = 0;
@@ -474,7 +468,6 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     int i = 0;
     const float sl2 = p.scale_log2;
     for (int c = c0; c < c1 && ok; ++c) {
-      if (c < p.n_pre && c * AT_BKV >= P) continue;
       ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i & 1], (uint32_t)(i >> 1) & 1u));
       tc_fence_after();
       float sc[64];
@@ -490,9 +483,9 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       mbar_arrive(&s_free[i & 1]);
       // keys of this chunk that exist (prefix shorter than the chunk, ragged
       // FOP + slot chunk) and, in the slot-isolated test mode, that are visible
-      const int kk0 = (c < p.n_pre) ? c * AT_BKV : (c - p.n_pre) * AT_BKV;
-      const int kvalid = (c < p.n_pre) ? P - kk0 : rows_per_robot - kk0;
-      const bool iso = (p.mask_mode == 1) && (c >= p.n_pre) && (kk0 < p.H);
+      const int kk0 = (c < npv) ? c * AT_BKV : (c - npv) * AT_BKV;
+      const int kvalid = (c < npv) ? P - kk0 : rows_per_robot - kk0;
+      const bool iso = (p.mask_mode == 1) && (c >= npv) && (kk0 < p.H);
       // (two compact loops: this code runs cold at batch 1, where each
       // instruction fetched costs more than it does)
       if (kvalid < AT_BKV) {
@@ -787,7 +780,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_enc = nullptr;
-int g_attn_max_cluster = 8;   // largest power-of-two cluster of key splits
+int g_attn_clusters[4] = {0, 0, 0, 0};   // resident clusters of 2, 4, 8, 16 CTAs (0: not to be had)
 
 cudaError_t enc3(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1_bytes,
                  uint64_t s2_bytes, uint32_t b0, uint32_t b1, uint32_t b2) {
@@ -814,20 +807,21 @@ cudaError_t init_attention_tc() {
   }
   cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  if (cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+  const bool big = cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  for (int i = 0; i < (big ? 4 : 3); ++i) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 1;
     attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 16;
-    cfg.gridDim = dim3(1, 1, 16);
+    attr.val.clusterDim.z = 2u << i;
+    cfg.gridDim = dim3(1, 1, 2u << i);
     cfg.blockDim = dim3(AT_THREADS);
     cfg.dynamicSmemBytes = AT_SMEM_MAX;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel, &cfg) == cudaSuccess && n > 0) g_attn_max_cluster = 16;
+    g_attn_clusters[i] = cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel, &cfg) == cudaSuccess && n > 0 ? n : 0;
   }
   cudaGetLastError();
   return cudaSuccess;
@@ -840,11 +834,7 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   AtParams p{};
   p.B = a.B; p.H = a.H; p.F = a.F; p.Hq = a.Hq; p.Hkv = a.Hkv; p.G = a.Hq / a.Hkv; p.hd = a.hd;
   p.hdp = (a.hd + 15) / 16 * 16;
-  const int tq_max = AT_BM / p.G;
-  p.q_tiles = (a.H + tq_max - 1) / tq_max;
-  p.TQ = (a.H + p.q_tiles - 1) / p.q_tiles;
   p.Pmax = a.Pmax;
-  p.n_pre = (a.Pmax + AT_BKV - 1) / AT_BKV;
   p.n_kv = (a.H + a.F + AT_BKV - 1) / AT_BKV;
   p.layer = a.layer; p.Bmax = a.Bmax; p.mask_mode = a.mask_mode;
   p.nblk = (a.hd + 63) / 64;
@@ -852,35 +842,43 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   p.out = (bf16*)a.out; p.ld_out = a.ld_out;
   p.err = a.err;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
-  const int C = p.n_pre + p.n_kv;
-  // when the keys will be split (the grid leaves most SMs idle), query tiles
-  // of 64 rows: the merge moves every split's rows x hd partial between the
-  // SMs of the cluster, so its time grows with the rows of a tile, while the
-  // MMAs (always 128 rows) and the key loads of a split do not; the grid
-  // (at up to 8 splits) stays within half the SMs, which are free while the
-  // previous kernel still holds the rest, so that every CTA starts early
-  {
-    const int tq_small = std::max(1, 64 / p.G);
-    const int qt_small = (a.H + tq_small - 1) / tq_small;
-    if (p.q_tiles * a.B * a.Hkv * 2 <= a.num_sms && tq_small < p.TQ && qt_small * a.B * a.Hkv * 8 <= a.num_sms / 2 &&
-        (C + 1) / 2 >= 2) {
-      p.q_tiles = qt_small;
-      p.TQ = (a.H + qt_small - 1) / qt_small;
+  // Query tiles of 128 rows, or of 64 where the keys are split, and the number
+  // of key splits (one cluster per query tile, a power of two whose head-dim
+  // slices are multiples of 4 columns): the least estimated time.  A CTA costs
+  // about 4 us and each of its 64-key chunks the issue of S (4 MMAs per 64 of
+  // head dim, 36 ns each) and of P V, or the softmax's 0.45 us; the merge moves
+  // every split's rows x hd partial between the SMs, so it grows with the rows
+  // of a tile (the MMAs are always 128 rows) and with the splits; a grid that
+  // does not fit the SMs at once (36 clusters of 4, 15 of 8, 7 of 16) takes
+  // another round.  16 robots, 16 slots, 2048 keys: 4 splits; 8 would run 16
+  // clusters in two rounds (27 us per layer against 16).
+  const int C = (a.Pmax + AT_BKV - 1) / AT_BKV + p.n_kv;
+  const float t_chunk = std::max(0.45f, 0.036f * 4.f * (float)p.nblk + 0.26f * std::max(0.55f, (float)p.hdp / 256.f));
+  float cost = 3.4e38f;
+  auto consider = [&](int rows, int splits, int resident) {
+    const int tq = std::max(1, rows / p.G);
+    const int qt = (a.H + tq - 1) / tq, ctas = qt * a.B * a.Hkv;
+    const int rounds = (ctas + resident - 1) / resident;
+    float t = (float)rounds * (4.f + t_chunk * (float)((C + splits - 1) / splits));
+    if (splits > 1) t += (float)rounds * (0.6f + 1.4f * (float)rows / 128.f + 0.15f * (float)splits);
+    if (t < cost) {
+      cost = t;
+      p.q_tiles = qt;
+      p.TQ = (a.H + qt - 1) / qt;
+      p.splits = splits;
+    }
+  };
+  consider(AT_BM, 1, a.num_sms);
+  for (int i = 0; i < 4; ++i) {
+    const int sp = 2 << i;
+    if (sp * 2 > C + 1 || (p.hdp / sp) % 4 != 0 || p.hdp % sp != 0 || !g_attn_clusters[i]) break;
+    for (int rows = AT_BM; rows >= 64; rows /= 2) {
+      const int tq = std::max(1, rows / p.G);
+      const size_t ctas = (size_t)((a.H + tq - 1) / tq) * a.B * a.Hkv;
+      if ((size_t)sp * ctas * AT_BM * (p.hdp + 2) * 4 <= a.ws_bytes) consider(rows, sp, g_attn_clusters[i]);
     }
   }
-  const int nctas = p.q_tiles * a.B * a.Hkv;
-  // split the key chunks only when the (b, g, q-tile) grid leaves most SMs
-  // idle; about two chunks per split so S(i+1) overlaps the softmax of i
-  // the splits of a query tile form one cluster (power of two, <= 16) whose
-  // head-dim slices are multiples of 4 columns
-  int splits = 1;
-  if (nctas * 2 <= a.num_sms) {
-    const int cap = std::min({(C + 1) / 2, std::max(1, a.num_sms / nctas), g_attn_max_cluster});
-    while (splits * 2 <= cap && (p.hdp / (splits * 2)) % 4 == 0 &&
-           (size_t)(splits * 2) * nctas * AT_BM * (p.hdp + 2) * 4 <= a.ws_bytes)
-      splits *= 2;
-  }
-  p.splits = splits;
+  const int splits = p.splits, nctas = p.q_tiles * a.B * a.Hkv;
   p.ws_o = a.ws;
   p.ws_ml = a.ws + (size_t)splits * nctas * AT_BM * p.hdp;
   // partials through shared memory: whole 8-column bf16 groups per rank
