@@ -513,6 +513,88 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
   }
 }
 
+// The same for rows in numbers: a block takes RB robots x RJ slots (RB RJ = 4), so
+// that each modulation row it reads serves several rows: a row then costs 14
+// KB of L2 traffic at width 1024 (its own 6 KB, half a slot's and half a
+// robot's modulation, a quarter of the bias) instead of 19 to 28, which is
+// what bounds the norm once the rows fill the SMs.  Every load is issued
+// before the one barrier.  FOP rows go four to a block.  The arithmetic is the
+// row kernel's, operation for operation.  (64 robots x 50 slots, width 1024, 35
+// launches: step 2701 -> 2682 us; from 1216 rows on, fewer gain nothing.)
+template <typename T, int RB, int RJ>
+__global__ void __launch_bounds__(256) ada_norm_tile_kernel(NormArgs a, int nb_b, int nb_j) {
+  constexpr int R = RB * RJ;
+  __shared__ float red[R][8];
+  pdl_trigger();
+  const int D = a.D, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = 4 * threadIdx.x;
+  const bool on = c < D;
+  const bool act = (int)blockIdx.x < nb_b * nb_j;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int b0 = act ? (blockIdx.x / nb_j) * RB : 0, j0 = act ? (blockIdx.x % nb_j) * RJ : 0;
+  const int f0 = act ? 0 : (blockIdx.x - nb_b * nb_j) * R;   // first FOP row (of B F)
+  float4 bsc = zero, bsh = zero;   // weights: independent of the earlier kernels
+  if (on) {
+    bsc = ld4(act ? a.mod_b + a.off + c : a.gamma + c);
+    if (act) bsh = ld4(a.mod_b + a.off + D + c);
+  }
+  pdl_wait();
+  float4 x[R], dsc[RB], dsh[RB], tsc[RJ], tsh[RJ];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    x[r] = zero;
+    if (!on) continue;
+    if (act) {
+      const int b = b0 + r / RJ, j = j0 + r % RJ;
+      if (b < a.B && j < a.H) x[r] = ld4(a.x + (size_t)(b * a.H + j) * D + c);
+    } else if (f0 + r < a.B * a.F) {
+      x[r] = ld4((const T*)a.fop + (size_t)(f0 + r) * D + c);
+    }
+  }
+  if (act && on) {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const int b = min(b0 + i, a.B - 1);
+      const float* md = a.modv + (size_t)(a.drow ? a.drow[b] : a.H + b) * a.mod_ld + a.off;
+      dsc[i] = ld4(md + c);
+      dsh[i] = ld4(md + D + c);
+    }
+#pragma unroll
+    for (int i = 0; i < RJ; ++i) {
+      const float* mt = a.modv + (size_t)(b0 * a.t_stride + min(j0 + i, a.H - 1)) * a.mod_ld + a.off;
+      tsc[i] = ld4(mt + c);
+      tsh[i] = ld4(mt + D + c);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float ss = warp_sum(x[r].x * x[r].x + x[r].y * x[r].y + x[r].z * x[r].z + x[r].w * x[r].w);
+    if (lane == 0) red[r][warp] = ss;
+  }
+  __syncthreads();
+  if (!on) return;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) tot += red[r][w];
+    const float inv = rsqrtf(tot / (float)D + 1e-6f);
+    const float4 v = x[r];
+    if (act) {
+      const int b = b0 + r / RJ, j = j0 + r % RJ;
+      if (b >= a.B || j >= a.H) continue;
+      const float4 sc = add2(add2(bsc, dsc[r / RJ]), tsc[r % RJ]), sh = add2(add2(bsh, dsh[r / RJ]), tsh[r % RJ]);
+      st4((T*)a.Y + ((size_t)b * a.row_pitch + j) * D + c,
+          make_float4(v.x * inv * (1.f + sc.x) + sh.x, v.y * inv * (1.f + sc.y) + sh.y,
+                      v.z * inv * (1.f + sc.z) + sh.z, v.w * inv * (1.f + sc.w) + sh.w));
+    } else if (f0 + r < a.B * a.F) {
+      const int b = (f0 + r) / a.F, f = (f0 + r) % a.F;
+      st4((T*)a.Y + ((size_t)b * a.row_pitch + a.H + f) * D + c,
+          make_float4(v.x * inv * (1.f + bsc.x), v.y * inv * (1.f + bsc.y), v.z * inv * (1.f + bsc.z),
+                      v.w * inv * (1.f + bsc.w)));
+    }
+  }
+}
+
 namespace {
 int g_norm_sms = 0;
 }
@@ -531,6 +613,18 @@ cudaError_t launch_ada_norm_t(const NormArgs& a, cudaStream_t st) {
   // SM (one row each when the rows fit)
   const int nf = a.fop ? a.F : 0;
   const int total = a.B * (a.H + nf);
+  // modulated rows of up to 1024 features that give every SM two tiles or more
+  if (a.D <= 1024 && !a.act_gain && a.H > 0 && total >= 8 * g_norm_sms) {
+    NormArgs b = a;
+    b.F = nf;
+    const int fop_blocks = (a.B * nf + 3) / 4;
+    if (a.t_stride == 0) {
+      const int nb = (a.B + 1) / 2, nj = (a.H + 1) / 2;
+      return launch_kernel(ada_norm_tile_kernel<T, 2, 2>, dim3(nb * nj + fop_blocks), dim3(256), 0, st, 1, b, nb, nj);
+    }
+    const int nj = (a.H + 3) / 4;   // a schedule per robot: slots of one robot
+    return launch_kernel(ada_norm_tile_kernel<T, 1, 4>, dim3(a.B * nj + fop_blocks), dim3(256), 0, st, 1, b, a.B, nj);
+  }
   int rb_all = (total + 8 * g_norm_sms - 1) / (8 * g_norm_sms);
   rb_all = (rb_all + R - 1) / R * R;
   auto rows_per_block = [&](int rows_per_robot) { return std::max(R, std::min(rb_all, rows_per_robot)); };
