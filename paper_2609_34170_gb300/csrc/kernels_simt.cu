@@ -682,89 +682,149 @@ cudaError_t launch_in_proj(const float* buf, int BH, int A, int D, const float* 
                        in_w, in_b, x, state, rel_mask, slot_times, H, t_stride);
 }
 
-// The in-projection of whole rows with the first layer's adaRMSNorm: one
-// CTA per row; an action row is projected (x, fp32), then normalised with its
-// modulation into Y; a FOP row is normalised with its gain.  (Rows of up to
-// 4096 features: a thread owns features tid, tid + 256, ...)
-template <typename T>
+// The in-projection of whole rows with the first layer's adaRMSNorm: a block
+// takes R consecutive slots of one robot (projected into x, fp32, then
+// normalised with their modulation into Y) or R FOP rows (normalised with their
+// gain).  A thread owns features 4 tid + 1024 g, so a row of W_in is one
+// 16-byte load per thread that serves R slots, eight of them in flight: one
+// slot per block and a load per feature re-read the 128 KB of W_in for every
+// slot (64 robots x 50 slots: step 2682 -> 2662 us) and waited for 32 loads in
+// turn (4 robots: 900 -> 891 us).
+template <typename T, int R, int G>
 __global__ void __launch_bounds__(256) in_proj_norm_kernel(const float* __restrict__ buf, int A, int D,
                                                            const float* __restrict__ in_w,
                                                            const float* __restrict__ in_b, float* __restrict__ x,
                                                            const float* __restrict__ state,
                                                            const float* __restrict__ rel_mask,
-                                                           const float* __restrict__ slot_times, RowNorm rn) {
+                                                           const float* __restrict__ slot_times, RowNorm rn, int nj) {
+  extern __shared__ float arow[];   // [R][A] the action rows of these slots
+  __shared__ float red[R][8];
   pdl_trigger();
   pdl_wait();
-  extern __shared__ float arow[];   // the action row of this slot
-  __shared__ float red[32];
-  const int r = blockIdx.x, BH = rn.B * rn.H;
-  float v[16];
-  float ss = 0.f;
-  if (r < BH) {
-    const int b = r / rn.H, j = r % rn.H;
-    for (int i = threadIdx.x; i < A; i += blockDim.x) {
-      float a = buf[(size_t)r * A + i];
-      if (state)   // relative coordinates of the expert: a - (1 - t_j) m s_b
-        a = __fsub_rn(a, __fmul_rn(__fsub_rn(1.f, slot_times[b * rn.t_stride + j]),
-                                   __fmul_rn(rel_mask[i], state[(size_t)b * A + i])));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool act = (int)blockIdx.x < rn.B * nj;
+  const int b = act ? blockIdx.x / nj : 0, j0 = act ? (blockIdx.x % nj) * R : 0;
+  const int f0 = act ? 0 : (blockIdx.x - rn.B * nj) * R;   // first FOP row (of B F)
+  float4 v[R][G];
+  if (act) {
+    for (int i = threadIdx.x; i < R * A; i += 256) {
+      const int j = j0 + i / A, d = i % A;
+      float a = 0.f;
+      if (j < rn.H) {
+        a = buf[(size_t)(b * rn.H + j) * A + d];
+        if (state)   // relative coordinates of the expert: a - (1 - t_j) m s_b
+          a = __fsub_rn(a, __fmul_rn(__fsub_rn(1.f, slot_times[b * rn.t_stride + j]),
+                                     __fmul_rn(rel_mask[d], state[(size_t)b * A + d])));
+      }
       arow[i] = a;
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int c = threadIdx.x + 256 * k;
-      v[k] = 0.f;
-      if (c < D) {
-        float acc = in_b[c];
-        for (int i = 0; i < A; ++i) acc = fmaf(arow[i], in_w[(size_t)i * D + c], acc);
-        x[(size_t)r * D + c] = acc;
-        v[k] = acc;
-        ss += acc * acc;
-      }
-    }
-    const float inv = rsqrtf(block_sum(ss, red) / (float)D + 1e-6f);
-    const float* mt = rn.modv + (size_t)(b * rn.t_stride + j) * rn.mod_ld + rn.off;
-    const float* md = rn.modv + (size_t)(rn.drow ? rn.drow[b] : rn.H + b) * rn.mod_ld + rn.off;
-    const float* mb = rn.mod_b + rn.off;
-    T* Y = (T*)rn.Y + (size_t)(b * rn.row_pitch + j) * D;
+    for (int g = 0; g < G; ++g) {
+      const int c = 4 * threadIdx.x + 1024 * g;
+      const float4 bias = c < D ? ld4(in_b + c) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int c = threadIdx.x + 256 * k;
-      if (c < D) {
-        const float sc = mt[c] + md[c] + mb[c], sh = mt[D + c] + md[D + c] + mb[D + c];
-        Y[c] = from_f32<T>(v[k] * inv * (1.f + sc) + sh);
+      for (int r = 0; r < R; ++r) v[r][g] = bias;
+      if (c >= D) continue;
+#pragma unroll 8
+      for (int i = 0; i < A; ++i) {
+        const float4 w = ld4(in_w + (size_t)i * D + c);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float a = arow[r * A + i];
+          v[r][g] = make_float4(fmaf(a, w.x, v[r][g].x), fmaf(a, w.y, v[r][g].y), fmaf(a, w.z, v[r][g].z),
+                                fmaf(a, w.w, v[r][g].w));
+        }
       }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (j0 + r < rn.H) st4(x + (size_t)(b * rn.H + j0 + r) * D + c, v[r][g]);
     }
   } else {
-    const int fr = r - BH, b = fr / rn.F, f = fr % rn.F;
-    const T* z = (const T*)rn.fop + (size_t)(b * rn.F + f) * D;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int c = threadIdx.x + 256 * k;
-      v[k] = c < D ? to_f32(z[c]) : 0.f;
-      ss += v[k] * v[k];
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int c = 4 * threadIdx.x + 1024 * g;
+        v[r][g] = (c < D && f0 + r < rn.B * rn.F) ? ld4((const T*)rn.fop + (size_t)(f0 + r) * D + c)
+                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    float ss = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      ss += v[r][g].x * v[r][g].x + v[r][g].y * v[r][g].y + v[r][g].z * v[r][g].z + v[r][g].w * v[r][g].w;
+    ss = warp_sum(ss);
+    if (lane == 0) red[r][warp] = ss;
+  }
+  __syncthreads();
+  const float* md = rn.modv + (size_t)(act ? (rn.drow ? rn.drow[b] : rn.H + b) : 0) * rn.mod_ld + rn.off;
+  const float* mb = rn.mod_b + rn.off;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int c = 4 * threadIdx.x + 1024 * g;
+    if (c >= D) continue;
+    float4 dsc, dsh, bsc, bsh;
+    if (act) {
+      dsc = ld4(md + c);
+      dsh = ld4(md + D + c);
+      bsc = ld4(mb + c);
+      bsh = ld4(mb + D + c);
+    } else {
+      bsc = ld4(rn.gamma + c);
     }
-    const float inv = rsqrtf(block_sum(ss, red) / (float)D + 1e-6f);
-    T* Y = (T*)rn.Y + (size_t)(b * rn.row_pitch + rn.H + f) * D;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int c = threadIdx.x + 256 * k;
-      if (c < D) Y[c] = from_f32<T>(v[k] * inv * (1.f + rn.gamma[c]));
+    for (int r = 0; r < R; ++r) {
+      float tot = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) tot += red[r][w];
+      const float inv = rsqrtf(tot / (float)D + 1e-6f);
+      const float4 q = v[r][g];
+      if (act) {
+        if (j0 + r >= rn.H) continue;
+        const float* mt = rn.modv + (size_t)(b * rn.t_stride + j0 + r) * rn.mod_ld + rn.off;
+        const float4 sc = add3(ld4(mt + c), dsc, bsc), sh = add3(ld4(mt + D + c), dsh, bsh);
+        st4((T*)rn.Y + ((size_t)b * rn.row_pitch + j0 + r) * D + c,
+            make_float4(q.x * inv * (1.f + sc.x) + sh.x, q.y * inv * (1.f + sc.y) + sh.y,
+                        q.z * inv * (1.f + sc.z) + sh.z, q.w * inv * (1.f + sc.w) + sh.w));
+      } else if (f0 + r < rn.B * rn.F) {
+        const int fb = (f0 + r) / rn.F, f = (f0 + r) % rn.F;
+        st4((T*)rn.Y + ((size_t)fb * rn.row_pitch + rn.H + f) * D + c,
+            make_float4(q.x * inv * (1.f + bsc.x), q.y * inv * (1.f + bsc.y), q.z * inv * (1.f + bsc.z),
+                        q.w * inv * (1.f + bsc.w)));
+      }
     }
   }
+}
+
+template <typename T, int R, int G>
+static cudaError_t launch_in_proj_norm_t(const float* buf, int A, int D, const float* in_w, const float* in_b,
+                                         float* x, const float* state, const float* rel_mask, const float* slot_times,
+                                         const RowNorm& rn, cudaStream_t st) {
+  const int nj = (rn.H + R - 1) / R, blocks = rn.B * nj + (rn.fop ? (rn.B * rn.F + R - 1) / R : 0);
+  return launch_kernel(in_proj_norm_kernel<T, R, G>, dim3(blocks), dim3(256), (size_t)R * A * sizeof(float), st, 1,
+                       buf, A, D, in_w, in_b, x, state, rel_mask, slot_times, rn, nj);
 }
 
 cudaError_t launch_in_proj_norm(const float* buf, int A, int D, const float* in_w, const float* in_b, float* x,
                                 const float* state, const float* rel_mask, const float* slot_times, const RowNorm& rn,
                                 Dtype dt, cudaStream_t st) {
-  if (D > 4096) return cudaErrorInvalidValue;
   const int rows = rn.B * rn.H + (rn.fop ? rn.B * rn.F : 0);
+  if (D > 4096 || D % 4) return cudaErrorInvalidValue;
   if (rows <= 0) return cudaSuccess;
-  if (dt == DT_BF16)
-    return launch_kernel(in_proj_norm_kernel<bf16>, dim3(rows), dim3(256), A * sizeof(float), st, 1, buf, A, D, in_w,
-                         in_b, x, state, rel_mask, slot_times, rn);
-  return launch_kernel(in_proj_norm_kernel<float>, dim3(rows), dim3(256), A * sizeof(float), st, 1, buf, A, D, in_w,
-                       in_b, x, state, rel_mask, slot_times, rn);
+  if (dt != DT_BF16) return cudaErrorNotSupported;   // (the fp32 step runs the two kernels)
+#define RAVEL_IPN(R, G) \
+  return launch_in_proj_norm_t<bf16, R, G>(buf, A, D, in_w, in_b, x, state, rel_mask, slot_times, rn, st)
+  if (D > 2048) RAVEL_IPN(1, 4);
+  if (D > 1024) RAVEL_IPN(1, 2);
+  // one slot per block while they leave SMs idle, then four, or eight (whose
+  // actions must fit the block's shared memory)
+  if (rows <= 2 * 152 || A > 1024) RAVEL_IPN(1, 1);
+  if (rows <= 8 * 152) RAVEL_IPN(4, 1);
+  RAVEL_IPN(8, 1);
+#undef RAVEL_IPN
 }
 
 __global__ void noop_kernel() {}
