@@ -3,15 +3,20 @@
 //
 // One CTA owns a tile of up to 128 query rows of one (robot b, KV head g)
 // pair -- row r = t*G + hh is slot j0+t of query head g*G+hh -- and walks the
-// pair's keys in chunks of 64: first the active VLM context's prefix
+// pair's keys in chunks of 128: first the active VLM context's prefix
 // (context slot, valid length read on the device), then the FOP tokens and
 // the H action slots of this step (the QKV buffer).  Per chunk:
-//   S = Q K^T        tcgen05.mma, M = 128 query rows, N = 64 keys, into TMEM
+//   S = Q K^T        tcgen05.mma, M = 128 query rows, N = 128 keys, into TMEM
 //   P = exp(S - m)   softmax warps: TMEM -> registers -> bf16 P back into TMEM
-//   O += P V         tcgen05.mma, M = 128, N = head dim, K = 64 keys, O in TMEM
-// Every operand is K-major with 128-byte swizzling; V is kept transposed
-// (keys contiguous) for that: the context's V is transposed when a context
-// is installed, and the step's own V by the QKV projection's epilogue.
+//   O += P V         tcgen05.mma, M = 128, N = head dim, K = 16 keys at a time, O in TMEM
+// What bounds it is the tensor pipe and the issue of its instructions (up to
+// N = 128 an MMA takes its warp 71 cycles whatever its N): chunks of 64 keys
+// spent 16 such MMAs on S for every 64 keys at head dim 256, 128-key chunks
+// spend them on 128.  Shared memory holds no two such chunks beside Q, so K
+// comes in units of 64 head dims (16 KB, freed as their four MMAs complete) and
+// V in halves of 64 keys: 4 K units + 3 V halves at head dim 256, the next
+// chunk's units streaming in behind the MMAs.  K is K-major, V the B operand of
+// P V in its natural layout (MN-major).
 // The online softmax rescales O in TMEM only when a row's running maximum
 // grows by more than 2^8 (the kept maximum is exact for the final
 // normalisation, so this is not an approximation).
@@ -28,8 +33,8 @@
 // publish unnormalised fp32 partials through L2 and the cluster barrier.  The
 // producer keeps the L2 warm a few prefix chunks ahead of its loads.
 //
-// Warp roles (192 threads): warp 0 TMA producer, warp 1 TMEM allocator + MMA
-// issuer, warps 2..5 softmax / epilogue (warp w owns TMEM lanes 32*(w%4)..).
+// Warp roles (320 threads): warp 0 TMA producer, warp 1 TMEM allocator + MMA
+// issuer, warps 2..9 softmax / epilogue (warp w owns TMEM lanes 32*(w%4)..).
 // Every wait is bounded (ERR_TIMEOUT, then unwind).
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -44,26 +49,33 @@
 namespace ravel {
 namespace {
 
-// warp 0: loads; warp 1: MMAs; warps 2-5: softmax (a thread per query row);
-// warps 6-7 join only the merge of the key splits, so that each thread takes
-// one (row, 8-column) item of a 64-row tile's slice instead of two
-constexpr int AT_THREADS = 256;
+// warp 0: loads; warp 1: MMAs; warps 2-9: softmax and epilogue, two threads per
+// query row (warps w and w + 4 share TMEM lanes): each takes 64 keys of a
+// chunk, and half of O's columns; all ten merge the key splits
+constexpr int AT_THREADS = 320;
 constexpr int AT_BM = 128;
-constexpr int AT_BKV = 64;
+constexpr int AT_BKV = 128;          // keys of a chunk
 constexpr int AT_SMEM_MAX = 227 * 1024;
 constexpr uint32_t AT_QBLK = AT_BM * 128;     // bytes of one 64-wide head-dim block of Q
-constexpr uint32_t AT_KBLK = AT_BKV * 128;    // bytes of one 64-wide head-dim block of a K chunk
+constexpr uint32_t AT_KUNIT = AT_BKV * 128;   // bytes of a K unit: 128 keys x 64 head dims
+constexpr uint32_t AT_VBLK = 64 * 128;        // bytes of one 64-wide head-dim block of a V half (64 keys)
+
+// Limit of the polling loops: a counter, because reading the global timer in
+// each turn left the tensor pipe idle between S and P V.  A turn takes at
+// least 30 cycles and at most some hundred: 0.5 to 5 s.
+constexpr uint32_t kPollLimit = 1u << 25;
 
 struct AtParams {
   int B, H, F, Hq, Hkv, G, hd, hdp;   // hdp: head dim rounded up to 16 (MMA N of P V)
   int TQ, q_tiles;
   int Pmax, n_kv, splits;
   int layer, Bmax, mask_mode;
-  int nblk, k_slots, v_slots;         // head-dim blocks of 64; K and V ring depths
+  int nblk, k_slots, v_slots;         // head-dim blocks of 64; K units and V halves in their rings
   int xch;                            // splits > 1: partials through L2 (0) or shared memory, sent once every
                                       // split's MMAs are done (1: cluster barrier) or once every split's S
                                       // MMAs are done (2: the receive area lies in Q and the K ring)
   const int* ctx_state;
+  const bf16 *ck[2], *cv[2];          // context slots [L][Bmax][Hkv][Pmax][hd]
   bf16* out;
   int ld_out;
   float* ws_o;
@@ -72,10 +84,10 @@ struct AtParams {
   float scale_log2;                   // log2(e) / sqrt(hd)
 };
 
-// K and V chunks alike: [64 keys][64-wide head-dim block] boxes, 128-byte
-// swizzled; V is the B operand of P V in its natural layout (MN-major)
+// boxes of [128 keys][64-wide head-dim block] (K) and [64 keys][64-wide block]
+// (V), 128-byte swizzled
 struct AtMaps {
-  CUtensorMap q, k, v, pk0, pk1, pv0, pv1;
+  CUtensorMap q, k, v, pk0, pk1, pv0, pv1, o;   // o: (hd, heads, slots, robots), boxes as Q's
 };
 
 // Rows of the split-KV combine: out = sum_s wgt[s] * O_s * inv over float4
@@ -173,27 +185,26 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   // compiler keeps it (and everything indexed from it) in the shared window
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const int SK = p.k_slots, SV = p.v_slots;   // K and V ring depths
-  const uint32_t k_bytes = (uint32_t)p.nblk * AT_KBLK;   // one K or V chunk
+  const uint32_t v_bytes = (uint32_t)p.nblk * AT_VBLK;   // one V half
   uint8_t* q_s = smem;
   uint8_t* kv_s = q_s + (size_t)p.nblk * AT_QBLK;   // K ring, then V ring
-  uint8_t* v_ring = kv_s + (size_t)SK * k_bytes;
-  uint64_t* bars = (uint64_t*)(v_ring + (size_t)SV * k_bytes);
-  // K and V of a stage have their own barriers: K is released as soon as
-  // S = Q K^T has been computed, V only after P V, so the next K load does
-  // not wait for the softmax and the PV of the chunk it replaces
+  uint8_t* v_ring = kv_s + (size_t)SK * AT_KUNIT;
+  uint64_t* bars = (uint64_t*)(v_ring + (size_t)SV * v_bytes);
+  // every K unit and V half has its own barriers: a K unit is released as its
+  // MMAs of S = Q K^T complete, a V half as its MMAs of P V do
   uint64_t* q_full = bars;
   uint64_t* k_full = bars + 1;
   uint64_t* v_full = k_full + SK;
   uint64_t* k_empty = v_full + SV;
   uint64_t* v_empty = k_empty + SK;
   uint64_t* s_full = v_empty + SV;
-  uint64_t* s_free = s_full + 2;
-  uint64_t* p_full = s_free + 2;
+  uint64_t* p_full = s_full + 2;
   uint64_t* pv_done = p_full + 2;   // [2]: PV of chunk i completes pv_done[i & 1]
   uint64_t* rcv_bar = pv_done + 2;  // xch: every split's share of this rank has arrived
   uint64_t* sdone = rcv_bar + 1;    // xch 2: every split's last S MMA has completed (one arrival each)
   uint32_t* tmem_slot = (uint32_t*)(sdone + 1);
-  int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] K issued, [2] K consumed, [3] V issued, [4] V consumed
+  float* xm = (float*)((uint8_t*)bars + 512);   // [2][128] row maxima, then sums, of the two halves
+  int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] K units issued, [2] consumed, [3] V halves issued, [4] consumed
 
   // (through a shuffle, so that the compiler knows it is uniform in the warp)
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -208,7 +219,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   const int npv = (P + AT_BKV - 1) / AT_BKV;
   const int C = npv + p.n_kv;
   const int c0 = split * C / p.splits, c1 = (split + 1) * C / p.splits;
-  const uint32_t ncols = (128 + p.hdp <= 256) ? 256u : 512u;
+  constexpr uint32_t ncols = 512;   // two S tiles of 128 columns, O
   const int ctx_z = (p.layer * p.Bmax + b) * p.Hkv + g;
   // query rows of this tile that hold a slot (rows 0 .. vrows-1)
   const int vrows = p.G * max(0, min(p.TQ, p.H - qt * p.TQ));
@@ -222,10 +233,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     return;
   }
   const int n = c1 - c0;
-  // the active context (slot, length and its prefix K/V) is fixed for the
-  // whole step, so the first prefix chunks are fetched before the wait on the
-  // previous kernel (the QKV projection)
-  int npre = 0;
+  // keys of chunk c that exist (the prefix may end inside its last chunk, the
+  // step's own keys inside theirs), from key `first` of the prefix / own keys on
+  auto keys_of = [&](int c) {
+    return min(AT_BKV, c < npv ? P - c * AT_BKV : rows_per_robot - (c - npv) * AT_BKV);
+  };
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -235,12 +247,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     }
     for (int s = 0; s < SV; ++s) {
       mbar_init(&v_full[s], 1);
-      mbar_init(&v_empty[s], 1);   // released by the PV commit
+      mbar_init(&v_empty[s], 1);   // released by the PV commits
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&s_free[i], 128);
-      mbar_init(&p_full[i], 128);
+      mbar_init(&p_full[i], 256);
     }
     mbar_init(&pv_done[0], 1);
     mbar_init(&pv_done[1], 1);
@@ -256,54 +267,83 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   const CUtensorMap* pv = slot ? &maps.pv1 : &maps.pv0;
   uint32_t el = 0;   // the issuing lane of warps 0 (TMA) and 1 (MMA)
   const uint32_t q0 = smem_u32(q_s), k0 = smem_u32(kv_s), v0 = smem_u32(v_ring);
-  // K and V of chunk c into stage s (warp 0), each CTA loading its own copy (query
-  // tiles of one (b, g) pair read the same chunk, which L2 serves to all)
-  auto load_k = [&](int c, int s, uint64_t pol) {
-    const uint32_t ks = k0 + (uint32_t)s * k_bytes, bar = smem_u32(&k_full[s]);
-    mbar_expect_tx_el(&k_full[s], k_bytes, el);
+  // K unit (chunk c, head-dim block blk) and V half h of chunk c into their
+  // slots (warp 0), each CTA loading its own copy (query tiles of one (b, g)
+  // pair read the same chunk, which L2 serves to all)
+  uint64_t pol_q = 0, pol_kv = 0;
+  auto load_k = [&](int c, int blk, int s) {
     const bool pre = c < npv;
-    const int cc = c - npv;
-    const CUtensorMap* km = pre ? pk : &maps.k;
-    const int ky = pre ? c * AT_BKV : g, kz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
-    #pragma unroll 1
-    for (int blk = 0; blk < p.nblk; ++blk)
-      tma_load_3d_el(km, bar, ks + (uint32_t)blk * AT_KBLK, blk * 64, ky, kz, pol, el);
+    mbar_expect_tx_el(&k_full[s], AT_KUNIT, el);
+    tma_load_3d_el(pre ? pk : &maps.k, smem_u32(&k_full[s]), k0 + (uint32_t)s * AT_KUNIT, blk * 64,
+                   pre ? c * AT_BKV : g, pre ? ctx_z : b * rows_per_robot + (c - npv) * AT_BKV, pre ? pol_kv : pol_q,
+                   el);
   };
-  auto load_v = [&](int c, int s, uint64_t pol) {
-    const uint32_t vs = v0 + (uint32_t)s * k_bytes, bar = smem_u32(&v_full[s]);
-    mbar_expect_tx_el(&v_full[s], k_bytes, el);
+  auto load_v = [&](int c, int h, int s) {
     const bool pre = c < npv;
-    const int cc = c - npv;
+    const uint32_t vs = v0 + (uint32_t)s * v_bytes, bar = smem_u32(&v_full[s]);
     const CUtensorMap* vm = pre ? pv : &maps.v;
-    const int vy = pre ? c * AT_BKV : g, vz = pre ? ctx_z : b * rows_per_robot + cc * AT_BKV;
+    const int key = (pre ? c : c - npv) * AT_BKV + 64 * h;
+    const int vy = pre ? key : g, vz = pre ? ctx_z : b * rows_per_robot + key;
+    mbar_expect_tx_el(&v_full[s], v_bytes, el);
     #pragma unroll 1
     for (int blk = 0; blk < p.nblk; ++blk)
-      tma_load_3d_el(vm, bar, vs + (uint32_t)blk * AT_KBLK, blk * 64, vy, vz, pol, el);
+      tma_load_3d_el(vm, bar, vs + (uint32_t)blk * AT_VBLK, blk * 64, vy, vz, pre ? pol_kv : pol_q, el);
   };
-  // prefix chunk c into L2
-  auto warm = [&](int c) {
-    #pragma unroll 1
-    for (int blk = 0; blk < p.nblk; ++blk) {
-      prefetch_l2_3d_el(pk, blk * 64, c * AT_BKV, ctx_z, el);
-      prefetch_l2_3d_el(pv, blk * 64, c * AT_BKV, ctx_z, el);
+  // next K unit (chunk kc, block kb, slot sk) and V half (chunk vc, half vh, slot
+  // sv) to load, and the parities their `empty` waits take
+  int kc = c0, kb = 0, nk = 0, sk = 0, vc = c0, vh = 0, nv = 0, sv = 0;
+  uint32_t phk = 1, phv = 1;
+  auto next_k = [&]() {
+    load_k(kc, kb, sk);
+    ++nk;
+    if (++kb == p.nblk) {
+      kb = 0;
+      ++kc;
+    }
+    if (++sk == SK) {
+      sk = 0;
+      phk ^= 1u;
     }
   };
-  const int n_pre_here = max(0, min(c1, npv) - c0);   // prefix chunks of this split (its first ones)
-  uint64_t pol_q = 0, pol_kv = 0;
+  auto next_v = [&]() {   // (a chunk of at most 64 keys has one half)
+    load_v(vc, vh, sv);
+    ++nv;
+    if (vh == 1 || keys_of(vc) <= 64) {
+      vh = 0;
+      ++vc;
+    } else {
+      vh = 1;
+    }
+    if (++sv == SV) {
+      sv = 0;
+      phv ^= 1u;
+    }
+  };
   if (warp == 0) {
     __syncwarp();   // the barriers initialised above
     el = elect_one();
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_q));
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_kv));
-    npre = min(n_pre_here, min(SK, SV));
+    // the active context (slot, length and its prefix K/V) is fixed for the
+    // whole step, so the first prefix units are fetched before the wait on the
+    // previous kernel (the QKV projection)
+    const int pre_end = min(c1, npv);
     #pragma unroll 1
-    for (int i = 0; i < npre; ++i) {
-      load_k(c0 + i, i, pol_kv);
-      load_v(c0 + i, i, pol_kv);
+    while (nk < SK && kc < pre_end) next_k();
+    #pragma unroll 1
+    while (nv < SV && vc < pre_end) next_v();
+    // the rest of the split's prefix goes to L2 now, K and V in one request
+    // each (the query tiles of a pair share it): loads that the loop below
+    // issues then find it there.  (Requests per chunk from the loop itself, a
+    // box at a time, held up the next K unit: 3900 cycles per chunk at batch
+    // 64, 2700 without them; the tensor pipe needs 2050.)
+    if (qt == 0 && kc < pre_end && el) {
+      const size_t row0 = (size_t)ctx_z * p.Pmax + (size_t)kc * AT_BKV;
+      const uint32_t bytes = (uint32_t)(min(pre_end * AT_BKV, P) - kc * AT_BKV) * (uint32_t)p.hd * 2u;
+      prefetch_l2_bulk(p.ck[slot ? 1 : 0] + row0 * p.hd, bytes);
+      prefetch_l2_bulk(p.cv[slot ? 1 : 0] + row0 * p.hd, bytes);
     }
-    // and warm L2 with the prefix chunks that will refill those stages
-    #pragma unroll 1
-    for (int i = npre; i < min(npre + SK, n_pre_here); ++i) warm(c0 + i);
+    __syncwarp();
   }
   // rows of the Q tile that no query fills are zeroed (their scores are unused)
   const int q_rows = p.TQ * p.G;
@@ -332,43 +372,24 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   cta_sync();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t o_col = 128;
+  const uint32_t o_col = 256;
 
   if (warp == 0) {
-    // K of chunk nk and V of chunk nv (nv <= nk), each as soon as its slot
-    // is free; K may run ahead of V.  Ring positions: slot and the parity its
-    // `empty` wait takes (npre <= SK <= SV).
-    int nk = npre, nv = npre;
-    int sk = npre == SK ? 0 : npre, sv = npre == SV ? 0 : npre;
-    uint32_t phk = npre == SK ? 0u : 1u, phv = npre == SV ? 0u : 1u;
-    unsigned long long t_last = globaltimer();
+    // K units and V halves, each as soon as its slot is free
+    uint32_t spins = 0;   // polls without progress (kPollLimit of them take seconds)
     bool ok = true;
-    while (ok && (nk < n || nv < n)) {
+    while (ok && (kc < c1 || vc < c1)) {
       bool progress = false;
-      if (nk < n && mbar_test_warp(&k_empty[sk], phk)) {
-        const bool pre = nk < n_pre_here;
-        load_k(c0 + nk, sk, pre ? pol_kv : pol_q);
-        // keep the L2 warm 2 SK chunks ahead of the loads (prefix chunks only)
-        if (nk + 2 * SK < n_pre_here) warm(c0 + nk + 2 * SK);
-        ++nk;
-        if (++sk == SK) {
-          sk = 0;
-          phk ^= 1u;
-        }
+      if (kc < c1 && mbar_test_warp(&k_empty[sk], phk)) {
+        next_k();
         progress = true;
       }
-      if (nv < nk && mbar_test_warp(&v_empty[sv], phv)) {
-        const bool pre = nv < n_pre_here;
-        load_v(c0 + nv, sv, pre ? pol_kv : pol_q);
-        ++nv;
-        if (++sv == SV) {
-          sv = 0;
-          phv ^= 1u;
-        }
+      if (vc < c1 && mbar_test_warp(&v_empty[sv], phv)) {
+        next_v();
         progress = true;
       }
-      if (progress) t_last = globaltimer();
-      else ok = __all_sync(0xffffffffu, globaltimer() - t_last <= kTcTimeoutNs);
+      spins = progress ? 0u : spins + 1u;
+      if (spins > kPollLimit) ok = false;
     }
     if (lane == 0) {
       if (!ok) flags[0] = 1;
@@ -383,40 +404,44 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     el = elect_one();
     const uint32_t idesc_s = idesc_bf16(AT_BM, AT_BKV);
     const uint32_t idesc_o = idesc_bf16_bmn(AT_BM, p.hdp);
-    const uint64_t qd0 = sw128_desc(q0), kd0 = sw128_desc(k0), vd0 = sw128_mn_desc(v0, AT_KBLK);
+    const uint64_t qd0 = sw128_desc(q0), kd0 = sw128_desc(k0), vd0 = sw128_mn_desc(v0, AT_VBLK);
     bool ok = mbar_wait_warp(q_full, 0);
     // Issue S of the next chunk and PV of the oldest chunk whose P is ready,
     // whichever can go: PV(i) never waits for chunk i+1's K/V (that would
     // chain every chunk's load behind the previous PV).  S runs at most one
     // chunk ahead of PV (two S buffers in TMEM).
     int ns = 0, i = 0;   // next S, next PV
-    int sk = 0, sv = 0;  // their ring slots, and the parities of their waits
-    uint32_t phk = 0, phv = 0;
+    int uk = 0, uv = 0;  // K units and V halves consumed
     bool sdone_sent = false;
     // xch 2: every split learns when this split's last S has completed
     // (its Q and K ring may then receive the partials of the merge)
     const uint16_t smask = (uint16_t)((1u << p.splits) - 1u);
-    unsigned long long t_last = globaltimer();
+    phk = phv = 0;
+    uint32_t spins = 0;   // polls without progress (kPollLimit of them take seconds)
     while (ok && i < n) {
       bool progress = false;
-      if (ns < n && ns <= i + 1 && mbar_test_warp(&k_full[sk], phk) &&
-          (ns < 2 || mbar_test_warp(&s_free[ns & 1], (uint32_t)((ns >> 1) - 1) & 1u))) {
-        tc_fence_after();
-        uint64_t ad = qd0, bd = kd0 + (uint32_t)sk * (k_bytes >> 4);
+      if (ns < n && ns <= i + 1 && mbar_test_warp(&k_full[sk], phk)) {
         const uint32_t sd = tmem + (uint32_t)(ns & 1) * AT_BKV;
+        uint64_t ad = qd0;
         #pragma unroll 1
-        for (int blk = 0; blk < p.nblk; ++blk, ad += AT_QBLK >> 4, bd += AT_KBLK >> 4) {
+        for (int blk = 0; blk < p.nblk; ++blk, ad += AT_QBLK >> 4) {
+          ok = mbar_wait_warp(&k_full[sk], phk);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t bd = kd0 + (uint32_t)sk * (AT_KUNIT >> 4);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             umma_bf16(sd, ad + 2 * k, bd + 2 * k, idesc_s, (blk > 0 || k > 0) ? 1u : 0u, el);
+          umma_commit(&k_empty[sk], el);
+          ++uk;
+          if (++sk == SK) {
+            sk = 0;
+            phk ^= 1u;
+          }
         }
+        if (!ok) break;
         umma_commit(&s_full[ns & 1], el);
-        umma_commit(&k_empty[sk], el);   // K of this stage is free once S is done
         ++ns;
-        if (++sk == SK) {
-          sk = 0;
-          phk ^= 1u;
-        }
         if (p.xch == 2 && ns == n) {
           umma_commit_mc(sdone, smask, el);
           sdone_sent = true;
@@ -424,94 +449,107 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         progress = true;
       }
       if (i < ns && mbar_test_warp(&p_full[i & 1], (uint32_t)(i >> 1) & 1u) && mbar_test_warp(&v_full[sv], phv)) {
-        tc_fence_after();
-        // A = P from TMEM (the S tile's first 32 columns, two bf16 per column)
+        // A = P from TMEM (the S tile's first 64 columns, two bf16 per column),
+        // B = V [64 keys][hd], MN-major: 16 keys (two 8-row groups) per MMA, only
+        // the groups that hold keys
         const uint32_t pa = tmem + (uint32_t)(i & 1) * AT_BKV;
-        // B = V [64 keys][hd], MN-major: 16 keys (two 8-row groups) per K step
-        const uint64_t bd = vd0 + (uint32_t)sv * (k_bytes >> 4);
+        const int groups = (keys_of(c0 + i) + 15) >> 4;
+        #pragma unroll 1
+        for (int h = 0; 4 * h < groups; ++h) {
+          ok = mbar_wait_warp(&v_full[sv], phv);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t bd = vd0 + (uint32_t)sv * (v_bytes >> 4);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          umma_bf16_ts(tmem + o_col, pa + 8 * k, bd + 128 * k, idesc_o, (i > 0 || k > 0) ? 1u : 0u, el);
-        umma_commit(&v_empty[sv], el);
+          for (int k = 0; k < 4; ++k)
+            if (4 * h + k < groups)
+              umma_bf16_ts(tmem + o_col, pa + 8 * (4 * h + k), bd + 128 * k, idesc_o, (i + h + k > 0) ? 1u : 0u, el);
+          umma_commit(&v_empty[sv], el);
+          ++uv;
+          if (++sv == SV) {
+            sv = 0;
+            phv ^= 1u;
+          }
+        }
+        if (!ok) break;
         umma_commit(&pv_done[i & 1], el);
         ++i;
-        if (++sv == SV) {
-          sv = 0;
-          phv ^= 1u;
-        }
         progress = true;
       }
-      if (progress) t_last = globaltimer();
-      else ok = __all_sync(0xffffffffu, globaltimer() - t_last <= kTcTimeoutNs);
+      spins = progress ? 0u : spins + 1u;
+      if (spins > kPollLimit) ok = false;
     }
     // (no chunk, or an abort: arrive all the same, once earlier MMAs are done)
     if (p.xch == 2 && !sdone_sent) umma_commit_mc(sdone, smask, el);
     if (lane == 0) {
       if (!ok) flags[0] = 1;
-      flags[2] = ns;   // chunks whose K arrival was consumed
-      flags[4] = i;    // chunks whose V arrival was consumed
+      flags[2] = uk;   // K units whose arrival was consumed
+      flags[4] = uv;   // V halves whose arrival was consumed
     }
     __syncwarp();
     if (p.xch == 1) cluster_arrive_release();
-  } else if (warp >= 6) {
-    // merge-only warps: one arrival on the cluster barrier that opens the exchange
-    if (p.xch == 1) cluster_arrive_release();
   } else {
-    // softmax / epilogue: thread owns query row r (TMEM lane r)
-    const int q4 = warp & 3;
+    // softmax / epilogue: two threads per query row r (TMEM lane r), half hf = 0, 1
+    const int q4 = warp & 3, hf = warp >= 6 ? 1 : 0;
     const int r = q4 * 32 + lane;
+    auto pair_bar = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + q4) : "memory"); };   // warps w and w + 4
     const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16);
     const int t = r / p.G;
     const int j = qt * p.TQ + t;
-    float m_used = -INFINITY, l = 0.f;   // running max (log2 domain, scaled) and sum of P
+    float m_used = -INFINITY, l = 0.f;   // running max (log2 domain, scaled) of the row, sum of this half's P
     bool ok = true;
     int i = 0;
     const float sl2 = p.scale_log2;
-    for (int c = c0; c < c1 && ok; ++c) {
-      ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i & 1], (uint32_t)(i >> 1) & 1u));
+    // (after a wait that ran out the loop goes on without waiting, so that the
+    // two warps of a pair meet at every barrier)
+    for (int c = c0; c < c1; ++c) {
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i & 1], (uint32_t)(i >> 1) & 1u));
       tc_fence_after();
-      float sc[64];
+      float sc[64];   // this half's keys 64 hf .. 64 hf + 63 of the chunk
       {
         uint32_t raw[64];
+        const uint32_t srow = lane_base + (uint32_t)(i & 1) * AT_BKV + 64 * hf;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tmem_ld16_async(lane_base + (uint32_t)(i & 1) * AT_BKV + 16 * q, raw + 16 * q);
+        for (int q = 0; q < 4; ++q) tmem_ld16_async(srow + 16 * q, raw + 16 * q);
         tmem_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tmem_reg_fence16(raw + 16 * q);
 #pragma unroll
         for (int k = 0; k < 64; ++k) sc[k] = __uint_as_float(raw[k]);
       }
-      tc_fence_before();
-      mbar_arrive(&s_free[i & 1]);
-      // keys of this chunk that exist (prefix shorter than the chunk, ragged
-      // FOP + slot chunk) and, in the slot-isolated test mode, that are visible
-      const int kk0 = (c < npv) ? c * AT_BKV : (c - npv) * AT_BKV;
-      const int kvalid = (c < npv) ? P - kk0 : rows_per_robot - kk0;
-      const bool iso = (p.mask_mode == 1) && (c >= npv) && (kk0 < p.H);
-      // (two compact loops: this code runs cold at batch 1, where each
-      // instruction fetched costs more than it does)
-      if (kvalid < AT_BKV) {
+      // keys of the chunk that do not exist and, in the slot-isolated test mode,
+      // that are not visible count as -inf
+      const int kleft = keys_of(c) - 64 * hf;
+      if (kleft < 64) {
 #pragma unroll
-        for (int k = 0; k < 64; ++k) sc[k] = k < kvalid ? sc[k] : -INFINITY;
+        for (int k = 0; k < 64; ++k) sc[k] = k < kleft ? sc[k] : -INFINITY;
       }
-      if (iso) {
+      const int own0 = (c - npv) * AT_BKV + 64 * hf;   // the step's own keys: index of this half's first
+      if (p.mask_mode == 1 && c >= npv && own0 < p.H) {
 #pragma unroll
         for (int k = 0; k < 64; ++k)
-          if (kk0 + k < p.H && kk0 + k != j) sc[k] = -INFINITY;
+          if (own0 + k < p.H && own0 + k != j) sc[k] = -INFINITY;
       }
       float m8[8];
 #pragma unroll
       for (int a = 0; a < 8; ++a)
         m8[a] = fmaxf(fmaxf(fmaxf(sc[8 * a], sc[8 * a + 1]), fmaxf(sc[8 * a + 2], sc[8 * a + 3])),
                       fmaxf(fmaxf(sc[8 * a + 4], sc[8 * a + 5]), fmaxf(sc[8 * a + 6], sc[8 * a + 7])));
-      const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
-                             fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7]))) * sl2;
+      // the row's maximum over both halves; past the first barrier both have
+      // read their scores (P may overwrite them), past the second the maxima
+      xm[hf * 128 + r] =
+          fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])), fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
+      pair_bar();
+      const float mx = fmaxf(xm[r], xm[128 + r]) * sl2;
+      pair_bar();
       const float m_new = fmaxf(m_used, mx);
       const bool need = m_new > m_used + 8.f;
       if (i > 0 && __any_sync(0xffffffffu, need)) {
         // O must hold PV of every earlier chunk before it is rescaled
-        ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[(i - 1) & 1], (uint32_t)((i - 1) >> 1) & 1u)) && ok;
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[(i - 1) & 1], (uint32_t)((i - 1) >> 1) & 1u));
         tc_fence_after();
         const float alpha = need ? exp2f(m_used - m_new) : 1.f;   // exp2(-inf) = 0
-        for (int cb = 0; cb < p.hdp; cb += 16) {
+        for (int cb = 16 * hf; cb < p.hdp; cb += 32) {   // (the halves take alternate columns)
           float o[16];
           tmem_ld16(lane_base + o_col + cb, o);
 #pragma unroll
@@ -523,10 +561,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       }
       if (need) m_used = m_new;
       const float nb = (m_used == -INFINITY) ? 0.f : -m_used;
-      // P (bf16) overwrites the first 32 columns of this chunk's S tile: S of
-      // chunk i + 2 reuses the tile only after PV of chunk i has been issued,
-      // and the tensor pipe runs them in order
-      const uint32_t prow = lane_base + (uint32_t)(i & 1) * AT_BKV;
+      // P (bf16) overwrites the first 64 columns of this chunk's S tile, 32 of
+      // them this half's: S of chunk i + 2 reuses the tile only after PV of chunk
+      // i has been issued, and the tensor pipe runs them in order
+      const uint32_t prow = lane_base + (uint32_t)(i & 1) * AT_BKV + 32 * hf;
       float ls[8];
 #pragma unroll
       for (int h2 = 0; h2 < 2; ++h2) {
@@ -553,6 +591,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       tc_fence_after();
     }
     if (!ok && lane == 0) flags[0] = 1;
+    {   // the row's sum of P over both halves
+      xm[hf * 128 + r] = l;
+      pair_bar();
+      l = xm[r] + xm[128 + r];
+    }
     if (p.xch == 1) {
       // past this barrier every split of the cluster has finished its MMAs
       // (its Q and rings may be overwritten) and armed its receive barrier;
@@ -566,19 +609,17 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       if (!okd && lane == 0) flags[0] = 1;
     }
     if (p.splits == 1) {
-      // O / l as bf16: this thread stages its row in the rings (every chunk
-      // has been consumed and every MMA has completed, so nothing writes
-      // there any more; rows padded by 16 bytes so that the warp's 16-byte
-      // stores hit distinct banks) and hands it to the bulk copy engine as one
-      // contiguous hd-wide output row
+      // O / l as bf16 into Q's place and layout (every S has completed), from
+      // where one TMA store per 64 head dims writes the tile's slots; the output
+      // map clips the slots past H (a bulk copy per row took each warp 32 issues)
       const float inv = (l > 0.f && n > 0) ? 1.f / l : 0.f;
-      const int rbytes = ((2 * p.hdp + 63) & ~63) + 16;   // whole 32-column writes, + 16 against bank conflicts
-      uint8_t* srow = kv_s + (size_t)r * rbytes;
-      for (int cb = 0; cb < p.hdp; cb += 32) {
+      for (int cb = 32 * hf; cb < p.hdp; cb += 64) {   // (the halves take alternate 32 columns)
         uint32_t raw[32];
-        tmem_ld16_async(lane_base + o_col + cb, raw);
-        tmem_ld16_async(lane_base + o_col + cb + 16, raw + 16);
+        tmem_ld32_async(lane_base + o_col + cb, raw);
         tmem_wait_ld();
+        tmem_reg_fence16(raw);
+        tmem_reg_fence16(raw + 16);
+        uint8_t* row = q_s + (size_t)(cb >> 6) * AT_QBLK + (size_t)r * 128;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           uint4 w;
@@ -586,14 +627,14 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
           w.y = pack_bf16x2(__uint_as_float(raw[8 * q + 2]) * inv, __uint_as_float(raw[8 * q + 3]) * inv);
           w.z = pack_bf16x2(__uint_as_float(raw[8 * q + 4]) * inv, __uint_as_float(raw[8 * q + 5]) * inv);
           w.w = pack_bf16x2(__uint_as_float(raw[8 * q + 6]) * inv, __uint_as_float(raw[8 * q + 7]) * inv);
-          *(uint4*)(srow + (cb / 8 + q) * 16) = w;
+          *(uint4*)(row + ((((cb & 32) >> 3) + q) ^ (r & 7)) * 16) = w;   // 128-byte swizzle
         }
       }
-      const int t = r / p.G, jj = qt * p.TQ + t;
-      if (r < q_rows && jj < p.H) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        bulk_copy_s2g(p.out + (size_t)(b * p.H + jj) * p.ld_out + (size_t)(g * p.G + r % p.G) * p.hd, srow,
-                      (uint32_t)(2 * p.hd));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("bar.sync 5, 256;" ::: "memory");
+      if (threadIdx.x == 64 && vrows > 0) {
+        for (int blk = 0; blk < p.nblk; ++blk)
+          tma_store_4d(&maps.o, q_s + (size_t)blk * AT_QBLK, blk * 64, g * p.G, qt * p.TQ, b);
         bulk_commit();
         bulk_wait_read<0>();   // read out before the shared memory goes away
       }
@@ -609,7 +650,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       const uint32_t base = smem_u32(smem);
       const uint32_t o0 = base + (uint32_t)(split * ngs * AT_BM + r) * 16u;
       const uint32_t bar0 = smem_u32(rcv_bar);
-      if (snd) {
+      if (snd && hf == 0) {
         const uint32_t ml0 = base + (uint32_t)(p.splits * ngs * AT_BM) * 16u + (uint32_t)(split * AT_BM + r) * 8u;
         const float m_s = has ? m_used : -INFINITY, l_s = has ? l : 0.f;
         for (int q = 0; q < p.splits; ++q) st_async_f2(mapa_shared(ml0, (uint32_t)q), m_s, l_s, mapa_shared(bar0, (uint32_t)q));
@@ -617,18 +658,18 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       // 32 columns per TMEM load (16 where hdp is not a multiple of 32), the
       // next load in flight while this one goes out
       const int cw = (p.hdp % 32 == 0) ? 32 : 16;
-      const int nch = p.hdp / cw;
-      int ch = (split * cps) / cw;
+      const int nch = p.hdp / cw, nown = (nch + 1 - hf) / 2;   // the halves take alternate chunks
+      int ch = ((split * cps) / cw + hf) % nch;
       uint32_t cur[32];
-      if (cw == 32) tmem_ld32_async(lane_base + o_col + 32 * ch, cur);
-      else tmem_ld16_async(lane_base + o_col + 16 * ch, cur);
+      if (cw == 32 && nown) tmem_ld32_async(lane_base + o_col + 32 * ch, cur);
+      else if (nown) tmem_ld16_async(lane_base + o_col + 16 * ch, cur);
       tmem_wait_ld();
       tmem_reg_fence16(cur);
       tmem_reg_fence16(cur + 16);
-      for (int jj = 0; jj < nch; ++jj) {
-        const int chn = ch + 1 == nch ? 0 : ch + 1;
+      for (int jj = 0; jj < nown; ++jj) {
+        const int chn = ch + 2 >= nch ? ch + 2 - nch : ch + 2;
         uint32_t nxt[32];
-        if (jj + 1 < nch) {
+        if (jj + 1 < nown) {
           if (cw == 32) tmem_ld32_async(lane_base + o_col + 32 * chn, nxt);
           else tmem_ld16_async(lane_base + o_col + 16 * chn, nxt);
         }
@@ -657,7 +698,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
             send8(3);
           }
         }
-        if (jj + 1 < nch) {
+        if (jj + 1 < nown) {
           tmem_wait_ld();
           tmem_reg_fence16(nxt);
           tmem_reg_fence16(nxt + 16);
@@ -671,7 +712,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       // contiguous 512-byte run per 4 columns), plus this split's (m, l)
       const size_t ti = ((size_t)bg * gridDim.x + qt) * p.splits + split;
       float* dst = p.ws_o + ti * (size_t)(p.hdp / 4) * 512 + (size_t)r * 4;
-      for (int cb = 0; cb < p.hdp; cb += 64) {   // up to four TMEM loads in flight, one wait
+      for (int cb = 64 * hf; cb < p.hdp; cb += 128) {   // up to four TMEM loads in flight, one wait
         const int nq = min(4, (p.hdp - cb) / 16);
         uint32_t raw[64];
 #pragma unroll
@@ -686,8 +727,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
                                          __uint_as_float(raw[4 * q + 2]), __uint_as_float(raw[4 * q + 3]))
                            : make_float4(0.f, 0.f, 0.f, 0.f));
       }
-      __stcg(p.ws_ml + (ti * 2) * AT_BM + r, (n > 0) ? m_used : -INFINITY);
-      __stcg(p.ws_ml + (ti * 2 + 1) * AT_BM + r, (n > 0) ? l : 0.f);
+      if (hf == 0) {
+        __stcg(p.ws_ml + (ti * 2) * AT_BM + r, (n > 0) ? m_used : -INFINITY);
+        __stcg(p.ws_ml + (ti * 2 + 1) * AT_BM + r, (n > 0) ? l : 0.f);
+      }
       __threadfence();
     }
   }
@@ -794,6 +837,19 @@ cudaError_t enc3(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uin
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The output as (hd, heads, slots, robots), boxes of 64 x G x TQ x 1: slots past
+// the robot's own are clipped.
+cudaError_t enc_out(CUtensorMap* m, void* base, int hd, int heads, int H, int B, int ld, int G, int TQ) {
+  cuuint64_t dims[4] = {(cuuint64_t)hd, (cuuint64_t)heads, (cuuint64_t)H, (cuuint64_t)B};
+  cuuint64_t strides[3] = {(cuuint64_t)hd * 2, (cuuint64_t)ld * 2, (cuuint64_t)H * ld * 2};
+  cuuint32_t box[4] = {64, (cuuint32_t)G, (cuuint32_t)TQ, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = g_enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 }  // namespace
 
 cudaError_t init_attention_tc() {
@@ -839,28 +895,34 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   p.layer = a.layer; p.Bmax = a.Bmax; p.mask_mode = a.mask_mode;
   p.nblk = (a.hd + 63) / 64;
   p.ctx_state = a.ctx_state;
+  for (int s = 0; s < 2; ++s) {
+    p.ck[s] = (const bf16*)a.ctx_k[s];
+    p.cv[s] = (const bf16*)a.ctx_v[s];
+  }
   p.out = (bf16*)a.out; p.ld_out = a.ld_out;
   p.err = a.err;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
-  // Query tiles of 128 rows, or of 64 where the keys are split, and the number
-  // of key splits (one cluster per query tile, a power of two whose head-dim
-  // slices are multiples of 4 columns): the least estimated time.  A CTA costs
-  // about 4 us and each of its 64-key chunks the issue of S (4 MMAs per 64 of
-  // head dim, 36 ns each) and of P V, or the softmax's 0.45 us; the merge moves
-  // every split's rows x hd partial between the SMs, so it grows with the rows
-  // of a tile (the MMAs are always 128 rows) and with the splits; a grid that
-  // does not fit the SMs at once (36 clusters of 4, 15 of 8, 7 of 16) takes
-  // another round.  16 robots, 16 slots, 2048 keys: 4 splits; 8 would run 16
-  // clusters in two rounds (27 us per layer against 16).
+  // Query tiles of 128 rows, or of 64 where the keys are split (32: one robot's
+  // 104 CTAs, 652 us per step against 635), and the number of key splits (one
+  // cluster per query tile, a power of two whose head-dim slices are multiples
+  // of 4 columns): the least estimated time.  A
+  // CTA costs about 4 us, each of its chunks the tensor pipe's time for S and
+  // P V (1.2 us at head dim 256) or the softmax's 0.95; the merge moves every
+  // split's rows x hd partial between the SMs at 16 bytes per clock (the MMAs
+  // are always 128 rows); a grid that does not fit the SMs at once (36 clusters
+  // of 4, 15 of 8, 7 of 16) takes another round.  (From per-CTA stamps.  16
+  // robots, 16 slots, 2048 keys: 4 splits; 8 would run 16 clusters in two
+  // rounds, 27 us per layer against 16.)
   const int C = (a.Pmax + AT_BKV - 1) / AT_BKV + p.n_kv;
-  const float t_chunk = std::max(0.45f, 0.036f * 4.f * (float)p.nblk + 0.26f * std::max(0.55f, (float)p.hdp / 256.f));
+  const float hd_rel = (float)p.hdp / 256.f;
+  const float t_chunk = std::max(0.95f, 0.1f + 0.144f * (float)p.nblk + 0.52f * std::max(0.55f, hd_rel));
   float cost = 3.4e38f;
   auto consider = [&](int rows, int splits, int resident) {
     const int tq = std::max(1, rows / p.G);
     const int qt = (a.H + tq - 1) / tq, ctas = qt * a.B * a.Hkv;
     const int rounds = (ctas + resident - 1) / resident;
     float t = (float)rounds * (4.f + t_chunk * (float)((C + splits - 1) / splits));
-    if (splits > 1) t += (float)rounds * (0.6f + 1.4f * (float)rows / 128.f + 0.15f * (float)splits);
+    if (splits > 1) t += (float)rounds * (1.f + 2.05f * hd_rel * (float)rows / 128.f + 0.1f * (float)splits);
     if (t < cost) {
       cost = t;
       p.q_tiles = qt;
@@ -871,7 +933,7 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   consider(AT_BM, 1, a.num_sms);
   for (int i = 0; i < 4; ++i) {
     const int sp = 2 << i;
-    if (sp * 2 > C + 1 || (p.hdp / sp) % 4 != 0 || p.hdp % sp != 0 || !g_attn_clusters[i]) break;
+    if (sp >= 2 * C || (p.hdp / sp) % 4 != 0 || p.hdp % sp != 0 || !g_attn_clusters[i]) break;
     for (int rows = AT_BM; rows >= 64; rows /= 2) {
       const int tq = std::max(1, rows / p.G);
       const size_t ctas = (size_t)((a.H + tq - 1) / tq) * a.B * a.Hkv;
@@ -885,19 +947,13 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   // slice, and the receive area (O groups + (m, l) of every split) within
   // Q + the rings (checked below)
   p.xch = splits > 1 && (p.hdp / splits) % 8 == 0 ? 1 : 0;
-  // K slots: as many whole K + V stages as fit (<= 4); V slots: the K count
-  // plus what the remaining bytes hold (<= 2 more): K is free again as soon
-  // as S = Q K^T is done, V only after P V, so V needs the depth
-  const size_t k_bytes = (size_t)p.nblk * AT_KBLK;
-  const size_t stage = 2 * k_bytes;
-  const size_t fixed = 1024 + (size_t)p.nblk * AT_QBLK + 512;
-  if (fixed + stage > (size_t)AT_SMEM_MAX) return cudaErrorInvalidConfiguration;
-  const int sk = (int)std::min<size_t>(4, (AT_SMEM_MAX - fixed) / stage);
-  const int sv = sk + (int)std::min<size_t>(2, (AT_SMEM_MAX - fixed - sk * stage) / k_bytes);
-  const size_t rings = (size_t)(sk + sv) * k_bytes;
-  // the epilogue stages 128 bf16 rows of O in the rings and stores them with
-  // 16-byte writes
-  if ((size_t)AT_BM * (size_t)(((2 * p.hdp + 63) & ~63) + 16) > rings) return cudaErrorInvalidConfiguration;
+  // K units and V halves beside Q: at head dim 256 one chunk's four units and
+  // three halves; smaller heads have room for more
+  const size_t v_bytes = (size_t)p.nblk * AT_VBLK;
+  const size_t fixed = 1024 + (size_t)p.nblk * AT_QBLK + 512 + 1024;   // alignment, Q, barriers, row maxima / sums
+  const int sk = p.nblk == 4 ? 4 : p.nblk == 1 ? 8 : 6;
+  const int sv = (int)std::min<size_t>(8, (AT_SMEM_MAX - fixed - sk * AT_KUNIT) / v_bytes);
+  const size_t rings = (size_t)sk * AT_KUNIT + (size_t)sv * v_bytes;
   if (a.ld_out % 8 != 0 || ((uintptr_t)a.out & 15u) != 0) return cudaErrorMisalignedAddress;
   p.k_slots = sk;
   p.v_slots = sv;
@@ -905,7 +961,7 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   if (p.xch && (size_t)AT_BM * p.hdp * 2 + (size_t)splits * AT_BM * 8 > (size_t)p.nblk * AT_QBLK + rings) p.xch = 0;
   // the receive area within Q and the K ring (free once S is done): send
   // without waiting for the other splits' PV
-  if (p.xch && (size_t)AT_BM * p.hdp * 2 + (size_t)splits * AT_BM * 8 <= (size_t)p.nblk * AT_QBLK + (size_t)sk * k_bytes)
+  if (p.xch && (size_t)AT_BM * p.hdp * 2 + (size_t)splits * AT_BM * 8 <= (size_t)p.nblk * AT_QBLK + (size_t)sk * AT_KUNIT)
     p.xch = 2;
 
   AtMaps m;
@@ -917,14 +973,15 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
              64, 1, AT_BKV);
   if (e == cudaSuccess)
     e = enc3(&m.v, (const bf16*)a.qkv + (size_t)(a.Hq + a.Hkv) * hd, hd, a.Hkv, rows, (uint64_t)hd * 2,
-             (uint64_t)a.ld_qkv * 2, 64, 1, AT_BKV);
+             (uint64_t)a.ld_qkv * 2, 64, 1, 64);
+  if (e == cudaSuccess) e = enc_out(&m.o, a.out, hd, a.Hq, a.H, a.B, a.ld_out, p.G, p.TQ);
   const uint64_t zc = (uint64_t)(a.layers * a.Bmax * a.Hkv);
   for (int s = 0; s < 2 && e == cudaSuccess; ++s) {
     e = enc3(s ? &m.pk1 : &m.pk0, a.ctx_k[s], hd, a.Pmax, zc, (uint64_t)hd * 2, (uint64_t)a.Pmax * hd * 2, 64,
              AT_BKV, 1);
     if (e == cudaSuccess)
-      e = enc3(s ? &m.pv1 : &m.pv0, a.ctx_v[s], hd, a.Pmax, zc, (uint64_t)hd * 2, (uint64_t)a.Pmax * hd * 2, 64,
-               AT_BKV, 1);
+      e = enc3(s ? &m.pv1 : &m.pv0, a.ctx_v[s], hd, a.Pmax, zc, (uint64_t)hd * 2, (uint64_t)a.Pmax * hd * 2, 64, 64,
+               1);
   }
   if (e != cudaSuccess) return e;
   dim3 grid(p.q_tiles, a.B * a.Hkv, splits);

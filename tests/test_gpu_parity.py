@@ -164,3 +164,18 @@ def test_full_size_configs_sampled(name, robots):
     s = gpu_session(case)
     check_step(case, s, robots=robots, label=name)
     s.close()
+
+
+# Chunks of 128 keys in two halves: prefixes that end inside the first or the
+# second half, at their edges and one key past them, own keys (slots + FOP) in
+# one and two halves and chunks, unsplit (many robots) and split; capacities
+# above the prefix.
+@pytest.mark.parametrize("prefix,capacity", [(1, 1), (63, 200), (64, 64), (65, 129), (127, 128), (128, 384), (129, 700)])
+@pytest.mark.parametrize("batch,slots,fop", [(1, 50, 16), (40, 20, 4), (2, 130, 3)])
+def test_attention_chunk_edges(prefix, capacity, batch, slots, fop):
+    cfg = synth.ExpertConfig(layers=1, width=128, n_q_heads=4, n_kv_heads=2, head_dim=64, mlp_dim=128, slots=slots,
+                             action_dim=4, prefix=capacity, fop_tokens=fop, batch=batch, dtype="bf16")
+    case = Case(cfg, prefix_len=prefix)
+    s = gpu_session(case)
+    check_step(case, s, robots=sorted({0, batch // 2, batch - 1}), label=f"prefix {prefix}")
+    s.close()
