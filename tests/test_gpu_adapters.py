@@ -46,3 +46,18 @@ def test_adapters_pi05_width_one_robot():
     s = gpu_session(case)
     check_step(case, s, label="pi05 width, adapters in every layer")
     s.close()
+
+
+# FOP adapter attention at the edges of its work split: one key, a key count that
+# fills a lane's first and second key, slots in one and two halves, and head
+# dims from one float4 per lane group to the largest
+@pytest.mark.parametrize("fop,slots,hd,dtype", [(1, 3, 8, "fp32"), (32, 9, 40, "fp32"), (33, 8, 256, "bf16"),
+                                                (64, 17, 64, "bf16"), (5, 30, 96, "fp32")])
+def test_adapter_attention_edges(fop, slots, hd, dtype):
+    from tests._harness import Case, check_step, gpu_session
+    cfg = synth.ExpertConfig(layers=2, width=128, n_q_heads=4, n_kv_heads=2, head_dim=hd, mlp_dim=128, slots=slots,
+                             action_dim=4, prefix=20, fop_tokens=fop, batch=2, dtype=dtype, fop_adapter_every=1)
+    case = Case(cfg)
+    s = gpu_session(case)
+    check_step(case, s, label=f"{fop} keys")
+    s.close()
