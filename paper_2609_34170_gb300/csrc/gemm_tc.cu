@@ -64,11 +64,11 @@ enum { RED_NONE = 0, RED_L2_CLUSTER = 1, RED_DSMEM = 2, RED_DSMEM32 = 3 };
 // Epilogue kind of an instantiation: outputs through TMA boxes as fp32, bf16,
 // a reduce-add into the fp32 residual stream or the GeGLU pair -- fixed, so
 // that a long persistent launch carries only the code of its own epilogue --
-// or any of these chosen at run time (EK_TMA_ANY: the
-// short split-K launches of one step then all run one binary, whose code the
-// previous launch has left in the SM's instruction cache), or stored by the
-// threads (EK_GENERIC: any epilogue; unaligned outputs).
-enum { EK_F32 = 0, EK_BF16 = 1, EK_ADD = 2, EK_GEGLU = 3, EK_GENERIC = 4, EK_TMA_ANY = 5 };
+// or stored by the threads: a split rank's slice (EK_SLICE: any epilogue, so
+// that the short split-K launches of one step all run one binary, whose code
+// the previous launch has left in the SM's instruction cache), or any tile
+// (EK_GENERIC: unaligned outputs).
+enum { EK_F32 = 0, EK_BF16 = 1, EK_ADD = 2, EK_GEGLU = 3, EK_GENERIC = 4, EK_SLICE = 5 };
 
 
 struct TcParams {
@@ -94,9 +94,7 @@ struct TcParams {
   uint32_t stg_off;     // SIMT transpose tile, or two TMA output boxes
   uint32_t xch_off;     // GeGLU exchange
   uint32_t rcv_off;     // RED_DSMEM*: the partials received from the splits, [split][cpr / 4][128 rows]
-                        // float4, overlaid on the operand ring (free once every CTA of the cluster
-                        // has finished its MMAs), else on the output boxes + exchange (used only
-                        // after the sum)
+                        // float4 (bf16: two rows per 16 bytes)
   uint32_t bar_off;     // mbarriers, TMEM slot, flags
   unsigned long long wait_ns;   // limit of every bounded wait (ERR_TIMEOUT after it)
   int withhold;         // fault injection (tests): the MMA thread first waits for an arrival that
@@ -105,11 +103,6 @@ struct TcParams {
                         // completes the copies it started and exits without computing
   uint32_t set_bytes;   // pair kernel: bytes from epilogue set 0's boxes / exchange to set 1's
 };
-
-// The TMA epilogue kind of a launch (EK_F32 .. EK_GEGLU).
-__device__ __forceinline__ int tma_kind(const TcParams& p) {
-  return p.epi == EPI_GEGLU ? EK_GEGLU : p.epi == EPI_ADD_F32 ? EK_ADD : p.out_bf16 ? EK_BF16 : EK_F32;
-}
 
 // The i-th work item of this CTA: a tile (tn, tm) and split sp.  With splits
 // the grid is (tiles_n, tiles_m, splits) and every CTA has one item; without,
@@ -346,7 +339,7 @@ __device__ __forceinline__ void epilogue_tma(const TcParams& p, const CUtensorMa
   if (issuer) bulk_wait_read<1>();
   epi_bar_set(set);
   uint8_t* box = boxes + (size_t)ebuf * p.box_bytes;
-  const int kind = EK == EK_TMA_ANY ? tma_kind(p) : EK;   // a constant in the fixed-kind instantiations
+  constexpr int kind = EK;
   if (kind == EK_GEGLU) {
     // tile rows 0..63 are gate features, 64..127 the matching up features:
     // transpose through xch so that every thread then forms 8 outputs of one
@@ -390,6 +383,82 @@ __device__ __forceinline__ void epilogue_tma(const TcParams& p, const CUtensorMa
   ebuf ^= 1;
 }
 
+// The outputs of a split rank's slice: v[i] is this thread's tile row r at token
+// m0+i (i < cpr <= 32), brow its bias; all 128 epilogue threads call it
+// together.  Stored (or added) by the threads, a warp 128 bytes of one token per
+// instruction: the slice is 4 to 16 KB, and a box in shared memory with its
+// proxy fence, barriers and TMA store took 1100 to 1900 cycles of the launch's
+// critical path.  xch: the idle operand ring (GeGLU's transpose).
+__device__ __forceinline__ void store_slice(const TcParams& p, int tile_n, int m0, int cpr, int r, const float* v,
+                                            float brow, float* xch) {
+  const int lim = min(cpr, p.M - m0);   // tokens that exist (may be <= 0)
+  const int n = tile_n * TC_BM + r;
+  if (p.epi == EPI_GEGLU) {
+    // rows 0..63 are gate features, 64..127 the matching up features: through
+    // xch, every thread then forms 8 outputs of one token
+    for_upto<32>(cpr, [&](int i) { xch[i * STG_LD + r] = v[i] + brow; });
+    epi_bar();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = (r >> 3) + 16 * h, fg = r & 7;
+      if (c < lim) {
+        const float4* g4 = (const float4*)(xch + c * STG_LD + fg * 8);
+        const float4* u4 = (const float4*)(xch + c * STG_LD + 64 + fg * 8);
+        const float4 ga = g4[0], gb = g4[1], ua = u4[0], ub = u4[1];
+        *(uint4*)((bf16*)p.out + (size_t)(m0 + c) * p.ldo + tile_n * 64 + fg * 8) =
+            make_uint4(pack_bf16x2(gelu_tanh_bf16out(ga.x) * ua.x, gelu_tanh_bf16out(ga.y) * ua.y),
+                       pack_bf16x2(gelu_tanh_bf16out(ga.z) * ua.z, gelu_tanh_bf16out(ga.w) * ua.w),
+                       pack_bf16x2(gelu_tanh_bf16out(gb.x) * ub.x, gelu_tanh_bf16out(gb.y) * ub.y),
+                       pack_bf16x2(gelu_tanh_bf16out(gb.z) * ub.z, gelu_tanh_bf16out(gb.w) * ub.w));
+      }
+    }
+  } else if (p.epi == EPI_ADD_F32) {
+    float* o = (float*)p.out + (size_t)m0 * p.ldo + n;
+    const bool in = n < p.N;
+#pragma unroll
+    for (int g = 0; g < 32; g += 4) {
+      if (g >= lim) break;
+#pragma unroll
+      for (int i = g; i < g + 4; ++i)   // one add per element: the result does not depend on an order
+        if (in && i < lim) atomicAdd(o + (size_t)i * p.ldo, v[i] + brow);
+    }
+  } else {
+    const bool silu = p.epi == EPI_STORE_SILU;
+    auto value = [&](int i) { return silu ? silu_f(v[i] + brow) : v[i] + brow; };
+    if (p.out_bf16) {
+      // lanes of rows r and r + 1 swap tokens i + 1 and i: each then stores both
+      // rows of one token
+      const bool odd = r & 1;
+      bf16* o = (bf16*)p.out + (size_t)(m0 + (odd ? 1 : 0)) * p.ldo + (n & ~1);
+      const bool both = (n | 1) < p.N, one = (n & ~1) < p.N;
+#pragma unroll
+      for (int g = 0; g < 32; g += 4) {
+        if (g >= lim) break;
+#pragma unroll
+        for (int i = g; i < g + 4; i += 2) {
+          const float a = value(i), b = value(i + 1);
+          const float got = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+          const uint32_t w = odd ? pack_bf16x2(got, b) : pack_bf16x2(a, got);
+          if (i + (odd ? 1 : 0) < lim) {
+            if (both) *(uint32_t*)(o + (size_t)i * p.ldo) = w;
+            else if (one) *(uint16_t*)(o + (size_t)i * p.ldo) = (uint16_t)w;
+          }
+        }
+      }
+    } else {
+      float* o = (float*)p.out + (size_t)m0 * p.ldo + n;
+      const bool in = n < p.N;
+#pragma unroll
+      for (int g = 0; g < 32; g += 4) {
+        if (g >= lim) break;
+#pragma unroll
+        for (int i = g; i < g + 4; ++i)
+          if (in && i < lim) o[(size_t)i * p.ldo] = value(i);
+      }
+    }
+  }
+}
+
 // RED = p.reduce and EK = the epilogue kind, fixed per instantiation so that
 // each reduction mode gets its own register allocation and each launch only
 // the code it runs.
@@ -429,7 +498,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const int kb1_first = (int)((long)(sp0 + 1) * p.num_kb / p.splits);
   const int npre = has_work ? min(S, kb1_first - kb0_first) : 0;
   const int cpr = BN / p.splits;   // tokens of the slice each split rank owns (a multiple of 4)
-  constexpr bool TMA_OUT = EK != EK_GENERIC;
+  constexpr bool TMA_OUT = EK < EK_GENERIC;
   // partials exchanged through distributed shared memory: RED_DSMEM in bf16
   // (two rows per message), RED_DSMEM32 in fp32
   constexpr bool DSM = RED == RED_DSMEM || RED == RED_DSMEM32;
@@ -492,6 +561,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     }
   };
   if (warp == 0 && !p.skip) issue_weight_prologue();
+  // RED_DSMEM*: this CTA's receive barrier is armed; the epilogue warps wait for
+  // the whole cluster's before they send
+  if constexpr (DSM) cluster_arrive_release();
   // everything below may read what earlier kernels wrote; TMEM is taken only
   // now, so a CTA waiting here never holds columns its predecessor needs
   pdl_wait();
@@ -553,9 +625,6 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     }
     if (lane == 0) flags[2] = it;
     __syncwarp();
-    // RED_DSMEM*: one arrival per thread on the cluster barrier that opens the
-    // exchange (the epilogue warps arrive once their MMAs are complete)
-    if constexpr (DSM) cluster_arrive_release();
   } else if (warp == 1) {
     el = elect_one();
     const uint32_t idesc = idesc_bf16(TC_BM, BN);
@@ -630,7 +699,6 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       flags[3] = it;
     }
     __syncwarp();
-    if constexpr (DSM) cluster_arrive_release();
   } else {
     // epilogue warps 2..5: TMEM lane quarter q = warp % 4, tile row r
     const int q = warp & 3;
@@ -640,13 +708,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     for (int i = 0; work_item(p, i, tn, tm, sp); ++i) {
       const int b = i & 1;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)(i >> 1) & 1u, p.wait_ns));
-      if constexpr (DSM) {
-        // past this barrier every CTA of the cluster has finished its MMAs
-        // (its operand ring may be overwritten) and armed its receive barrier;
-        // every thread arrives exactly once, whatever happened before
-        cluster_arrive_release();
-        cluster_wait_acquire();
-      }
+      if constexpr (DSM) cluster_wait_acquire();   // every CTA of the cluster has armed its receive barrier
       if (!ok) {
         if (lane == 0) flags[0] = 1;
         break;
@@ -715,7 +777,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             const uint32_t got0 = __shfl_xor_sync(0xffffffffu, odd ? p0 : p2, 1);
             const uint32_t got1 = __shfl_xor_sync(0xffffffffu, odd ? p1 : p3, 1);
             const uint4 w = odd ? make_uint4(got0, got1, p2, p3) : make_uint4(p0, p1, got0, got1);
-            st_async_u4(mapa_shared(rcv0 + (uint32_t)gl * 1024u, (uint32_t)dst), w, mapa_shared(bar0, (uint32_t)dst));
+            const uint32_t to = mapa_shared(rcv0, (uint32_t)dst);
+            st_async_u4(to + (uint32_t)gl * 1024u, w, to + (bar0 - rcv0));
             // two groups on: a select per rank boundary, not a branch
             gl += 2;
             bool wrap = gl >= ngs;
@@ -802,9 +865,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     // Rank q sums its slice of tokens [q*cpr, (q+1)*cpr) over the splits in
     // order once every split's bytes have arrived (the wait also keeps this
     // CTA alive until no store into its shared memory is in flight), then
-    // sends the whole slice out as one box.  (When the partials overlay the
-    // output boxes, epilogue_tma passes a barrier of all 128 threads before it
-    // writes over what was just read.)
+    // stores the slice from the threads (store_slice).
     if (warp >= 2) {
       const int r = (warp & 3) * 32 + lane;
       const bool ok = __all_sync(0xffffffffu, mbar_wait_cluster(rcv_bar, 0, p.wait_ns));
@@ -841,9 +902,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             default: reduce_slice_smem<8>(b0, p.splits, v); break;
           }
         }
-        int ebuf = 0;
-        if constexpr (TMA_OUT) epilogue_tma<EK, 32>(p, &tmO, tn0, tm0 * BN + sp0 * cpr, r, v, brow, stg_raw, xch, ebuf);
-        if (threadIdx.x == 64) bulk_wait_read<0>();
+        store_slice(p, tn0, tm0 * BN + sp0 * cpr, cpr, r, v, brow, (float*)smem);
       }
     }
   }
@@ -1164,7 +1223,7 @@ TcKernel tc_kernel(int red, int ek) {
   RAVEL_TC_K(RED_NONE, EK_F32) RAVEL_TC_K(RED_NONE, EK_BF16) RAVEL_TC_K(RED_NONE, EK_ADD)
   RAVEL_TC_K(RED_NONE, EK_GEGLU) RAVEL_TC_K(RED_NONE, EK_GENERIC)
   RAVEL_TC_K(RED_L2_CLUSTER, EK_GENERIC)
-  RAVEL_TC_K(RED_DSMEM, EK_TMA_ANY) RAVEL_TC_K(RED_DSMEM32, EK_TMA_ANY)
+  RAVEL_TC_K(RED_DSMEM, EK_SLICE) RAVEL_TC_K(RED_DSMEM32, EK_SLICE)
 #undef RAVEL_TC_K
   return nullptr;
 }
@@ -1365,7 +1424,7 @@ cudaError_t init_tc_gemm() {
   if (e != cudaSuccess) return e;
   std::vector<const void*> kernels;
   for (int red = 0; red <= RED_DSMEM32; ++red)
-    for (int ek = 0; ek <= EK_TMA_ANY; ++ek)
+    for (int ek = 0; ek <= EK_SLICE; ++ek)
       if (TcKernel k = tc_kernel(red, ek)) kernels.push_back((const void*)k);
   for (int ek = 0; ek < EK_GENERIC; ++ek) kernels.push_back((const void*)tc_pair_kernel(ek));
   for (const void* k : kernels) {
@@ -1389,7 +1448,7 @@ cudaError_t init_tc_gemm() {
     cfg.numAttrs = 1;
     int n = 0;
     g_max_clusters[i] =
-        cudaOccupancyMaxActiveClusters(&n, tc_kernel(RED_DSMEM, EK_TMA_ANY), &cfg) == cudaSuccess && n > 0 ? n : 0;
+        cudaOccupancyMaxActiveClusters(&n, tc_kernel(RED_DSMEM, EK_SLICE), &cfg) == cudaSuccess && n > 0 ? n : 0;
   }
   cudaGetLastError();
   return cudaSuccess;
@@ -1435,29 +1494,27 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   // range when that fits, so that no operand load waits for a freed stage
   if (splits > 1) stages = std::min(stages, std::max(2, TC_RING_SPLIT / stage_bytes));
   stages = std::max(2, std::min(stages, std::max(2, kb_per_item * items)));
-  // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
-  // takes its weight and token k-tiles in one box each (K a multiple of 64)
-  const bool oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
-                       (size_t)kb_per_item * stage_bytes <= (size_t)TC_SMEM_BUDGET;
-  if (oneshot) stages = kb_per_item;   // the ring is exactly one box deep
-  const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
   // partials exchanged in bf16 where the caller allows it, else in fp32
   const bool xbf = g.xbf16 != 0;
   const bool dsmem = splits > 1 && tma_out;
+  const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
+  // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
+  // takes its weight and token k-tiles in one box each (K a multiple of 64)
+  const bool oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
+                       (size_t)kb_per_item * stage_bytes <=
+                           std::min<size_t>(TC_SMEM_BUDGET, TC_SMEM_MAX - 4096 - (rcv_bytes + 1023) / 1024 * 1024);
+  if (oneshot) stages = kb_per_item;   // the ring is exactly one box deep
+  const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
   const int reduce = splits == 1 ? RED_NONE : !dsmem ? RED_L2_CLUSTER : xbf ? RED_DSMEM : RED_DSMEM32;
-  // tokens per output box: a split's whole slice through shared memory
-  const int box_m = splits == 1 ? 16 : dsmem ? cpr : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
+  // tokens per output box; a split's slice is stored by the threads, its
+  // received partials (all splits' slices of this rank) behind the ring
+  const int box_m = splits == 1 ? 16 : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
   const uint32_t box_bytes =
       (uint32_t)(((size_t)box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
-  const size_t stg_bytes = tma_out ? 2 * (size_t)box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
-  const size_t xch_bytes = (tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
-  // received partials (all splits' slices of this rank) overlay the operand
-  // ring, else the boxes + exchange
-  const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
-  const bool in_ring = rcv_bytes <= ring;
-  const uint32_t stg_off = (uint32_t)ring, xch_off = stg_off + (uint32_t)stg_bytes;
-  const uint32_t rcv_off = in_ring ? 0u : stg_off;
-  const uint32_t bar_off = stg_off + (uint32_t)std::max(stg_bytes + xch_bytes, in_ring ? (size_t)0 : rcv_bytes);
+  const size_t stg_bytes = dsmem ? rcv_bytes : tma_out ? 2 * (size_t)box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
+  const size_t xch_bytes = (splits == 1 && tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
+  const uint32_t stg_off = (uint32_t)ring, xch_off = stg_off + (uint32_t)stg_bytes, rcv_off = stg_off;
+  const uint32_t bar_off = xch_off + (uint32_t)xch_bytes;
   const size_t smem = 1024 + bar_off + (size_t)(2 * stages + 5) * 8 + 4 + 16 + 64;
   if (smem > (size_t)TC_SMEM_MAX) return cudaErrorInvalidConfiguration;
   CUtensorMap mw, mx, mo;
@@ -1466,7 +1523,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
                           : encode_2d(&mw, g.W, g.N, g.K, g.ldw, TC_BM);
   if (e == cudaSuccess)
     e = oneshot ? encode_kt(&mx, g.A, g.M, g.K, g.lda, bn, kb_per_item) : encode_2d(&mx, g.A, g.M, g.K, g.lda, bn);
-  if (e == cudaSuccess && tma_out)
+  if (e == cudaSuccess && tma_out && !dsmem)
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, box_m);
   if (e != cudaSuccess) return e;
@@ -1483,9 +1540,9 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   const dim3 grid = splits > 1 ? dim3(tiles_n, tiles_m, splits) : dim3(grid_ctas);
   const dim3 block(TC_THREADS);
   // persistent launches: one instantiation per epilogue kind; split-K
-  // launches: one for all TMA epilogues
+  // launches: one for all
   const int ek = !tma_out ? EK_GENERIC
-                 : reduce != RED_NONE ? EK_TMA_ANY
+                 : dsmem ? EK_SLICE
                  : g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32;
   const TcKernel k = tc_kernel(reduce, ek);
   if (!k) return cudaErrorInvalidConfiguration;
