@@ -396,9 +396,14 @@ __device__ __forceinline__ void store_slice(const TcParams& p, int tile_n, int m
   if (p.epi == EPI_GEGLU) {
     // rows 0..63 are gate features, 64..127 the matching up features: through
     // xch, every thread then forms 8 outputs of one token
-    for_upto<32>(cpr, [&](int i) { xch[i * STG_LD + r] = v[i] + brow; });
-    epi_bar();
 #pragma unroll
+    for (int g = 0; g < 32; g += 4) {
+      if (g >= cpr) break;
+#pragma unroll
+      for (int i = g; i < g + 4; ++i) xch[i * STG_LD + r] = v[i] + brow;
+    }
+    epi_bar();
+    #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
       const int c = (r >> 3) + 16 * h, fg = r & 7;
       if (c < lim) {
@@ -768,7 +773,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
           tmem_wait_ld();
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq) tmem_reg_fence16(raw + 16 * qq);
-          for_upto<8, 2>(2 * nq, [&](int k) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (k >= 2 * nq) break;
             const uint32_t* a = raw + 8 * k;
             const uint32_t p0 = pack_bf16x2(__uint_as_float(a[0]), __uint_as_float(a[1]));
             const uint32_t p1 = pack_bf16x2(__uint_as_float(a[2]), __uint_as_float(a[3]));
@@ -787,7 +794,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             wrap = gl >= ngs;
             gl = wrap ? gl - ngs : gl;
             dst += wrap ? 1 : 0;
-          });
+          }
         }
       } else if constexpr (RED == RED_DSMEM32) {
         // token slice q of this split's partial goes to rank q (= split q) of
@@ -809,7 +816,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq)
             if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, lacc, raw + 16 * qq);
-          for_upto<16>(4 * nq, [&](int qq) {
+#pragma unroll
+          for (int qq = 0; qq < 16; ++qq) {
+            if (qq >= 4 * nq) break;
             st_async_f4(mapa_shared(rcv0 + (uint32_t)gl * (TC_BM * 16), (uint32_t)dst),
                         make_float4(__uint_as_float(raw[4 * qq]), __uint_as_float(raw[4 * qq + 1]),
                                     __uint_as_float(raw[4 * qq + 2]), __uint_as_float(raw[4 * qq + 3])),
@@ -817,7 +826,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             const bool wrap = ++gl == ngs;   // next rank: a select, not a branch
             gl = wrap ? 0 : gl;
             dst += wrap ? 1 : 0;
-          });
+          }
         }
       } else {   // RED_L2_CLUSTER
         // this split's fp32 partial to the workspace as [col/4][row][4]: each
