@@ -278,7 +278,7 @@ ravel_status ravel_profile_step(ravel_t* r, float* buffer, const float* slot_tim
  * Enqueued on `stream`; uses the handle's split-K workspace, so it must not
  * overlap another call on the same handle.  Like ravel_roll_step it first
  * reports a device error raised by earlier work (RAVEL_EDEVICE /
- * RAVEL_ETIMEOUT) and mirrors the error word after its own launch. */
+ * RAVEL_ETIMEOUT). */
 ravel_status ravel_gemm(ravel_t* r, const void* X, int M, int K, int lda, const void* W, int N, int ldw, int epi,
                         void* out, int ldo, int out_dtype, const float* bias, void* stream);
 

@@ -44,8 +44,15 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return warp_sum(t);
 }
 
+// err: the word of an ErrorWord.  The kernel that raises an error also writes it
+// to the host's mirror, so that a call without one copies nothing back (a
+// 4-byte copy per call cost a batch-1 step 5 of 608 us, a tiny fp32 one 7 of
+// 139, and a single projection, M 800 x N 1024 x K 4096, 7 of 22).
 __device__ __forceinline__ void raise_error(int* err, int bits) {
-  if (err) atomicOr(err, bits);
+  if (!err) return;
+  atomicOr(err, bits);
+  int* mirror = ((ErrorWord*)err)->mirror;
+  if (mirror) atomicOr_system(mirror, bits);
 }
 
 // Programmatic Dependent Launch: let the next kernel in the stream start

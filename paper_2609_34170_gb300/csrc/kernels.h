@@ -16,6 +16,13 @@ enum : int {
   ERR_SHAPE = 1 << 2,        // a kernel was launched with sizes it cannot handle
 };
 
+// The device error word and where its bits are also OR-ed for the host (pinned,
+// mapped memory; null: only the word).
+struct ErrorWord {
+  int bits;
+  int* mirror;
+};
+
 // Kernel attributes (dynamic shared memory limits); called once per handle,
 // outside any stream capture.
 cudaError_t init_simt_kernels();

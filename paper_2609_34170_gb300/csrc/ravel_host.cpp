@@ -49,8 +49,7 @@ struct ravel_ctx {
   cudaGraphExec_t dn_gexec = nullptr;
   StepIO dn_io{};
   int dn_batch = -1, dn_steps = 0;
-  // asynchronously mirrored device error word
-  int* err_host = nullptr;     // pinned
+  int* err_host = nullptr;     // pinned, mapped: the error word's mirror, written by the kernel that raises
   std::string last_error;
 };
 
@@ -111,11 +110,17 @@ ravel_status ravel_create(const ravel_config* cfg, const ravel_weights* w, int d
     if (cudaEventCreateWithFlags(&r->ev_step_done, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&r->ev_ctx_ready, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithFlags(&r->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaHostAlloc((void**)&r->err_host, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cudaHostAlloc((void**)&r->err_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
       r->last_error = "event / stream / pinned allocation failed";
       s = RAVEL_ECUDA;
     } else {
       *r->err_host = 0;
+      ErrorWord w{0, nullptr};
+      if (cudaHostGetDevicePointer((void**)&w.mirror, r->err_host, 0) != cudaSuccess ||
+          cudaMemcpy(r->plan.err, &w, sizeof w, cudaMemcpyHostToDevice) != cudaSuccess) {
+        r->last_error = "error mirror set-up failed";
+        s = RAVEL_ECUDA;
+      }
     }
   }
   if (s != RAVEL_OK) {
@@ -245,8 +250,8 @@ ravel_status ravel_set_context_robots(ravel_t* r, const int* robots, int n, cons
 }
 
 static ravel_status check_device_errors(ravel_t* r) {
-  // the pinned mirror is written by an async copy after each step; reading a
-  // stale value only delays the report to a later call
+  // the mirror is written when a kernel raises an error; reading it before the
+  // write has arrived only delays the report to a later call
   const int bits = *(volatile int*)r->err_host;
   if (bits) {
     char buf[96];
@@ -321,7 +326,6 @@ static ravel_status roll_step_impl(ravel_t* r, float* buffer, const float* slot_
   }
   RV_CUDA(r, cudaGraphLaunch(r->gexec, st), "graph launch");
   RV_CUDA(r, cudaEventRecord(r->ev_step_done, st), "record step");
-  RV_CUDA(r, cudaMemcpyAsync(r->err_host, r->plan.err, sizeof(int), cudaMemcpyDeviceToHost, st), "error mirror");
   r->any_step = true;
   return RAVEL_OK;
 }
@@ -400,7 +404,6 @@ ravel_status ravel_denoise_chunk(ravel_t* r, float* chunk, int n_steps, const vo
   }
   RV_CUDA(r, cudaGraphLaunch(r->dn_gexec, st), "graph launch");
   RV_CUDA(r, cudaEventRecord(r->ev_step_done, st), "record step");
-  RV_CUDA(r, cudaMemcpyAsync(r->err_host, r->plan.err, sizeof(int), cudaMemcpyDeviceToHost, st), "error mirror");
   r->any_step = true;
   return RAVEL_OK;
 }
@@ -423,7 +426,6 @@ ravel_status ravel_gemm(ravel_t* r, const void* X, int M, int K, int lda, const 
   GemmArgs g{X, lda, W, ldw, M, N, K, (Epi)epi, out, ldo, out_dtype ? DT_BF16 : DT_F32, bias};
   cudaStream_t st = (cudaStream_t)stream;
   RV_CUDA(r, run_gemm(r->plan, g, st), "gemm");
-  RV_CUDA(r, cudaMemcpyAsync(r->err_host, r->plan.err, sizeof(int), cudaMemcpyDeviceToHost, st), "error mirror");
   return RAVEL_OK;
 }
 

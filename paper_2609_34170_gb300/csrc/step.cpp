@@ -168,7 +168,7 @@ ravel_status plan_create(StepPlan* p, const ravel_config& c, const ravel_weights
   AL(p->seeds, Bm * sizeof(uint64_t));
   AL(p->counters, Bm * sizeof(uint64_t));
   AL(p->head_cnt, Bm * sizeof(int));
-  AL(p->err, sizeof(int));
+  AL(p->err, sizeof(ErrorWord));
 #undef AL
   p->tcws.err = p->err;
   if (e == cudaSuccess) {

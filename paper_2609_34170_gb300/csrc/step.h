@@ -76,7 +76,7 @@ struct StepPlan {
   void *Ya = nullptr, *Za = nullptr, *Qa = nullptr, *KVa = nullptr, *XA = nullptr;
   uint64_t* seeds = nullptr;
   uint64_t* counters = nullptr;
-  int* err = nullptr;
+  int* err = nullptr;          // an ErrorWord; the handle sets its mirror
   std::vector<void*> allocs;
 };
 
