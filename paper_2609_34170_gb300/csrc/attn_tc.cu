@@ -903,26 +903,30 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   p.err = a.err;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
   // Query tiles of 128 rows, or of 64 where the keys are split (32: one robot's
-  // 104 CTAs, 652 us per step against 635), and the number of key splits (one
+  // 104 CTAs, 612 us per step against 601), and the number of key splits (one
   // cluster per query tile, a power of two whose head-dim slices are multiples
-  // of 4 columns): the least estimated time.  A
-  // CTA costs about 4 us, each of its chunks the tensor pipe's time for S and
-  // P V (1.2 us at head dim 256) or the softmax's 0.95; the merge moves every
-  // split's rows x hd partial between the SMs at 16 bytes per clock (the MMAs
-  // are always 128 rows); a grid that does not fit the SMs at once (36 clusters
-  // of 4, 15 of 8, 7 of 16) takes another round.  (From per-CTA stamps.  16
-  // robots, 16 slots, 2048 keys: 4 splits; 8 would run 16 clusters in two
-  // rounds, 27 us per layer against 16.)
+  // of 4 columns): the least estimated time, fitted to whole steps of 1 to 16
+  // robots with every tile height and split count.  A CTA costs about 4 us and
+  // each chunk 1.65 at head dim 256 (the tensor pipe's turns of S and P V), 0.95
+  // at 64 (the softmax); the merge moves every split's rows x hd partial
+  // between the SMs; CTAs past half the SMs delay the next kernel's; a grid that
+  // does not fit at once (36 clusters of 4, 15 of 8, 7 of 16) takes another
+  // round.  16 robots, 16 slots, 2048 keys: 4 splits of 64 rows, 964 us; of 128
+  // rows 1005, 2 splits 1061, 8 (16 clusters in two rounds) 1118.
   const int C = (a.Pmax + AT_BKV - 1) / AT_BKV + p.n_kv;
   const float hd_rel = (float)p.hdp / 256.f;
-  const float t_chunk = std::max(0.95f, 0.1f + 0.144f * (float)p.nblk + 0.52f * std::max(0.55f, hd_rel));
+  const float t_chunk = std::max(0.95f, 1.65f * hd_rel);
   float cost = 3.4e38f;
   auto consider = [&](int rows, int splits, int resident) {
     const int tq = std::max(1, rows / p.G);
     const int qt = (a.H + tq - 1) / tq, ctas = qt * a.B * a.Hkv;
-    const int rounds = (ctas + resident - 1) / resident;
+    const int rounds = (ctas + resident - 1) / resident, half = a.num_sms / 2;
     float t = (float)rounds * (4.f + t_chunk * (float)((C + splits - 1) / splits));
-    if (splits > 1) t += (float)rounds * (1.f + 2.05f * hd_rel * (float)rows / 128.f + 0.1f * (float)splits);
+    if (splits > 1) {
+      const float tile_rows = (float)((a.H + qt - 1) / qt * p.G);
+      t += (float)rounds * hd_rel * (2.4f + 1.5f * tile_rows / 128.f);
+      t += 0.6f * (float)std::max(0, ctas * splits - half) / (float)half;
+    }
     if (t < cost) {
       cost = t;
       p.q_tiles = qt;
