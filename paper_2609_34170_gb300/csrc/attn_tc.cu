@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         uint64_t ad = qd0;
         #pragma unroll 1
         for (int blk = 0; blk < p.nblk; ++blk, ad += AT_QBLK >> 4) {
-          ok = mbar_wait_warp(&k_full[sk], phk);
+          if (blk) ok = mbar_wait_warp(&k_full[sk], phk);   // (the first is known to have arrived)
           if (!ok) break;
           tc_fence_after();
           const uint64_t bd = kd0 + (uint32_t)sk * (AT_KUNIT >> 4);
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         const int groups = (keys_of(c0 + i) + 15) >> 4;
         #pragma unroll 1
         for (int h = 0; 4 * h < groups; ++h) {
-          ok = mbar_wait_warp(&v_full[sv], phv);
+          if (h) ok = mbar_wait_warp(&v_full[sv], phv);   // (as above)
           if (!ok) break;
           tc_fence_after();
           const uint64_t bd = vd0 + (uint32_t)sv * (v_bytes >> 4);
@@ -632,9 +632,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("bar.sync 5, 256;" ::: "memory");
-      if (threadIdx.x == 64 && vrows > 0) {
+      if (warp == 2 && vrows > 0) {
+        el = elect_one();
+        #pragma unroll 1
         for (int blk = 0; blk < p.nblk; ++blk)
-          tma_store_4d(&maps.o, q_s + (size_t)blk * AT_QBLK, blk * 64, g * p.G, qt * p.TQ, b);
+          tma_store_4d_el(&maps.o, q0 + (uint32_t)blk * AT_QBLK, blk * 64, g * p.G, qt * p.TQ, b, el);
         bulk_commit();
         bulk_wait_read<0>();   // read out before the shared memory goes away
       }
