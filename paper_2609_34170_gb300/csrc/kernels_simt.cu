@@ -440,18 +440,8 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
   const float* md = modulated ? a.modv + (size_t)(a.drow ? a.drow[b] : a.H + b) * a.mod_ld + a.off : nullptr;
   int buf = 0;
   for (int j = j0; j < j1; j += R, buf ^= 1) {
-    float4 xv[R][G], ts[R][G], th[R][G];
+    float4 xv[R][G], ts[R][G], th[R][G], dsc[G], dsh[G];
     float ss[R];
-    if (modulated && j == j0) {   // M_delta[b] joins the first batch's loads (one round trip)
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const int c = 4 * threadIdx.x + 1024 * g;
-        if (c < D) {
-          csc[g] = add2(csc[g], ld4(md + c));
-          csh[g] = add2(csh[g], ld4(md + D + c));
-        }
-      }
-    }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) {
       ss[rr] = 0.f;
@@ -473,11 +463,27 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
           }
         }
       }
+    }
+    // M_delta[b] after the row's own loads: its address waits for drow[b], and a
+    // warp issues in order (before them, the row waited for two round trips:
+    // 36 to 47 launches of a step, 6 us at batch 1, 17 on the wide expert)
+    const bool first = modulated && j == j0;
+    if (first) {
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int c = 4 * threadIdx.x + 1024 * g;
+        if (c < D) {
+          dsc[g] = ld4(md + c);
+          dsh[g] = ld4(md + D + c);
+        }
+      }
+    }
+#pragma unroll
+    for (int rr = 0; rr < R; ++rr)
 #pragma unroll
       for (int g = 0; g < G; ++g)
         ss[rr] += xv[rr][g].x * xv[rr][g].x + xv[rr][g].y * xv[rr][g].y + xv[rr][g].z * xv[rr][g].z +
                   xv[rr][g].w * xv[rr][g].w;
-    }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) {
 #pragma unroll
@@ -485,6 +491,14 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
       if (lane == 0) red[buf][rr][warp] = ss[rr];
     }
     __syncthreads();
+    if (first) {
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (4 * (int)threadIdx.x + 1024 * g < D) {
+          csc[g] = add2(csc[g], dsc[g]);
+          csh[g] = add2(csh[g], dsh[g]);
+        }
+    }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) {
       const int jj = j + rr;
@@ -520,7 +534,7 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
 // what bounds the norm once the rows fill the SMs.  Every load is issued
 // before the one barrier.  FOP rows go four to a block.  The arithmetic is the
 // row kernel's, operation for operation.  (64 robots x 50 slots, width 1024, 35
-// launches: step 2701 -> 2682 us; from 1216 rows on, fewer gain nothing.)
+// launches: step 2701 -> 2682 us; 1056 rows: 1288 -> 1264.)
 template <typename T, int RB, int RJ>
 __global__ void __launch_bounds__(256) ada_norm_tile_kernel(NormArgs a, int nb_b, int nb_j) {
   constexpr int R = RB * RJ;
@@ -552,17 +566,17 @@ __global__ void __launch_bounds__(256) ada_norm_tile_kernel(NormArgs a, int nb_b
   }
   if (act && on) {
 #pragma unroll
+    for (int i = 0; i < RJ; ++i) {
+      const float* mt = a.modv + (size_t)(b0 * a.t_stride + min(j0 + i, a.H - 1)) * a.mod_ld + a.off;
+      tsc[i] = ld4(mt + c);
+      tsh[i] = ld4(mt + D + c);
+    }
+#pragma unroll
     for (int i = 0; i < RB; ++i) {
       const int b = min(b0 + i, a.B - 1);
       const float* md = a.modv + (size_t)(a.drow ? a.drow[b] : a.H + b) * a.mod_ld + a.off;
       dsc[i] = ld4(md + c);
       dsh[i] = ld4(md + D + c);
-    }
-#pragma unroll
-    for (int i = 0; i < RJ; ++i) {
-      const float* mt = a.modv + (size_t)(b0 * a.t_stride + min(j0 + i, a.H - 1)) * a.mod_ld + a.off;
-      tsc[i] = ld4(mt + c);
-      tsh[i] = ld4(mt + D + c);
     }
   }
 #pragma unroll
@@ -613,8 +627,9 @@ cudaError_t launch_ada_norm_t(const NormArgs& a, cudaStream_t st) {
   // SM (one row each when the rows fit)
   const int nf = a.fop ? a.F : 0;
   const int total = a.B * (a.H + nf);
-  // modulated rows of up to 1024 features that give every SM two tiles or more
-  if (a.D <= 1024 && !a.act_gain && a.H > 0 && total >= 8 * g_norm_sms) {
+  // modulated rows of up to 1024 features, from where the row kernel's blocks no
+  // longer fit the SMs at once (five each)
+  if (a.D <= 1024 && !a.act_gain && a.H > 0 && total > 5 * g_norm_sms) {
     NormArgs b = a;
     b.F = nf;
     const int fop_blocks = (a.B * nf + 3) / 4;
