@@ -237,6 +237,13 @@ ravel_status ravel_set_relative_dims(ravel_t* r, const float* mask);
 ravel_status ravel_denoise_chunk(ravel_t* r, float* chunk, int n_steps, const void* obs_tokens, const float* delta,
                                  float* velocity, void* stream);
 
+/* Copies n (1 .. 4) device arrays, dst[i] <- src[i] (bytes[i] bytes, even; dst
+ * and src 2-byte aligned, not overlapping), in one launch on `stream`: a step's
+ * inputs into the places that its graph was captured on.  dst, src and bytes
+ * are host arrays, read before the call returns. */
+ravel_status ravel_copy_inputs(ravel_t* r, int n, void* const* dst, const void* const* src, const size_t* bytes,
+                               void* stream);
+
 /* Per-robot action counters (the index of the next appended action), host
  * uint64 [B].  get synchronises the handle's device; set is synchronous and
  * lets a rollout resume bit-exactly. */

@@ -73,6 +73,7 @@ def load(path: str | None = None):
         "ravel_denoise_chunk": (i, [vp, vp, i, vp, vp, vp, vp]),
         "ravel_roll_step_rel": (i, [vp, vp, vp, vp, vp, vp, vp, vp, vp]),
         "ravel_set_relative_dims": (i, [vp, vp]),
+        "ravel_copy_inputs": (i, [vp, i, vp, vp, vp, vp]),
         "ravel_get_state": (i, [vp, vp]),
         "ravel_set_state": (i, [vp, vp]),
         "ravel_step_kernel_count": (i, [vp]),
@@ -256,6 +257,12 @@ def ravel_gemm_noalloc_status(stream=None) -> int:
 def ravel_debug_inject(h, fault: int, count: int = 1, stream=None):
     """Fault injection of the failure-path tests (see ravel.h)."""
     _check(h, load().ravel_debug_inject(h, fault, count, _stream_ptr(stream)), "ravel_debug_inject")
+
+
+def ravel_copy_inputs(h, n: int, dst, src, nbytes, stream=None):
+    """dst[i] <- src[i] for n device arrays in one launch: ctypes arrays of
+    addresses (c_void_p) and sizes (c_size_t)."""
+    _check(h, load().ravel_copy_inputs(h, n, dst, src, nbytes, _stream_ptr(stream)), "ravel_copy_inputs")
 
 
 def ravel_get_state(h, batch: int) -> np.ndarray:

@@ -232,6 +232,15 @@ cudaError_t launch_chunk_noise(float* buffer, const uint64_t* seeds, uint64_t* c
 cudaError_t launch_reset(float* buffer, const uint64_t* seeds, uint64_t* counters, int B, int H, int A,
                          cudaStream_t st);
 
+// Up to four device arrays in one launch (bytes even, 2-byte aligned).
+struct CopyList {
+  int n;
+  void* dst[4];
+  const void* src[4];
+  size_t bytes[4];
+};
+cudaError_t launch_copy_list(const CopyList& c, cudaStream_t st);
+
 // Busy-wait on the device for `ns` nanoseconds (globaltimer), then return.
 cudaError_t launch_delay(unsigned long long ns, cudaStream_t st);
 

@@ -1371,6 +1371,26 @@ cudaError_t launch_reset(float* buffer, const uint64_t* seeds, uint64_t* counter
   return cudaGetLastError();
 }
 
+__global__ void copy_list_kernel(CopyList c) {
+  const int i = blockIdx.y;
+  const size_t bytes = c.bytes[i], t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t step = (size_t)gridDim.x * blockDim.x;
+  if ((((uintptr_t)c.dst[i] | (uintptr_t)c.src[i] | bytes) & 15) == 0) {
+    for (size_t k = t0; k < bytes / 16; k += step) ((uint4*)c.dst[i])[k] = ((const uint4*)c.src[i])[k];
+  } else {
+    for (size_t k = t0; k < bytes / 2; k += step) ((uint16_t*)c.dst[i])[k] = ((const uint16_t*)c.src[i])[k];
+  }
+}
+
+cudaError_t launch_copy_list(const CopyList& c, cudaStream_t st) {
+  size_t most = 0;
+  for (int i = 0; i < c.n; ++i) most = std::max(most, c.bytes[i]);
+  if (most == 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)std::min<size_t>((most / 16 + 255) / 256 + 1, 256);
+  copy_list_kernel<<<dim3(blocks, c.n), 256, 0, st>>>(c);
+  return cudaGetLastError();
+}
+
 __global__ void delay_kernel(unsigned long long ns) {
   unsigned long long t0, t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));

@@ -408,6 +408,23 @@ ravel_status ravel_denoise_chunk(ravel_t* r, float* chunk, int n_steps, const vo
   return RAVEL_OK;
 }
 
+ravel_status ravel_copy_inputs(ravel_t* r, int n, void* const* dst, const void* const* src, const size_t* bytes,
+                               void* stream) {
+  if (!r || n < 1 || n > 4 || !dst || !src || !bytes) return fail(r, RAVEL_EINVAL, "copy_inputs: bad argument");
+  CopyList c{};
+  c.n = n;
+  for (int i = 0; i < n; ++i) {
+    if (!dst[i] || !src[i] || ((bytes[i] | (uintptr_t)dst[i] | (uintptr_t)src[i]) & 1))
+      return fail(r, RAVEL_EINVAL, "copy_inputs: null or odd array");
+    c.dst[i] = dst[i];
+    c.src[i] = src[i];
+    c.bytes[i] = bytes[i];
+  }
+  RV_CUDA(r, cudaSetDevice(r->device), "cudaSetDevice");
+  RV_CUDA(r, launch_copy_list(c, (cudaStream_t)stream), "copy_inputs");
+  return RAVEL_OK;
+}
+
 const char* ravel_kernel_kind_name(int kind) { return kernel_kind_name(kind); }
 
 ravel_status ravel_gemm(ravel_t* r, const void* X, int M, int K, int lda, const void* W, int N, int ldw, int epi,

@@ -12,7 +12,7 @@ import pytest
 
 import synth
 from oracle import expert
-from tests._harness import TOL, Case, rel_l2
+from tests._harness import TOL, Case, gpu_session, rel_l2
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -117,3 +117,31 @@ def test_per_robot_swap_rules():
     ctx.install([2], kc, vc, 20)
     _step_and_check(case, s, ctx, "contexts assembled from two calls")
     s.close()
+
+
+# The session's step inputs: plain CUDA tensors go in one launch, everything else
+# one by one; all forms give the same step, and what cannot fill an input is
+# refused as before.
+@pytest.mark.parametrize("fop", [0, 3])
+def test_step_inputs_in_every_form(fop):
+    cfg = synth.ExpertConfig(layers=1, width=72, n_q_heads=2, n_kv_heads=1, head_dim=24, mlp_dim=64, slots=5,
+                             action_dim=3, prefix=9, fop_tokens=fop, batch=3, dtype="bf16")
+    case = Case(cfg)
+    outs = []
+    dev = lambda a, dt=torch.float32: torch.from_numpy(np.ascontiguousarray(a)).to("cuda", dt)  # noqa: E731
+    t, d, z = dev(case.t), dev(case.delta), dev(case.fop, torch.bfloat16)
+    odd = torch.zeros(t.numel() + 1, device="cuda")[1:]   # 4-byte aligned only
+    odd.copy_(t)
+    forms = [(case.t, case.fop, case.delta), (t, z, d), (odd, z, d), (t.reshape(1, -1), z.float(), d.double()),
+             (t, z.transpose(0, 1).contiguous().transpose(0, 1), d), (t, z, case.delta)]
+    for tt, zz, dd in forms:
+        s = gpu_session(case)
+        s.step(tt, zz, dd, want_velocity=True)
+        outs.append((s.released.clone(), s.velocity.clone()))
+        with pytest.raises(RuntimeError):
+            s.step(t, z, d.reshape(-1, 1))
+        with pytest.raises(RuntimeError):
+            s.step(torch.cat([t, t]), z, d)
+        s.close()
+    for r, v in outs[1:]:
+        assert torch.equal(r, outs[0][0]) and torch.equal(v, outs[0][1])
