@@ -265,8 +265,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 // lanes split K in float4 steps, so W streams once per 8 rows in 512-byte
 // requests and the rows come from L1 (the 8 warps of a block read the same
 // ones); the 16 sums then halve across the lanes.  Bound by load latency and
-// the L1: at M 10, K 1024 the tile kernel above, whose only CTAs walk K in
-// serial 32-wide steps with two barriers each, takes 75 us, this one 4.
+// the L1: at M 10, N 256, K 1024 the tile kernel above, whose only CTAs walk K in
+// serial 32-wide steps with two barriers each, takes 75 us, this one 8.  The
+// row loads of two steps go out together, and no branch on the row count stands
+// between them: with one, each load waited for the one before (14 us; a tiny
+// step 125 instead of 87).
 constexpr int RG_M = 8, RG_N = 2, RG_WARPS = 8;
 
 template <int EPI, typename TO>
@@ -281,17 +284,22 @@ __global__ void __launch_bounds__(RG_WARPS * 32) gemm_rows_kernel(const float* _
   const int mr = min(RG_M, M - m0);
   const float* w0 = W + (size_t)min(n0, N - 1) * ldw;
   const float* w1 = W + (size_t)min(n0 + 1, N - 1) * ldw;
+  const float* x[RG_M];   // rows past M repeat the last one; their sums are not stored
+#pragma unroll
+  for (int r = 0; r < RG_M; ++r) x[r] = A + (size_t)min(m0 + r, M - 1) * lda;
   pdl_wait();
   if (skip && *skip) return;
   float acc[RG_M][RG_N] = {};
+#pragma unroll 2
   for (int k = 4 * lane; k < K; k += 128) {
     const float4 wa = ld4(w0 + k), wb = ld4(w1 + k);
+    float4 xr[RG_M];
+#pragma unroll
+    for (int r = 0; r < RG_M; ++r) xr[r] = ld4(x[r] + k);
 #pragma unroll
     for (int r = 0; r < RG_M; ++r) {
-      if (r >= mr) break;
-      const float4 x = ld4(A + (size_t)(m0 + r) * lda + k);
-      acc[r][0] = fmaf(x.x, wa.x, fmaf(x.y, wa.y, fmaf(x.z, wa.z, fmaf(x.w, wa.w, acc[r][0]))));
-      acc[r][1] = fmaf(x.x, wb.x, fmaf(x.y, wb.y, fmaf(x.z, wb.z, fmaf(x.w, wb.w, acc[r][1]))));
+      acc[r][0] = fmaf(xr[r].x, wa.x, fmaf(xr[r].y, wa.y, fmaf(xr[r].z, wa.z, fmaf(xr[r].w, wa.w, acc[r][0]))));
+      acc[r][1] = fmaf(xr[r].x, wb.x, fmaf(xr[r].y, wb.y, fmaf(xr[r].z, wb.z, fmaf(xr[r].w, wb.w, acc[r][1]))));
     }
   }
   // lanes 2i and 2i + 1 end with the warp's sum i (row i / 2, column i % 2):
