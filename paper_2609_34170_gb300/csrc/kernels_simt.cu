@@ -899,15 +899,23 @@ cudaError_t launch_geglu(const float* GU, int M, int Fm, void* Hm, Dtype dt, cud
 // (b, g) pair is slot j = r / G of query head g*G + r % G.  Keys are visited
 // in chunks of KT: [0, P) the active context's prefix, [P, P+F) the FOP
 // tokens, [P+F, P+F+H) the action slots; online softmax in fp32.  Eight
-// threads copy a key's K and V row in float4 steps; rows of Q and K are padded
-// by four floats, so that the 16-byte reads of a score (8 keys per phase) fall
-// into distinct banks.  (Unpadded rows put the 16 keys of a request into one
-// bank, and an integer division found every element's row: 40 us at 40 query
-// rows, 78 keys and head dim 64, against 8 now.)
+// threads copy a key's K and V row in float4 steps, into registers while the
+// chunk before is worked on; rows of Q and K are padded by four floats, so that
+// the 16-byte reads of a score (8 keys per phase) fall into distinct banks.
+// Bound by a few blocks' shared-memory reads, hence 16-byte ones throughout: 40
+// query rows, 78 keys and head dim 64 take 6 us; with scalar reads of the
+// probabilities and V, and each chunk's loads in front of its work, 10; with
+// unpadded rows (16 keys of a request in one bank) and an integer division for
+// every element's row, 40.  NC: 32-column groups of the head dim, rounded up to
+// 2, 4 or 8.
 constexpr int ATT_QT = 16, ATT_KT = 32, ATT_THREADS = 256;
 
-template <typename T>
-__global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a) {
+__device__ __forceinline__ void fma4(float4& d, float p, float4 v) {
+  d = make_float4(fmaf(p, v.x, d.x), fmaf(p, v.y, d.y), fmaf(p, v.z, d.z), fmaf(p, v.w, d.w));
+}
+
+template <typename T, int NC>
+__global__ void __launch_bounds__(ATT_THREADS, 2) attention_simt_kernel(AttnArgs a) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ float sm[];
@@ -936,58 +944,74 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
   const int rpr = a.H + a.F;   // QKV rows per robot: H action slots, then F FOP tokens
   const float scale = rsqrtf((float)hd);
   // 16 threads per query row: its Q, its scores (keys qlane, qlane + 16), its
-  // softmax and its output columns qlane + 16 i
+  // softmax and its output columns 4 qlane + 64 i (four each)
   const int qrow = threadIdx.x >> 4, qlane = threadIdx.x & 15;
   const int r = r0 + qrow, j = r < nrows ? r / G : -1, h = g * G + r % G;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int c = 4 * qlane; c < hd; c += 64) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 v = zero;
     if (r < nrows) v = ld4(qkv + (size_t)(b * rpr + j) * a.ld_qkv + h * hd + c);
     st4(Qs + qrow * ld + c, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
   }
-  float m_run = -INFINITY, l_run = 0.f;
-  float acc[16];
+  // the K and V row of key k0 + threadIdx.x / 8: columns 4 (threadIdx.x % 8) + 32 i
+  const int kk = threadIdx.x >> 3, kc = 4 * (threadIdx.x & 7);
+  float4 kv[NC], vv[NC];
+  auto fetch = [&](int key) {
+    const T *kr = nullptr, *vr = nullptr;
+    if (key < P) {
+      kr = pk + (size_t)key * hd;
+      vr = pv + (size_t)key * hd;
+    } else if (key < nk) {   // the step's own rows: FOP tokens, then slots
+      const int row = key < P + a.F ? a.H + (key - P) : key - P - a.F;
+      kr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + kofs;
+      vr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + vofs;
+    }
 #pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+    for (int i = 0; i < NC; ++i) {
+      kv[i] = vv[i] = zero;
+      if (kr && kc + 32 * i < hd) {
+        kv[i] = ld4(kr + kc + 32 * i);
+        vv[i] = ld4(vr + kc + 32 * i);
+      }
+    }
+  };
+  float m_run = -INFINITY, l_run = 0.f;
+  float4 acc[NC / 2];
+#pragma unroll
+  for (int i = 0; i < NC / 2; ++i) acc[i] = zero;
 
+  fetch(kk);
   for (int k0 = 0; k0 < nk; k0 += ATT_KT) {
     __syncthreads();
-    {
-      const int kk = threadIdx.x >> 3, key = k0 + kk;
-      const T *kr = nullptr, *vr = nullptr;
-      if (key < P) {
-        kr = pk + (size_t)key * hd;
-        vr = pv + (size_t)key * hd;
-      } else if (key < nk) {   // the step's own rows: FOP tokens, then slots
-        const int row = key < P + a.F ? a.H + (key - P) : key - P - a.F;
-        kr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + kofs;
-        vr = qkv + (size_t)(b * rpr + row) * a.ld_qkv + vofs;
-      }
-      for (int c = 4 * (threadIdx.x & 7); c < hd; c += 32) {
-        float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
-        if (kr) {
-          kv = ld4(kr + c);
-          vv = ld4(vr + c);
-        }
-        st4(Ks + kk * ld + c, kv);
-        st4(Vs + kk * hd + c, vv);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      if (kc + 32 * i < hd) {
+        st4(Ks + kk * ld + kc + 32 * i, kv[i]);
+        st4(Vs + kk * hd + kc + 32 * i, vv[i]);
       }
     }
     __syncthreads();
+    fetch(k0 + ATT_KT + kk);
+    float4 d[2] = {zero, zero};
+#pragma unroll 4
+    for (int c = 0; c < hd; c += 4) {
+      const float4 q = ld4(Qs + qrow * ld + c);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const float4 k = ld4(Ks + (qlane + 16 * t) * ld + c);
+        d[t].x = fmaf(q.x, k.x, d[t].x);
+        d[t].y = fmaf(q.y, k.y, d[t].y);
+        d[t].z = fmaf(q.z, k.z, d[t].z);
+        d[t].w = fmaf(q.w, k.w, d[t].w);
+      }
+    }
     float s[2];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-      const int kk = qlane + 16 * t, key = k0 + kk;
-      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int c = 0; c < hd; c += 4) {
-        const float4 q = ld4(Qs + qrow * ld + c), k = ld4(Ks + kk * ld + c);
-        d.x = fmaf(q.x, k.x, d.x);
-        d.y = fmaf(q.y, k.y, d.y);
-        d.z = fmaf(q.z, k.z, d.z);
-        d.w = fmaf(q.w, k.w, d.w);
-      }
+      const int key = k0 + qlane + 16 * t;
       bool vis = key < nk;
       if (a.mask_mode == 1 && key >= P + a.F && key < nk) vis = vis && (key - P - a.F == j);
-      s[t] = vis ? (d.x + d.y) + (d.z + d.w) : -INFINITY;
+      s[t] = vis ? (d[t].x + d[t].y) + (d[t].z + d[t].w) : -INFINITY;
     }
     float cmax = fmaxf(s[0], s[1]);
 #pragma unroll
@@ -1007,16 +1031,20 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
     m_run = m_new;
     __syncwarp();   // a row's 16 threads are half a warp
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int c = qlane + 16 * i;
+    for (int i = 0; i < NC / 2; ++i) {
+      const int c = 4 * qlane + 64 * i;
       if (c < hd) {
-        float v0 = acc[i] * corr, v1 = 0.f;
-#pragma unroll 8
-        for (int kk = 0; kk < ATT_KT; kk += 2) {
-          v0 = fmaf(Ss[qrow * ATT_KT + kk], Vs[kk * hd + c], v0);
-          v1 = fmaf(Ss[qrow * ATT_KT + kk + 1], Vs[(kk + 1) * hd + c], v1);
+        float4 v0 = make_float4(acc[i].x * corr, acc[i].y * corr, acc[i].z * corr, acc[i].w * corr), v1 = zero;
+#pragma unroll(NC <= 4 ? 8 : 2)
+        for (int q = 0; q < ATT_KT; q += 4) {
+          const float4 p = ld4(Ss + qrow * ATT_KT + q);
+          const float* vs = Vs + q * hd + c;
+          fma4(v0, p.x, ld4(vs));
+          fma4(v1, p.y, ld4(vs + hd));
+          fma4(v0, p.z, ld4(vs + 2 * hd));
+          fma4(v1, p.w, ld4(vs + 3 * hd));
         }
-        acc[i] = v0 + v1;
+        acc[i] = make_float4(v0.x + v1.x, v0.y + v1.y, v0.z + v1.z, v0.w + v1.w);
       }
     }
   }
@@ -1024,9 +1052,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attention_simt_kernel(AttnArgs a)
     T* o = (T*)a.out + (size_t)(b * a.H + j) * a.ld_out + h * hd;
     const float inv = 1.f / l_run;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int c = qlane + 16 * i;
-      if (c < hd) o[c] = from_f32<T>(acc[i] * inv);
+    for (int i = 0; i < NC / 2; ++i) {
+      const int c = 4 * qlane + 64 * i;
+      if (c < hd) st4(o + c, make_float4(acc[i].x * inv, acc[i].y * inv, acc[i].z * inv, acc[i].w * inv));
     }
   }
 }
@@ -1039,9 +1067,13 @@ cudaError_t launch_attention_simt(const AttnArgs& a, Dtype dt, cudaStream_t st) 
   if (a.hd > 256 || a.hd % 8) return cudaErrorInvalidValue;
   const int G = a.Hq / a.Hkv;
   dim3 grid(a.B * a.Hkv, (a.H * G + ATT_QT - 1) / ATT_QT);
-  if (dt == DT_BF16)
-    return launch_kernel(attention_simt_kernel<bf16>, grid, dim3(ATT_THREADS), att_smem(a.hd), st, 1, a);
-  return launch_kernel(attention_simt_kernel<float>, grid, dim3(ATT_THREADS), att_smem(a.hd), st, 1, a);
+  const size_t smem = att_smem(a.hd);
+  const bool bf = dt == DT_BF16;
+  if (a.hd <= 64)
+    return launch_kernel(bf ? attention_simt_kernel<bf16, 2> : attention_simt_kernel<float, 2>, grid, dim3(ATT_THREADS), smem, st, 1, a);
+  if (a.hd <= 128)
+    return launch_kernel(bf ? attention_simt_kernel<bf16, 4> : attention_simt_kernel<float, 4>, grid, dim3(ATT_THREADS), smem, st, 1, a);
+  return launch_kernel(bf ? attention_simt_kernel<bf16, 8> : attention_simt_kernel<float, 8>, grid, dim3(ATT_THREADS), smem, st, 1, a);
 }
 
 // ============================================================================ FOP adapter cross-attention
@@ -1361,9 +1393,9 @@ cudaError_t launch_chunk_noise(float* buffer, const uint64_t* seeds, uint64_t* c
 
 cudaError_t init_simt_kernels() {
   const int att = (int)att_smem(256);
-  cudaError_t e = cudaFuncSetAttribute(attention_simt_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);
+  cudaError_t e = cudaFuncSetAttribute(attention_simt_kernel<bf16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(attention_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);
+    e = cudaFuncSetAttribute(attention_simt_kernel<float, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, att);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * (int)sizeof(float));
   const int xa = (int)xattn_smem(64, 256);

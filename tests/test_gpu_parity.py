@@ -179,3 +179,17 @@ def test_attention_chunk_edges(prefix, capacity, batch, slots, fop):
     s = gpu_session(case)
     check_step(case, s, robots=sorted({0, batch // 2, batch - 1}), label=f"prefix {prefix}")
     s.close()
+
+
+# The fp32 attention: head dims at the edges of its column groups (8 columns, a
+# whole and a part group of 64, 128 and 256), keys that fill a chunk of 32, end
+# one past it and span several.
+@pytest.mark.parametrize("hd", [8, 64, 72, 128, 136, 256])
+@pytest.mark.parametrize("prefix,slots,fop", [(24, 5, 3), (25, 5, 3), (70, 17, 0)])
+@pytest.mark.parametrize("mask", ["full", "slot_isolated"])
+def test_fp32_attention_edges(hd, prefix, slots, fop, mask):
+    cfg = synth.ExpertConfig(layers=1, width=64, n_q_heads=6, n_kv_heads=2, head_dim=hd, mlp_dim=64, slots=slots,
+                             action_dim=3, prefix=prefix, fop_tokens=fop, batch=2, dtype="fp32")
+    s = gpu_session(Case(cfg), mask_mode=int(mask != "full"))
+    check_step(Case(cfg), s, mask=mask, label=f"head dim {hd}")
+    s.close()
