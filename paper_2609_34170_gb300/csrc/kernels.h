@@ -96,7 +96,9 @@ struct GemmArgs {
   // the step's projections take; 0 keeps them in fp32
   int xbf16 = 0;
 };
+// EPI_GEGLU: fp32 with a float output where the row kernel takes it (few rows)
 cudaError_t launch_gemm_simt(const GemmArgs& g, Dtype dt, cudaStream_t st);
+bool rows_gemm_supported(const GemmArgs& g);
 
 // tcgen05 / TMEM / TMA path (bf16 operands only).  EPI_GEGLU: W rows come in
 // 128-row blocks of 64 gate rows then the 64 matching up rows; out is bf16

@@ -269,7 +269,9 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 // serial 32-wide steps with two barriers each, takes 75 us, this one 8.  The
 // row loads of two steps go out together, and no branch on the row count stands
 // between them: with one, each load waited for the one before (14 us; a tiny
-// step 125 instead of 87).
+// step 125 instead of 87).  EPI_GEGLU: a warp's two columns are a feature's gate and
+// up, W rows in groups of 64 gates and their 64 ups (the separate launch and its
+// fp32 round trip took a two-layer tiny step 4 of 69 us).
 constexpr int RG_M = 8, RG_N = 2, RG_WARPS = 8;
 
 template <int EPI, typename TO, int KS>
@@ -282,8 +284,11 @@ __global__ void __launch_bounds__(RG_WARPS * 32) gemm_rows_kernel(const float* _
   const int warp = (threadIdx.x >> 5) / KS, part = (threadIdx.x >> 5) % KS, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * RG_M, n0 = (blockIdx.x * (RG_WARPS / KS) + warp) * RG_N;
   const int mr = min(RG_M, M - m0);
-  const float* w0 = W + (size_t)min(n0, N - 1) * ldw;
-  const float* w1 = W + (size_t)min(n0 + 1, N - 1) * ldw;
+  // GeGLU: a gate row and its up row, 64 below it (N = 2 mlp, n0 / 2 the feature)
+  const int f = min(n0, N - 1) / 2;
+  const int nw = EPI == EPI_GEGLU ? f / 64 * 128 + f % 64 : min(n0, N - 1);
+  const float* w0 = W + (size_t)nw * ldw;
+  const float* w1 = W + (size_t)(EPI == EPI_GEGLU ? nw + 64 : min(n0 + 1, N - 1)) * ldw;
   const float* x[RG_M];   // rows past M repeat the last one; their sums are not stored
 #pragma unroll
   for (int r = 0; r < RG_M; ++r) x[r] = A + (size_t)min(m0 + r, M - 1) * lda;
@@ -326,6 +331,12 @@ __global__ void __launch_bounds__(RG_WARPS * 32) gemm_rows_kernel(const float* _
 #pragma unroll
     for (int i = 1; i < KS; ++i) t += sums[warp][i][lane];
   }
+  if (EPI == EPI_GEGLU) {
+    const float up = __shfl_xor_sync(0xffffffffu, t, 2);
+    if ((lane & 3) == 0 && (lane >> 2) < mr && n0 < N)
+      out[(size_t)(m0 + (lane >> 2)) * ldo + n0 / 2] = from_f32<TO>(gelu_tanh_f(t) * up);
+    return;
+  }
   const int m = m0 + (lane >> 2), n = n0 + ((lane >> 1) & 1);
   if ((lane & 1) || (lane >> 2) >= mr || n >= N) return;
   t += bias ? bias[n] : 0.f;
@@ -343,7 +354,7 @@ constexpr int RG_KS = 4, RG_SPLIT_COLS = 1024;
 
 // The row kernel re-reads W for every 8 rows (from L2): up to 256 rows, where
 // the tile kernel would leave SMs idle.
-static bool rows_gemm_supported(const GemmArgs& g) {
+bool rows_gemm_supported(const GemmArgs& g) {
   return g.M <= 256 && g.K % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
          (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
 }
@@ -360,6 +371,7 @@ static cudaError_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st) {
 
 static cudaError_t gemm_rows_dispatch(const GemmArgs& g, cudaStream_t st) {
   if (g.epi == EPI_ADD_F32) return launch_gemm_rows<EPI_ADD_F32, float>(g, st);
+  if (g.epi == EPI_GEGLU) return launch_gemm_rows<EPI_GEGLU, float>(g, st);
   if (g.out_dt == DT_BF16)
     return g.epi == EPI_STORE_SILU ? launch_gemm_rows<EPI_STORE_SILU, bf16>(g, st) : launch_gemm_rows<EPI_STORE, bf16>(g, st);
   return g.epi == EPI_STORE_SILU ? launch_gemm_rows<EPI_STORE_SILU, float>(g, st) : launch_gemm_rows<EPI_STORE, float>(g, st);

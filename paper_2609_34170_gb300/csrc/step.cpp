@@ -412,6 +412,8 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     gu.xbf16 = 1;
     if (p.use_tc && tc_gemm_supported(gu)) {
       RUN(KK_GEMM_GATE_UP, launch_gemm_tc(gu, p.tcws, p.num_sms, st));   // GeGLU fused in the epilogue
+    } else if (dt == DT_F32 && rows_gemm_supported(gu)) {
+      RUN(KK_GEMM_GATE_UP, launch_gemm_simt(gu, dt, st));   // likewise (few rows)
     } else {
       RUN(KK_GEMM_GATE_UP, gemm(p.Y, D, wgu, BH, 2 * Fm, D, EPI_STORE, p.GU, 2 * Fm, DT_F32, nullptr));
       RUN(KK_GEGLU, launch_geglu(p.GU, BH, Fm, p.Hm, dt, st));

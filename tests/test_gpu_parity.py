@@ -193,3 +193,16 @@ def test_fp32_attention_edges(hd, prefix, slots, fop, mask):
     s = gpu_session(Case(cfg), mask_mode=int(mask != "full"))
     check_step(Case(cfg), s, mask=mask, label=f"head dim {hd}")
     s.close()
+
+
+# fp32 GeGLU in the row kernel: part and whole row chunks, the last row count it
+# takes and the first that goes through the separate launch, one and several
+# gate/up groups, widths on either side of the split of K.
+@pytest.mark.parametrize("batch,slots", [(1, 2), (3, 3), (8, 32), (1, 257)])
+@pytest.mark.parametrize("width,mlp", [(64, 64), (512, 192), (520, 1024)])
+def test_fp32_geglu_rows(batch, slots, width, mlp):
+    cfg = synth.ExpertConfig(layers=2, width=width, n_q_heads=2, n_kv_heads=1, head_dim=16, mlp_dim=mlp, slots=slots,
+                             action_dim=3, prefix=9, fop_tokens=2, batch=batch, dtype="fp32")
+    s = gpu_session(Case(cfg))
+    check_step(Case(cfg), s, robots=sorted({0, batch - 1}), label=f"rows {batch * slots}")
+    s.close()
