@@ -214,9 +214,8 @@ struct HeadArgs {
   const float* x; int D;                       // residual stream [B*H][D]
   const float* modv; int mod_ld; const float* mod_b; int off; const int* drow;   // as NormArgs
   const void* w; const float* b;               // W_out [A][D] bf16, b_out [A]
-  float* v;                                    // [B*H][A] velocity (= a.vel)
+  float* v;                                    // [B*H][A] scratch: the slots' new values (a.vel is not read)
   int* cnt;                                    // [B] zero-initialised counters
-  int rows_per_cta;
   int t_stride = 0;                            // as NormArgs
 };
 cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, cudaStream_t st);

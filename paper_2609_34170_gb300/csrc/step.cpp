@@ -429,7 +429,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     TailArgs ta{io.buffer, p.V, io.slot_times, io.released, io.velocity, p.seeds, p.counters, B, H, A, io.state,
                 p.rel_mask};
     ta.t_stride = t_stride;
-    HeadArgs hd{p.x, D, p.modv, p.mod_dim, p.mod_b, 4 * L * D, p.cond_drow, p.out_w, p.out_b, p.V, p.head_cnt, 1};
+    HeadArgs hd{p.x, D, p.modv, p.mod_dim, p.mod_b, 4 * L * D, p.cond_drow, p.out_w, p.out_b, p.V, p.head_cnt};
     hd.t_stride = t_stride;
     RUN(KK_HEAD_TAIL, launch_head_tail(hd, ta, st));
     if (n_kernels) *n_kernels = nk;

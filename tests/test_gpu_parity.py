@@ -206,3 +206,17 @@ def test_fp32_geglu_rows(batch, slots, width, mlp):
     s = gpu_session(Case(cfg))
     check_step(Case(cfg), s, robots=sorted({0, batch - 1}), label=f"rows {batch * slots}")
     s.close()
+
+
+# The fused head and tail: action widths at the edges of a noise group and of its
+# 32 outputs, one and several passes over the row, few slots and the most rows.
+@pytest.mark.parametrize("batch,slots", [(1, 2), (5, 9), (1, 152)])
+@pytest.mark.parametrize("width,actions", [(64, 1), (1024, 20), (1032, 32), (2056, 5)])
+def test_head_tail_edges(batch, slots, width, actions):
+    cfg = synth.ExpertConfig(layers=1, width=width, n_q_heads=2, n_kv_heads=1, head_dim=64, mlp_dim=64, slots=slots,
+                             action_dim=actions, prefix=9, fop_tokens=2, batch=batch, dtype="bf16")
+    case = Case(cfg)
+    s = gpu_session(case)
+    for _ in range(2):   # (the second step starts from the first one's buffer and counters)
+        check_step(case, s, label=f"{batch * slots} rows")
+    s.close()
