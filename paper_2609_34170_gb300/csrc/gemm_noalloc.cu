@@ -18,7 +18,7 @@
 // theirs through the shared memory of their cluster, and the call is the GEMM
 // launch alone (M 51, N 3000, K 1024 with SiLU: the earlier reduction through
 // this array, with counters cleared by a memset before each launch, took 30.7
-// us per call, 15.0 of them on the GPU; now 14.2 and 5.5).  The error word is
+// us per call, 15.0 of them on the GPU; now 11.5 to 12.4 and 5.5).  The error word is
 // sticky: a bounded wait that runs out inside a GEMM sets it, and it stays set
 // until ravel_gemm_noalloc_status reads it.
 #include <cuda_runtime.h>

@@ -10,7 +10,8 @@
 // large-batch case (many 128 x 256 tiles).
 //
 // Warp roles (192 threads): warp 0 = TMA producer, warp 1 = TMEM allocator +
-// single-thread MMA issuer, warps 2..5 = epilogue (warp w reads TMEM lanes
+// MMA issuer (both stay converged: every lane waits, the elected one's
+// instruction is predicated), warps 2..5 = epilogue (warp w reads TMEM lanes
 // 32*(w%4)..+31).  Operand tiles are 64 K-elements wide (one 128-byte
 // swizzle row) in an S-stage shared-memory ring guarded by mbarriers.  Every
 // wait is bounded: on timeout the kernel raises ERR_TIMEOUT in the device
@@ -25,8 +26,8 @@
 //    form a thread-block cluster and rank q sums a token slice over the splits
 //    in order (deterministic) and applies the epilogue.  The partials travel
 //    by st.async straight into rank q's shared memory, completing on an
-//    mbarrier there (slices of up to 32 tokens), else through L2 and the
-//    cluster barrier.
+//    mbarrier there, or, where the output is not 16-byte aligned, through L2
+//    and the cluster barrier.
 // Epilogue: a chunk of tokens is written into a shared-memory box in the
 // output layout and leaves through one TMA store (or a TMA reduce-add for the
 // residual-stream epilogue), double-buffered so that the epilogue threads

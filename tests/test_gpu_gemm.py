@@ -1,8 +1,8 @@
 """The projection GEMM building block (tcgen05 / TMEM / TMA for bf16, SIMT
 for fp32) against numpy fp64 matmul of the same bf16 operands, through the C
 ABI (ravel_gemm).  Shapes cover single and multiple tiles, ragged token /
-feature / K tails, split-K (partials exchanged through shared memory for token
-slices of 4..32, through L2 for wider ones), persistent launches on one SM
+feature / K tails, split-K (partials exchanged through shared memory, or
+through L2 for unaligned outputs), persistent launches on one SM
 or on SM pairs (one 256-row MMA per K step across two CTAs) and every
 epilogue."""
 import numpy as np
