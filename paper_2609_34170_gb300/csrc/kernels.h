@@ -61,13 +61,12 @@ struct CondArgs {
   float* modv; int mod_ld;
   int enabled;                  // 0: always compute, drow = H + b
 };
-cudaError_t launch_cond_check(const CondArgs& a, cudaStream_t st);
 cudaError_t launch_cond_commit(const CondArgs& a, cudaStream_t st);
-// E[r][:] = sinusoidal(x_r) for r < H (x = slot_times[r]) and H <= r < H+B
-// (x = delta[r-H]); periods geometric from 4e-3 to 4; fp64 angles reduced mod 2 pi.
-// omega: device fp64 [D/2] angular frequencies 2 pi / p_i.
-cudaError_t launch_embed(const float* slot_times, int H, const float* delta, int B, int D, const double* omega,
-                         void* E, Dtype dt, cudaStream_t st, const int* skip = nullptr);
+// cond_check, and in the same launch E[r][:] = sinusoidal(x_r) for r < H (x =
+// slot_times[r]) and H <= r < H+B (x = delta[r-H]); periods geometric from 4e-3
+// to 4 (fp64 angles reduced mod 2 pi).  omega: device fp64 [D/2] angular
+// frequencies 2 pi / p_i.
+cudaError_t launch_cond_embed(const CondArgs& a, int D, const double* omega, void* E, Dtype dt, cudaStream_t st);
 
 // ---- generic projection GEMM: out[m][n] = sum_k A[m][k] W[n][k] (W K-major) ----
 enum Epi { EPI_STORE = 0, EPI_STORE_SILU = 1, EPI_ADD_F32 = 2, EPI_GEGLU = 3 };

@@ -58,60 +58,30 @@ cudaError_t launch_convert(const float* src, size_t n, void* dst, Dtype dt, cuda
   return cudaGetLastError();
 }
 
-// ============================================================================ embedding
+// ============================================================================ conditioning: cache check, embedding
 
-// Sinusoidal embedding of a scalar (flow time or context offset): component
-// i < D/2 is sin(x w_i), i >= D/2 is cos(x w_{i-D/2}), w_i = 2 pi / p_i with
-// periods p_i geometric from 4e-3 to 4 (w_i precomputed in fp64).  x w
-// reaches ~1.6e3 rad, where a float32 product would already be off by ~1e-4:
-// the angle is formed and reduced modulo 2 pi in fp64, then sin / cos of the
-// reduced angle (|a| <= pi) in fp32.
-template <typename T>
-__global__ void embed_kernel(const float* __restrict__ slot_times, int H, const float* __restrict__ delta, int D,
-                             const double* __restrict__ omega, T* __restrict__ E, const int* __restrict__ skip) {
-  pdl_trigger();
-  pdl_wait();
-  if (skip && *skip) return;
-  const int r = blockIdx.y;
-  const double x = (r < H) ? (double)slot_times[r] : (double)delta[r - H];
-  const int half = D / 2;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= half) return;
-  const double ang = x * omega[i];
-  const double red = ang - 6.283185307179586 * rint(ang * 0.15915494309189535);
-  float s, c;
-  sincosf((float)red, &s, &c);
-  E[(size_t)r * D + i] = from_f32<T>(s);
-  E[(size_t)r * D + half + i] = from_f32<T>(c);
-}
-
-cudaError_t launch_embed(const float* slot_times, int H, const float* delta, int B, int D, const double* omega,
-                         void* E, Dtype dt, cudaStream_t st, const int* skip) {
-  dim3 grid((D / 2 + 127) / 128, H + B);
-  if (dt == DT_BF16)
-    return launch_kernel(embed_kernel<bf16>, grid, dim3(128), 0, st, 1, slot_times, H, delta, D, omega, (bf16*)E,
-                         skip);
-  return launch_kernel(embed_kernel<float>, grid, dim3(128), 0, st, 1, slot_times, H, delta, D, omega, (float*)E,
-                       skip);
-}
-
-// ============================================================================ conditioning cache
-
-// One block: which rows of this step's conditioning are cached already (see
-// CondCache).  The slot times hit when every one equals the cached key; a
-// robot's offset hits when its value is one of the cached offsets.  Misses
-// get a cache slot (a slot already referenced in this step is never taken;
-// with no slot left the robot keeps this step's fresh row), and their keys
-// are written now: the rows themselves arrive through cond_commit before
-// any reader of this step, and a later step reads them only after that.
-__global__ void cond_check_kernel(CondArgs a) {
-  __shared__ int s_tmiss;
+// Which rows of this step's conditioning are cached already (see CondCache).
+// The slot times hit when every one equals the cached key; a robot's offset
+// hits when its value is one of the cached offsets.  Misses get a cache slot (a
+// slot already referenced in this step is never taken; with no slot left the
+// robot keeps this step's fresh row), and their keys are written now: the rows
+// themselves arrive through cond_commit before any reader of this step, and a
+// later step reads them only after that.  One block; bound by load latency, so
+// every key is read once, in parallel, and the loop over the robots runs only
+// where one misses (that loop and one key after the other took 64 robots 3 us
+// more, hit or miss).
+__device__ void cond_check(const CondArgs& a) {
+  __shared__ int s_tmiss, s_bmiss, s_used[kCondCache];
+  __shared__ float s_key[kCondCache];
   __shared__ unsigned s_ref;   // cache slots referenced by this step
-  pdl_trigger();
-  pdl_wait();
   CondCache* cc = a.cc;
+  if (threadIdx.x < kCondCache) {
+    s_used[threadIdx.x] = cc->used[threadIdx.x];
+    s_key[threadIdx.x] = cc->delta[threadIdx.x];
+  }
   if (threadIdx.x == 0) {
     s_tmiss = a.enabled ? !cc->t_valid : 1;
+    s_bmiss = 0;
     s_ref = 0u;
   }
   __syncthreads();
@@ -119,54 +89,52 @@ __global__ void cond_check_kernel(CondArgs a) {
     if (a.slot_times[j] != a.t_key[j]) s_tmiss = 1;   // benign race: every writer stores 1
   // offsets: look up in parallel; -1 = miss
   for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
-    int row = -1;
+    int row = a.enabled ? -1 : a.H + b;
     if (a.enabled) {
       const float d = a.delta[b];
       for (int c = 0; c < kCondCache; ++c)
-        if (cc->used[c] && cc->delta[c] == d) {
+        if (s_used[c] && s_key[c] == d) {
           row = a.H + a.Bmax + c;
           atomicOr(&s_ref, 1u << c);
           break;
         }
+      if (row < 0) s_bmiss = 1;
     }
     a.drow[b] = row;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int any_miss = s_tmiss, nc = 0;
+    int nc = 0;
     unsigned ref = s_ref;
-    for (int b = 0; b < a.B; ++b) {
+    for (int b = 0; s_bmiss && b < a.B; ++b) {
       if (a.drow[b] >= 0) continue;
-      any_miss = 1;
       const float d = a.delta[b];
       int row = a.H + b;   // this step's fresh row unless a cache slot is found
-      if (a.enabled) {
-        int c = -1;
-        for (int k = 0; k < kCondCache; ++k)   // assigned to an earlier robot of this step?
-          if ((ref >> k & 1u) && cc->used[k] && cc->delta[k] == d) c = k;
-        if (c < 0) {
-          for (int k = 0; k < kCondCache && c < 0; ++k) {
-            const int v = (cc->next + k) % kCondCache;
-            if (!(ref >> v & 1u)) c = v;
-          }
-          if (c >= 0) {
-            cc->next = (c + 1) % kCondCache;
-            cc->delta[c] = d;
-            cc->used[c] = 1;
-            a.commit[2 * nc] = a.H + b;
-            a.commit[2 * nc + 1] = a.H + a.Bmax + c;
-            ++nc;
-          }
+      int c = -1;
+      for (int k = 0; k < kCondCache; ++k)   // assigned to an earlier robot of this step?
+        if ((ref >> k & 1u) && cc->used[k] && cc->delta[k] == d) c = k;
+      if (c < 0) {
+        for (int k = 0; k < kCondCache && c < 0; ++k) {
+          const int v = (cc->next + k) % kCondCache;
+          if (!(ref >> v & 1u)) c = v;
         }
         if (c >= 0) {
-          ref |= 1u << c;
-          row = a.H + a.Bmax + c;
+          cc->next = (c + 1) % kCondCache;
+          cc->delta[c] = d;
+          cc->used[c] = 1;
+          a.commit[2 * nc] = a.H + b;
+          a.commit[2 * nc + 1] = a.H + a.Bmax + c;
+          ++nc;
         }
+      }
+      if (c >= 0) {
+        ref |= 1u << c;
+        row = a.H + a.Bmax + c;
       }
       a.drow[b] = row;
     }
     cc->n_commit = nc;
-    cc->skip = any_miss ? 0 : 1;
+    cc->skip = s_tmiss || s_bmiss ? 0 : 1;
     if (a.enabled) cc->t_valid = 1;
   }
   // the slot times become the key (a miss recomputes rows [0, H) this step)
@@ -174,8 +142,40 @@ __global__ void cond_check_kernel(CondArgs a) {
     for (int j = threadIdx.x; j < a.H; j += blockDim.x) a.t_key[j] = a.slot_times[j];
 }
 
-cudaError_t launch_cond_check(const CondArgs& a, cudaStream_t st) {
-  return launch_kernel(cond_check_kernel, dim3(1), dim3(256), 0, st, 1, a);
+// Sinusoidal embedding of a scalar (flow time or context offset): component
+// i < D/2 is sin(x w_i), i >= D/2 is cos(x w_{i-D/2}), w_i = 2 pi / p_i with
+// periods p_i geometric from 4e-3 to 4 (w_i precomputed in fp64).  x w
+// reaches ~1.6e3 rad, where a float32 product would already be off by ~1e-4:
+// the angle is formed and reduced modulo 2 pi in fp64, then sin / cos of the
+// reduced angle (|a| <= pi) in fp32.  The first block checks the cache; the
+// others, a row each, don't wait for its answer: a launch of its own behind the
+// check cost more than rows that nobody reads (3 of a batch-1 step's 582 us).
+template <typename T>
+__global__ void __launch_bounds__(256) cond_embed_kernel(CondArgs a, int D, const double* __restrict__ omega,
+                                                         T* __restrict__ E) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0) {
+    cond_check(a);
+    return;
+  }
+  const int r = blockIdx.x - 1, half = D / 2;
+  const double x = r < a.H ? (double)a.slot_times[r] : (double)a.delta[r - a.H];
+  for (int i = threadIdx.x; i < half; i += blockDim.x) {
+    const double ang = x * omega[i];
+    const double red = ang - 6.283185307179586 * rint(ang * 0.15915494309189535);
+    float s, c;
+    sincosf((float)red, &s, &c);
+    E[(size_t)r * D + i] = from_f32<T>(s);
+    E[(size_t)r * D + half + i] = from_f32<T>(c);
+  }
+}
+
+cudaError_t launch_cond_embed(const CondArgs& a, int D, const double* omega, void* E, Dtype dt, cudaStream_t st) {
+  const dim3 grid(1 + a.H + a.B);
+  if (dt == DT_BF16)
+    return launch_kernel(cond_embed_kernel<bf16>, grid, dim3(256), 0, st, 1, a, D, omega, (bf16*)E);
+  return launch_kernel(cond_embed_kernel<float>, grid, dim3(256), 0, st, 1, a, D, omega, (float*)E);
 }
 
 // Copies the rows that cond_check listed (this step's fresh offset rows) into

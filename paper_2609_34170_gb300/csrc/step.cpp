@@ -331,9 +331,8 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
               p.modv, p.mod_dim, (p.cond_cache && !c.per_robot_times) ? 1 : 0};
   const int* skip = &p.cond->skip;
   pdl_enabled() = false;
-  RUN(KK_COND_CACHE, launch_cond_check(ca, st));
+  RUN(KK_EMBED, launch_cond_embed(ca, D, p.omega, p.E, dt, st));
   pdl_enabled() = p.use_pdl && !trace;
-  RUN(KK_EMBED, launch_embed(io.slot_times, Ht, io.delta, B, D, p.omega, p.E, dt, st, skip));
   RUN(KK_GEMM_COND, gemm(p.E, D, p.t_w1, Ht, D, D, EPI_STORE_SILU, p.H1, D, dt, p.t_b1, skip));
   RUN(KK_GEMM_COND, gemm(rowp(p.E, Ht, D), D, p.d_w1, B, D, D, EPI_STORE_SILU, (void*)rowp(p.H1, Ht, D), D, dt, p.d_b1,
                          skip));
