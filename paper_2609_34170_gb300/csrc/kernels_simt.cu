@@ -701,12 +701,16 @@ cudaError_t launch_ada_norm(const NormArgs& a, Dtype dt, cudaStream_t st) {
 
 // ============================================================================ in-proj
 
+// The in-projection reads what the step starts from (buffer, slot times, state,
+// weights) and x's last readers were the step before, while the launches in
+// front of it, back to the step's first one, which waits for all earlier work,
+// are the conditioning: it runs beside them, and waits for them only where it
+// needs the modulation (or at its end, for the kernels that follow).
 __global__ void in_proj_kernel(const float* __restrict__ buf, int A, int D, const float* __restrict__ in_w,
                                const float* __restrict__ in_b, float* __restrict__ x, const float* __restrict__ state,
                                const float* __restrict__ rel_mask, const float* __restrict__ slot_times, int H,
                                int t_stride) {
   pdl_trigger();
-  pdl_wait();
   extern __shared__ float arow[];   // the action row of this slot
   const int r = blockIdx.y;
   for (int i = threadIdx.x; i < A; i += blockDim.x) {
@@ -720,10 +724,12 @@ __global__ void in_proj_kernel(const float* __restrict__ buf, int A, int D, cons
   }
   __syncthreads();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= D) return;
-  float acc = in_b[c];
-  for (int i = 0; i < A; ++i) acc = fmaf(arow[i], in_w[(size_t)i * D + c], acc);
-  x[(size_t)r * D + c] = acc;
+  if (c < D) {
+    float acc = in_b[c];
+    for (int i = 0; i < A; ++i) acc = fmaf(arow[i], in_w[(size_t)i * D + c], acc);
+    x[(size_t)r * D + c] = acc;
+  }
+  pdl_wait();   // (the kernels after this one wait for it alone)
 }
 
 cudaError_t launch_in_proj(const float* buf, int BH, int A, int D, const float* in_w, const float* in_b, float* x,
@@ -741,7 +747,9 @@ cudaError_t launch_in_proj(const float* buf, int BH, int A, int D, const float* 
 // 16-byte load per thread that serves R slots, eight of them in flight: one
 // slot per block and a load per feature re-read the 128 KB of W_in for every
 // slot (64 robots x 50 slots: step 2682 -> 2662 us) and waited for 32 loads in
-// turn (4 robots: 900 -> 891 us).
+// turn (4 robots: 900 -> 891 us).  All but the modulation runs before the wait
+// (see above; where the modulation GEMM runs in front of it: four robots on
+// schedules of their own 999 -> 992 us, ten denoising passes 6068 -> 6029).
 template <typename T, int R, int G>
 __global__ void __launch_bounds__(256) in_proj_norm_kernel(const float* __restrict__ buf, int A, int D,
                                                            const float* __restrict__ in_w,
@@ -752,7 +760,6 @@ __global__ void __launch_bounds__(256) in_proj_norm_kernel(const float* __restri
   extern __shared__ float arow[];   // [R][A] the action rows of these slots
   __shared__ float red[R][8];
   pdl_trigger();
-  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool act = (int)blockIdx.x < rn.B * nj;
   const int b = act ? blockIdx.x / nj : 0, j0 = act ? (blockIdx.x % nj) * R : 0;
@@ -812,6 +819,7 @@ __global__ void __launch_bounds__(256) in_proj_norm_kernel(const float* __restri
     if (lane == 0) red[r][warp] = ss;
   }
   __syncthreads();
+  pdl_wait();   // the modulation
   const float* md = rn.modv + (size_t)(act ? (rn.drow ? rn.drow[b] : rn.H + b) : 0) * rn.mod_ld + rn.off;
   const float* mb = rn.mod_b + rn.off;
 #pragma unroll
