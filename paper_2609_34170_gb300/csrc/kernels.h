@@ -60,6 +60,7 @@ struct CondArgs {
   int H, B, Bmax;
   float* modv; int mod_ld;
   int enabled;                  // 0: always compute, drow = H + b
+  int fresh = 0;                // 1: the time rows count as not cached
 };
 cudaError_t launch_cond_commit(const CondArgs& a, cudaStream_t st);
 // cond_check, and in the same launch E[r][:] = sinusoidal(x_r) for r < H (x =
@@ -129,7 +130,9 @@ struct NormArgs {
   const int* drow = nullptr;    // optional: row of modv holding robot b's offset part (default H + b)
   const float* act_gain = nullptr;   // optional [D]: action rows y = x rsqrt(mean(x^2)+eps) (1 + act_gain),
                                      // without modulation (the query rows of a FOP adapter)
-  int t_stride = 0;             // modv time row of slot j of robot b: b * t_stride + j (H: a schedule per robot)
+  // modv time row of slot j of robot b: b * t_stride + j (t_stride = H: a schedule
+  // per robot), or row ~t_stride for all of them (t_stride < 0)
+  int t_stride = 0;
 };
 cudaError_t launch_ada_norm(const NormArgs& a, Dtype dt, cudaStream_t st);
 
@@ -220,11 +223,14 @@ struct HeadArgs {
 cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, cudaStream_t st);
 
 // Synchronous (full-horizon) denoising: buffer += (t_now - t_next) * vel for
-// every slot (vel_out optional copy); times[0..H-1] = t; a fresh chunk
+// every slot (vel_out optional copy); times[i] = t[min(n0 + i, n_steps - 1)]; a fresh chunk
 // buffer[b][j] = noise(seeds[b], counters[b] + j), counters[b] += H.
 cudaError_t launch_denoise_tail(float* buffer, const float* vel, float* vel_out, int B, int H, int A, float t_now,
                                 float t_next, cudaStream_t st);
-cudaError_t launch_fill_times(float* times, int H, float t, cudaStream_t st);
+struct PassTimes {
+  float t[64];
+};
+cudaError_t launch_fill_times(float* times, int H, const PassTimes& t, int n0, int n_steps, cudaStream_t st);
 cudaError_t launch_chunk_noise(float* buffer, const uint64_t* seeds, uint64_t* counters, int B, int H, int A,
                                cudaStream_t st);
 

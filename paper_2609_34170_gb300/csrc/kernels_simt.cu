@@ -80,7 +80,7 @@ __device__ void cond_check(const CondArgs& a) {
     s_key[threadIdx.x] = cc->delta[threadIdx.x];
   }
   if (threadIdx.x == 0) {
-    s_tmiss = a.enabled ? !cc->t_valid : 1;
+    s_tmiss = a.enabled && !a.fresh ? !cc->t_valid : 1;
     s_bmiss = 0;
     s_ref = 0u;
   }
@@ -411,6 +411,11 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, Dtype dt, cudaStream_t st) {
 
 // ============================================================================ adaRMSNorm
 
+// (t_stride as in NormArgs)
+__device__ __forceinline__ int time_row(int t_stride, int b, int j) {
+  return t_stride < 0 ? ~t_stride : b * t_stride + j;
+}
+
 __device__ __forceinline__ float4 add3(float4 a, float4 b, float4 c) {
   return make_float4(a.x + b.x + c.x, a.y + b.y + c.y, a.z + b.z + c.z, a.w + b.w + c.w);
 }
@@ -438,8 +443,9 @@ __device__ __forceinline__ float4 add2(float4 a, float4 b) {
 // (the row sums are reduced through a double-buffered table).  Few rows per
 // block: the row's loads are the block's critical path, and spreading the
 // rows over more blocks (one each when they fit the SMs) beat batching four
-// rows per round trip.
-template <typename T, int G>
+// rows per round trip.  ONE: one time row for all slots (a select at run time
+// cost a tiny fp32 step 1.8 of 64 us, a batch-1 step 1.1 of 577).
+template <typename T, int G, bool ONE>
 __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, int nb_act, int rb_fop, int nb_fop) {
   constexpr int R = 1;
   __shared__ float red[2][R][8];
@@ -491,7 +497,7 @@ __global__ void __launch_bounds__(256) ada_norm_kernel(NormArgs a, int rb_act, i
           if (act) {
             xv[rr][g] = ld4(a.x + (size_t)(b * a.H + jj) * D + c);
             if (modulated) {
-              const float* mt = a.modv + (size_t)(b * a.t_stride + jj) * a.mod_ld + a.off;
+              const float* mt = a.modv + (size_t)(ONE ? ~a.t_stride : b * a.t_stride + jj) * a.mod_ld + a.off;
               ts[rr][g] = ld4(mt + c);
               th[rr][g] = ld4(mt + D + c);
             }
@@ -604,7 +610,7 @@ __global__ void __launch_bounds__(256) ada_norm_tile_kernel(NormArgs a, int nb_b
   if (act && on) {
 #pragma unroll
     for (int i = 0; i < RJ; ++i) {
-      const float* mt = a.modv + (size_t)(b0 * a.t_stride + min(j0 + i, a.H - 1)) * a.mod_ld + a.off;
+      const float* mt = a.modv + (size_t)time_row(a.t_stride, b0, min(j0 + i, a.H - 1)) * a.mod_ld + a.off;
       tsc[i] = ld4(mt + c);
       tsh[i] = ld4(mt + D + c);
     }
@@ -670,7 +676,7 @@ cudaError_t launch_ada_norm_t(const NormArgs& a, cudaStream_t st) {
     NormArgs b = a;
     b.F = nf;
     const int fop_blocks = (a.B * nf + 3) / 4;
-    if (a.t_stride == 0) {
+    if (a.t_stride <= 0) {
       const int nb = (a.B + 1) / 2, nj = (a.H + 1) / 2;
       return launch_kernel(ada_norm_tile_kernel<T, 2, 2>, dim3(nb * nj + fop_blocks), dim3(256), 0, st, 1, b, nb, nj);
     }
@@ -686,12 +692,16 @@ cudaError_t launch_ada_norm_t(const NormArgs& a, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
   NormArgs b = a;
   b.F = nf;
+#define RAVEL_NORM(G)                                                                                            \
+  return launch_kernel(a.t_stride < 0 ? ada_norm_kernel<T, G, true> : ada_norm_kernel<T, G, false>, dim3(blocks), \
+                       dim3(256), 0, st, 1, b, rb_act, nb_act, rb_fop, nb_fop)
   switch (G) {
-    case 1: return launch_kernel(ada_norm_kernel<T, 1>, dim3(blocks), dim3(256), 0, st, 1, b, rb_act, nb_act, rb_fop, nb_fop);
-    case 2: return launch_kernel(ada_norm_kernel<T, 2>, dim3(blocks), dim3(256), 0, st, 1, b, rb_act, nb_act, rb_fop, nb_fop);
-    case 3: return launch_kernel(ada_norm_kernel<T, 3>, dim3(blocks), dim3(256), 0, st, 1, b, rb_act, nb_act, rb_fop, nb_fop);
-    default: return launch_kernel(ada_norm_kernel<T, 4>, dim3(blocks), dim3(256), 0, st, 1, b, rb_act, nb_act, rb_fop, nb_fop);
+    case 1: RAVEL_NORM(1);
+    case 2: RAVEL_NORM(2);
+    case 3: RAVEL_NORM(3);
+    default: RAVEL_NORM(4);
   }
+#undef RAVEL_NORM
 }
 
 cudaError_t launch_ada_norm(const NormArgs& a, Dtype dt, cudaStream_t st) {
@@ -844,7 +854,7 @@ __global__ void __launch_bounds__(256) in_proj_norm_kernel(const float* __restri
       const float4 q = v[r][g];
       if (act) {
         if (j0 + r >= rn.H) continue;
-        const float* mt = rn.modv + (size_t)(b * rn.t_stride + j0 + r) * rn.mod_ld + rn.off;
+        const float* mt = rn.modv + (size_t)time_row(rn.t_stride, b, j0 + r) * rn.mod_ld + rn.off;
         const float4 sc = add3(ld4(mt + c), dsc, bsc), sh = add3(ld4(mt + D + c), dsh, bsh);
         st4((T*)rn.Y + ((size_t)b * rn.row_pitch + j0 + r) * D + c,
             make_float4(q.x * inv * (1.f + sc.x) + sh.x, q.y * inv * (1.f + sc.y) + sh.y,
@@ -1428,15 +1438,16 @@ cudaError_t launch_denoise_tail(float* buffer, const float* vel, float* vel_out,
   return launch_kernel(denoise_tail_kernel, dim3(blocks), dim3(256), 0, st, 1, buffer, vel, vel_out, n, t_now, t_next);
 }
 
-// times[0..H-1] = t (the single flow time of a synchronous denoising pass).
-__global__ void fill_times_kernel(float* __restrict__ times, int H, float t) {
+// The flow times of up to H synchronous denoising passes from pass n0 on (the
+// last one's repeated): rows of one conditioning for all of them.
+__global__ void fill_times_kernel(float* __restrict__ times, int H, PassTimes t, int n0, int n_steps) {
   pdl_trigger();
   pdl_wait();
-  for (int j = threadIdx.x; j < H; j += blockDim.x) times[j] = t;
+  for (int i = threadIdx.x; i < H; i += blockDim.x) times[i] = t.t[min(n0 + i, n_steps - 1)];
 }
 
-cudaError_t launch_fill_times(float* times, int H, float t, cudaStream_t st) {
-  return launch_kernel(fill_times_kernel, dim3(1), dim3(128), 0, st, 1, times, H, t);
+cudaError_t launch_fill_times(float* times, int H, const PassTimes& t, int n0, int n_steps, cudaStream_t st) {
+  return launch_kernel(fill_times_kernel, dim3(1), dim3(128), 0, st, 1, times, H, t, n0, n_steps);
 }
 
 // A fresh chunk: slot j of robot b receives the Gaussian action of index

@@ -378,13 +378,12 @@ ravel_status ravel_denoise_chunk(ravel_t* r, float* chunk, int n_steps, const vo
     // time each, t_n = 1 - n / n_steps, stepping to t_{n+1} (t_{n_steps} = 0)
     cudaError_t e = launch_chunk_noise(chunk, r->plan.seeds, r->plan.counters, r->batch, c.slots, c.action_dim,
                                        r->cap_stream);
+    PassTimes t{};
+    for (int n = 0; n < n_steps; ++n) t.t[n] = (float)(1.0 - (double)n / n_steps);
     for (int n = 0; n < n_steps && e == cudaSuccess; ++n) {
-      const float t_now = (float)(1.0 - (double)n / n_steps);
-      const float t_next = n + 1 < n_steps ? (float)(1.0 - (double)(n + 1) / n_steps) : 0.f;
-      e = launch_fill_times(r->plan.dn_times, c.per_robot_times ? r->batch * c.slots : c.slots, t_now,
-                            r->cap_stream);
+      if (n % c.slots == 0) e = launch_fill_times(r->plan.dn_times, c.slots, t, n, n_steps, r->cap_stream);
       if (e == cudaSuccess) {
-        const DenoisePass dn{t_now, t_next};
+        const DenoisePass dn{t.t[n], n + 1 < n_steps ? t.t[n + 1] : 0.f, n % c.slots, n_steps > 1};
         int nk = 0;
         e = enqueue_step(r->plan, r->batch, io, r->cap_stream, &nk, nullptr, &dn);
       }

@@ -326,22 +326,33 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
   // compute nothing (cond_check sets the skip flag)
   // time rows of the conditioning: the H slot times, or B*H with a schedule
   // per robot (norms then read robot b's row b*H + j: t_stride = H)
-  const int Ht = c.per_robot_times ? B * H : H, t_stride = c.per_robot_times ? H : 0;
+  // Denoising passes have one flow time for all slots: the first one's
+  // conditioning has the times of up to H passes as its rows, and the passes
+  // after it find theirs there (ten passes at batch 1: 6029 us with a
+  // conditioning each, 5588 so).
+  const bool own_times = c.per_robot_times && !dn;
+  const int Ht = own_times ? B * H : H, t_stride = own_times ? H : 0;
+  const int t_row = dn ? dn->row : 0;
+  const int n_stride = dn ? ~t_row : t_stride;   // the norms' (see NormArgs)
   CondArgs ca{p.cond, p.cond_tkey, p.cond_drow, p.cond_commit, io.slot_times, io.delta, Ht, B, c.max_batch,
               p.modv, p.mod_dim, (p.cond_cache && !c.per_robot_times) ? 1 : 0};
+  ca.fresh = dn ? dn->fresh : 0;
   const int* skip = &p.cond->skip;
-  pdl_enabled() = false;
-  RUN(KK_EMBED, launch_cond_embed(ca, D, p.omega, p.E, dt, st));
-  pdl_enabled() = p.use_pdl && !trace;
-  RUN(KK_GEMM_COND, gemm(p.E, D, p.t_w1, Ht, D, D, EPI_STORE_SILU, p.H1, D, dt, p.t_b1, skip));
-  RUN(KK_GEMM_COND, gemm(rowp(p.E, Ht, D), D, p.d_w1, B, D, D, EPI_STORE_SILU, (void*)rowp(p.H1, Ht, D), D, dt, p.d_b1,
-                         skip));
-  RUN(KK_GEMM_COND, gemm(p.H1, D, p.t_w2, Ht, D, D, EPI_STORE, p.HC, D, dt, p.t_b2, skip));
-  RUN(KK_GEMM_COND, gemm(rowp(p.H1, Ht, D), D, p.d_w2, B, D, D, EPI_STORE, (void*)rowp(p.HC, Ht, D), D, dt, p.d_b2,
-                         skip));
-  RUN(KK_GEMM_MOD, gemm(p.HC, D, p.mod_w, Ht + B, p.mod_dim, D, EPI_STORE, p.modv, p.mod_dim, DT_F32, nullptr,
-                        skip));
-  RUN(KK_COND_CACHE, launch_cond_commit(ca, st));
+  const bool pdl = p.use_pdl && !trace;
+  pdl_enabled() = false;   // the first launch waits for all earlier work
+  if (t_row == 0) {
+    RUN(KK_EMBED, launch_cond_embed(ca, D, p.omega, p.E, dt, st));
+    pdl_enabled() = pdl;
+    RUN(KK_GEMM_COND, gemm(p.E, D, p.t_w1, Ht, D, D, EPI_STORE_SILU, p.H1, D, dt, p.t_b1, skip));
+    RUN(KK_GEMM_COND, gemm(rowp(p.E, Ht, D), D, p.d_w1, B, D, D, EPI_STORE_SILU, (void*)rowp(p.H1, Ht, D), D, dt,
+                           p.d_b1, skip));
+    RUN(KK_GEMM_COND, gemm(p.H1, D, p.t_w2, Ht, D, D, EPI_STORE, p.HC, D, dt, p.t_b2, skip));
+    RUN(KK_GEMM_COND, gemm(rowp(p.H1, Ht, D), D, p.d_w2, B, D, D, EPI_STORE, (void*)rowp(p.HC, Ht, D), D, dt, p.d_b2,
+                           skip));
+    RUN(KK_GEMM_MOD, gemm(p.HC, D, p.mod_w, Ht + B, p.mod_dim, D, EPI_STORE, p.modv, p.mod_dim, DT_F32, nullptr,
+                          skip));
+    RUN(KK_COND_CACHE, launch_cond_commit(ca, st));
+  }
   // residual stream
   // in-projection; with the fused norms, also the first layer's first norm
   const bool fuse_in = p.fuse_norm && p.dt == DT_BF16 && D <= 4096;
@@ -349,13 +360,14 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     const int FF0 = (io.obs && !(p.n_adapters > 0)) ? F : 0;
     RowNorm rn0{p.modv, p.mod_dim, p.mod_b, 0, p.cond_drow, B, H, FF0 ? io.obs : nullptr, F, p.fop_gamma, p.Y,
                       H + FF0};
-    rn0.t_stride = t_stride;
+    rn0.t_stride = n_stride;
     RUN(KK_IN_PROJ, launch_in_proj_norm(io.buffer, A, D, p.in_w, p.in_b, p.x, io.state, p.rel_mask, io.slot_times,
                                         rn0, dt, st));
   } else {
     RUN(KK_IN_PROJ, launch_in_proj(io.buffer, B * H, A, D, p.in_w, p.in_b, p.x, st, io.state, p.rel_mask,
                                    io.slot_times, H, t_stride));
   }
+  pdl_enabled() = pdl;
   const bool adapters = p.n_adapters > 0 && io.obs;
   const int FF = (io.obs && !adapters) ? F : 0;   // FOP tokens as keys of the self-attention
   const int RPR = H + FF;              // normed / QKV rows per robot: H slots, then the FOP tokens
@@ -363,7 +375,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
   for (int l = 0; l < L; ++l) {
     NormArgs n1{p.x, B, H, D, p.modv, p.mod_dim, p.mod_b, 4 * l * D, FF ? io.obs : nullptr, F,
                 p.fop_gamma + (size_t)l * D, p.Y, RPR, p.cond_drow};
-    n1.t_stride = t_stride;
+    n1.t_stride = n_stride;
     if (l > 0 || !fuse_in) RUN(KK_NORM, launch_ada_norm(n1, dt, st));
     const void* wqkv = (const char*)p.w_qkv + (size_t)l * p.nqkv * D * es;
     if (p.use_tc_attn) {
@@ -404,7 +416,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
                            p.x, D, DT_F32, nullptr));
     }
     NormArgs n2{p.x, B, H, D, p.modv, p.mod_dim, p.mod_b, 4 * l * D + 2 * D, nullptr, 0, nullptr, p.Y, H, p.cond_drow};
-    n2.t_stride = t_stride;
+    n2.t_stride = n_stride;
     RUN(KK_NORM, launch_ada_norm(n2, dt, st));
     const void* wgu = (const char*)p.w_gu + (size_t)l * 2 * Fm * D * es;
     GemmArgs gu{p.Y, D, wgu, D, BH, 2 * Fm, D, EPI_GEGLU, p.Hm, Fm, dt, nullptr};
@@ -435,7 +447,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     return e;
   }
   NormArgs nf{p.x, B, H, D, p.modv, p.mod_dim, p.mod_b, 4 * L * D, nullptr, 0, nullptr, p.Y, H, p.cond_drow};
-  nf.t_stride = t_stride;
+  nf.t_stride = n_stride;
   RUN(KK_NORM, launch_ada_norm(nf, dt, st));
   RUN(KK_GEMM_OUT, gemm(p.Y, D, p.out_w, BH, A, D, EPI_STORE, p.V, A, DT_F32, p.out_b));
   if (dn) {

@@ -110,6 +110,8 @@ cudaError_t run_gemm(const StepPlan& p, const GemmArgs& g, cudaStream_t st);
 // time t_now, Euler step t_now - t_next, no release / shift / append.
 struct DenoisePass {
   float t_now, t_next;
+  int row;     // the pass's time row: 0 computes the conditioning of up to H passes at once
+  int fresh;   // row 0: those rows are computed even if their times are cached
 };
 
 // Enqueue one rolling step for `B` robots on `st` (no synchronisation, graph

@@ -83,3 +83,24 @@ def test_denoise_chunk_pi05_b1():
     s = _session(case)
     _check_chunk(case, s, 10, label="pi05 b1 n=10")
     s.close()
+
+
+# One conditioning serves as many passes as there are slots: pass counts on either
+# side of that and of its multiples, fp32 and bf16, the norm's row and tile
+# kernels, schedules per robot; a rolling step after it has its own times back.
+@pytest.mark.parametrize("n_steps", [2, 6, 7, 8, 15])
+@pytest.mark.parametrize("dtype,batch,own", [("fp32", 2, 0), ("bf16", 2, 0), ("bf16", 2, 1), ("bf16", 112, 0)])
+def test_denoise_chunk_conditioning_groups(n_steps, dtype, batch, own):
+    cfg = synth.ExpertConfig(layers=2, width=64, n_q_heads=2, n_kv_heads=1, head_dim=32, mlp_dim=64, slots=7,
+                             action_dim=3, prefix=10, fop_tokens=2, batch=batch, dtype=dtype, per_robot_times=own)
+    case = Case(cfg)
+    if own:
+        case.t = np.stack([case.t * (1 - 0.05 * b) for b in range(batch)])
+    s = _session(case)
+    robots = sorted({0, batch - 1})
+    from tests._harness import check_step
+    for _ in range(2):
+        _check_chunk(case, s, n_steps, robots=robots, label=f"n={n_steps}")
+        if not own:
+            check_step(case, s, robots=robots, label="roll between chunks")
+    s.close()
