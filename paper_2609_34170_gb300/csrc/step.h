@@ -65,7 +65,7 @@ struct StepPlan {
   TcWorkspace tcws{};       // split-K workspace of the tensor-core GEMM
   int num_sms = 0;
   bool use_tc = false;      // bf16 projections on tcgen05
-  float* dn_times = nullptr;   // [H] flow times of a synchronous denoising pass (all equal)
+  float* dn_times = nullptr;   // [H] flow times of the next synchronous denoising passes, one each
   float* rel_mask = nullptr;   // [A] 1 = a dimension the expert predicts relative to the robot state
   bool fuse_norm = true;       // bf16: the in-projection also writes the first layer's first norm
   // FOP adapters (cfg.fop_adapter_every > 0): packed K-major weights, gains,
