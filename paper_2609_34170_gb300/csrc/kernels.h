@@ -53,7 +53,7 @@ struct CondCache {
   float delta[kCondCache];
 };
 struct CondArgs {
-  CondCache* cc; float* t_key;  // [H]
+  CondCache* cc; float* t_key;  // [slots], touched only when enabled
   int* drow;                    // [Bmax] out: modv row of robot b's offset part
   int* commit;                  // [Bmax] pairs (src row, dst row) as 2 ints each -> [2 Bmax]
   const float* slot_times; const float* delta;
