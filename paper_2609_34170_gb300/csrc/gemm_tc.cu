@@ -56,6 +56,7 @@ constexpr int TC_PAIR_THREADS = 320;   // pair kernel: TMA, MMA and two sets of 
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;
 constexpr int TC_SMEM_BUDGET = 200 * 1024;   // operand ring
 constexpr int TC_SMEM_MAX = 227 * 1024;
+constexpr size_t TC_SMEM_SM = 228 * 1024;
 constexpr int TC_RING_SPLIT = 128 * 1024;    // operand ring of a split-K launch
 constexpr int STG_LD = 132;                  // SIMT staging pitch (floats): 16 tokens x 128 tile rows
 constexpr uint32_t STG_BYTES = 16 * STG_LD * 4;
@@ -1298,7 +1299,10 @@ constexpr unsigned long long kWithholdWaitNs = 2000000ull;   // their wait limit
 // Resident clusters of 2, 4, 8, 16 split CTAs (one CTA per SM; 0: that
 // cluster size is not to be had).  The split-K kernels take a whole SM each,
 // and clusters stay inside a GPC: 76, 36, 15 and 7 on this part.
-int g_max_clusters[4] = {0, 0, 0, 0};
+struct TcClusters {
+  int n[4];
+};
+TcClusters g_max_clusters = {{0, 0, 0, 0}};
 
 // How a GEMM is cut: token-tile width, K splits (a cluster), or SM pairs.
 struct TcPlan {
@@ -1325,7 +1329,8 @@ struct TcPlan {
 // 64 robots, each projection's width and splits varied in turn: the rule is
 // 0 to 3.5 % of the step away from the best combination (batch 1 at it: 652
 // us, 685 with the chain's terms alone).
-TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t ws_bytes, bool pairs, int num_sms) {
+TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t ws_bytes, bool pairs, int num_sms,
+                 const TcClusters& clusters) {
   const int tiles_n = (N + TC_BM - 1) / TC_BM, num_kb = (K + TC_BK - 1) / TC_BK;
   TcPlan best;
   float cost = 3.4e38f;
@@ -1350,9 +1355,9 @@ TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t
       // 4-token groups, of at most 32 tokens through shared memory, and
       // through L2 the partials have to fit the workspace
       const int sp = 2 << i;
-      if (sp > num_kb || bn % (4 * sp) || !g_max_clusters[i] || (long)tiles * sp > 2L * num_sms) break;
+      if (sp > num_kb || bn % (4 * sp) || !clusters.n[i] || (long)tiles * sp > 2L * num_sms) break;
       if (dsmem ? bn / sp > 32 : (size_t)sp * tiles * bn * TC_BM * 4 > ws_bytes) continue;
-      const int w = (tiles + g_max_clusters[i] - 1) / g_max_clusters[i];
+      const int w = (tiles + clusters.n[i] - 1) / clusters.n[i];
       consider(false, bn, sp,
                2.6f + epi / (float)sp + (float)w * (float)((num_kb + sp - 1) / sp) * step +
                    (xbf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * 2.5f +
@@ -1379,49 +1384,126 @@ TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t
 // 2e-3.
 bool short_sums(const GemmArgs& g) { return !g.xbf16 && (g.epi == EPI_ADD_F32 || (g.epi != EPI_GEGLU && g.out_dt == DT_F32)); }
 
+// Sizes of a launch: the operand ring, TMEM and the shared memory around them.
+struct TcLayout {
+  int stages = 0, lacc = 0, reduce = RED_NONE, box_m = 0;
+  bool oneshot = false;
+  uint32_t acc_cols = 32, ncols = 0, box_bytes = 0, stg_off = 0, xch_off = 0, rcv_off = 0, bar_off = 0, set_bytes = 0;
+  size_t ring = 0, smem = 0;   // smem 0: no such launch
+};
+
+bool out_is_bf16(const GemmArgs& g) { return g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16); }
+
+// outputs through TMA boxes when the output rows are 16-byte aligned
+bool out_aligned(const GemmArgs& g) {
+  return ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * (out_is_bf16(g) ? 2 : 4)) % 16 == 0;
+}
+
+// Two-SM launch with token tiles of bn (a multiple of 32 in [64, 256]).
+TcLayout pair_layout(const GemmArgs& g, int bn) {
+  TcLayout l;
+  while ((int)l.acc_cols < bn) l.acc_cols <<= 1;
+  l.ncols = 2 * l.acc_cols;
+  l.box_m = 32;
+  l.box_bytes = (uint32_t)(((size_t)l.box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * (out_is_bf16(g) ? 2 : 4) + 1023) /
+                           1024 * 1024);
+  const size_t stg_bytes = 2 * (size_t)l.box_bytes;
+  const size_t xch_bytes = g.epi == EPI_GEGLU ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
+  // each of the two epilogue warp sets has its own boxes and exchange tile
+  l.set_bytes = (uint32_t)(stg_bytes + xch_bytes);
+  const size_t fixed = 1024 + 2 * (size_t)l.set_bytes + 256;
+  const int stage_bytes = TC_A_BYTES + (bn / 2) * TC_BK * 2;
+  l.stages = std::min(8, (int)((TC_SMEM_MAX - fixed) / stage_bytes));
+  if (l.stages < 2) return l;
+  l.ring = ((size_t)l.stages * stage_bytes + 1023) / 1024 * 1024;
+  l.stg_off = (uint32_t)l.ring;
+  l.xch_off = l.stg_off + (uint32_t)stg_bytes;
+  l.bar_off = l.stg_off + 2 * l.set_bytes;
+  const size_t smem = 1024 + l.bar_off + (size_t)(2 * l.stages + 4) * 8 + 4 + 16 + 64;
+  l.smem = smem > (size_t)TC_SMEM_MAX ? 0 : smem;
+  return l;
+}
+
+// One-SM launch of a plan.
+TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
+  TcLayout l;
+  const bool tma_out = out_aligned(g);
+  const int bn = plan.bn, splits = plan.splits, es = out_is_bf16(g) ? 2 : 4;
+  const int tiles = (g.N + TC_BM - 1) / TC_BM * ((g.M + bn - 1) / bn);
+  const int num_kb = (g.K + TC_BK - 1) / TC_BK;
+  const int cpr = bn / splits;   // a multiple of 4 whenever the splits form a cluster
+  while ((int)l.acc_cols < bn) l.acc_cols <<= 1;
+  const int stage_bytes = TC_A_BYTES + bn * TC_BK * 2;
+  const int kb_per_item = (num_kb + splits - 1) / splits;
+  // (more than one k-tile per accumulator, so every one is written)
+  if (short_sums(g))
+    while (kb_per_item > (3 << l.lacc) && (l.acc_cols << (l.lacc + (splits > 1 ? 1 : 2))) <= 512u) ++l.lacc;
+  l.ncols = l.acc_cols << (l.lacc + (splits > 1 ? 0 : 1));
+  const int grid_ctas = splits > 1 ? tiles * splits : std::min(tiles, num_sms);
+  const int items = splits > 1 ? 1 : (tiles + grid_ctas - 1) / grid_ctas;
+  l.stages = std::min(8, TC_SMEM_BUDGET / stage_bytes);
+  // a split-K launch is latency-bound: enough stages for its whole (short) K
+  // range when that fits, so that no operand load waits for a freed stage
+  if (splits > 1) l.stages = std::min(l.stages, std::max(2, TC_RING_SPLIT / stage_bytes));
+  l.stages = std::max(2, std::min(l.stages, std::max(2, kb_per_item * items)));
+  // partials exchanged in bf16 where the caller allows it, else in fp32
+  const bool xbf = g.xbf16 != 0;
+  const bool dsmem = splits > 1 && tma_out;
+  const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
+  // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
+  // takes its weight and token k-tiles in one box each (K a multiple of 64)
+  l.oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
+              (size_t)kb_per_item * stage_bytes <=
+                  std::min<size_t>(TC_SMEM_BUDGET, TC_SMEM_MAX - 4096 - (rcv_bytes + 1023) / 1024 * 1024);
+  if (l.oneshot) l.stages = kb_per_item;   // the ring is exactly one box deep
+  l.ring = ((size_t)l.stages * stage_bytes + 1023) / 1024 * 1024;
+  l.reduce = splits == 1 ? RED_NONE : !dsmem ? RED_L2_CLUSTER : xbf ? RED_DSMEM : RED_DSMEM32;
+  // tokens per output box; a split's slice is stored by the threads, its
+  // received partials (all splits' slices of this rank) behind the ring
+  l.box_m = splits == 1 ? 16 : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
+  l.box_bytes = (uint32_t)(((size_t)l.box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
+  const size_t stg_bytes = dsmem ? rcv_bytes : tma_out ? 2 * (size_t)l.box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
+  const size_t xch_bytes = (splits == 1 && tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
+  l.stg_off = l.rcv_off = (uint32_t)l.ring;
+  l.xch_off = l.stg_off + (uint32_t)stg_bytes;
+  l.bar_off = l.xch_off + (uint32_t)xch_bytes;
+  size_t smem = 1024 + l.bar_off + (size_t)(2 * l.stages + 5) * 8 + 4 + 16 + 64;
+  // The CTAs of a split wait for one another with their TMEM taken.  Beside a
+  // CTA of another stream's split launch, one could wait for columns that the
+  // other frees only after a peer that waits likewise, until both time out:
+  // a launch takes no larger share of the SM's TMEM than of its shared memory
+  // (1 KB per CTA is the system's), so that what fits together fits in both.
+  if (splits > 1) smem = std::max(smem, (size_t)l.ncols * TC_SMEM_SM / 512 - 1024);
+  l.smem = smem > (size_t)TC_SMEM_MAX ? 0 : smem;
+  return l;
+}
+
 // Two-SM launch of a persistent GEMM (see tc_gemm_pair_kernel) with token
-// tiles of bn (a multiple of 32 in [64, 256]) and the usual TMA epilogue
-// layout.
-cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st, int ek,
-                             bool out_bf, int es, int bn) {
+// tiles of bn and the usual TMA epilogue layout.
+cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st, int bn) {
+  const TcLayout l = pair_layout(g, bn);
+  if (!l.smem) return cudaErrorInvalidConfiguration;
+  const bool out_bf = out_is_bf16(g);
+  const int ek = g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32;
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
   const int tiles_n2 = (g.N + 2 * TC_BM - 1) / (2 * TC_BM);
   const int slots = num_sms / 2;
   const int tiles_m = (g.M + bn - 1) / bn;
   const int num_tiles = tiles_n2 * tiles_m;
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
-  uint32_t acc_cols = 32;
-  while ((int)acc_cols < bn) acc_cols <<= 1;
-  const int box_m = 32;
-  const uint32_t box_bytes =
-      (uint32_t)(((size_t)box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
-  const size_t stg_bytes = 2 * (size_t)box_bytes;
-  const size_t xch_bytes = g.epi == EPI_GEGLU ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
-  // each of the two epilogue warp sets has its own boxes and exchange tile
-  const size_t set_bytes = stg_bytes + xch_bytes;
-  const size_t fixed = 1024 + 2 * set_bytes + 256;
-  const int stage_bytes = TC_A_BYTES + (bn / 2) * TC_BK * 2;
-  const int stages = std::min(8, (int)((TC_SMEM_MAX - fixed) / stage_bytes));
-  if (stages < 2) return cudaErrorInvalidConfiguration;
-  const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
-  const uint32_t stg_off = (uint32_t)ring;
-  const uint32_t xch_off = stg_off + (uint32_t)stg_bytes;
-  const uint32_t bar_off = stg_off + 2 * (uint32_t)set_bytes;
-  const size_t smem = 1024 + bar_off + (size_t)(2 * stages + 4) * 8 + 4 + 16 + 64;
-  if (smem > (size_t)TC_SMEM_MAX) return cudaErrorInvalidConfiguration;
   CUtensorMap mw, mx, mo;
   cudaError_t e = encode_2d(&mw, g.W, g.N, g.K, g.ldw, TC_BM);
   if (e == cudaSuccess) e = encode_2d(&mx, g.A, g.M, g.K, g.lda, bn / 2);
   if (e == cudaSuccess)
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
-                   g.epi == EPI_GEGLU ? 64 : TC_BM, box_m);
+                   g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, stages, 1, num_kb, RED_NONE, (uint32_t)ring, acc_cols, 0, tiles_n, tiles_m, num_tiles,
-             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
-             1, 0, box_m, box_bytes, stg_off, xch_off, 0, bar_off, kTcTimeoutNs, 0, g.skip};
-  p.set_bytes = (uint32_t)set_bytes;
+  TcParams p{g.M, g.N, g.K, bn, l.stages, 1, num_kb, RED_NONE, (uint32_t)l.ring, l.acc_cols, 0, tiles_n, tiles_m,
+             num_tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
+             1, 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, 0, l.bar_off, kTcTimeoutNs, 0, g.skip};
+  p.set_bytes = l.set_bytes;
   const int npairs = std::min(num_tiles, slots);
-  return launch_kernel_cluster(tc_pair_kernel(ek), dim3(2 * npairs), dim3(TC_PAIR_THREADS), smem, st, dim3(2, 1, 1),
+  return launch_kernel_cluster(tc_pair_kernel(ek), dim3(2 * npairs), dim3(TC_PAIR_THREADS), l.smem, st, dim3(2, 1, 1),
                                mw, mx, mo, p);
 }
 
@@ -1457,7 +1539,7 @@ cudaError_t init_tc_gemm() {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    g_max_clusters[i] =
+    g_max_clusters.n[i] =
         cudaOccupancyMaxActiveClusters(&n, tc_kernel(RED_DSMEM, EK_SLICE), &cfg) == cudaSuccess && n > 0 ? n : 0;
   }
   cudaGetLastError();
@@ -1474,59 +1556,20 @@ bool tc_gemm_supported(const GemmArgs& g) {
 
 cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st) {
   if (!g_encode) return cudaErrorInitializationError;
-  // outputs through TMA boxes when the output rows are 16-byte aligned
-  const bool out_bf = g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16);
-  const int es = out_bf ? 2 : 4;
-  const bool tma_out = ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * es) % 16 == 0;
-  const TcPlan plan = plan_gemm(g.M, g.N, g.K, g.epi == EPI_GEGLU, g.xbf16 != 0, tma_out, ws.ws_bytes, tma_out, num_sms);
-  if (plan.pair)
-    return launch_gemm_pair(g, ws, num_sms, st,
-                            g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32,
-                            out_bf, es, plan.bn);
+  const bool out_bf = out_is_bf16(g), tma_out = out_aligned(g);
+  const TcPlan plan = plan_gemm(g.M, g.N, g.K, g.epi == EPI_GEGLU, g.xbf16 != 0, tma_out, ws.ws_bytes, tma_out, num_sms,
+                                g_max_clusters);
+  if (plan.pair) return launch_gemm_pair(g, ws, num_sms, st, plan.bn);
+  const TcLayout l = one_layout(g, plan, num_sms);
+  if (!l.smem) return cudaErrorInvalidConfiguration;
   const int bn = plan.bn, splits = plan.splits;
   const int tiles_n = (g.N + TC_BM - 1) / TC_BM;
   const int tiles_m = (g.M + bn - 1) / bn;
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
   const int tiles = tiles_n * tiles_m;
-  const int cpr = bn / splits;   // a multiple of 4 whenever the splits form a cluster
-  uint32_t acc_cols = 32;
-  while ((int)acc_cols < bn) acc_cols <<= 1;
-  const int stage_bytes = TC_A_BYTES + bn * TC_BK * 2;
   const int kb_per_item = (num_kb + splits - 1) / splits;
-  // (more than one k-tile per accumulator, so every one is written)
-  int lacc = 0;
-  if (short_sums(g))
-    while (kb_per_item > (3 << lacc) && (acc_cols << (lacc + (splits > 1 ? 1 : 2))) <= 512u) ++lacc;
   const int grid_ctas = splits > 1 ? tiles * splits : std::min(tiles, num_sms);
-  const int items = splits > 1 ? 1 : (tiles + grid_ctas - 1) / grid_ctas;
-  int stages = std::min(8, TC_SMEM_BUDGET / stage_bytes);
-  // a split-K launch is latency-bound: enough stages for its whole (short) K
-  // range when that fits, so that no operand load waits for a freed stage
-  if (splits > 1) stages = std::min(stages, std::max(2, TC_RING_SPLIT / stage_bytes));
-  stages = std::max(2, std::min(stages, std::max(2, kb_per_item * items)));
-  // partials exchanged in bf16 where the caller allows it, else in fp32
-  const bool xbf = g.xbf16 != 0;
-  const bool dsmem = splits > 1 && tma_out;
-  const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
-  // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
-  // takes its weight and token k-tiles in one box each (K a multiple of 64)
-  const bool oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
-                       (size_t)kb_per_item * stage_bytes <=
-                           std::min<size_t>(TC_SMEM_BUDGET, TC_SMEM_MAX - 4096 - (rcv_bytes + 1023) / 1024 * 1024);
-  if (oneshot) stages = kb_per_item;   // the ring is exactly one box deep
-  const size_t ring = ((size_t)stages * stage_bytes + 1023) / 1024 * 1024;
-  const int reduce = splits == 1 ? RED_NONE : !dsmem ? RED_L2_CLUSTER : xbf ? RED_DSMEM : RED_DSMEM32;
-  // tokens per output box; a split's slice is stored by the threads, its
-  // received partials (all splits' slices of this rank) behind the ring
-  const int box_m = splits == 1 ? 16 : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
-  const uint32_t box_bytes =
-      (uint32_t)(((size_t)box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
-  const size_t stg_bytes = dsmem ? rcv_bytes : tma_out ? 2 * (size_t)box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
-  const size_t xch_bytes = (splits == 1 && tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
-  const uint32_t stg_off = (uint32_t)ring, xch_off = stg_off + (uint32_t)stg_bytes, rcv_off = stg_off;
-  const uint32_t bar_off = xch_off + (uint32_t)xch_bytes;
-  const size_t smem = 1024 + bar_off + (size_t)(2 * stages + 5) * 8 + 4 + 16 + 64;
-  if (smem > (size_t)TC_SMEM_MAX) return cudaErrorInvalidConfiguration;
+  const bool oneshot = l.oneshot, dsmem = splits > 1 && tma_out;
   CUtensorMap mw, mx, mo;
   memset(&mo, 0, sizeof(mo));
   cudaError_t e = oneshot ? encode_kt(&mw, g.W, g.N, g.K, g.ldw, TC_BM, kb_per_item)
@@ -1535,15 +1578,15 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
     e = oneshot ? encode_kt(&mx, g.A, g.M, g.K, g.lda, bn, kb_per_item) : encode_2d(&mx, g.A, g.M, g.K, g.lda, bn);
   if (e == cudaSuccess && tma_out && !dsmem)
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
-                   g.epi == EPI_GEGLU ? 64 : TC_BM, box_m);
+                   g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, stages, splits, num_kb, reduce, (uint32_t)ring, acc_cols, lacc, tiles_n, tiles_m, tiles,
-             (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
-             tma_out ? 1 : 0, oneshot ? 1 : 0, box_m, box_bytes, stg_off, xch_off, rcv_off, bar_off, kTcTimeoutNs, 0,
-             g.skip};
+  TcParams p{g.M, g.N, g.K, bn, l.stages, splits, num_kb, l.reduce, (uint32_t)l.ring, l.acc_cols, l.lacc, tiles_n,
+             tiles_m, tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
+             tma_out ? 1 : 0, oneshot ? 1 : 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, l.rcv_off, l.bar_off,
+             kTcTimeoutNs, 0, g.skip};
   // fault injection (tests): a launch without a cluster may be told to wait
   // for an arrival that never comes, with a short limit
-  if (reduce == RED_NONE && g_withhold.load() > 0 && g_withhold.fetch_sub(1) > 0) {
+  if (l.reduce == RED_NONE && g_withhold.load() > 0 && g_withhold.fetch_sub(1) > 0) {
     p.withhold = 1;
     p.wait_ns = kWithholdWaitNs;
   }
@@ -1554,9 +1597,26 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
   const int ek = !tma_out ? EK_GENERIC
                  : dsmem ? EK_SLICE
                  : g.epi == EPI_GEGLU ? EK_GEGLU : g.epi == EPI_ADD_F32 ? EK_ADD : out_bf ? EK_BF16 : EK_F32;
-  const TcKernel k = tc_kernel(reduce, ek);
+  const TcKernel k = tc_kernel(l.reduce, ek);
   if (!k) return cudaErrorInvalidConfiguration;
-  return launch_kernel(k, grid, block, smem, st, (unsigned)splits, mw, mx, mo, p);
+  return launch_kernel(k, grid, block, l.smem, st, (unsigned)splits, mw, mx, mo, p);
 }
 
 }  // namespace ravel
+
+// What a tensor-core GEMM of these sizes is cut into, for tests: out = {1 on SM
+// pairs, token-tile width, K splits, how they exchange (0 none, 1 fp32 through
+// L2, 2 bf16 and 3 fp32 through shared memory), accumulators per item, TMEM
+// columns, shared-memory bytes}.  clusters: how many clusters of 2, 4, 8, 16 fit.
+extern "C" void ravel_debug_gemm_plan(int M, int N, int K, int epi, int out_bf16, int xbf16, int aligned,
+                                      size_t ws_bytes, int num_sms, const int* clusters, int* out) {
+  using namespace ravel;
+  GemmArgs g{nullptr, K, nullptr, K, M, N, K, (Epi)epi, (void*)(uintptr_t)(aligned ? 16 : 4), (N + 7) / 8 * 8,
+             out_bf16 ? DT_BF16 : DT_F32, nullptr};
+  g.xbf16 = xbf16;
+  const TcPlan plan = plan_gemm(M, N, K, epi == EPI_GEGLU, xbf16 != 0, aligned != 0, ws_bytes, aligned != 0, num_sms,
+                                TcClusters{{clusters[0], clusters[1], clusters[2], clusters[3]}});
+  const TcLayout l = plan.pair ? pair_layout(g, plan.bn) : one_layout(g, plan, num_sms);
+  const int v[7] = {plan.pair, plan.bn, plan.splits, l.reduce, 1 << l.lacc, (int)l.ncols, (int)l.smem};
+  for (int i = 0; i < 7; ++i) out[i] = v[i];
+}

@@ -1,0 +1,58 @@
+"""What the tensor-core GEMM is cut into (host code, no GPU): the plan's
+tile width, splits, exchange, accumulators, TMEM and shared memory over sizes
+drawn from the whole range."""
+import ctypes as C
+import random
+
+import pytest
+
+STORE, SILU, ADD, GEGLU = 0, 1, 2, 3
+NONE, L2, BF16, FP32 = 0, 1, 2, 3   # how splits exchange their partials
+SMS, SM_SMEM, TMEM = 152, 228 * 1024, 512
+
+
+@pytest.fixture(scope="module")
+def plan():
+    from paper_2609_34170_gb300 import build, load
+    build.build()
+    fn = load().ravel_debug_gemm_plan
+    fn.restype = None
+    fn.argtypes = [C.c_int] * 7 + [C.c_size_t, C.c_int, C.c_void_p, C.c_void_p]
+    clusters = (C.c_int * 4)(76, 36, 15, 7)
+    out = (C.c_int * 7)()
+
+    def call(m, n, k, epi, out_bf16, xbf16, aligned=1, ws=24 << 20):
+        fn(m, n, k, epi, out_bf16, xbf16, aligned, ws, SMS, clusters, out)
+        return dict(zip(("pair", "bn", "splits", "exchange", "accs", "cols", "smem"), out))
+
+    return call
+
+
+def _draws(n, seed):
+    rng = random.Random(seed)
+    for _ in range(n):
+        m = int(4225 ** rng.random())
+        k = 8 * rng.randint(1, 512) if rng.random() < 0.5 else rng.choice([64, 128, 256, 512, 1024, 2048, 4096])
+        nn = rng.choice([32, 100, 1024, 1536, 2560, 8192, rng.randint(16, 4096)])
+        epi = rng.choice([STORE, STORE, SILU, ADD, GEGLU])
+        yield (m, (nn + 127) // 128 * 128 if epi == GEGLU else nn, k, epi,
+               1 if epi == GEGLU else 0 if epi == ADD else rng.randint(0, 1), rng.randint(0, 1), rng.random() < 0.8)
+
+
+def test_waiting_launches_share_an_sm_only_if_tmem_holds_both(plan):
+    """CTAs that wait for others of their cluster may meet another stream's on
+    an SM, each holding TMEM that the other's peers need: whatever fits the
+    SM's shared memory together must fit its TMEM."""
+    splits, pairs = set(), set()
+    for m, n, k, epi, bf, xb, al in _draws(20000, 1):
+        p = plan(m, n, k, epi, bf, xb, int(al))
+        assert 0 < p["smem"] <= 227 * 1024 and 32 <= p["cols"] <= TMEM, (m, n, k, p)
+        if p["splits"] > 1:
+            splits.add((p["smem"] + 1024, p["cols"]))   # 1 KB of each CTA is the system's
+        elif p["pair"]:
+            pairs.add((p["smem"] + 1024, p["cols"]))
+    for smem, cols in splits:   # at most its share of TMEM: any set of them fits
+        assert cols * SM_SMEM <= TMEM * smem, (smem, cols)
+    for smem, cols in pairs:
+        for s2, c2 in splits:
+            assert smem + s2 > SM_SMEM or cols + c2 <= TMEM, (smem, cols, s2, c2)
