@@ -85,7 +85,11 @@ struct AtParams {
 };
 
 // boxes of [128 keys][64-wide head-dim block] (K) and [64 keys][64-wide block]
-// (V), 128-byte swizzled
+// (V), 128-byte swizzled.  V's maps end at the robot's last row, so that the rows
+// of a 16-key group past it are zeros: their probability is 0, but 0 times
+// another robot's Inf or NaN is not.  (K needs no such end: those scores are
+// replaced.  The context's V rows up to the group's end are zeroed when it is
+// installed.)
 struct AtMaps {
   CUtensorMap q, k, v, pk0, pk1, pv0, pv1, o;   // o: (hd, heads, slots, robots), boxes as Q's
 };
@@ -283,11 +287,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     const uint32_t vs = v0 + (uint32_t)s * v_bytes, bar = smem_u32(&v_full[s]);
     const CUtensorMap* vm = pre ? pv : &maps.v;
     const int key = (pre ? c : c - npv) * AT_BKV + 64 * h;
-    const int vy = pre ? key : g, vz = pre ? ctx_z : b * rows_per_robot + key;
     mbar_expect_tx_el(&v_full[s], v_bytes, el);
     #pragma unroll 1
     for (int blk = 0; blk < p.nblk; ++blk)
-      tma_load_3d_el(vm, bar, vs + (uint32_t)blk * AT_VBLK, blk * 64, vy, vz, pre ? pol_kv : pol_q, el);
+      tma_load_4d_el(vm, bar, vs + (uint32_t)blk * AT_VBLK, blk * 64, pre ? 0 : g, key, pre ? ctx_z : b,
+                     pre ? pol_kv : pol_q, el);
   };
   // next K unit (chunk kc, block kb, slot sk) and V half (chunk vc, half vh, slot
   // sv) to load, and the parities their `empty` waits take
@@ -839,15 +843,17 @@ cudaError_t enc3(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uin
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// The output as (hd, heads, slots, robots), boxes of 64 x G x TQ x 1: slots past
-// the robot's own are clipped.
-cudaError_t enc_out(CUtensorMap* m, void* base, int hd, int heads, int H, int B, int ld, int G, int TQ) {
-  cuuint64_t dims[4] = {(cuuint64_t)hd, (cuuint64_t)heads, (cuuint64_t)H, (cuuint64_t)B};
-  cuuint64_t strides[3] = {(cuuint64_t)hd * 2, (cuuint64_t)ld * 2, (cuuint64_t)H * ld * 2};
-  cuuint32_t box[4] = {64, (cuuint32_t)G, (cuuint32_t)TQ, 1};
+// Rows as (hd, heads, rows of a group, groups), boxes of 64 x heads_box x rows_box
+// x 1: rows past the group's own are clipped (stores) or zeros (loads).
+cudaError_t enc4(CUtensorMap* m, const void* base, int hd, int heads, int rows, uint64_t groups, uint64_t row_bytes,
+                 int heads_box, int rows_box, bool load) {
+  cuuint64_t dims[4] = {(cuuint64_t)hd, (cuuint64_t)heads, (cuuint64_t)rows, (cuuint64_t)groups};
+  cuuint64_t strides[3] = {(cuuint64_t)hd * 2, (cuuint64_t)row_bytes, (cuuint64_t)rows * row_bytes};
+  cuuint32_t box[4] = {64, (cuuint32_t)heads_box, (cuuint32_t)rows_box, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = g_enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+  CUresult r = g_enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                     load ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_NONE,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -978,16 +984,15 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
     e = enc3(&m.k, (const bf16*)a.qkv + (size_t)a.Hq * hd, hd, a.Hkv, rows, (uint64_t)hd * 2, (uint64_t)a.ld_qkv * 2,
              64, 1, AT_BKV);
   if (e == cudaSuccess)
-    e = enc3(&m.v, (const bf16*)a.qkv + (size_t)(a.Hq + a.Hkv) * hd, hd, a.Hkv, rows, (uint64_t)hd * 2,
-             (uint64_t)a.ld_qkv * 2, 64, 1, 64);
-  if (e == cudaSuccess) e = enc_out(&m.o, a.out, hd, a.Hq, a.H, a.B, a.ld_out, p.G, p.TQ);
+    e = enc4(&m.v, (const bf16*)a.qkv + (size_t)(a.Hq + a.Hkv) * hd, hd, a.Hkv, rpr, a.B, (uint64_t)a.ld_qkv * 2, 1,
+             64, true);
+  if (e == cudaSuccess) e = enc4(&m.o, a.out, hd, a.Hq, a.H, a.B, (uint64_t)a.ld_out * 2, p.G, p.TQ, false);
   const uint64_t zc = (uint64_t)(a.layers * a.Bmax * a.Hkv);
   for (int s = 0; s < 2 && e == cudaSuccess; ++s) {
     e = enc3(s ? &m.pk1 : &m.pk0, a.ctx_k[s], hd, a.Pmax, zc, (uint64_t)hd * 2, (uint64_t)a.Pmax * hd * 2, 64,
              AT_BKV, 1);
     if (e == cudaSuccess)
-      e = enc3(s ? &m.pv1 : &m.pv0, a.ctx_v[s], hd, a.Pmax, zc, (uint64_t)hd * 2, (uint64_t)a.Pmax * hd * 2, 64, 64,
-               1);
+      e = enc4(s ? &m.pv1 : &m.pv0, a.ctx_v[s], hd, 1, a.Pmax, zc, (uint64_t)hd * 2, 1, 64, true);
   }
   if (e != cudaSuccess) return e;
   dim3 grid(p.q_tiles, a.B * a.Hkv, splits);

@@ -262,8 +262,9 @@ struct CtxList {
 // ctx_state [Bmax][2] = {slot, prefix length} per robot
 cudaError_t launch_flip(int* ctx_state, const CtxList& f, cudaStream_t st);
 // src [L][src_n][Hkv][P] rows of row_bytes, list entry i at source position
-// i0 + i -> dst_{f.slot[i]} [L][Bmax][Hkv][Pmax] rows of robot f.robot[i]
+// i0 + i -> dst_{f.slot[i]} [L][Bmax][Hkv][Pmax] rows of robot f.robot[i];
+// rows P .. Pz - 1 (P <= Pz <= Pmax) become zeros
 cudaError_t launch_ctx_scatter(const void* src, int src_n, int i0, void* dst0, void* dst1, int L, int Bmax, int Hkv,
-                               int P, int Pmax, size_t row_bytes, const CtxList& f, cudaStream_t st);
+                               int P, int Pz, int Pmax, size_t row_bytes, const CtxList& f, cudaStream_t st);
 
 }  // namespace ravel

@@ -1482,28 +1482,30 @@ cudaError_t launch_flip(int* ctx_state, const CtxList& f, cudaStream_t st) {
 
 // Context rows of the listed robots into their slots: source [L][src_n][Hkv]
 // [P][row] with the list's robots at positions i0 .. i0 + f.n - 1 of each
-// layer, destination [slot][L][Bmax][Hkv][Pmax][row] (16-byte words).
+// layer, destination [slot][L][Bmax][Hkv][Pmax][row] (16-byte words); rows P ..
+// Pz - 1 become zeros.
 __global__ void ctx_scatter_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst0, uint4* __restrict__ dst1,
-                                   int src_n, int i0, int Bmax, int Hkv, int P, int Pmax, int row_words, CtxList f) {
+                                   int src_n, int i0, int Bmax, int Hkv, int P, int Pz, int Pmax, int row_words,
+                                   CtxList f) {
   const int z = blockIdx.y;                  // (l * f.n + i) * Hkv + g
   const int g = z % Hkv, li = z / Hkv;
   const int i = li % f.n, l = li / f.n;
-  const size_t words = (size_t)P * row_words;
+  const size_t words = (size_t)P * row_words, all = (size_t)Pz * row_words;
   const uint4* s = src + ((size_t)(l * src_n + i0 + i) * Hkv + g) * words;
   uint4* d = (f.slot[i] ? dst1 : dst0) + (((size_t)l * Bmax + f.robot[i]) * Hkv + g) * (size_t)Pmax * row_words;
-  for (size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += (size_t)gridDim.x * blockDim.x)
-    d[w] = s[w];
+  for (size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x; w < all; w += (size_t)gridDim.x * blockDim.x)
+    d[w] = w < words ? s[w] : make_uint4(0, 0, 0, 0);
 }
 
 cudaError_t launch_ctx_scatter(const void* src, int src_n, int i0, void* dst0, void* dst1, int L, int Bmax, int Hkv,
-                               int P, int Pmax, size_t row_bytes, const CtxList& f, cudaStream_t st) {
+                               int P, int Pz, int Pmax, size_t row_bytes, const CtxList& f, cudaStream_t st) {
   if (f.n <= 0 || P <= 0) return cudaSuccess;
   if (row_bytes % 16 || ((uintptr_t)src | (uintptr_t)dst0 | (uintptr_t)dst1) % 16) return cudaErrorMisalignedAddress;
   const int row_words = (int)(row_bytes / 16);
   const size_t words = (size_t)P * row_words;
   dim3 grid((unsigned)std::min<size_t>((words + 255) / 256, 64), (unsigned)(L * f.n * Hkv));
   ctx_scatter_kernel<<<grid, 256, 0, st>>>((const uint4*)src, (uint4*)dst0, (uint4*)dst1, src_n, i0, Bmax, Hkv, P,
-                                           Pmax, row_words, f);
+                                           Pz, Pmax, row_words, f);
   return cudaGetLastError();
 }
 

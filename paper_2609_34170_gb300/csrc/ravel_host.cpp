@@ -218,10 +218,12 @@ static ravel_status set_context_impl(ravel_t* r, const int* robots, int n, const
       f.len[i] = prefix_len;
     }
     RV_CUDA(r, launch_ctx_scatter(k, n, i0, p.ctx_k[0], p.ctx_k[1], c.layers, c.max_batch, c.n_kv_heads, prefix_len,
-                                  c.max_prefix, (size_t)c.head_dim * es, f, side),
+                                  prefix_len, c.max_prefix, (size_t)c.head_dim * es, f, side),
             (w + ": copy K").c_str());
+    // P V takes whole groups of 16 keys: the rest of V's last group, which may
+    // hold an earlier, longer context's rows, becomes zeros
     RV_CUDA(r, launch_ctx_scatter(v, n, i0, p.ctx_v[0], p.ctx_v[1], c.layers, c.max_batch, c.n_kv_heads, prefix_len,
-                                  c.max_prefix, (size_t)c.head_dim * es, f, side),
+                                  std::min((prefix_len + 15) / 16 * 16, c.max_prefix), c.max_prefix, (size_t)c.head_dim * es, f, side),
             (w + ": copy V").c_str());
     for (int i = 0; i < f.n; ++i) {
       r->ctx_pend[f.robot[i]] = f.slot[i];

@@ -141,6 +141,15 @@ __device__ __forceinline__ void tma_load_3d_el(const CUtensorMap* map, uint32_t 
       "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy), "r"(el)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_4d_el(const CUtensorMap* map, uint32_t bar, uint32_t dst, int x, int y, int z,
+                                               int w, uint64_t policy, uint32_t el) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %8, 0;\n\t"
+      "@q cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;\n\t}" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy), "r"(el)
+      : "memory");
+}
 // 2D TMA load into this CTA's shared memory whose completion is counted on an
 // mbarrier that may sit in the peer CTA of the pair (bar: shared::cluster
 // address).

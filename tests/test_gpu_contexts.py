@@ -145,3 +145,54 @@ def test_step_inputs_in_every_form(fop):
         s.close()
     for r, v in outs[1:]:
         assert torch.equal(r, outs[0][0]) and torch.equal(v, outs[0][1])
+
+
+def _raw_step(case, s, bad=None):
+    """One step from a fresh rollout: released actions and velocity.  Robot
+    `bad`'s actions and observation are not numbers."""
+    s.reset(case.seeds)
+    fop = case.fop.copy()
+    if bad is not None:
+        s.buffer[bad] = float("nan")
+        fop[bad] = np.nan
+    s.step(case.t, fop, case.delta, want_velocity=True)
+    torch.cuda.synchronize()
+    return s.released.cpu().numpy(), s.velocity.cpu().numpy()
+
+
+# head dims with one and four 64-wide blocks; slots + FOP tokens that end inside
+# a group of 16 keys; one robot group whose keys are split and one whose are not
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("heads,kv,hd", [(6, 2, 40), (4, 1, 64), (4, 1, 256)])
+@pytest.mark.parametrize("B,slots", [(2, 7), (48, 50)])
+def test_a_robots_bad_values_stay_its_own(dtype, heads, kv, hd, B, slots):
+    # keys of another robot have probability 0, but 0 x NaN is NaN
+    cfg = synth.ExpertConfig(layers=2, width=192, n_q_heads=heads, n_kv_heads=kv, head_dim=hd, mlp_dim=320,
+                             slots=slots, action_dim=5, prefix=45, fop_tokens=3, batch=B, dtype=dtype)
+    case = Case(cfg)
+    s = gpu_session(case)
+    clean, got = _raw_step(case, s), _raw_step(case, s, bad=1)
+    others = [b for b in range(B) if b != 1]
+    for c, g in zip(clean, got):
+        np.testing.assert_array_equal(g[others], c[others])
+    s.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("P", [1, 18, 32])
+def test_rows_of_an_earlier_longer_context_are_never_used(dtype, P):
+    cfg = _cfg(dtype)
+    case = Case(cfg, prefix_len=P)
+    s = gpu_session(case)
+    want = _raw_step(case, s)
+    s.close()
+    k, v = synth.make_context(cfg, 5000, cfg.batch, cfg.prefix)
+    v[..., P:, :] = np.nan
+    s = gpu_session(case)
+    for c in ((k, v, cfg.prefix), (k, v, cfg.prefix), (case.k, case.v, P)):   # the slots alternate
+        s.step(case.t, case.fop, case.delta)
+        s.set_context(*c)
+    got = _raw_step(case, s)
+    for c, g in zip(want, got):
+        np.testing.assert_array_equal(g, c)
+    s.close()
