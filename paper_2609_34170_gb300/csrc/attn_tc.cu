@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       // splits send to different ranks at any moment.  The TMEM loads are
       // warp-collective: every lane runs them, only rows that hold a slot send.
       const bool snd = r < vrows;
-      const bool has = n > 0 && l > 0.f;
+      const bool has = n > 0 && !(l <= 0.f);   // (a sum that is not a number goes out as it is)
       const float inv = has ? 1.f / l : 0.f;
       const int ngs = cps / 8;
       const uint32_t base = smem_u32(smem);

@@ -175,6 +175,7 @@ def test_a_robots_bad_values_stay_its_own(dtype, heads, kv, hd, B, slots):
     others = [b for b in range(B) if b != 1]
     for c, g in zip(clean, got):
         np.testing.assert_array_equal(g[others], c[others])
+        assert np.isnan(g[1]).all()   # and the robot itself is told
     s.close()
 
 
