@@ -1304,6 +1304,18 @@ struct TcClusters {
 };
 TcClusters g_max_clusters = {{0, 0, 0, 0}};
 
+// Whether a step's launch (xbf16) exchanges its splits' shares in bf16: where
+// tiles of 64 (M <= 64) or 128 tokens leave so many SMs idle that a split's slice
+// is at most 32 tokens, and that many splits have a k-tile each.  Elsewhere
+// shares stay fp32, whatever the plan: a share in bf16 costs a sum 2^-9 of its
+// size, and the estimated time is no reason to take that where it was not taken
+// (QKV of 2560 features from 129 tokens on, O and down of 1024 from 513 on).
+bool bf16_shares(const GemmArgs& g, int num_sms) {
+  const int s = g.M <= 64 ? 2 : 4;
+  const long tiles = (long)((g.N + TC_BM - 1) / TC_BM) * ((g.M + 127) / 128);
+  return g.xbf16 && tiles * s <= num_sms && (g.K + TC_BK - 1) / TC_BK >= s;
+}
+
 // How a GEMM is cut: token-tile width, K splits (a cluster), or SM pairs.
 struct TcPlan {
   bool pair = false;
@@ -1329,8 +1341,9 @@ struct TcPlan {
 // 64 robots, each projection's width and splits varied in turn: the rule is
 // 0 to 3.5 % of the step away from the best combination (batch 1 at it: 652
 // us, 685 with the chain's terms alone).
-TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t ws_bytes, bool pairs, int num_sms,
-                 const TcClusters& clusters) {
+TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int num_sms, const TcClusters& clusters) {
+  const int M = g.M, N = g.N, K = g.K;
+  const bool geglu = g.epi == EPI_GEGLU, xbf16 = g.xbf16 != 0, shares_bf16 = bf16_shares(g, num_sms);
   const int tiles_n = (N + TC_BM - 1) / TC_BM, num_kb = (K + TC_BK - 1) / TC_BK;
   TcPlan best;
   float cost = 3.4e38f;
@@ -1360,7 +1373,7 @@ TcPlan plan_gemm(int M, int N, int K, bool geglu, bool xbf16, bool dsmem, size_t
       const int w = (tiles + clusters.n[i] - 1) / clusters.n[i];
       consider(false, bn, sp,
                2.6f + epi / (float)sp + (float)w * (float)((num_kb + sp - 1) / sp) * step +
-                   (xbf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * 2.5f +
+                   (shares_bf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * 2.5f +
                    (xbf16 ? 0.7f * (float)std::max(0, tiles * sp - num_sms / 2) / (float)(num_sms / 2) : 0.f));
     }
   }
@@ -1446,8 +1459,7 @@ TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
   // range when that fits, so that no operand load waits for a freed stage
   if (splits > 1) l.stages = std::min(l.stages, std::max(2, TC_RING_SPLIT / stage_bytes));
   l.stages = std::max(2, std::min(l.stages, std::max(2, kb_per_item * items)));
-  // partials exchanged in bf16 where the caller allows it, else in fp32
-  const bool xbf = g.xbf16 != 0;
+  const bool xbf = bf16_shares(g, num_sms);   // partials exchanged in bf16, else in fp32
   const bool dsmem = splits > 1 && tma_out;
   const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
   // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
@@ -1557,8 +1569,7 @@ bool tc_gemm_supported(const GemmArgs& g) {
 cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms, cudaStream_t st) {
   if (!g_encode) return cudaErrorInitializationError;
   const bool out_bf = out_is_bf16(g), tma_out = out_aligned(g);
-  const TcPlan plan = plan_gemm(g.M, g.N, g.K, g.epi == EPI_GEGLU, g.xbf16 != 0, tma_out, ws.ws_bytes, tma_out, num_sms,
-                                g_max_clusters);
+  const TcPlan plan = plan_gemm(g, tma_out, ws.ws_bytes, tma_out, num_sms, g_max_clusters);
   if (plan.pair) return launch_gemm_pair(g, ws, num_sms, st, plan.bn);
   const TcLayout l = one_layout(g, plan, num_sms);
   if (!l.smem) return cudaErrorInvalidConfiguration;
@@ -1614,7 +1625,7 @@ extern "C" void ravel_debug_gemm_plan(int M, int N, int K, int epi, int out_bf16
   GemmArgs g{nullptr, K, nullptr, K, M, N, K, (Epi)epi, (void*)(uintptr_t)(aligned ? 16 : 4), (N + 7) / 8 * 8,
              out_bf16 ? DT_BF16 : DT_F32, nullptr};
   g.xbf16 = xbf16;
-  const TcPlan plan = plan_gemm(M, N, K, epi == EPI_GEGLU, xbf16 != 0, aligned != 0, ws_bytes, aligned != 0, num_sms,
+  const TcPlan plan = plan_gemm(g, aligned != 0, ws_bytes, aligned != 0, num_sms,
                                 TcClusters{{clusters[0], clusters[1], clusters[2], clusters[3]}});
   const TcLayout l = plan.pair ? pair_layout(g, plan.bn) : one_layout(g, plan, num_sms);
   const int v[7] = {plan.pair, plan.bn, plan.splits, l.reduce, 1 << l.lacc, (int)l.ncols, (int)l.smem};

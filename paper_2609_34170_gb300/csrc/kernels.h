@@ -91,9 +91,9 @@ struct GemmArgs {
   Dtype out_dt;
   const float* bias;            // [N] or null
   const int* skip = nullptr;    // optional device flag: nonzero at run time -> the launch computes nothing
-  // tcgen05 split-K inside a cluster: the splits' partials may travel between
-  // the SMs in bf16 (half the bytes of fp32; the sum itself stays fp32), which
-  // the step's projections take; 0 keeps them in fp32
+  // a projection of the step: where splits of the tcgen05 kernel are many, their
+  // partials may travel between the SMs in bf16 (half the bytes of fp32; the sum
+  // itself stays fp32); 0 keeps them in fp32
   int xbf16 = 0;
 };
 // EPI_GEGLU: fp32 with a float output where the row kernel takes it (few rows)

@@ -56,3 +56,25 @@ def test_waiting_launches_share_an_sm_only_if_tmem_holds_both(plan):
     for smem, cols in pairs:
         for s2, c2 in splits:
             assert smem + s2 > SM_SMEM or cols + c2 <= TMEM, (smem, cols, s2, c2)
+
+
+def test_shares_in_bf16_only_where_splits_are_many(plan):
+    """A share rounded to bf16 loses 2^-9 of its size: only a step's launch does
+    that, and only where 64- or 128-token tiles split into slices of at most 32
+    tokens on the SMs that there are."""
+    def check(m, n, k, epi, bf, xb, al):
+        p = plan(m, n, k, epi, bf, xb, al)
+        many = 2 if m <= 64 else 4
+        if not xb or (n + 127) // 128 * ((m + 127) // 128) * many > SMS or (k + 63) // 64 < many:
+            assert p["exchange"] != BF16, (m, n, k, epi, p)
+        assert (p["exchange"] == NONE) == (p["splits"] == 1), p
+        return p
+
+    for d in _draws(20000, 2):
+        check(*d[:6], int(d[6]))
+    for m in range(1, 1200):   # the projections of the two experts, all token counts
+        for n, k, epi, bf in ((2560, 1024, STORE, 1), (1024, 2048, ADD, 0), (1024, 4096, ADD, 0), (8192, 1024, GEGLU, 1),
+                              (1536, 1024, STORE, 1), (1024, 1024, ADD, 0)):
+            p = check(m, n, k, epi, bf, 1, 1)
+            if m == 50:   # one robot: the exchange that the step was tuned with
+                assert p["exchange"] == (BF16 if p["splits"] > 1 else NONE)
