@@ -77,9 +77,9 @@ struct TcParams {
   int M, N, K;
   int bn, stages, splits, num_kb;
   int reduce;           // how the splits of a tile are combined (splits > 1)
-  uint32_t ring_bytes;  // operand ring bytes (1024-aligned)
+  uint32_t ncols;       // TMEM columns of the launch
   uint32_t acc_cols;    // TMEM columns of one accumulator
-  int lacc;             // log2 of the accumulators an item's K range is cut into (short_sums)
+  int accs;             // accumulators that an item's K range is cut into, at most one per k-tile (sum_accumulators)
   int tiles_n, tiles_m, num_tiles;
   int epi;              // Epi
   int out_bf16;
@@ -202,10 +202,10 @@ __device__ __forceinline__ void reduce_slice_smem(const float4* b0, int S, float
 
 // v[k] += the item's other accumulators (in K order) at this thread's row,
 // columns taddr + k of the first one.
-__device__ __forceinline__ void add_accumulators(uint32_t taddr, uint32_t acc_cols, int lacc, uint32_t v[16]) {
+__device__ __forceinline__ void add_accumulators(uint32_t taddr, uint32_t acc_cols, int accs, uint32_t v[16]) {
   #pragma unroll 1
-  for (int j = 1; j < (1 << lacc); j += 3) {   // up to three loads in flight
-    const int n = (1 << lacc) - j;
+  for (int j = 1; j < accs; j += 3) {   // up to three loads in flight
+    const int n = accs - j;
     uint32_t x[3][16];
 #pragma unroll
     for (int u = 0; u < 3; ++u)
@@ -494,16 +494,16 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 
   // (through a shuffle, so that the compiler knows it is uniform in the warp)
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  // the K range of an item in 1 << lacc accumulators, summed in the epilogue
-  constexpr bool MULTI = RED != RED_DSMEM;
-  const int lacc = MULTI ? p.lacc : 0;
-  const uint32_t item_cols = p.acc_cols << lacc;
-  const uint32_t ncols = (p.splits > 1) ? item_cols : 2 * item_cols;
   int tn0 = 0, tm0 = 0, sp0 = 0;
   const bool has_work = work_item(p, 0, tn0, tm0, sp0);
   const int kb0_first = (int)((long)sp0 * p.num_kb / p.splits);
   const int kb1_first = (int)((long)(sp0 + 1) * p.num_kb / p.splits);
   const int npre = has_work ? min(S, kb1_first - kb0_first) : 0;
+  // the K range of an item in several accumulators, summed in the epilogue
+  // (every item of a launch without splits has the same range)
+  constexpr bool MULTI = RED != RED_DSMEM;
+  const int accs = MULTI ? min(p.accs, kb1_first - kb0_first) : 1;
+  const uint32_t item_cols = p.acc_cols * (uint32_t)p.accs;
   const int cpr = BN / p.splits;   // tokens of the slice each split rank owns (a multiple of 4)
   constexpr bool TMA_OUT = EK < EK_GENERIC;
   // partials exchanged through distributed shared memory: RED_DSMEM in bf16
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(ncols)
+                 "r"(p.ncols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -636,6 +636,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     el = elect_one();
     const uint32_t idesc = idesc_bf16(TC_BM, BN);
     const uint64_t ad0 = sw128_desc(a0), bd0 = sw128_desc(b0);
+    // accumulator j takes acc_q k-tiles, the first acc_r of them one more
+    const int cnt = kb1_first - kb0_first, acc_q = accs > 1 ? cnt / accs : cnt, acc_r = accs > 1 ? cnt - acc_q * accs : 0;
     int it = 0;
     bool ok = true;
     // fault injection: an arrival that never comes (rcv_bar is armed by
@@ -646,14 +648,13 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       if (ok) {
         tc_fence_after();
         uint64_t ad = ad0, bd = bd0;
-        const int cnt = kb1_first - kb0_first;
-        int j = 0, first = 0, next = cnt >> lacc;   // accumulator j takes k-tiles [first, next)
+        int j = 0, first = 0, next = acc_q + (acc_r > 0 ? 1 : 0);   // accumulator j takes k-tiles [first, next)
         uint32_t d = tmem;
         #pragma unroll 1
         for (int kb = 0; kb < cnt; ++kb, ad += TC_A_BYTES >> 4, bd += b_bytes >> 4) {
           if (MULTI && kb == next) {
             first = kb;
-            next = (cnt * (++j + 1)) >> lacc;
+            next += acc_q + (++j < acc_r ? 1 : 0);
             d += p.acc_cols;
           }
 #pragma unroll
@@ -674,12 +675,12 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       tc_fence_after();
       uint32_t d = tmem + (uint32_t)b * item_cols;
       const int kb0 = (int)((long)sp * p.num_kb / p.splits), kb1 = (int)((long)(sp + 1) * p.num_kb / p.splits);
-      int j = 0, first = kb0, next = kb0 + ((kb1 - kb0) >> lacc);   // accumulator j takes k-tiles [first, next)
+      int j = 0, first = kb0, next = kb0 + acc_q + (acc_r > 0 ? 1 : 0);   // as above
       #pragma unroll 1
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
         if (MULTI && kb == next) {
           first = kb;
-          next = kb0 + (((kb1 - kb0) * (++j + 1)) >> lacc);
+          next += acc_q + (++j < acc_r ? 1 : 0);
           d += p.acc_cols;
         }
         ok = mbar_wait_warp(&full[s], ph, p.wait_ns);
@@ -735,7 +736,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 16) {
           float v[16];
-          add_accumulators(trow + c0, p.acc_cols, lacc, nxt);
+          add_accumulators(trow + c0, p.acc_cols, accs, nxt);
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(nxt[k]);
           const bool more = c0 + 16 < BN;
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
           for (int qq = 0; qq < 4; ++qq) tmem_reg_fence16(raw + 16 * qq);
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq)
-            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, lacc, raw + 16 * qq);
+            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, accs, raw + 16 * qq);
 #pragma unroll
           for (int qq = 0; qq < 16; ++qq) {
             if (qq >= 4 * nq) break;
@@ -847,7 +848,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
           for (int qq = 0; qq < 4; ++qq) tmem_reg_fence16(raw + 16 * qq);
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq)
-            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, lacc, raw + 16 * qq);
+            if (qq < nq) add_accumulators(trow + c0 + 16 * qq, p.acc_cols, accs, raw + 16 * qq);
 #pragma unroll
           for (int qq = 0; qq < 16; ++qq)
             if (qq < 4 * nq)
@@ -945,7 +946,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   }
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.ncols) : "memory");
   }
 }
 
@@ -988,7 +989,6 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
-  const uint32_t ncols = 2 * p.acc_cols;
   // work item i of this pair: pair tile pair + i * npairs = (256-row block tn2, token tile tm)
   auto item = [&](int i, int& tn2, int& tm) -> bool {
     const int t = pair + i * npairs;
@@ -1061,7 +1061,7 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(ncols)
+                 "r"(p.ncols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
@@ -1210,7 +1210,7 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
   cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.ncols) : "memory");
   }
 }
 
@@ -1390,16 +1390,25 @@ TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int
 
 // The tensor cores truncate each fp32 accumulation, so a sum's error grows
 // with its length: about 1e-9 of the result per K element (N(0, 1) x N(0,
-// 0.02) operands: 2.7e-7 at K = 256, 1.7e-6 at 2048).  Where the result is
-// stored in fp32 and the splits' shares are exchanged in fp32 too, an item's
-// K range therefore goes through accumulators of at most 192 elements each
-// (as far as TMEM holds them), added in the epilogue; bf16 results round at
+// 0.02) operands: 1.2e-7 at K = 128, 9.9e-7 at 1024).  Where the result is
+// stored in fp32 and no share is rounded to bf16, an item's K range therefore
+// goes through an accumulator per k-tile (64 elements), as far as TMEM holds
+// them beside the accumulators of the tile before, added in the epilogue.  Past
+// 32 k-tiles four take a quarter each: M 800 x N 1024 x K 4096 errs by 7.9e-7 with
+// four, 3.7e-7 with eight, which add 1.6 to its 14.8 us.  A step's projections,
+// whose operands are bf16 activations, take two halves, what the widest split of
+// the same tokens would sum.  The two-SM kernel sums all of
+// K in one (its tiles fill TMEM), as it does for bf16 results, which round at
 // 2e-3.
-bool short_sums(const GemmArgs& g) { return !g.xbf16 && (g.epi == EPI_ADD_F32 || (g.epi != EPI_GEGLU && g.out_dt == DT_F32)); }
+int sum_accumulators(const GemmArgs& g, bool bf16_exchange, int kb_per_item, uint32_t acc_cols, bool two_items) {
+  if (bf16_exchange || g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16)) return 1;
+  const int fit = std::max(1, 512 / (int)acc_cols / (two_items ? 2 : 1));
+  return std::min({kb_per_item, fit, g.xbf16 ? 2 : kb_per_item > 32 ? 4 : fit});
+}
 
 // Sizes of a launch: the operand ring, TMEM and the shared memory around them.
 struct TcLayout {
-  int stages = 0, lacc = 0, reduce = RED_NONE, box_m = 0;
+  int stages = 0, accs = 1, reduce = RED_NONE, box_m = 0;
   bool oneshot = false;
   uint32_t acc_cols = 32, ncols = 0, box_bytes = 0, stg_off = 0, xch_off = 0, rcv_off = 0, bar_off = 0, set_bytes = 0;
   size_t ring = 0, smem = 0;   // smem 0: no such launch
@@ -1448,10 +1457,6 @@ TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
   while ((int)l.acc_cols < bn) l.acc_cols <<= 1;
   const int stage_bytes = TC_A_BYTES + bn * TC_BK * 2;
   const int kb_per_item = (num_kb + splits - 1) / splits;
-  // (more than one k-tile per accumulator, so every one is written)
-  if (short_sums(g))
-    while (kb_per_item > (3 << l.lacc) && (l.acc_cols << (l.lacc + (splits > 1 ? 1 : 2))) <= 512u) ++l.lacc;
-  l.ncols = l.acc_cols << (l.lacc + (splits > 1 ? 0 : 1));
   const int grid_ctas = splits > 1 ? tiles * splits : std::min(tiles, num_sms);
   const int items = splits > 1 ? 1 : (tiles + grid_ctas - 1) / grid_ctas;
   l.stages = std::min(8, TC_SMEM_BUDGET / stage_bytes);
@@ -1462,6 +1467,10 @@ TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
   const bool xbf = bf16_shares(g, num_sms);   // partials exchanged in bf16, else in fp32
   const bool dsmem = splits > 1 && tma_out;
   const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
+  // a CTA with several items works on two at a time
+  l.accs = sum_accumulators(g, dsmem && xbf, kb_per_item, l.acc_cols, items > 1);
+  l.ncols = 32;
+  while (l.ncols < l.acc_cols * (uint32_t)l.accs * (items > 1 ? 2u : 1u)) l.ncols <<= 1;
   // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
   // takes its weight and token k-tiles in one box each (K a multiple of 64)
   l.oneshot = splits > 1 && g.K % TC_BK == 0 && g.K / TC_BK <= 256 &&
@@ -1510,7 +1519,7 @@ cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_s
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, l.stages, 1, num_kb, RED_NONE, (uint32_t)l.ring, l.acc_cols, 0, tiles_n, tiles_m,
+  TcParams p{g.M, g.N, g.K, bn, l.stages, 1, num_kb, RED_NONE, l.ncols, l.acc_cols, 1, tiles_n, tiles_m,
              num_tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
              1, 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, 0, l.bar_off, kTcTimeoutNs, 0, g.skip};
   p.set_bytes = l.set_bytes;
@@ -1591,7 +1600,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, l.stages, splits, num_kb, l.reduce, (uint32_t)l.ring, l.acc_cols, l.lacc, tiles_n,
+  TcParams p{g.M, g.N, g.K, bn, l.stages, splits, num_kb, l.reduce, l.ncols, l.acc_cols, l.accs, tiles_n,
              tiles_m, tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
              tma_out ? 1 : 0, oneshot ? 1 : 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, l.rcv_off, l.bar_off,
              kTcTimeoutNs, 0, g.skip};
@@ -1628,6 +1637,6 @@ extern "C" void ravel_debug_gemm_plan(int M, int N, int K, int epi, int out_bf16
   const TcPlan plan = plan_gemm(g, aligned != 0, ws_bytes, aligned != 0, num_sms,
                                 TcClusters{{clusters[0], clusters[1], clusters[2], clusters[3]}});
   const TcLayout l = plan.pair ? pair_layout(g, plan.bn) : one_layout(g, plan, num_sms);
-  const int v[7] = {plan.pair, plan.bn, plan.splits, l.reduce, 1 << l.lacc, (int)l.ncols, (int)l.smem};
+  const int v[7] = {plan.pair, plan.bn, plan.splits, l.reduce, l.accs, (int)l.ncols, (int)l.smem};
   for (int i = 0; i < 7; ++i) out[i] = v[i];
 }

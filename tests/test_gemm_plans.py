@@ -11,8 +11,7 @@ NONE, L2, BF16, FP32 = 0, 1, 2, 3   # how splits exchange their partials
 SMS, SM_SMEM, TMEM = 152, 228 * 1024, 512
 
 
-@pytest.fixture(scope="module")
-def plan():
+def load_plan():
     from paper_2609_34170_gb300 import build, load
     build.build()
     fn = load().ravel_debug_gemm_plan
@@ -26,6 +25,11 @@ def plan():
         return dict(zip(("pair", "bn", "splits", "exchange", "accs", "cols", "smem"), out))
 
     return call
+
+
+@pytest.fixture(scope="module")
+def plan():
+    return load_plan()
 
 
 def _draws(n, seed):
@@ -78,3 +82,28 @@ def test_shares_in_bf16_only_where_splits_are_many(plan):
             p = check(m, n, k, epi, bf, 1, 1)
             if m == 50:   # one robot: the exchange that the step was tuned with
                 assert p["exchange"] == (BF16 if p["splits"] > 1 else NONE)
+
+
+def test_fp32_results_sum_one_k_tile_per_accumulator(plan):
+    """The tensor cores truncate, so a sum's error grows with its length: where
+    the result stays fp32, each k-tile has an accumulator of its own as far as
+    TMEM holds them (two tiles' worth where a CTA has several); past 32 k-tiles
+    four share them."""
+    for m, n, k, epi, bf, _, al in _draws(20000, 3):
+        for xb in (0, 1):
+            p = plan(m, n, k, epi, bf, xb, int(al))
+            per_item = -(-((k + 63) // 64) // p["splits"])
+            items = -(-((n + 127) // 128 * -(-m // p["bn"])) // SMS) if p["splits"] == 1 else 1
+            width = 32
+            while width < p["bn"]:
+                width *= 2
+            fit = max(1, TMEM // width // (2 if items > 1 else 1))
+            if bf or p["pair"] or p["exchange"] == BF16:
+                assert p["accs"] == 1, (m, n, k, p)
+            else:
+                assert p["accs"] == min(per_item, fit, 2 if xb else 4 if per_item > 32 else fit), (m, n, k, xb, p)
+    for m, n, k in ((1, 32, 128), (16, 128, 128), (50, 1024, 1024), (128, 1024, 1024), (240, 512, 560), (256, 100, 4096)):
+        p = plan(m, n, k, STORE, 0, 0)
+        assert -(-((k + 63) // 64) // (p["splits"] * p["accs"])) == 1, (m, n, k, p)
+    # a step's O and down without splits: two halves, as the widest split of 128 tokens summed
+    assert plan(800, 1024, 2048, ADD, 0, 1)["accs"] == plan(800, 1024, 4096, ADD, 0, 1)["accs"] == 2

@@ -81,6 +81,34 @@ def test_gemm_bf16_plans(handles, M, N, K):
                                atol=1e-2 * scale)
 
 
+# fp32 results against 64 bits, on each kind of plan: one K range per CTA, split
+# and on SM pairs, with as many accumulators as k-tiles, fewer, and 9 (no power
+# of two).  Bound: each of an accumulator's K / 16 truncating steps loses half an
+# ulp (2^-24) of the sum, and the fp32 additions around them a few (what one
+# accumulator gives at K = 4096, 4e-6, is above it wherever there are several).
+@pytest.mark.parametrize("M,N,K", [(16, 128, 128), (50, 1024, 1024), (50, 1024, 4096), (240, 512, 560), (800, 1024, 4096),
+                                   (1200, 1024, 4096), (1600, 1024, 4096), (3200, 1024, 1024), (431, 1025, 2048)])
+@pytest.mark.parametrize("alloc", [True, False])
+def test_gemm_fp32_results_are_short_sums(handles, M, N, K, alloc):
+    from paper_2609_34170_gb300 import ravel_gemm, ravel_gemm_noalloc
+    from tests.test_gemm_plans import SMS, load_plan
+    g = torch.Generator("cuda").manual_seed(M + N + K)
+    X = torch.randn((M, K), generator=g, device="cuda").bfloat16()
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.02).bfloat16()
+    out = torch.empty((M, N), device="cuda")
+    if alloc:
+        ravel_gemm(handles["bf16"], X, W, 0, out)
+    else:
+        ravel_gemm_noalloc(X, W, 0, out)
+    p = load_plan()(M, N, K, 0, 0, 0, int(N % 4 == 0), (24 if alloc else 8) << 20)
+    length = 64 * -(-((K + 63) // 64) // (p["splits"] * p["accs"]))
+    ref = X.double() @ W.double().T
+    err = float((out.double() - ref).norm() / ref.norm())
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bound = ((length if sms == SMS else K) / 16 + 4) * 2.0 ** -24
+    assert err < bound, (err, bound, p)
+
+
 @pytest.mark.parametrize("M,N,K", [(50, 256, 1024), (50, 8192, 1024), (66, 4096, 1024), (66, 8192, 1024),
                                    (300, 1024, 256), (3200, 2048, 1024), (3200, 8192, 1024)])
 @pytest.mark.parametrize("with_bias", [False, True])
