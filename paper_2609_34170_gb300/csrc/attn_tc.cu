@@ -829,7 +829,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_enc = nullptr;
-int g_attn_clusters[4] = {0, 0, 0, 0};   // resident clusters of 2, 4, 8, 16 CTAs (0: not to be had)
+struct AtClusters {
+  int n[4];   // resident clusters of 2, 4, 8, 16 CTAs (0: not to be had)
+};
+AtClusters g_attn_clusters = {{0, 0, 0, 0}};
 
 cudaError_t enc3(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1_bytes,
                  uint64_t s2_bytes, uint32_t b0, uint32_t b1, uint32_t b2) {
@@ -856,6 +859,94 @@ cudaError_t enc4(CUtensorMap* m, const void* base, int hd, int heads, int rows, 
                      load ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_NONE,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// How a launch is cut: query tiles, key splits and how they merge, ring depths.
+struct AtPlan {
+  int q_tiles = 0, TQ = 0, splits = 1;
+  bool smem_merge = false;   // partials normalised, in bf16, through shared memory; else fp32 through L2
+  int k_slots = 0, v_slots = 0;
+  size_t smem = 0;
+};
+
+// The most splits that 64-key pieces, two each, and SMs that half the grid leaves
+// idle allow.  It is what the precision goes by, not the plan of least time: with
+// one, keys are not split at all (a split rounds its share to bf16), and where its
+// head-dim slices are not whole 8-column groups the partials stay in fp32
+// through L2 however few the splits are (head dim 64 with 16 splits, 80, 96).
+int most_splits(const AttnTcArgs& a, int hdp, bool clusters_of_16) {
+  const int G = a.Hq / a.Hkv, pairs = a.B * a.Hkv;
+  const int pieces = (a.Pmax + 63) / 64 + (a.H + a.F + 63) / 64;
+  auto tiles = [&](int rows) { return (a.H + std::max(1, rows / G) - 1) / std::max(1, rows / G); };
+  int qt = tiles(AT_BM);
+  const int tq = (a.H + qt - 1) / qt, qt64 = tiles(64);
+  if (qt * pairs * 2 <= a.num_sms && std::max(1, 64 / G) < tq && qt64 * pairs * 8 <= a.num_sms / 2 && pieces >= 3)
+    qt = qt64;
+  const int ctas = qt * pairs;
+  if (ctas * 2 > a.num_sms) return 1;
+  const int cap = std::min({(pieces + 1) / 2, a.num_sms / ctas, clusters_of_16 ? 16 : 8});
+  int s = 1;
+  while (s * 2 <= cap && (hdp / (s * 2)) % 4 == 0 && (size_t)(s * 2) * ctas * AT_BM * (hdp + 2) * 4 <= a.ws_bytes) s *= 2;
+  return s;
+}
+
+AtPlan plan_attention(const AttnTcArgs& a, const AtClusters& clusters) {
+  AtPlan p;
+  const int G = a.Hq / a.Hkv, hdp = (a.hd + 15) / 16 * 16, nblk = (a.hd + 63) / 64;
+  const int most = most_splits(a, hdp, clusters.n[3] > 0);
+  // Query tiles of 128 rows, or of 64 where the keys are split (32: one robot's
+  // 104 CTAs, 612 us per step against 601), and the number of key splits (one
+  // cluster per query tile, a power of two whose head-dim slices are multiples
+  // of 4 columns): the least estimated time, fitted to whole steps of 1 to 16
+  // robots with every tile height and split count.  A CTA costs about 4 us and
+  // each chunk 1.65 at head dim 256 (the tensor pipe's turns of S and P V), 0.95
+  // at 64 (the softmax); the merge moves every split's rows x hd partial
+  // between the SMs; CTAs past half the SMs delay the next kernel's; a grid that
+  // does not fit at once (36 clusters of 4, 15 of 8, 7 of 16) takes another
+  // round.  16 robots, 16 slots, 2048 keys: 4 splits of 64 rows, 964 us; of 128
+  // rows 1005, 2 splits 1061, 8 (16 clusters in two rounds) 1118.
+  const int C = (a.Pmax + AT_BKV - 1) / AT_BKV + (a.H + a.F + AT_BKV - 1) / AT_BKV;
+  const float hd_rel = (float)hdp / 256.f;
+  const float t_chunk = std::max(0.95f, 1.65f * hd_rel);
+  float cost = 3.4e38f;
+  auto consider = [&](int rows, int splits, int resident) {
+    const int tq = std::max(1, rows / G);
+    const int qt = (a.H + tq - 1) / tq, ctas = qt * a.B * a.Hkv;
+    const int rounds = (ctas + resident - 1) / resident, half = a.num_sms / 2;
+    float t = (float)rounds * (4.f + t_chunk * (float)((C + splits - 1) / splits));
+    if (splits > 1) {
+      const float tile_rows = (float)((a.H + qt - 1) / qt * G);
+      t += (float)rounds * hd_rel * (2.4f + 1.5f * tile_rows / 128.f);
+      t += 0.6f * (float)std::max(0, ctas * splits - half) / (float)half;
+    }
+    if (t < cost) {
+      cost = t;
+      p.q_tiles = qt;
+      p.TQ = (a.H + qt - 1) / qt;
+      p.splits = splits;
+    }
+  };
+  consider(AT_BM, 1, a.num_sms);
+  for (int i = 0; i < 4 && most > 1; ++i) {
+    const int sp = 2 << i;
+    if (sp >= 2 * C || (hdp / sp) % 4 != 0 || hdp % sp != 0 || !clusters.n[i]) break;
+    for (int rows = AT_BM; rows >= 64; rows /= 2) {
+      const int tq = std::max(1, rows / G);
+      const size_t ctas = (size_t)((a.H + tq - 1) / tq) * a.B * a.Hkv;
+      if ((size_t)sp * ctas * AT_BM * (hdp + 2) * 4 <= a.ws_bytes) consider(rows, sp, clusters.n[i]);
+    }
+  }
+  p.smem_merge = p.splits > 1 && (hdp / most) % 8 == 0 && (hdp / p.splits) % 8 == 0;
+  // K units and V halves beside Q: at head dim 256 one chunk's four units and
+  // three halves; smaller heads have room for more.  (The receive area of a merge
+  // -- 128 rows of bf16, as large as Q, and (m, l) of up to 16 splits, 16 KB --
+  // always lies in Q and the K ring.)
+  const size_t v_bytes = (size_t)nblk * AT_VBLK;
+  const size_t fixed = 1024 + (size_t)nblk * AT_QBLK + 512 + 1024;   // alignment, Q, barriers, row maxima / sums
+  p.k_slots = nblk == 4 ? 4 : nblk == 1 ? 8 : 6;
+  p.v_slots = (int)std::min<size_t>(8, (AT_SMEM_MAX - fixed - p.k_slots * AT_KUNIT) / v_bytes);
+  p.smem = fixed + (size_t)p.k_slots * AT_KUNIT + (size_t)p.v_slots * v_bytes;
+  return p;
 }
 
 }  // namespace
@@ -885,7 +976,7 @@ cudaError_t init_attention_tc() {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    g_attn_clusters[i] = cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel, &cfg) == cudaSuccess && n > 0 ? n : 0;
+    g_attn_clusters.n[i] = cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel, &cfg) == cudaSuccess && n > 0 ? n : 0;
   }
   cudaGetLastError();
   return cudaSuccess;
@@ -910,71 +1001,17 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   p.out = (bf16*)a.out; p.ld_out = a.ld_out;
   p.err = a.err;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
-  // Query tiles of 128 rows, or of 64 where the keys are split (32: one robot's
-  // 104 CTAs, 612 us per step against 601), and the number of key splits (one
-  // cluster per query tile, a power of two whose head-dim slices are multiples
-  // of 4 columns): the least estimated time, fitted to whole steps of 1 to 16
-  // robots with every tile height and split count.  A CTA costs about 4 us and
-  // each chunk 1.65 at head dim 256 (the tensor pipe's turns of S and P V), 0.95
-  // at 64 (the softmax); the merge moves every split's rows x hd partial
-  // between the SMs; CTAs past half the SMs delay the next kernel's; a grid that
-  // does not fit at once (36 clusters of 4, 15 of 8, 7 of 16) takes another
-  // round.  16 robots, 16 slots, 2048 keys: 4 splits of 64 rows, 964 us; of 128
-  // rows 1005, 2 splits 1061, 8 (16 clusters in two rounds) 1118.
-  const int C = (a.Pmax + AT_BKV - 1) / AT_BKV + p.n_kv;
-  const float hd_rel = (float)p.hdp / 256.f;
-  const float t_chunk = std::max(0.95f, 1.65f * hd_rel);
-  float cost = 3.4e38f;
-  auto consider = [&](int rows, int splits, int resident) {
-    const int tq = std::max(1, rows / p.G);
-    const int qt = (a.H + tq - 1) / tq, ctas = qt * a.B * a.Hkv;
-    const int rounds = (ctas + resident - 1) / resident, half = a.num_sms / 2;
-    float t = (float)rounds * (4.f + t_chunk * (float)((C + splits - 1) / splits));
-    if (splits > 1) {
-      const float tile_rows = (float)((a.H + qt - 1) / qt * p.G);
-      t += (float)rounds * hd_rel * (2.4f + 1.5f * tile_rows / 128.f);
-      t += 0.6f * (float)std::max(0, ctas * splits - half) / (float)half;
-    }
-    if (t < cost) {
-      cost = t;
-      p.q_tiles = qt;
-      p.TQ = (a.H + qt - 1) / qt;
-      p.splits = splits;
-    }
-  };
-  consider(AT_BM, 1, a.num_sms);
-  for (int i = 0; i < 4; ++i) {
-    const int sp = 2 << i;
-    if (sp >= 2 * C || (p.hdp / sp) % 4 != 0 || p.hdp % sp != 0 || !g_attn_clusters[i]) break;
-    for (int rows = AT_BM; rows >= 64; rows /= 2) {
-      const int tq = std::max(1, rows / p.G);
-      const size_t ctas = (size_t)((a.H + tq - 1) / tq) * a.B * a.Hkv;
-      if ((size_t)sp * ctas * AT_BM * (p.hdp + 2) * 4 <= a.ws_bytes) consider(rows, sp, g_attn_clusters[i]);
-    }
-  }
-  const int splits = p.splits, nctas = p.q_tiles * a.B * a.Hkv;
+  const AtPlan plan = plan_attention(a, g_attn_clusters);
+  const int splits = plan.splits, nctas = plan.q_tiles * a.B * a.Hkv;
+  p.q_tiles = plan.q_tiles;
+  p.TQ = plan.TQ;
+  p.splits = splits;
+  p.xch = plan.smem_merge ? 2 : 0;
   p.ws_o = a.ws;
   p.ws_ml = a.ws + (size_t)splits * nctas * AT_BM * p.hdp;
-  // partials through shared memory: whole 8-column bf16 groups per rank
-  // slice, and the receive area (O groups + (m, l) of every split) within
-  // Q + the rings (checked below)
-  p.xch = splits > 1 && (p.hdp / splits) % 8 == 0 ? 1 : 0;
-  // K units and V halves beside Q: at head dim 256 one chunk's four units and
-  // three halves; smaller heads have room for more
-  const size_t v_bytes = (size_t)p.nblk * AT_VBLK;
-  const size_t fixed = 1024 + (size_t)p.nblk * AT_QBLK + 512 + 1024;   // alignment, Q, barriers, row maxima / sums
-  const int sk = p.nblk == 4 ? 4 : p.nblk == 1 ? 8 : 6;
-  const int sv = (int)std::min<size_t>(8, (AT_SMEM_MAX - fixed - sk * AT_KUNIT) / v_bytes);
-  const size_t rings = (size_t)sk * AT_KUNIT + (size_t)sv * v_bytes;
+  p.k_slots = plan.k_slots;
+  p.v_slots = plan.v_slots;
   if (a.ld_out % 8 != 0 || ((uintptr_t)a.out & 15u) != 0) return cudaErrorMisalignedAddress;
-  p.k_slots = sk;
-  p.v_slots = sv;
-  const size_t smem = fixed + rings;
-  if (p.xch && (size_t)AT_BM * p.hdp * 2 + (size_t)splits * AT_BM * 8 > (size_t)p.nblk * AT_QBLK + rings) p.xch = 0;
-  // the receive area within Q and the K ring (free once S is done): send
-  // without waiting for the other splits' PV
-  if (p.xch && (size_t)AT_BM * p.hdp * 2 + (size_t)splits * AT_BM * 8 <= (size_t)p.nblk * AT_QBLK + (size_t)sk * AT_KUNIT)
-    p.xch = 2;
 
   AtMaps m;
   const int hd = a.hd, rpr = a.H + a.F;
@@ -996,9 +1033,30 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   }
   if (e != cudaSuccess) return e;
   dim3 grid(p.q_tiles, a.B * a.Hkv, splits);
-  e = launch_kernel_cluster(attn_tc_kernel, grid, dim3(AT_THREADS), smem, st, dim3(1, 1, splits), m, p);
+  e = launch_kernel_cluster(attn_tc_kernel, grid, dim3(AT_THREADS), plan.smem, st, dim3(1, 1, splits), m, p);
   if (a.n_launched) ++*a.n_launched;
   return e;
 }
 
 }  // namespace ravel
+
+// What the tensor-core attention of these sizes is cut into, for tests: out =
+// {query tiles, slots per tile, key splits, 1 if they merge in bf16 through
+// shared memory, shared-memory bytes}.
+extern "C" void ravel_debug_attention_plan(int B, int H, int F, int Hq, int Hkv, int hd, int Pmax, size_t ws_bytes,
+                                           int num_sms, const int* clusters, int* out) {
+  using namespace ravel;
+  AttnTcArgs a{};
+  a.B = B;
+  a.H = H;
+  a.F = F;
+  a.Hq = Hq;
+  a.Hkv = Hkv;
+  a.hd = hd;
+  a.Pmax = Pmax;
+  a.ws_bytes = ws_bytes;
+  a.num_sms = num_sms;
+  const AtPlan p = plan_attention(a, AtClusters{{clusters[0], clusters[1], clusters[2], clusters[3]}});
+  const int v[5] = {p.q_tiles, p.TQ, p.splits, p.smem_merge, (int)p.smem};
+  for (int i = 0; i < 5; ++i) out[i] = v[i];
+}
