@@ -1396,14 +1396,17 @@ TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int
 // them beside the accumulators of the tile before, added in the epilogue.  Past
 // 32 k-tiles four take a quarter each: M 800 x N 1024 x K 4096 errs by 7.9e-7 with
 // four, 3.7e-7 with eight, which add 1.6 to its 14.8 us.  A step's projections,
-// whose operands are bf16 activations, take two halves, what the widest split of
-// the same tokens would sum.  The two-SM kernel sums all of
+// whose operands are bf16 activations, take two halves where 128-token tiles
+// leave half the SMs idle, as a split of those would (800 tokens: 0.3 us per
+// launch; 3200: 16 of a step's 2630, and no split to match).  The two-SM kernel sums all of
 // K in one (its tiles fill TMEM), as it does for bf16 results, which round at
 // 2e-3.
-int sum_accumulators(const GemmArgs& g, bool bf16_exchange, int kb_per_item, uint32_t acc_cols, bool two_items) {
+int sum_accumulators(const GemmArgs& g, bool bf16_exchange, int kb_per_item, uint32_t acc_cols, bool two_items,
+                     int num_sms) {
   if (bf16_exchange || g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16)) return 1;
   const int fit = std::max(1, 512 / (int)acc_cols / (two_items ? 2 : 1));
-  return std::min({kb_per_item, fit, g.xbf16 ? 2 : kb_per_item > 32 ? 4 : fit});
+  const long tiles = (long)((g.N + TC_BM - 1) / TC_BM) * ((g.M + 127) / 128);
+  return std::min({kb_per_item, fit, g.xbf16 ? (tiles * 2 <= num_sms ? 2 : 1) : kb_per_item > 32 ? 4 : fit});
 }
 
 // Sizes of a launch: the operand ring, TMEM and the shared memory around them.
@@ -1468,7 +1471,7 @@ TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
   const bool dsmem = splits > 1 && tma_out;
   const size_t rcv_bytes = dsmem ? (size_t)TC_BM * bn * (xbf ? 2 : 4) : 0;
   // a CTA with several items works on two at a time
-  l.accs = sum_accumulators(g, dsmem && xbf, kb_per_item, l.acc_cols, items > 1);
+  l.accs = sum_accumulators(g, dsmem && xbf, kb_per_item, l.acc_cols, items > 1, num_sms);
   l.ncols = 32;
   while (l.ncols < l.acc_cols * (uint32_t)l.accs * (items > 1 ? 2u : 1u)) l.ncols <<= 1;
   // one-shot: a cluster split whose whole K range fits a ring of up to 200 KB
