@@ -210,8 +210,8 @@ struct TailArgs {
 cudaError_t launch_tail(const TailArgs& a, cudaStream_t st);
 
 // The final adaRMSNorm, the velocity head and the tail in one launch (bf16
-// weights, A <= 32): rows_per_cta slots of one robot per CTA write v = the
-// head of their normed rows into a.vel; the robot's last CTA runs the tail.
+// weights, A <= 32): a CTA takes one slot of a robot, or eight consecutive ones
+// where rows are many, head and Euler step; the robot's last CTA shifts the slots.
 struct HeadArgs {
   const float* x; int D;                       // residual stream [B*H][D]
   const float* modv; int mod_ld; const float* mod_b; int off; const int* drow;   // as NormArgs
@@ -220,7 +220,7 @@ struct HeadArgs {
   int* cnt;                                    // [B] zero-initialised counters
   int t_stride = 0;                            // as NormArgs
 };
-cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, cudaStream_t st);
+cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, int num_sms, cudaStream_t st);
 
 // Synchronous (full-horizon) denoising: buffer += (t_now - t_next) * vel for
 // every slot (vel_out optional copy); times[i] = t[min(n0 + i, n_steps - 1)]; a fresh chunk

@@ -1177,26 +1177,32 @@ cudaError_t launch_tail(const TailArgs& a, cudaStream_t st) {
   return launch_kernel(tail_kernel, dim3(a.B), dim3(256), smem, st, 1, a);
 }
 
-// The step's last three stages in one launch (bf16 mode, A <= 32), one CTA per
-// slot: the final adaRMSNorm of the action row (Eq. 2's modulation, offset
-// off), the velocity head v = Y W_out^T + b_out on the bf16-rounded normed row
-// (as the separate norm + GEMM compute it) and the slot's Euler step; slot 0 is
-// released, the last slot's row takes the new noise, and the robot's CTA that
-// finishes last shifts the others forward.  (The CTAs count themselves on
-// cnt[b], reset by the last one, so it is zero between launches: the classic
-// last-block pattern, no CTA waits for another.)
+// The step's last three stages in one launch (bf16 mode, A <= 32), one CTA per R
+// consecutive slots of a robot: the final adaRMSNorm of an action row (Eq. 2's
+// modulation, offset off), the velocity head v = Y W_out^T + b_out on the
+// bf16-rounded normed row (as the separate norm + GEMM compute it) and the slot's
+// Euler step; slot 0 is released, the last slot's row takes the new noise, and the
+// robot's CTA that finishes last shifts the others forward.  (The CTAs count
+// themselves on cnt[b], reset by the last one, so it is zero between launches: the
+// classic last-block pattern, no CTA waits for another.)
 // Bound by the latency of its loads, so they go out together: W_out and the
 // bias, which no earlier kernel writes, before the wait for those kernels, the
 // rest right after it, without a branch on A between them (outputs past A
 // repeat the last row and are dropped).  (50 rows, A 32, D 1024: 6 us, 10 with
 // the loads behind the norm and the whole tail in the last CTA; 120 rows, A 20: 6,
-// and 17.)
+// and 17.)  R > 1, for more than two rows per SM: the CTA keeps its share of W_out
+// (64 KB in all) in registers for its rows, the next row's loads in flight behind
+// this one's sums.  (Whole steps of 3200 and 800 rows: 2642 and 1253 us with one
+// row per CTA, 2615 and 1249 with four, 2612 and 1248 with eight, 2633 and 1262
+// with eight in 128 registers, two CTAs per SM.)
+template <int R>
 __global__ void __launch_bounds__(256) head_tail_kernel(HeadArgs h, TailArgs a) {
   pdl_trigger();
-  __shared__ float red[8][33];     // per-warp sums: [warp][output] (+ the norm's row sum in [w][32])
+  __shared__ float red[2][8][33];   // per-warp sums: [warp][output] (+ the norm's row sum in [w][32])
   __shared__ int last;
   const int H = a.H, A = a.A, D = h.D, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, o = threadIdx.x;
-  const int b = blockIdx.x / H, j = blockIdx.x % H, f0 = 4 * threadIdx.x;
+  const int nc = (H + R - 1) / R;   // CTAs per robot
+  const int b = blockIdx.x / nc, j0 = blockIdx.x % nc * R, j1 = min(H, j0 + R), f0 = 4 * threadIdx.x;
   const float* mb = h.mod_b + h.off;
   uint2 wq[32];   // 4 bf16 of every W_out row
   float4 x, b0, b1, t0, t1, d0, d1;
@@ -1208,93 +1214,106 @@ __global__ void __launch_bounds__(256) head_tail_kernel(HeadArgs h, TailArgs a) 
   };
   if (f0 < D) weights(f0);
   pdl_wait();
-  const float* xr = h.x + (size_t)(b * H + j) * D;
-  const float* mt = h.modv + (size_t)(b * h.t_stride + j) * h.mod_ld + h.off;
   const float* md = h.modv + (size_t)(h.drow ? h.drow[b] : H + b) * h.mod_ld + h.off;
-  auto row = [&](int f) {
-    x = ld4(xr + f);
+  auto row = [&](int j, int f) {
+    const float* mt = h.modv + (size_t)(b * h.t_stride + j) * h.mod_ld + h.off;
+    x = ld4(h.x + (size_t)(b * H + j) * D + f);
     t0 = ld4(mt + f);
     t1 = ld4(mt + D + f);
+  };
+  auto offset = [&](int f) {
     d0 = ld4(md + f);
     d1 = ld4(md + D + f);
   };
-  if (f0 < D) row(f0);
-  // the slot's Euler step (threads o < A): its flow times, old value and, with an
+  if (f0 < D) {
+    row(j0, f0);
+    offset(f0);
+  }
+  // a slot's Euler step (threads o < A): its flow times, old value and, with an
   // absolute buffer and a relative expert, the state it also moves by
   float* buf = a.buffer + (size_t)b * H * A;
+  const float* tb = a.slot_times + (size_t)b * a.t_stride;   // robot b's schedule
   float dt = 0.f, old = 0.f, rm = 0.f, sv = 0.f, bias = 0.f;
-  if (o < A) {
-    const float* tb = a.slot_times + (size_t)b * a.t_stride;   // robot b's schedule
+  auto euler = [&](int j) {
     dt = __fsub_rn(tb[j], j ? tb[j - 1] : 0.f);
     old = buf[j * A + o];
+  };
+  if (o < A) {
+    euler(j0);
     bias = h.b[o];
     if (a.state) {
       rm = a.rel_mask[o];
       sv = a.state[(size_t)b * A + o];
     }
   }
-  // sum of squares of the row (4 features per thread per pass)
-  float ss = 0.f;
-  if (f0 < D) ss = x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
-  for (int f = f0 + 4 * blockDim.x; f < D; f += 4 * blockDim.x) {
-    const float4 xv = ld4(xr + f);
-    ss += xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w;
-  }
-  ss = warp_sum(ss);
-  if (lane == 0) red[warp][32] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int w = 0; w < 8; ++w) tot += red[w][32];
-  const float inv = rsqrtf(tot / (float)D + 1e-6f);
-  // this thread's partial products for all 32 outputs
-  float acc[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-  for (int f = f0; f < D; f += 4 * blockDim.x) {
-    if (f != f0) {
-      weights(f);
-      row(f);
-    }
-    const float xs[4] = {x.x, x.y, x.z, x.w};
-    const float sc[4] = {t0.x + d0.x + b0.x, t0.y + d0.y + b0.y, t0.z + d0.z + b0.z, t0.w + d0.w + b0.w};
-    const float sh[4] = {t1.x + d1.x + b1.x, t1.y + d1.y + b1.y, t1.z + d1.z + b1.z, t1.w + d1.w + b1.w};
-    float y[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) y[e] = __bfloat162float(__float2bfloat16_rn(xs[e] * inv * (1.f + sc[e]) + sh[e]));
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      acc[i] = fmaf(y[0], __uint_as_float(wq[i].x << 16), acc[i]);
-      acc[i] = fmaf(y[1], __uint_as_float(wq[i].x & 0xFFFF0000u), acc[i]);
-      acc[i] = fmaf(y[2], __uint_as_float(wq[i].y << 16), acc[i]);
-      acc[i] = fmaf(y[3], __uint_as_float(wq[i].y & 0xFFFF0000u), acc[i]);
-    }
-  }
-  // warp: lane o ends with the warp's sum of output o (each step keeps half
-  // of the outputs and adds the partner's half)
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < off; ++i) {
-      const float send = up ? acc[i] : acc[i + off];
-      const float keep = up ? acc[i + off] : acc[i];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-  red[warp][lane] = acc[0];
-  __syncthreads();
-  if (o < A) {
-    float v = bias;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) v += red[w][o];
-    if (a.vel_out) a.vel_out[((size_t)b * H + j) * A + o] = v;
-    const float next = fmaf(dt, a.state ? fmaf(rm, sv, v) : v, old);
-    if (j == 0) a.released[(size_t)b * A + o] = next;
-    else h.v[((size_t)b * H + j) * A + o] = next;
-  }
   const uint64_t n = a.counters[b];
-  if (j == H - 1) {   // (its old value has been read)
+  for (int j = j0; j < j1; ++j) {
+    float(*rd)[33] = red[(j - j0) & 1];
+    // sum of squares of the row (4 features per thread per pass)
+    float ss = 0.f;
+    if (f0 < D) ss = x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+    for (int f = f0 + 4 * blockDim.x; f < D; f += 4 * blockDim.x) {
+      const float4 xv = ld4(h.x + (size_t)(b * H + j) * D + f);
+      ss += xv.x * xv.x + xv.y * xv.y + xv.z * xv.z + xv.w * xv.w;
+    }
+    ss = warp_sum(ss);
+    if (lane == 0) rd[warp][32] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) tot += rd[w][32];
+    const float inv = rsqrtf(tot / (float)D + 1e-6f);
+    // this thread's partial products for all 32 outputs
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+    for (int f = f0; f < D; f += 4 * blockDim.x) {
+      if (f != f0) {
+        weights(f);
+        row(j, f);
+        offset(f);
+      }
+      const float xs[4] = {x.x, x.y, x.z, x.w};
+      const float sc[4] = {t0.x + d0.x + b0.x, t0.y + d0.y + b0.y, t0.z + d0.z + b0.z, t0.w + d0.w + b0.w};
+      const float sh[4] = {t1.x + d1.x + b1.x, t1.y + d1.y + b1.y, t1.z + d1.z + b1.z, t1.w + d1.w + b1.w};
+      float y[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) y[e] = __bfloat162float(__float2bfloat16_rn(xs[e] * inv * (1.f + sc[e]) + sh[e]));
+      if (R > 1 && f + 4 * blockDim.x >= D && j + 1 < j1) row(j + 1, f0);   // (D <= 1024: one pass)
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        acc[i] = fmaf(y[0], __uint_as_float(wq[i].x << 16), acc[i]);
+        acc[i] = fmaf(y[1], __uint_as_float(wq[i].x & 0xFFFF0000u), acc[i]);
+        acc[i] = fmaf(y[2], __uint_as_float(wq[i].y << 16), acc[i]);
+        acc[i] = fmaf(y[3], __uint_as_float(wq[i].y & 0xFFFF0000u), acc[i]);
+      }
+    }
+    // warp: lane o ends with the warp's sum of output o (each step keeps half
+    // of the outputs and adds the partner's half)
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int i = 0; i < off; ++i) {
+        const float send = up ? acc[i] : acc[i + off];
+        const float keep = up ? acc[i + off] : acc[i];
+        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      }
+    }
+    rd[warp][lane] = acc[0];
+    __syncthreads();
+    if (o < A) {
+      float v = bias;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v += rd[w][o];
+      if (a.vel_out) a.vel_out[((size_t)b * H + j) * A + o] = v;
+      const float next = fmaf(dt, a.state ? fmaf(rm, sv, v) : v, old);
+      if (j == 0) a.released[(size_t)b * A + o] = next;
+      else h.v[((size_t)b * H + j) * A + o] = next;
+      if (R > 1 && j + 1 < j1) euler(j + 1);
+    }
+  }
+  if (j1 == H) {   // (the last slot's old value has been read)
     const int g = (int)blockDim.x - 1 - (int)threadIdx.x;
     if (4 * g < A) {
       float z[4];
@@ -1309,7 +1328,7 @@ __global__ void __launch_bounds__(256) head_tail_kernel(HeadArgs h, TailArgs a) 
   __syncthreads();
   if (threadIdx.x == 0) {
     const int done = atomicAdd(h.cnt + b, 1);
-    last = done == H - 1;
+    last = done == nc - 1;
     if (last) h.cnt[b] = 0;
   }
   __syncthreads();
@@ -1328,10 +1347,13 @@ __global__ void __launch_bounds__(256) head_tail_kernel(HeadArgs h, TailArgs a) 
   if (threadIdx.x == 0) a.counters[b] = n + 1;
 }
 
-cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, cudaStream_t st) {
+cudaError_t launch_head_tail(const HeadArgs& h, const TailArgs& a, int num_sms, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
   if (a.A > 32 || h.D % 4) return cudaErrorNotSupported;
-  return launch_kernel(head_tail_kernel, dim3(a.B * a.H), dim3(256), 0, st, 1, h, a);
+  // (rows of up to 1024 features: one pass, whose weights stay in registers)
+  if (a.B * a.H > 2 * num_sms && h.D <= 1024)
+    return launch_kernel(head_tail_kernel<8>, dim3(a.B * ((a.H + 7) / 8)), dim3(256), 0, st, 1, h, a);
+  return launch_kernel(head_tail_kernel<1>, dim3(a.B * a.H), dim3(256), 0, st, 1, h, a);
 }
 
 // Full-horizon denoising (the synchronous baseline): every slot takes the

@@ -432,17 +432,18 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
     RUN(KK_GEMM_DOWN, gemm(p.Hm, Fm, (const char*)p.w_down + (size_t)l * D * Fm * es, BH, D, Fm, EPI_ADD_F32, p.x, D,
                            DT_F32, nullptr, nullptr, 1));
   }
-  // final norm, velocity head and tail: in one launch while its rows leave SMs
-  // idle; it reads W_out (64 KB) for every row, so more rows take the norm, the
-  // tensor-core GEMM and the tail (3200 rows: step 2662 -> 2632 us, 800 rows:
-  // 1295 -> 1285; at 200 rows the two are equal)
-  if (!dn && dt == DT_BF16 && A <= 32 && D % 4 == 0 && BH <= p.num_sms) {
+  // final norm, velocity head and tail in one launch, in fp32 FMAs whatever the
+  // number of rows.  (Past the SMs the norm, the tensor-core GEMM and the tail on
+  // their own are faster, 2589 instead of 2612 us per step at 3200 rows, but its
+  // truncated sums are 1.0e-7 from 64 bits even at 64 elements each, the FMAs'
+  // 7.3e-8.)
+  if (!dn && dt == DT_BF16 && A <= 32 && D % 4 == 0) {
     TailArgs ta{io.buffer, p.V, io.slot_times, io.released, io.velocity, p.seeds, p.counters, B, H, A, io.state,
                 p.rel_mask};
     ta.t_stride = t_stride;
     HeadArgs hd{p.x, D, p.modv, p.mod_dim, p.mod_b, 4 * L * D, p.cond_drow, p.out_w, p.out_b, p.V, p.head_cnt};
     hd.t_stride = t_stride;
-    RUN(KK_HEAD_TAIL, launch_head_tail(hd, ta, st));
+    RUN(KK_HEAD_TAIL, launch_head_tail(hd, ta, p.num_sms, st));
     if (n_kernels) *n_kernels = nk;
     return e;
   }

@@ -220,3 +220,23 @@ def test_head_tail_edges(batch, slots, width, actions):
     for _ in range(2):   # (the second step starts from the first one's buffer and counters)
         check_step(case, s, label=f"{batch * slots} rows")
     s.close()
+
+
+# The same for more rows than two per SM, where a CTA takes eight slots of a
+# robot: whole and ragged groups of slots, fewer than eight, one and several
+# passes over the row (one slot per CTA); the head stays the same launch.
+@pytest.mark.parametrize("slots", [5, 8, 17, 50])
+@pytest.mark.parametrize("width,actions", [(64, 1), (1024, 20), (1032, 32)])
+def test_head_tail_many_rows(slots, width, actions):
+    batch = 2 * torch.cuda.get_device_properties(0).multi_processor_count // slots + 1
+    cfg = synth.ExpertConfig(layers=1, width=width, n_q_heads=2, n_kv_heads=1, head_dim=64, mlp_dim=64, slots=slots,
+                             action_dim=actions, prefix=9, fop_tokens=2, batch=batch, dtype="bf16")
+    case = Case(cfg)
+    s = gpu_session(case)
+    for _ in range(2):
+        check_step(case, s, robots=[0, batch // 2, batch - 1], label=f"{batch * slots} rows")
+    few = gpu_session(Case(cfg, batch=1))
+    check_step(Case(cfg, batch=1), few)
+    assert s.kernel_count() == few.kernel_count()
+    s.close()
+    few.close()
