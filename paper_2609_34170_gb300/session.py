@@ -32,23 +32,30 @@ class RollingSession:
 
     def _put(self, *inputs):
         """The persistent step inputs take their new values (pairs of input and
-        value), on the current stream: all plain CUDA tensors of the input's
-        type, shape and device in one launch, anything else (arrays, other
-        types, broadcasts) one by one.  (A batch-1 step call took the host 56 us
-        with one tensor copy per input, 26 so, and the step's stream 595 us
-        instead of 588; a tiny fp32 step 130 instead of 125.)"""
+        value), on the current stream: plain CUDA tensors of the inputs' types,
+        shapes and device that share no memory with another input in one
+        launch, anything else (arrays, other types, broadcasts, views of the
+        inputs) one by one in order.  (A batch-1 step call took the host 56 us
+        with one tensor copy per input, 26 in one launch, and the step's stream
+        595 us instead of 588; a tiny fp32 step 130 instead of 125.)"""
         whole = []
         for dst, value in inputs:
-            if (type(value) is self.torch.Tensor and value.dtype == dst.dtype and value.device == dst.device
+            if not (type(value) is self.torch.Tensor and value.dtype == dst.dtype and value.device == dst.device
                     and value.shape == dst.shape and value.is_contiguous() and not value.is_neg()):
+                break
+            if dst.numel():
                 whole.append((dst.data_ptr(), value.data_ptr(), dst.numel() * dst.element_size()))
-            else:
-                dst.copy_(self.to_dev(value, dst.dtype))
-        if whole:
-            n = len(whole)
-            dst, src, size = zip(*whole)
-            B.ravel_copy_inputs(self.handle, n, (ctypes.c_void_p * n)(*dst), (ctypes.c_void_p * n)(*src),
-                                (ctypes.c_size_t * n)(*size), self.torch.cuda.current_stream(self.device))
+        else:
+            if all(src and not any(src < d + n and d < src + size and not d == own == src for d, _, n in whole)
+                   for own, src, size in whole):
+                if whole:
+                    n = len(whole)
+                    dst, src, size = zip(*whole)
+                    B.ravel_copy_inputs(self.handle, n, (ctypes.c_void_p * n)(*dst), (ctypes.c_void_p * n)(*src),
+                                        (ctypes.c_size_t * n)(*size), self.torch.cuda.current_stream(self.device))
+                return
+        for dst, value in inputs:
+            dst.copy_(self.to_dev(value, dst.dtype))
 
     def _times(self, slot_times):
         """Slot times of any shape, flat: the input that they fill."""
@@ -92,9 +99,10 @@ class RollingSession:
         targets and the expert works relative to that state (see
         ravel_roll_step_rel and set_relative_dims)."""
         t = self.torch
-        inputs = [self._times(slot_times), (self.delta, delta)]
+        inputs = [self._times(slot_times)]
         if self.cfg.fop_tokens:
             inputs.append((self.obs, obs))
+        inputs.append((self.delta, delta))
         if state is not None:
             if not hasattr(self, "state"):
                 self.state = t.zeros((self.batch, self.cfg.action_dim), device=self.device, dtype=t.float32)
@@ -119,7 +127,7 @@ class RollingSession:
         t = self.torch
         if not hasattr(self, "chunk"):
             self.chunk = t.empty_like(self.buffer)
-        self._put((self.delta, delta), *([(self.obs, obs)] if self.cfg.fop_tokens else []))
+        self._put(*([(self.obs, obs)] if self.cfg.fop_tokens else []), (self.delta, delta))
         B.ravel_denoise_chunk(self.handle, self.chunk, n_steps, self.obs if self.cfg.fop_tokens else None, self.delta,
                               self.velocity if want_velocity else None, stream)
         return self.chunk
