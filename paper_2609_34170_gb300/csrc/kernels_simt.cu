@@ -271,11 +271,16 @@ __global__ void __launch_bounds__(RG_WARPS * 32) gemm_rows_kernel(const float* _
 // 8.2.
 constexpr int RG_KS = 4, RG_SPLIT_COLS = 1024;
 
-// The row kernel re-reads W for every 8 rows (from L2): up to 256 rows, where
-// the tile kernel would leave SMs idle.
+// The row kernel re-reads W for every 8 rows (from L2), the tile kernel pads rows
+// to 64 and takes K x 72 ns however few its tiles are: rows while the products
+// are few or the tile kernel's rows mostly padding.  Measured per call, rows and
+// tiles: M 64 x N 2560 x K 1024 29 and 76 us, 192 x 2560 x 1024 72 and 73, 96 x 4096
+// x 4096 352 and 450, 128 x 4096 x 4096 436 and 430, 256 x 4096 x 4096 832 and 468,
+// 128 x 8192 x 1024 125 and 106; at K 256, 128 x 2048 17 and 21, 256 x 2048 29 and
+// 21; 24 x 75776 x 1024 306 and 394, 32 x 75776 x 1024 406 and 394.
 bool rows_gemm_supported(const GemmArgs& g) {
-  return g.M <= 256 && g.K % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
-         (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
+  return (g.M <= 24 || (g.M <= 256 && (int64_t)g.M * g.N < (g.K < 512 ? 5 : 8) << 16)) && g.K % 4 == 0 &&
+         g.lda % 4 == 0 && g.ldw % 4 == 0 && (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
 }
 
 template <int EPI, typename TO>
@@ -1532,3 +1537,9 @@ cudaError_t launch_ctx_scatter(const void* src, int src_n, int i0, void* dst0, v
 }
 
 }  // namespace ravel
+
+// 1 if an fp32 GEMM of these sizes (16-byte aligned rows) takes the row kernel, for tests.
+extern "C" int ravel_debug_rows_gemm(int M, int N, int K) {
+  using namespace ravel;
+  return rows_gemm_supported(GemmArgs{nullptr, K, nullptr, K, M, N, K, EPI_STORE, nullptr, N, DT_F32, nullptr}) ? 1 : 0;
+}

@@ -108,3 +108,17 @@ def test_fp32_results_sum_one_k_tile_per_accumulator(plan):
         assert -(-((k + 63) // 64) // (p["splits"] * p["accs"])) == 1, (m, n, k, p)
     # a step's O and down without splits: two halves, as the widest split of 128 tokens summed
     assert plan(800, 1024, 2048, ADD, 0, 1)["accs"] == plan(800, 1024, 4096, ADD, 0, 1)["accs"] == 2
+
+
+def test_fp32_rows_only_where_they_were_measured_faster():
+    """Each side of the line between the fp32 row and tile kernels, at sizes
+    whose times its comment gives."""
+    from paper_2609_34170_gb300 import build, load
+    build.build()
+    rows = load().ravel_debug_rows_gemm
+    for m, n, k in ((1, 75776, 4096), (24, 75776, 1024), (64, 2560, 1024), (192, 2560, 1024), (256, 1024, 4096),
+                    (96, 4096, 4096), (128, 2048, 256)):
+        assert rows(m, n, k) == 1, (m, n, k)
+    for m, n, k in ((25, 75776, 1024), (128, 4096, 4096), (256, 4096, 4096), (128, 8192, 1024), (256, 2048, 256),
+                    (257, 33, 516), (8, 100, 250)):
+        assert rows(m, n, k) == 0, (m, n, k)

@@ -162,9 +162,11 @@ def test_gemm_two_sm_is_deterministic(handles):
 # the row kernel: one ragged 8-row chunk, exact chunks, its last M and the
 # first of the tile kernel; odd N, K that ends inside a lane's stride, and a K
 # that is not whole float4s (the tile kernel); K split over warps with a ragged
-# last step and row chunk, and either side of where that ends
+# last step and row chunk, and either side of where that ends; either side of the
+# lines on the products and on the rows
 @pytest.mark.parametrize("M,N,K", [(1, 1, 4), (8, 16, 128), (10, 1027, 1024), (256, 33, 516), (257, 33, 516), (7, 40, 250),
-                                   (5, 41, 516), (17, 300, 1024), (1, 1024, 512), (1, 1025, 512), (8, 1024, 508)])
+                                   (5, 41, 516), (17, 300, 1024), (1, 1024, 512), (1, 1025, 512), (8, 1024, 508),
+                                   (24, 30000, 64), (25, 30000, 64), (64, 8191, 512), (64, 8192, 512)])
 @pytest.mark.parametrize("epi", [0, 1, 2])
 def test_gemm_fp32_rows(handles, M, N, K, epi):
     from paper_2609_34170_gb300 import ravel_gemm
