@@ -274,13 +274,17 @@ constexpr int RG_KS = 4, RG_SPLIT_COLS = 1024;
 // The row kernel re-reads W for every 8 rows (from L2), the tile kernel pads rows
 // to 64 and takes K x 72 ns however few its tiles are: rows while the products
 // are few or the tile kernel's rows mostly padding.  Measured per call, rows and
-// tiles: M 64 x N 2560 x K 1024 29 and 76 us, 192 x 2560 x 1024 72 and 73, 96 x 4096
-// x 4096 352 and 450, 128 x 4096 x 4096 436 and 430, 256 x 4096 x 4096 832 and 468,
-// 128 x 8192 x 1024 125 and 106; at K 256, 128 x 2048 17 and 21, 256 x 2048 29 and
-// 21; 24 x 75776 x 1024 306 and 394, 32 x 75776 x 1024 406 and 394.
+// tiles: M 64 x N 2560 x K 1024 29 and 76 us, 192 x 2560 x 1024 72 and 77, 192 x 3000
+// x 1024 84 and 77, 128 x 8192 x 1024 125 and 106; 96 x 4096 x 4096 352 and 450, 192 x 4096 x 4096 605 and 457; at K
+// 256, 192 x 2048 23 and 26, 256 x 2048 29 and 26; 24 x 75776 x 1024 306 and 394, 32 x
+// 75776 x 1024 406 and 394.  GeGLU saves a launch and its fp32 round trip on top:
+// steps of four 1024-wide layers, 100 rows 1239 and 1493 us, 200 rows 2169 and 1951;
+// of two 256-wide ones, 250 rows 252 and 277.
 bool rows_gemm_supported(const GemmArgs& g) {
-  return (g.M <= 24 || (g.M <= 256 && (int64_t)g.M * g.N < (g.K < 512 ? 5 : 8) << 16)) && g.K % 4 == 0 &&
-         g.lda % 4 == 0 && g.ldw % 4 == 0 && (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
+  const bool glu = g.epi == EPI_GEGLU;
+  const int limit = g.K < 512 ? (glu ? 18 : 13) : glu && g.K < 2048 ? 26 : 16;   // in 2^15 products
+  return (g.M <= 24 || (g.M <= 256 && (int64_t)g.M * g.N < limit << 15)) && g.K % 4 == 0 && g.lda % 4 == 0 &&
+         g.ldw % 4 == 0 && (((uintptr_t)g.A | (uintptr_t)g.W) & 15u) == 0;
 }
 
 template <int EPI, typename TO>
@@ -1539,7 +1543,7 @@ cudaError_t launch_ctx_scatter(const void* src, int src_n, int i0, void* dst0, v
 }  // namespace ravel
 
 // 1 if an fp32 GEMM of these sizes (16-byte aligned rows) takes the row kernel, for tests.
-extern "C" int ravel_debug_rows_gemm(int M, int N, int K) {
+extern "C" int ravel_debug_rows_gemm(int M, int N, int K, int epi) {
   using namespace ravel;
-  return rows_gemm_supported(GemmArgs{nullptr, K, nullptr, K, M, N, K, EPI_STORE, nullptr, N, DT_F32, nullptr}) ? 1 : 0;
+  return rows_gemm_supported(GemmArgs{nullptr, K, nullptr, K, M, N, K, (Epi)epi, nullptr, N, DT_F32, nullptr}) ? 1 : 0;
 }

@@ -117,8 +117,10 @@ def test_fp32_rows_only_where_they_were_measured_faster():
     build.build()
     rows = load().ravel_debug_rows_gemm
     for m, n, k in ((1, 75776, 4096), (24, 75776, 1024), (64, 2560, 1024), (192, 2560, 1024), (256, 1024, 4096),
-                    (96, 4096, 4096), (128, 2048, 256)):
-        assert rows(m, n, k) == 1, (m, n, k)
-    for m, n, k in ((25, 75776, 1024), (128, 4096, 4096), (256, 4096, 4096), (128, 8192, 1024), (256, 2048, 256),
+                    (96, 4096, 4096), (192, 2048, 256)):
+        assert rows(m, n, k, STORE) == rows(m, n, k, GEGLU) == 1, (m, n, k)
+    for m, n, k in ((25, 75776, 1024), (128, 4096, 4096), (192, 4096, 4096), (128, 8192, 1024), (200, 8192, 1024),
                     (257, 33, 516), (8, 100, 250)):
-        assert rows(m, n, k) == 0, (m, n, k)
+        assert rows(m, n, k, STORE) == rows(m, n, k, GEGLU) == 0, (m, n, k)
+    for m, n, k in ((100, 8192, 1024), (192, 3000, 1024), (250, 2048, 256)):   # GeGLU saves a launch
+        assert (rows(m, n, k, STORE), rows(m, n, k, GEGLU)) == (0, 1), (m, n, k)
