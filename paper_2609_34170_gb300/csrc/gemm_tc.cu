@@ -1316,6 +1316,9 @@ bool bf16_shares(const GemmArgs& g, int num_sms) {
   return g.xbf16 && tiles * s <= num_sms && (g.K + TC_BK - 1) / TC_BK >= s;
 }
 
+// Tokens per chunk of a split's slice of cpr tokens (a multiple of 4).
+int split_chunk(int cpr) { return cpr % 16 == 0 ? 16 : cpr % 8 == 0 ? 8 : 4; }
+
 // How a GEMM is cut: token-tile width, K splits (a cluster), or SM pairs.
 struct TcPlan {
   bool pair = false;
@@ -1366,14 +1369,19 @@ TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int
     for (int i = 0; i < 4; ++i) {
       // the splits of a tile form one cluster; each sums a slice of whole
       // 4-token groups, of at most 32 tokens through shared memory, and
-      // through L2 the partials have to fit the workspace
+      // through L2 the partials have to fit the workspace; there the slice goes
+      // out in chunks of 16, 8 or 4 tokens, each a round trip (two with the
+      // residual stream's reads: M 200 x N 2049 x K 6216 in seven chunks of 4
+      // tokens took 48 us, in two of 16 29, of 64-token tiles in two waves 41)
       const int sp = 2 << i;
       if (sp > num_kb || bn % (4 * sp) || !clusters.n[i] || (long)tiles * sp > 2L * num_sms) break;
       if (dsmem ? bn / sp > 32 : (size_t)sp * tiles * bn * TC_BM * 4 > ws_bytes) continue;
+      const int chunks = bn / sp / split_chunk(bn / sp);
       const int w = (tiles + clusters.n[i] - 1) / clusters.n[i];
       consider(false, bn, sp,
                2.6f + epi / (float)sp + (float)w * (float)((num_kb + sp - 1) / sp) * step +
-                   (shares_bf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * 2.5f +
+                   (shares_bf16 ? 0.47f : 2.14f) * (float)bn / 64.f + (float)(w - 1) * (dsmem ? 2.5f : 10.f) +
+                   (dsmem ? 0.f : (float)(chunks - 1) * (g.epi == EPI_ADD_F32 ? 4.f : 0.8f)) +
                    (xbf16 ? 0.7f * (float)std::max(0, tiles * sp - num_sms / 2) / (float)(num_sms / 2) : 0.f));
     }
   }
@@ -1388,13 +1396,21 @@ TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int
   return best;
 }
 
+bool out_is_bf16(const GemmArgs& g) { return g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16); }
+
+// outputs through TMA boxes when the output rows are 16-byte aligned
+bool out_aligned(const GemmArgs& g) {
+  return ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * (out_is_bf16(g) ? 2 : 4)) % 16 == 0;
+}
+
 // The tensor cores truncate each fp32 accumulation, so a sum's error grows
 // with its length: about 1e-9 of the result per K element (N(0, 1) x N(0,
 // 0.02) operands: 1.2e-7 at K = 128, 9.9e-7 at 1024).  Where the result is
 // stored in fp32 and no share is rounded to bf16, an item's K range therefore
 // goes through an accumulator per k-tile (64 elements), as far as TMEM holds
 // them beside the accumulators of the tile before, added in the epilogue.  Past
-// 32 k-tiles four take a quarter each: M 800 x N 1024 x K 4096 errs by 7.9e-7 with
+// 32 k-tiles four take a quarter each (outputs through TMA boxes; the others have
+// fewer splits than they had): M 800 x N 1024 x K 4096 errs by 7.9e-7 with
 // four, 3.7e-7 with eight, which add 1.6 to its 14.8 us.  A step's projections,
 // whose operands are bf16 activations, take two halves where 128-token tiles
 // leave half the SMs idle, as a split of those would (800 tokens: 0.3 us per
@@ -1406,7 +1422,7 @@ int sum_accumulators(const GemmArgs& g, bool bf16_exchange, int kb_per_item, uin
   if (bf16_exchange || g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16)) return 1;
   const int fit = std::max(1, 512 / (int)acc_cols / (two_items ? 2 : 1));
   const long tiles = (long)((g.N + TC_BM - 1) / TC_BM) * ((g.M + 127) / 128);
-  return std::min({kb_per_item, fit, g.xbf16 ? (tiles * 2 <= num_sms ? 2 : 1) : kb_per_item > 32 ? 4 : fit});
+  return std::min({kb_per_item, fit, g.xbf16 ? (tiles * 2 <= num_sms ? 2 : 1) : kb_per_item > 32 && out_aligned(g) ? 4 : fit});
 }
 
 // Sizes of a launch: the operand ring, TMEM and the shared memory around them.
@@ -1416,13 +1432,6 @@ struct TcLayout {
   uint32_t acc_cols = 32, ncols = 0, box_bytes = 0, stg_off = 0, xch_off = 0, rcv_off = 0, bar_off = 0, set_bytes = 0;
   size_t ring = 0, smem = 0;   // smem 0: no such launch
 };
-
-bool out_is_bf16(const GemmArgs& g) { return g.epi == EPI_GEGLU || (g.epi != EPI_ADD_F32 && g.out_dt == DT_BF16); }
-
-// outputs through TMA boxes when the output rows are 16-byte aligned
-bool out_aligned(const GemmArgs& g) {
-  return ((uintptr_t)g.out & 15) == 0 && ((size_t)g.ldo * (out_is_bf16(g) ? 2 : 4)) % 16 == 0;
-}
 
 // Two-SM launch with token tiles of bn (a multiple of 32 in [64, 256]).
 TcLayout pair_layout(const GemmArgs& g, int bn) {
@@ -1484,7 +1493,7 @@ TcLayout one_layout(const GemmArgs& g, const TcPlan& plan, int num_sms) {
   l.reduce = splits == 1 ? RED_NONE : !dsmem ? RED_L2_CLUSTER : xbf ? RED_DSMEM : RED_DSMEM32;
   // tokens per output box; a split's slice is stored by the threads, its
   // received partials (all splits' slices of this rank) behind the ring
-  l.box_m = splits == 1 ? 16 : (cpr % 16 == 0 ? 16 : (cpr % 8 == 0 ? 8 : 4));
+  l.box_m = splits == 1 ? 16 : split_chunk(cpr);
   l.box_bytes = (uint32_t)(((size_t)l.box_m * (g.epi == EPI_GEGLU ? 64 : TC_BM) * es + 1023) / 1024 * 1024);
   const size_t stg_bytes = dsmem ? rcv_bytes : tma_out ? 2 * (size_t)l.box_bytes : (STG_BYTES + 1023) / 1024 * 1024;
   const size_t xch_bytes = (splits == 1 && tma_out && g.epi == EPI_GEGLU) ? (XCH_BYTES + 1023) / 1024 * 1024 : 0;
