@@ -1307,8 +1307,8 @@ TcClusters g_max_clusters = {{0, 0, 0, 0}};
 // Whether a step's launch (xbf16) exchanges its splits' shares in bf16: where
 // tiles of 64 (M <= 64) or 128 tokens leave so many SMs idle that a split's slice
 // is at most 32 tokens, and that many splits have a k-tile each.  Elsewhere
-// shares stay fp32, whatever the plan: a share in bf16 costs a sum 2^-9 of its
-// size, and the estimated time is no reason to take that where it was not taken
+// shares stay fp32, whatever the plan: a share in bf16 costs a sum up to 2^-8 of
+// the share, and the estimated time is no reason to take that where it was not taken
 // (QKV of 2560 features from 129 tokens on, O and down of 1024 from 513 on).
 bool bf16_shares(const GemmArgs& g, int num_sms) {
   const int s = g.M <= 64 ? 2 : 4;

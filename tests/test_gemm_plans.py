@@ -63,7 +63,7 @@ def test_waiting_launches_share_an_sm_only_if_tmem_holds_both(plan):
 
 
 def test_shares_in_bf16_only_where_splits_are_many(plan):
-    """A share rounded to bf16 loses 2^-9 of its size: only a step's launch does
+    """A share rounded to bf16 loses up to 2^-8 of its size: only a step's launch does
     that, and only where 64- or 128-token tiles split into slices of at most 32
     tokens on the SMs that there are."""
     def check(m, n, k, epi, bf, xb, al):

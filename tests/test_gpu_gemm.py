@@ -128,6 +128,28 @@ def test_gemm_geglu_bf16(handles, M, N, K, with_bias):
     np.testing.assert_allclose(got, ref, rtol=1e-2, atol=1e-2 * (np.abs(ref).max() + 1e-3))
 
 
+# GeGLU of given gates (one product each, exact in fp32) on each kind of epilogue:
+# one item per CTA, split slices, SM pairs and an unaligned output.  Bound: bf16's 8
+# significant bits (2^-8 of the result) and tanh.approx's 2^-11 of tanh, times g / 2
+# (the larger one for gates below -1.5, where 1 + tanh cancels).
+@pytest.mark.parametrize("M,K,ld", [(4, 64, 1024), (50, 1024, 1024), (3200, 64, 1024), (50, 1024, 1028)])
+def test_gemm_geglu_of_negative_gates(handles, M, K, ld):
+    from paper_2609_34170_gb300 import _binding as B
+    N = 2048
+    gates = torch.linspace(-5, 5, N // 2, device="cuda").bfloat16()
+    X = torch.zeros((M, K), device="cuda", dtype=torch.bfloat16)
+    X[:, 0] = 1
+    W = torch.zeros((N // 128, 2, 64, K), device="cuda", dtype=torch.bfloat16)
+    W[:, 0, :, 0], W[:, 1, :, 0] = gates.view(-1, 64), 1
+    out = torch.zeros((M, ld), device="cuda", dtype=torch.bfloat16)
+    s = B.load().ravel_gemm(handles["bf16"], X.data_ptr(), M, K, K, W.data_ptr(), N, K, 3, out.data_ptr(), ld, 1, None,
+                            torch.cuda.current_stream().cuda_stream)
+    assert s == 0
+    ref = torch.nn.functional.gelu(gates.double(), approximate="tanh")
+    bound = ref.abs() * 2.0 ** -8 + gates.double().abs() * 2.0 ** -12 + 1e-6
+    assert bool(((out[:, :N // 2].double() - ref).abs() <= bound).all())
+
+
 def test_gemm_bf16_output_and_determinism(handles):
     from paper_2609_34170_gb300 import ravel_gemm
     M, N, K = 50, 1024, 4096      # split-K across the grid
