@@ -27,11 +27,10 @@
 // precision of every activation between kernels of the bf16 path), by
 // st.async straight into the owning rank's shared memory, overlaid on Q and
 // the K ring, as soon as its own PV is done and every split's last S MMA has
-// completed (a multicast tcgen05.commit on each split's "S done" barrier; a
-// cluster barrier after all MMAs where the area reaches the V ring); an
+// completed (a multicast tcgen05.commit on each split's "S done" barrier); an
 // mbarrier at the owner counts the bytes.  Where that does not apply, the splits
 // publish unnormalised fp32 partials through L2 and the cluster barrier.  The
-// producer keeps the L2 warm a few prefix chunks ahead of its loads.
+// producer asks for the rest of its split's prefix in L2 as it starts.
 //
 // Warp roles (320 threads): warp 0 TMA producer, warp 1 TMEM allocator + MMA
 // issuer, warps 2..9 softmax / epilogue (warp w owns TMEM lanes 32*(w%4)..).
@@ -66,14 +65,13 @@ constexpr uint32_t AT_VBLK = 64 * 128;        // bytes of one 64-wide head-dim b
 constexpr uint32_t kPollLimit = 1u << 25;
 
 struct AtParams {
-  int B, H, F, Hq, Hkv, G, hd, hdp;   // hdp: head dim rounded up to 16 (MMA N of P V)
+  int H, F, Hkv, G, hd, hdp;   // hdp: head dim rounded up to 16 (MMA N of P V)
   int TQ, q_tiles;
   int Pmax, n_kv, splits;
   int layer, Bmax, mask_mode;
   int nblk, k_slots, v_slots;         // head-dim blocks of 64; K units and V halves in their rings
-  int xch;                            // splits > 1: partials through L2 (0) or shared memory, sent once every
-                                      // split's MMAs are done (1: cluster barrier) or once every split's S
-                                      // MMAs are done (2: the receive area lies in Q and the K ring)
+  int xch;                            // splits > 1: partials through shared memory (1; the receive area lies in
+                                      // Q and the K ring) or L2 (0)
   const int* ctx_state;
   const bf16 *ck[2], *cv[2];          // context slots [L][Bmax][Hkv][Pmax][hd]
   bf16* out;
@@ -205,7 +203,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
   uint64_t* p_full = s_full + 2;
   uint64_t* pv_done = p_full + 2;   // [2]: PV of chunk i completes pv_done[i & 1]
   uint64_t* rcv_bar = pv_done + 2;  // xch: every split's share of this rank has arrived
-  uint64_t* sdone = rcv_bar + 1;    // xch 2: every split's last S MMA has completed (one arrival each)
+  uint64_t* sdone = rcv_bar + 1;    // xch: every split's last S MMA has completed (one arrival each)
   uint32_t* tmem_slot = (uint32_t*)(sdone + 1);
   float* xm = (float*)((uint8_t*)bars + 512);   // [2][128] row maxima, then sums, of the two halves
   int* flags = (int*)(tmem_slot + 1);   // [0] abort, [1] K units issued, [2] consumed, [3] V halves issued, [4] consumed
@@ -265,8 +263,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (p.xch) mbar_expect_tx(rcv_bar, (uint32_t)(p.splits * vrows * (2 * cps + 8)));
   }
-  // (xch 2) every split's barriers must exist before a peer targets them
-  if (p.xch == 2) cluster_sync();
+  // (xch) every split's barriers must exist before a peer targets them
+  if (p.xch) cluster_sync();
   const CUtensorMap* pk = slot ? &maps.pk1 : &maps.pk0;
   const CUtensorMap* pv = slot ? &maps.pv1 : &maps.pv0;
   uint32_t el = 0;   // the issuing lane of warps 0 (TMA) and 1 (MMA)
@@ -401,9 +399,6 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       flags[3] = nv;
     }
     __syncwarp();
-    // xch 1: one arrival per thread on the cluster barrier that opens the
-    // exchange (the softmax warps arrive once their last PV is complete)
-    if (p.xch == 1) cluster_arrive_release();
   } else if (warp == 1) {
     el = elect_one();
     const uint32_t idesc_s = idesc_bf16(AT_BM, AT_BKV);
@@ -417,7 +412,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
     int ns = 0, i = 0;   // next S, next PV
     int uk = 0, uv = 0;  // K units and V halves consumed
     bool sdone_sent = false;
-    // xch 2: every split learns when this split's last S has completed
+    // xch: every split learns when this split's last S has completed
     // (its Q and K ring may then receive the partials of the merge)
     const uint16_t smask = (uint16_t)((1u << p.splits) - 1u);
     phk = phv = 0;
@@ -446,7 +441,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
         if (!ok) break;
         umma_commit(&s_full[ns & 1], el);
         ++ns;
-        if (p.xch == 2 && ns == n) {
+        if (p.xch && ns == n) {
           umma_commit_mc(sdone, smask, el);
           sdone_sent = true;
         }
@@ -484,14 +479,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       if (spins > kPollLimit) ok = false;
     }
     // (no chunk, or an abort: arrive all the same, once earlier MMAs are done)
-    if (p.xch == 2 && !sdone_sent) umma_commit_mc(sdone, smask, el);
+    if (p.xch && !sdone_sent) umma_commit_mc(sdone, smask, el);
     if (lane == 0) {
       if (!ok) flags[0] = 1;
       flags[2] = uk;   // K units whose arrival was consumed
       flags[4] = uv;   // V halves whose arrival was consumed
     }
     __syncwarp();
-    if (p.xch == 1) cluster_arrive_release();
   } else {
     // softmax / epilogue: two threads per query row r (TMEM lane r), half hf = 0, 1
     const int q4 = warp & 3, hf = warp >= 6 ? 1 : 0;
@@ -600,13 +594,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) attn_tc_kernel(const __grid_con
       pair_bar();
       l = xm[r] + xm[128 + r];
     }
-    if (p.xch == 1) {
-      // past this barrier every split of the cluster has finished its MMAs
-      // (its Q and rings may be overwritten) and armed its receive barrier;
-      // every thread arrives exactly once, whatever happened before
-      cluster_arrive_release();
-      cluster_wait_acquire();
-    } else if (p.xch == 2) {
+    if (p.xch) {
       // every split's S MMAs are done: their Q and K rings, where the
       // partials land, are no longer read
       const bool okd = __all_sync(0xffffffffu, mbar_wait_cluster(sdone, 0));
@@ -987,7 +975,7 @@ bool attention_tc_supported(int hd, int G) { return hd % 8 == 0 && hd <= 256 && 
 cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   if (!g_enc) return cudaErrorInitializationError;
   AtParams p{};
-  p.B = a.B; p.H = a.H; p.F = a.F; p.Hq = a.Hq; p.Hkv = a.Hkv; p.G = a.Hq / a.Hkv; p.hd = a.hd;
+  p.H = a.H; p.F = a.F; p.Hkv = a.Hkv; p.G = a.Hq / a.Hkv; p.hd = a.hd;
   p.hdp = (a.hd + 15) / 16 * 16;
   p.Pmax = a.Pmax;
   p.n_kv = (a.H + a.F + AT_BKV - 1) / AT_BKV;
@@ -1006,7 +994,7 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   p.q_tiles = plan.q_tiles;
   p.TQ = plan.TQ;
   p.splits = splits;
-  p.xch = plan.smem_merge ? 2 : 0;
+  p.xch = plan.smem_merge ? 1 : 0;
   p.ws_o = a.ws;
   p.ws_ml = a.ws + (size_t)splits * nctas * AT_BM * p.hdp;
   p.k_slots = plan.k_slots;
@@ -1034,7 +1022,6 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   dim3 grid(p.q_tiles, a.B * a.Hkv, splits);
   e = launch_kernel_cluster(attn_tc_kernel, grid, dim3(AT_THREADS), plan.smem, st, dim3(1, 1, splits), m, p);
-  if (a.n_launched) ++*a.n_launched;
   return e;
 }
 

@@ -31,19 +31,6 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Sum over the whole block (blockDim.x a multiple of 32, at most 1024); every
-// thread gets the result.  `red` is 32 floats of shared memory.
-__device__ __forceinline__ float block_sum(float v, float* red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  float t = (l < nw) ? red[l] : 0.f;
-  return warp_sum(t);
-}
-
 // err: the word of an ErrorWord.  The kernel that raises an error also writes it
 // to the host's mirror, so that a call without one copies nothing back (a
 // 4-byte copy per call cost a batch-1 step 5 of 608 us, a tiny fp32 one 7 of

@@ -74,9 +74,8 @@ enum { EK_F32 = 0, EK_BF16 = 1, EK_ADD = 2, EK_GEGLU = 3, EK_GENERIC = 4, EK_SLI
 
 
 struct TcParams {
-  int M, N, K;
+  int M, N;
   int bn, stages, splits, num_kb;
-  int reduce;           // how the splits of a tile are combined (splits > 1)
   uint32_t ncols;       // TMEM columns of the launch
   uint32_t acc_cols;    // TMEM columns of one accumulator
   int accs;             // accumulators that an item's K range is cut into, at most one per k-tile (sum_accumulators)
@@ -88,7 +87,6 @@ struct TcParams {
   const float* bias;
   float* ws;
   int* err;
-  int tma_out;          // outputs leave through TMA boxes
   int oneshot;          // split launch whose whole K range fits the ring: tmW / tmX are 3-D maps
                         // (64, rows, K / 64) and one box each brings all of its k-tiles
   int box_m;            // tokens per epilogue chunk (= rows of a TMA output box)
@@ -466,9 +464,9 @@ __device__ __forceinline__ void store_slice(const TcParams& p, int tile_n, int m
   }
 }
 
-// RED = p.reduce and EK = the epilogue kind, fixed per instantiation so that
-// each reduction mode gets its own register allocation and each launch only
-// the code it runs.
+// RED, how the splits of a tile are combined, and EK, the epilogue kind, are
+// fixed per instantiation, so that each reduction mode gets its own register
+// allocation and each launch only the code it runs.
 template <int RED, int EK>
 __global__ void __launch_bounds__(TC_THREADS, 2)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
@@ -962,7 +960,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 // shared memory and count the bytes on the even CTA's `full` barrier; the
 // MMA completion is multicast to both CTAs' `empty` / `acc_full` barriers;
 // both CTAs run the epilogue of their own rows, whose drained accumulators
-// the even CTA's `acc_empty` counts (256 arrivals).
+// the even CTA's `acc_empty` counts (512 arrivals, 256 epilogue threads each).
 template <int EK>
 __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
     tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
@@ -1165,7 +1163,7 @@ __global__ void __launch_bounds__(TC_PAIR_THREADS, 1)
       const int m_base = tm * BN;
       const int n = tile_n * TC_BM + r;
       const float brow = (p.bias && n < p.N) ? p.bias[n] : 0.f;
-      // 32-token chunks (BN is a multiple of 32, at least 128): this set's
+      // 32-token chunks (BN is a multiple of 32, at least 64): this set's
       // every other chunk, the next one's TMEM load in flight meanwhile
       uint32_t nxt[32];
       const int cf = 32 * set;
@@ -1531,9 +1529,9 @@ cudaError_t launch_gemm_pair(const GemmArgs& g, const TcWorkspace& ws, int num_s
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, l.stages, 1, num_kb, RED_NONE, l.ncols, l.acc_cols, 1, tiles_n, tiles_m,
+  TcParams p{g.M, g.N, bn, l.stages, 1, num_kb, l.ncols, l.acc_cols, 1, tiles_n, tiles_m,
              num_tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
-             1, 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, 0, l.bar_off, kTcTimeoutNs, 0, g.skip};
+             0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, 0, l.bar_off, kTcTimeoutNs, 0, g.skip};
   p.set_bytes = l.set_bytes;
   const int npairs = std::min(num_tiles, slots);
   return launch_kernel_cluster(tc_pair_kernel(ek), dim3(2 * npairs), dim3(TC_PAIR_THREADS), l.smem, st, dim3(2, 1, 1),
@@ -1612,9 +1610,9 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const TcWorkspace& ws, int num_sms
     e = encode_out(&mo, g.out, g.M, g.epi == EPI_GEGLU ? g.N / 2 : g.N, g.ldo, out_bf,
                    g.epi == EPI_GEGLU ? 64 : TC_BM, l.box_m);
   if (e != cudaSuccess) return e;
-  TcParams p{g.M, g.N, g.K, bn, l.stages, splits, num_kb, l.reduce, l.ncols, l.acc_cols, l.accs, tiles_n,
+  TcParams p{g.M, g.N, bn, l.stages, splits, num_kb, l.ncols, l.acc_cols, l.accs, tiles_n,
              tiles_m, tiles, (int)g.epi, g.out_dt == DT_BF16 ? 1 : 0, g.out, g.ldo, g.bias, ws.ws, ws.err,
-             tma_out ? 1 : 0, oneshot ? 1 : 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, l.rcv_off, l.bar_off,
+             oneshot ? 1 : 0, l.box_m, l.box_bytes, l.stg_off, l.xch_off, l.rcv_off, l.bar_off,
              kTcTimeoutNs, 0, g.skip};
   // fault injection (tests): a launch without a cluster may be told to wait
   // for an arrival that never comes, with a short limit

@@ -147,7 +147,7 @@ cudaError_t launch_in_proj(const float* buf, int BH, int A, int D, const float* 
 // adaRMSNorm into rn.Y (action rows and, with rn.fop, FOP rows).
 cudaError_t launch_in_proj_norm(const float* buf, int A, int D, const float* in_w, const float* in_b, float* x,
                                 const float* state, const float* rel_mask, const float* slot_times, const RowNorm& rn,
-                                Dtype dt, cudaStream_t st);
+                                Dtype dt, int num_sms, cudaStream_t st);
 
 // An empty kernel (one thread): the launch overhead of a timed eager replay.
 cudaError_t launch_noop(cudaStream_t st);
@@ -180,7 +180,6 @@ struct AttnTcArgs {
   void* out; int ld_out;
   float* ws; size_t ws_bytes;
   int* err; int num_sms;
-  int* n_launched = nullptr;   // optional: incremented by the number of kernels launched (1 or 2)
 };
 cudaError_t init_attention_tc();
 bool attention_tc_supported(int hd, int G);

@@ -808,7 +808,7 @@ static cudaError_t launch_in_proj_norm_t(const float* buf, int A, int D, const f
 
 cudaError_t launch_in_proj_norm(const float* buf, int A, int D, const float* in_w, const float* in_b, float* x,
                                 const float* state, const float* rel_mask, const float* slot_times, const RowNorm& rn,
-                                Dtype dt, cudaStream_t st) {
+                                Dtype dt, int num_sms, cudaStream_t st) {
   const int rows = rn.B * rn.H + (rn.fop ? rn.B * rn.F : 0);
   if (D > 4096 || D % 4) return cudaErrorInvalidValue;
   if (rows <= 0) return cudaSuccess;
@@ -819,8 +819,8 @@ cudaError_t launch_in_proj_norm(const float* buf, int A, int D, const float* in_
   if (D > 1024) RAVEL_IPN(1, 2);
   // one slot per block while they leave SMs idle, then four, or eight (whose
   // actions must fit the block's shared memory)
-  if (rows <= 2 * 152 || A > 1024) RAVEL_IPN(1, 1);
-  if (rows <= 8 * 152) RAVEL_IPN(4, 1);
+  if (rows <= 2 * num_sms || A > 1024) RAVEL_IPN(1, 1);
+  if (rows <= 8 * num_sms) RAVEL_IPN(4, 1);
   RAVEL_IPN(8, 1);
 #undef RAVEL_IPN
 }

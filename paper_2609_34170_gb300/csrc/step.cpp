@@ -362,7 +362,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
                       H + FF0};
     rn0.t_stride = n_stride;
     RUN(KK_IN_PROJ, launch_in_proj_norm(io.buffer, A, D, p.in_w, p.in_b, p.x, io.state, p.rel_mask, io.slot_times,
-                                        rn0, dt, st));
+                                        rn0, dt, p.num_sms, st));
   } else {
     RUN(KK_IN_PROJ, launch_in_proj(io.buffer, B * H, A, D, p.in_w, p.in_b, p.x, st, io.state, p.rel_mask,
                                    io.slot_times, H, t_stride));
@@ -386,10 +386,7 @@ cudaError_t enqueue_step(const StepPlan& p, int B, const StepIO& io, cudaStream_
       AttnTcArgs at{p.QKV, p.nqkv, {p.ctx_k[0], p.ctx_k[1]}, {p.ctx_v[0], p.ctx_v[1]}, L, l,
                     c.max_batch, c.max_prefix, p.ctx_state, B, H, FF, c.n_q_heads, c.n_kv_heads, c.head_dim,
                     c.mask_mode, p.O, p.qdim, p.attn_ws, p.attn_ws_bytes, p.err, p.num_sms};
-      int launched = 0;
-      at.n_launched = &launched;
       RUN(KK_ATTENTION, launch_attention_tc(at, st));
-      nk += launched - 1;   // RUN counted one launch; a split attention adds its combine kernel
     } else {
       RUN(KK_GEMM_QKV, gemm(p.Y, D, wqkv, BY, p.nqkv, D, EPI_STORE, p.QKV, p.nqkv, dt, nullptr));
       AttnArgs at{p.QKV, p.nqkv, p.ctx_k[0], p.ctx_k[1], p.ctx_v[0], p.ctx_v[1], p.ctx_state, l, c.max_batch,
