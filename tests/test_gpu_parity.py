@@ -240,3 +240,19 @@ def test_head_tail_many_rows(slots, width, actions):
     assert s.kernel_count() == few.kernel_count()
     s.close()
     few.close()
+
+
+# Token counts where a step's projections exchange fp32 shares or sum two halves
+# (QKV at 129 to 192 tokens; O and down at 513 to 576 and at 577 to 1152), and
+# attentions whose few splits merge in fp32 through L2 or whose one prefix chunk
+# is not split.
+@pytest.mark.parametrize("batch,slots,heads,kv,hd,prefix", [(2, 50, 8, 1, 256, 300), (11, 50, 8, 1, 256, 100),
+                                                            (16, 50, 8, 1, 256, 64), (19, 8, 8, 2, 80, 384),
+                                                            (2, 30, 16, 4, 64, 2048), (3, 30, 16, 4, 64, 64)])
+def test_exchange_in_fp32(batch, slots, heads, kv, hd, prefix):
+    cfg = synth.ExpertConfig(layers=1, width=1024, n_q_heads=heads, n_kv_heads=kv, head_dim=hd, mlp_dim=4096,
+                             slots=slots, action_dim=7, prefix=prefix, fop_tokens=16, batch=batch, dtype="bf16")
+    case = Case(cfg)
+    s = gpu_session(case)
+    check_step(case, s, robots=[0, batch - 1], label=f"{batch * slots} tokens")
+    s.close()
