@@ -299,9 +299,10 @@ ravel_status ravel_gemm(ravel_t* r, const void* X, int M, int K, int lda, const 
  * (X and W bf16, 16-byte aligned, K, lda, ldw multiples of 8), on the
  * current CUDA device.  It calls no cudaMalloc / cudaFree: its split-K
  * scratch is one fixed device array inside the library (8 MiB of partial
- * sums), held by every GPU that loads the library until the process exits.  The split plan is chosen to fit that array.  M, N, K
- * above RAVEL_NOALLOC_MAX_M / _N / _K return RAVEL_ESHAPE; bad pointers or
- * modes RAVEL_EINVAL.  The first call on a device resolves the array's device
+ * sums), held by every GPU that loads the library until the process exits.
+ * The split plan is chosen to fit that array.  M, N, K above
+ * RAVEL_NOALLOC_MAX_M / _N / _K return RAVEL_ESHAPE; bad pointers or modes
+ * RAVEL_EINVAL.  The first call on a device resolves the array's device
  * address (and the kernel set-up) for that device; make that first call
  * before any stream capture (a first call on a capturing stream returns
  * RAVEL_EINVAL and does nothing).  Every call shares the array, so calls

@@ -1336,12 +1336,12 @@ struct TcPlan {
 // rule before it was 19 % slower (M 50 x N 1024 x K 2048: 16 splits, 5.9 us;
 // now 4.1 us; M 240 x 1024 x 4096: 12.4, now 7.3 us).  Inside a step (xbf16)
 // the neighbours of a launch are other kernels: there the exchange of bf16
-// shares weighs less, an unsplit launch 0.3 more (its code is another
-// binary's than the split launches'), and split CTAs past half the SMs, which
-// the next kernel could have started on, up to 0.7 more.  Whole steps at 1 to
-// 64 robots, each projection's width and splits varied in turn: the rule is
-// 0 to 3.5 % of the step away from the best combination (batch 1 at it: 652
-// us, 685 with the chain's terms alone).
+// shares, where bf16_shares allows it, weighs less, an unsplit launch 0.3 more
+// (its code is another binary's than the split launches'), and split CTAs past
+// half the SMs, which the next kernel could have started on, up to 0.7 more.
+// Whole steps at 1 to 64 robots, each projection's width and splits varied in
+// turn: the rule is 0 to 3.5 % of the step away from the best combination
+// (batch 1 at it: 652 us, 685 with the chain's terms alone).
 TcPlan plan_gemm(const GemmArgs& g, bool dsmem, size_t ws_bytes, bool pairs, int num_sms, const TcClusters& clusters) {
   const int M = g.M, N = g.N, K = g.K;
   const bool geglu = g.epi == EPI_GEGLU, xbf16 = g.xbf16 != 0, shares_bf16 = bf16_shares(g, num_sms);

@@ -209,7 +209,7 @@ def test_fp32_geglu_rows(batch, slots, width, mlp):
 
 
 # The fused head and tail: action widths at the edges of a noise group and of its
-# 32 outputs, one and several passes over the row, few slots and the most rows.
+# 32 outputs, one and several passes over the row, a slot per CTA: few and many.
 @pytest.mark.parametrize("batch,slots", [(1, 2), (5, 9), (1, 152)])
 @pytest.mark.parametrize("width,actions", [(64, 1), (1024, 20), (1032, 32), (2056, 5)])
 def test_head_tail_edges(batch, slots, width, actions):
